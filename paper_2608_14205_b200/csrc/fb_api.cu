@@ -50,7 +50,7 @@ struct fb_ctx {
   int max_pairs = 0;
   int pair_limit = 0;
   int stage_limit = 0;                 // diagnostic: pipeline stages at most (0 = as many as fit)
-  int dispatch_blocks_max = 296;       // resident blocks of the dispatch-index kernel (2 per SM)
+  int n_sm = 148;                      // SMs of the device
   // k-range split of the one-tile pair kernel: block pairs that fit on the GPU at once, the
   // partial tiles and their flags (one slot per helper item; set by the helper, put back by the
   // owner), and the caller's switch / tuning value
@@ -64,8 +64,7 @@ struct fb_ctx {
   uint32_t* counts_scratch = nullptr;   // [256], zero between calls
   uint32_t* ticket = nullptr;           // [1],   zero between calls
   int32_t* status = nullptr;            // [1]
-  uint32_t* tile_counts = nullptr;      // [max_tiles][E]
-  uint32_t* super_counts = nullptr;     // [ceil(max_tiles / 32)][E]
+  uint8_t* slice_counts = nullptr;      // [max_tiles][slice_row_bytes(E)]: per-tile histograms for the dispatch index
   // descriptor cache
   MapEntry x_maps[kMapCache];
   MapEntry w_maps[kMapCache];
@@ -270,7 +269,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.topk_ids = topk_ids;
   p.topk_w = topk_w;
   p.logits = logits;
-  p.tile_counts = ctx->tile_counts;
+  p.slice_counts = ctx->slice_counts;
   p.stamps = ctx->stamps;
   p.probe = probe;
   if (plan) p.plan = *plan;
@@ -395,16 +394,9 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, const int32_t* expert_to
   dp.T = T; dp.k = c.k; dp.E = c.E; dp.R = c.R;
   dp.num_tiles = (T + fb::kDispatchTile - 1) / fb::kDispatchTile;
   dp.topk_ids = topk_ids;
-  dp.tile_counts = ctx->tile_counts;
-  dp.super_counts = nullptr;
-  if (dp.num_tiles > 4 * fb::kSuperTiles) {                 // beyond 16k tokens the two-level sums pay off
-    const int n_super = (dp.num_tiles + fb::kSuperTiles - 1) / fb::kSuperTiles;
-    fb::fb_tile_sums_kernel<<<n_super, FB_MAX_EXPERTS, 0, stream>>>(ctx->tile_counts, ctx->super_counts,
-                                                                     dp.num_tiles, c.E);
-    ++ctx->launches;
-    if (cudaGetLastError() != cudaSuccess) return FB_ERR_CUDA;
-    dp.super_counts = ctx->super_counts;
-  }
+  dp.slices_per_tile = 1;
+  dp.num_slices = dp.num_tiles;
+  dp.slice_counts = ctx->slice_counts;
   dp.expert_to_slot = expert_to_slot;
   dp.slot_offsets = slot_offsets;
   dp.rank_offsets = rank_offsets;
@@ -412,11 +404,24 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, const int32_t* expert_to
   dp.inv_perm = inv_perm;
   dp.rank_load = rank_load;
   dp.status = ctx->status;
-  // at most two blocks per SM are resident (1024 threads each): more tiles than that are walked in runs
-  const int dispatch_blocks = dp.num_tiles < ctx->dispatch_blocks_max ? dp.num_tiles : ctx->dispatch_blocks_max;
-  fb::fb_dispatch_kernel<<<dispatch_blocks, fb::kDispatchThreads, 0, stream>>>(dp);
+  // one block per SM at most: more tiles than that are walked in runs (every block reads the whole
+  // histogram table once, so more blocks would only read it more often)
+  const int dispatch_blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;
+  // May start under the router kernel's last blocks; it waits for that kernel's completion before
+  // it reads anything.
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(static_cast<unsigned>(dispatch_blocks), 1, 1);
+  cfg.blockDim = dim3(fb::kDispatchThreads, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, fb::fb_dispatch_kernel, dp);
   ++ctx->launches;
-  return cudaGetLastError() == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
 fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* counts, cudaStream_t stream) {
@@ -465,7 +470,7 @@ static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
     ctx->smem_bytes[pair] = dyn + 1024;
   }
   ctx->max_tiles = (cfg.T_max + fb::kTileM - 1) / fb::kTileM;
-  ctx->dispatch_blocks_max = 2 * prop.multiProcessorCount;
+  ctx->n_sm = prop.multiProcessorCount;
   return FB_OK;
 }
 
@@ -612,9 +617,7 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
   }
   ok = ok && dev_alloc(&ctx->counts_scratch, FB_MAX_EXPERTS) && dev_alloc(&ctx->ticket, 1) &&
        dev_alloc(&ctx->status, 1) &&
-       dev_alloc(&ctx->tile_counts, static_cast<size_t>(ctx->max_tiles) * cfg->E) &&
-       dev_alloc(&ctx->super_counts,
-                 static_cast<size_t>((ctx->max_tiles + fb::kSuperTiles - 1) / fb::kSuperTiles) * cfg->E);
+       dev_alloc(&ctx->slice_counts, static_cast<size_t>(ctx->max_tiles) * fb::slice_row_bytes(cfg->E));
   ok = ok && cudaMemset(ctx->counts_scratch, 0, FB_MAX_EXPERTS * sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->ticket, 0, sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess;
@@ -628,7 +631,7 @@ fb_status fb_destroy(fb_ctx* ctx) {
   DeviceGuard guard(ctx->device);
   cudaDeviceSynchronize();
   void* ptrs[] = {ctx->split_partial, ctx->split_flags,
-                  ctx->counts_scratch, ctx->ticket, ctx->status, ctx->tile_counts, ctx->super_counts, ctx->st_hprev, ctx->st_H,
+                  ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->st_hprev, ctx->st_H,
                   ctx->st_pi, ctx->st_pi_out, ctx->st_counts, ctx->st_swaps, ctx->st_nswaps, ctx->st_load_before,
                   ctx->st_load_after, ctx->st_ids, ctx->st_w, ctx->st_slot_offsets, ctx->st_rank_offsets,
                   ctx->st_perm, ctx->st_inv_perm, ctx->st_rank_load};
@@ -1083,7 +1086,7 @@ fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int
   const long long n = static_cast<long long>(T_local) * ctx->cfg.k;
   long long blocks = (n + fb::kGlobalizeThreads - 1) / fb::kGlobalizeThreads;
   if (blocks < 1) blocks = 1;
-  if (blocks > 2 * ctx->dispatch_blocks_max) blocks = 2 * ctx->dispatch_blocks_max;
+  if (blocks > 4 * ctx->n_sm) blocks = 4 * ctx->n_sm;
   fb::fb_dispatch_globalize_kernel<<<static_cast<unsigned>(blocks), fb::kGlobalizeThreads, 0,
                                      static_cast<cudaStream_t>(stream_)>>>(gp);
   ++ctx->launches;
@@ -1285,7 +1288,7 @@ extern "C" fb_status fb_predict_load_static(const fb_config* cfg, int device, co
   ctx.counts_scratch = st.scratch;
   ctx.ticket = st.scratch + FB_STATIC_MAX_EXPERTS;
   ctx.status = status_word ? status_word : reinterpret_cast<int32_t*>(st.scratch + FB_STATIC_MAX_EXPERTS + 1);
-  ctx.tile_counts = nullptr;                             // unused by the prediction pass
+  ctx.slice_counts = nullptr;                            // unused by the prediction pass
   if (T == 0)
     return cudaMemsetAsync(counts, 0, cfg->E * sizeof(uint32_t), stream) == cudaSuccess ? FB_OK : FB_ERR_CUDA;
   // The array keeps whatever the previous call (possibly one that was cut short) left in it.

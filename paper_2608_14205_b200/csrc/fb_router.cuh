@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fb_dispatch.cuh"
 #include "fb_planner.cuh"
 #include "fb_ptx.cuh"
 
@@ -97,7 +98,7 @@ struct RouterParams {
   int32_t* topk_ids;                 // [T][k] or nullptr
   float* topk_w;                     // [T][k] or nullptr
   float* logits;                     // [T][E] or nullptr
-  uint32_t* tile_counts;             // [tiles][E]    (dispatch mode)
+  uint8_t* slice_counts;             // [tiles][slice_row_bytes(E)] (dispatch mode)
   unsigned long long* stamps;        // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
   int32_t probe;                     // measurement aid: 1 = operands are loaded but no MMA is issued and nothing
                                      // follows the main loop; 2 = with the MMAs, still nothing after them
@@ -199,7 +200,7 @@ struct RouterShared {
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS + 32];     // + 32: a partial last chunk is read in full
   alignas(16) float select_bias[FB_MAX_EXPERTS + 32];
-  uint32_t hist[FB_MAX_EXPERTS];
+  alignas(16) uint32_t hist[FB_MAX_EXPERTS];
   uint32_t cand_count[kTileM];               // fast selection path: candidates claimed per row
   PlanShared plan;
 };
@@ -388,6 +389,17 @@ __device__ __forceinline__ void publish_counts(Shared& sh, const RouterParams& p
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
       plan_write_placement(p.plan, sh.plan, et, kEpilogueThreads);
     }
+  }
+}
+
+// A tile's histogram as one table row of the dispatch index: one byte per expert (a count is at most
+// kTileM), four per store.  Bins from E up to the row's end are zero.
+__device__ __forceinline__ void write_slice_counts(uint8_t* table, int slice, int E, const uint32_t* hist, int et) {
+  const int row_bytes = slice_row_bytes(E);
+  for (int w = et; w < row_bytes / 4; w += kEpilogueThreads) {
+    const uint4 h = *reinterpret_cast<const uint4*>(hist + 4 * w);
+    reinterpret_cast<uint32_t*>(table + static_cast<size_t>(slice) * row_bytes)[w] =
+        h.x | h.y << 8 | h.z << 16 | h.w << 24;
   }
 }
 
@@ -1214,8 +1226,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       }
       if (mode == kModeDispatch) {
         if (static_cast<long long>(tile) * kTileM < p.T)       // the padding block of an odd pair owns no tile
-          for (int e = et; e < E; e += kEpilogueThreads)
-            p.tile_counts[static_cast<size_t>(tile) * E + e] = sh.hist[e];
+          write_slice_counts(p.slice_counts, tile, E, sh.hist, et);
       } else if (p.probe == 0) {
         publish_counts(sh, p, et, warp, lane, mode == kModePredictPlan && p.fuse_planner != 0);
       }

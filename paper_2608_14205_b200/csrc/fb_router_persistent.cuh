@@ -44,7 +44,7 @@ struct PersistShared {
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];
-  uint32_t hist[FB_MAX_EXPERTS];
+  alignas(16) uint32_t hist[FB_MAX_EXPERTS];
   uint32_t cand_count[kTileM];
   PlanShared plan;
 };
@@ -458,10 +458,9 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       if (et == 0) sh.any_overflow = 0;                       // everyone has read it
       if (mode == kModeDispatch) {
         const bool owns = static_cast<long long>(tile) * kTileM < p.T;   // the padding block of an odd pair owns no tile
-        for (int e = et; e < E; e += kEpilogueThreads) {
-          if (owns) p.tile_counts[static_cast<size_t>(tile) * E + e] = sh.hist[e];
-          sh.hist[e] = 0;
-        }
+        if (owns) write_slice_counts(p.slice_counts, tile, E, sh.hist, et);
+        named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+        for (int e = et; e < E; e += kEpilogueThreads) sh.hist[e] = 0;
       } else if (pt + pair_stride >= pairs_per_pass) {
         // The histogram keeps accumulating over this block's tiles of the pass and is published
         // once, after the last of them (one fence and one ticket per block, not per tile).

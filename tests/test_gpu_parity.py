@@ -709,6 +709,20 @@ def test_dispatch_index_with_several_tiles_per_block():
     assert rep["early_mismatch_unflagged"] == 0 and rep["final_mismatch_unflagged"] == 0
 
 
+@pytest.mark.parametrize("E,k,R,T", [
+    (8, 2, 4, 128 * 148 + 1),       # one 16-expert unit per row of the histogram table; runs of two tiles, the last of one row
+    (40, 3, 5, 128 * 149),          # three units: a count that does not divide a warp
+    (160, 6, 8, 128 * 148 * 5 - 3), # ten units; runs of five tiles: a batch of four and a single tile
+    (256, 8, 64, 128 * 148 * 4),    # sixteen units, full batches
+    (96, 7, 6, 100), (256, 1, 8, 129),   # one tile per block
+])
+def test_dispatch_index_over_table_widths_and_runs_of_tiles(E, k, R, T):
+    # whole numbers only: the index is checked entry by entry against the oracle's on the GPU's own ids
+    wl = _wl(E=E, k=k, R=R, gate=0, d=64, max_swaps=3)
+    sample = None if T <= 2500 else np.sort(np.random.default_rng(3).choice(T, size=200, replace=False))
+    _run(wl, T, want_logits=False, sample=sample)
+
+
 def test_contexts_of_different_shapes_alive_together():
     # Kernel attributes (the dynamic shared-memory ceiling) belong to the kernel, not to a context:
     # a large-shape context must keep working after a small-shape one was created, and the

@@ -419,7 +419,8 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, const int32_t* expert_to
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t err = cudaLaunchKernelEx(&cfg, fb::fb_dispatch_kernel, dp);
+  const cudaError_t err = cudaLaunchKernelEx(
+      &cfg, dispatch_blocks < dp.num_tiles ? fb::fb_dispatch_kernel<true> : fb::fb_dispatch_kernel<false>, dp);
   ++ctx->launches;
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }

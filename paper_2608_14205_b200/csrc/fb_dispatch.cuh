@@ -53,21 +53,26 @@ __device__ __forceinline__ void add_bytes(uint32_t& even, uint32_t& odd, uint32_
   odd += (w >> 8) & 0x00ff00ffu;
 }
 
+// kRuns: a block walks several tiles (more tiles than SMs).  The instance for one tile per block carries
+// none of that: in a launch of a few microseconds the instructions themselves have to be fetched, and
+// the code for runs costs it 1 us (512 tokens, 8 experts: layer step 21.1 -> 20.1 us without it).
+template <bool kRuns>
 __global__ void __launch_bounds__(kDispatchThreads, 1)
 fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
+  constexpr int kBatch = kRuns ? kDispatchBatch : 1;
   __shared__ int32_t slot_of[FB_MAX_EXPERTS];
   __shared__ int32_t owner[FB_MAX_EXPERTS];
   __shared__ uint32_t gbase[FB_MAX_EXPERTS];       // position of the slot's first assignment of this batch of tiles
   __shared__ uint32_t total[FB_MAX_EXPERTS];       // assignments to this slot in all tiles; later: in this batch
   __shared__ uint32_t offs[FB_MAX_EXPERTS + 1];    // exclusive prefix of total over slots; later: of the batch's counts
-  __shared__ uint16_t ahead_of[kDispatchBatch][FB_MAX_EXPERTS];   // the batch's assignments to this slot in earlier tiles
+  __shared__ uint16_t ahead_of[kBatch][FB_MAX_EXPERTS];   // the batch's assignments to this slot in earlier tiles
   // The per-warp sums of the histogram table are read before the tile loop starts and share their
   // memory with what the loop works on.
   __shared__ union {
     uint32_t part[kDispatchWarps][2][FB_MAX_EXPERTS / 2];   // [all / earlier slices][two 16-bit counters per word]
     struct {
-      uint4 mask[kDispatchBatch][FB_MAX_EXPERTS];           // rows of the tile that go to the slot
-      uint32_t sorted[kDispatchBatch * kDispatchThreads];   // the batch's assignments in slot order: slot << 16 | tile, thread
+      uint4 mask[kBatch][FB_MAX_EXPERTS];                   // rows of the tile that go to the slot
+      uint32_t sorted[kBatch * kDispatchThreads];   // the batch's assignments in slot order: slot << 16 | tile, thread
     } b;
   } u;
   __shared__ int32_t bad;
@@ -98,9 +103,9 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   };
   pdl_wait();                                    // from here on: what the router kernel wrote
   const int my_slot_in = t < E ? p.expert_to_slot[t] : 0;
-  int ids[kDispatchBatch];
+  int ids[kBatch];
 #pragma unroll
-  for (int i = 0; i < kDispatchBatch; ++i) ids[i] = load_id(tile_begin + i);
+  for (int i = 0; i < kBatch; ++i) ids[i] = load_id(tile_begin + i);
   // ---- column sums of the histogram table, split at this block's first slice.  Thread (part, unit)
   // adds 16 experts of every P-th slice; a warp's threads of the same unit are then combined by
   // shuffles.  16-bit counters: a thread adds at most 2^16 / 2^7 / (32 / U) slices between two flushes.
@@ -182,8 +187,8 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     if (e0 < E) { total[slot_of[e0]] = sum_all0; gbase[slot_of[e0]] = sum_bef0; }
     if (e1 < E) { total[slot_of[e1]] = sum_all1; gbase[slot_of[e1]] = sum_bef1; }
   }
-  u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
   static_assert(kDispatchThreads == kDispatchBatch * FB_MAX_EXPERTS, "one mask per thread");
+  if (t < kBatch * FB_MAX_EXPERTS) u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
   __syncthreads();
   // Exclusive scan of total[] over slots into offs[], by one warp, 8 slots per lane.
   auto scan = [&]() {
@@ -203,7 +208,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   };
   auto mark_rows = [&]() {
 #pragma unroll
-    for (int i = 0; i < kDispatchBatch; ++i)
+    for (int i = 0; i < kBatch; ++i)
       if (ids[i] >= 0) {
         uint32_t* m = reinterpret_cast<uint32_t*>(&u.b.mask[i][slot_of[ids[i]]]);
         atomicOr(m + (row >> 5), 1u << (row & 31));
@@ -222,12 +227,12 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   // Up to four tiles at a time.  With more than one, their assignments are first put into slot
   // order in shared memory, so that perm is written in runs (4-byte stores to as many sectors as
   // threads took 4 us of the 18 us at 131072 tokens); a single tile has runs of a few entries only and writes directly.
-  for (int tile0 = tile_begin; tile0 < tile_end; tile0 += kDispatchBatch) {
-    const bool several = tile_end - tile0 > 1;                  // (the same for the whole block)
+  for (int tile0 = tile_begin; tile0 < tile_end; tile0 += kBatch) {
+    const bool several = kRuns && tile_end - tile0 > 1;         // (the same for the whole block)
     if (several && t < E) {
       uint32_t run = 0;
 #pragma unroll
-      for (int i = 0; i < kDispatchBatch; ++i) {
+      for (int i = 0; i < kBatch; ++i) {
         ahead_of[i][t] = static_cast<uint16_t>(run);
         const uint4 m = u.b.mask[i][t];
         run += __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
@@ -239,11 +244,11 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
       if (warp == 0) scan();
       __syncthreads();
     }
-    int next_ids[kDispatchBatch];
+    int next_ids[kBatch];
 #pragma unroll
-    for (int i = 0; i < kDispatchBatch; ++i) next_ids[i] = load_id(tile0 + kDispatchBatch + i);
+    for (int i = 0; i < kBatch; ++i) next_ids[i] = kRuns ? load_id(tile0 + kBatch + i) : -1;
 #pragma unroll
-    for (int i = 0; i < kDispatchBatch; ++i) {
+    for (int i = 0; i < kBatch; ++i) {
       if (ids[i] < 0) continue;
       const int my_slot = slot_of[ids[i]];
       const uint4 m = u.b.mask[i][my_slot];
@@ -266,13 +271,13 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
       }
       if (several) {
         const uint32_t at = offs[my_slot] + ahead;
-        if (at < kDispatchBatch * kDispatchThreads)
+        if (at < kBatch * kDispatchThreads)
           u.b.sorted[at] = static_cast<uint32_t>(my_slot) << 16 | static_cast<uint32_t>(i) << 10 | static_cast<uint32_t>(t);
       }
     }
     if (!several) break;
     __syncthreads();
-    const uint32_t count = min(offs[E], static_cast<uint32_t>(kDispatchBatch * kDispatchThreads));
+    const uint32_t count = min(offs[E], static_cast<uint32_t>(kBatch * kDispatchThreads));
     for (uint32_t at = t; at < count; at += kDispatchThreads) {
       const uint32_t v = u.b.sorted[at];
       const uint32_t slot = v >> 16;
@@ -280,12 +285,12 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
       if (pos < n_assign)
         p.perm[pos] = static_cast<int32_t>((tile0 + static_cast<int>((v >> 10) & 3u)) * kDispatchTile * k + static_cast<int>(v & 1023u));
     }
-    if (tile0 + kDispatchBatch >= tile_end) break;
-    u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
+    if (tile0 + kBatch >= tile_end) break;
+    u.b.mask[(t / FB_MAX_EXPERTS) % kBatch][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     if (t < E) gbase[t] += total[t];
 #pragma unroll
-    for (int i = 0; i < kDispatchBatch; ++i) ids[i] = next_ids[i];
+    for (int i = 0; i < kBatch; ++i) ids[i] = next_ids[i];
     mark_rows();
     __syncthreads();
   }

@@ -228,6 +228,29 @@ static RouterKernelFn persistent_kernel_fn(bool sigmoid, bool lb) {
   return lb ? fb::fb_router_persistent_kernel<false, true> : fb::fb_router_persistent_kernel<false, false>;
 }
 
+// Launch of a small kernel that may start under the end of the stream's previous kernel (it waits for
+// that kernel's completion - griddepcontrol.wait - before it touches global memory).
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), int blocks, int threads, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* counts, cudaStream_t stream) {
+  const cudaError_t err = launch_dependent(fb::fb_plan_kernel, 1, fb::kPlanThreads, stream, pp, counts, ctx->status);
+  ++ctx->launches;
+  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+}
+
 // Launch the router kernel in one of its three modes.
 // x2 is the second input of kModeLayer (the normal router input), nullptr otherwise.
 fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T, int mode,
@@ -377,11 +400,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   ++ctx->launches;
   if (persistent) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
-  if (plan_wanted && !p.fuse_planner) {
-    fb::fb_plan_kernel<<<1, fb::kPlanThreads, 0, stream>>>(*plan, counts_out, ctx->status);
-    ++ctx->launches;
-    if (cudaGetLastError() != cudaSuccess) return FB_ERR_CUDA;
-  }
+  if (plan_wanted && !p.fuse_planner) return launch_plan(ctx, *plan, counts_out, stream);
   return FB_OK;
 }
 
@@ -407,28 +426,10 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, const int32_t* expert_to
   // one block per SM at most: more tiles than that are walked in runs (every block reads the whole
   // histogram table once, so more blocks would only read it more often)
   const int dispatch_blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;
-  // May start under the router kernel's last blocks; it waits for that kernel's completion before
-  // it reads anything.
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(static_cast<unsigned>(dispatch_blocks), 1, 1);
-  cfg.blockDim = dim3(fb::kDispatchThreads, 1, 1);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t err = cudaLaunchKernelEx(
-      &cfg, dispatch_blocks < dp.num_tiles ? fb::fb_dispatch_kernel<true> : fb::fb_dispatch_kernel<false>, dp);
+  const cudaError_t err = launch_dependent(dispatch_blocks < dp.num_tiles ? fb::fb_dispatch_kernel<true> : fb::fb_dispatch_kernel<false>,
+                                           dispatch_blocks, fb::kDispatchThreads, stream, dp);
   ++ctx->launches;
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
-}
-
-fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* counts, cudaStream_t stream) {
-  fb::fb_plan_kernel<<<1, fb::kPlanThreads, 0, stream>>>(pp, counts, ctx->status);
-  ++ctx->launches;
-  return cudaGetLastError() == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
 // The device that owns a device pointer (-1 if it is not device memory).

@@ -11,7 +11,7 @@
 
 namespace fb {
 
-constexpr int kPlanThreads = 32;          // the stand-alone planner kernel is one warp
+constexpr int kPlanThreads = 256;         // the stand-alone planner kernel: one thread per expert; one warp decides
 constexpr uint32_t kPlanBarrierId = 1;    // named barrier of the router kernel's epilogue warps
 
 struct PlanParams {
@@ -70,8 +70,6 @@ struct PlanShared {
   // fast loop: one word per slot - bits 0..21 the count of the expert placed there, bits 22..29
   // that expert's id, bit 31 set once the expert has moved
   uint32_t slot_cnt[FB_MAX_EXPERTS];
-  uint8_t cand_a[FB_MAX_EXPERTS];        // fast loop: candidate c pairs slot c / m of the heavy rank ...
-  uint8_t cand_b[FB_MAX_EXPERTS];        // ... with slot c % m of the light rank
   uint8_t rank_of[FB_MAX_EXPERTS];       // expert -> rank under the placement as given
   uint8_t node_of[FB_MAX_RANKS];         // rank -> node (all 0 when every rank is in one node)
   uint32_t load[FB_MAX_RANKS];           // rank loads under the placement as given
@@ -129,10 +127,6 @@ __device__ __forceinline__ void plan_load_placement(const PlanParams& p, PlanSha
   }
   for (int r = t; r < p.R; r += nthreads)
     sh.node_of[r] = static_cast<uint8_t>(p.ranks_per_node > 0 ? r / p.ranks_per_node : 0);
-  for (int c = t; c < FB_MAX_EXPERTS; c += nthreads) {
-    sh.cand_a[c] = static_cast<uint8_t>(c / m);
-    sh.cand_b[c] = static_cast<uint8_t>(c % m);
-  }
 }
 __device__ __forceinline__ void plan_clear(PlanShared& sh, int t, int nthreads) {
   if (t == 0) { sh.bad = 0; sh.bad_range = 0; sh.fast = 0; }
@@ -165,38 +159,36 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 }
 
 // Greedy loop specialised for the common case: one cost per link class (no per-expert
-// size table) and at most 256 candidate pairs per iteration (m <= 16), kPerLane fixed (slot,
-// slot) pairs per lane.  One warp runs alone here, so what counts is the length of the
-// dependent instruction chain of an iteration, not the instruction count: every load of an
-// iteration is issued before the first result is needed, nothing branches on a loaded value
-// until the candidates are evaluated, and the accepted pair's slots and counts come from the
-// winning lane's registers by shuffle instead of a second trip through shared memory.  Same
-// decisions as the general loop below; 32-bit arithmetic where the ranges allow (loads < 2^22).
+// size table) and at most 256 candidate pairs per iteration (m <= 16).  One warp runs alone here,
+// so what counts is the length of the dependent instruction chain of an iteration.
+//
+// All pairs of an iteration have the same cost, so the largest benefit / cost is the largest
+// benefit.  With d tokens moved from the heavy rank (load La) to the light one (Lb), D = La - Lb and
+// v = |2 d - D|: the larger of the two new loads is (La + Lb + v) / 2 and d (D - d) = (D^2 - v^2) / 4, so
+//     gamma_den (Phi(L) - Phi(L')) = gamma_den (La - max((La + Lb + v) / 2, M2)) + gamma_num (D^2 - v^2) / 2
+// (M2: largest load of the other ranks) falls with v - strictly when gamma_num > 0; when it is 0, it is
+// constant up to v = 2 M2 - La - Lb.  A pair is useful exactly if v < D (0 < d < D), and with
+// gamma_num = 0 also M2 < La, which the same comparison tests.  The best pair is therefore the one
+// with the smallest v (clamped from below when gamma_num = 0), ties to the smallest pair: 32-bit
+// keys and one warp minimum, no products and no bound on the benefits.  (Benefits formed and
+// compared per candidate took 0.41 us per swap with 8 experts per rank and 0.75 us with 16; now 0.25 and 0.3.)
 // L0 / L1: this lane's rank loads (ranks lane and lane + 32, -1 if absent).
-// k32: every benefit of the call is known to stay below 2^32 (the caller checks the bound
-// gamma_den * Lmax + 2 gamma_num * Lmax^2 / 4 for the largest rank load Lmax, which no swap
-// raises), so benefits are formed and compared in 32 bits and the winner needs two warp
-// reductions instead of three plus a ballot.
+// Lane l tries expert slot l / g of the heavy rank with kPerLane slots of the light one, g lanes per
+// heavy slot (kPerLane g >= m).
 // kSide: the per-rank or the per-link budget can bind.  With a uniform cost per link class
 // a rank or a link is never charged more than the whole plan, so a side budget that starts at
 // or above the global one (the usual case: all three start at the same B) can never stop a
 // swap the global budget admits; the instance without them keeps no per-rank or per-link
 // books at all.
-template <int kPerLane, bool k32, bool kSide>
+template <int kPerLane, bool kSide>
 __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanShared& sh, int lane,
                                                       int& L0, int& L1) {
-  const int R = p.R, m = p.E / R, mm = m * m;
+  const int R = p.R, m = p.E / R;
   const uint32_t full = 0xffffffffu;
-  int cand_sa[kPerLane], cand_sb[kPerLane];                     // slot offsets inside the two ranks
-  bool cand_ok[kPerLane];
-#pragma unroll
-  for (int t = 0; t < kPerLane; ++t) {
-    cand_ok[t] = lane + 32 * t < mm;
-    cand_sa[t] = cand_ok[t] ? sh.cand_a[lane + 32 * t] : 0;
-    cand_sb[t] = cand_ok[t] ? sh.cand_b[lane + 32 * t] : 0;
-  }
-  const uint32_t gden = p.gamma_den ? p.gamma_den : 1u;
-  const uint32_t gnum2 = p.gamma_den ? 2u * p.gamma_num : 0u;   // <= 2^21
+  constexpr uint32_t kNone = 0xffffffffu;
+  constexpr int g = kPerLane == 8 ? 2 : (kPerLane == 2 ? 4 : 8);     // m <= 16, <= 8, <= 4
+  const int ia = lane / g, j0 = (lane % g) * kPerLane;
+  const bool flat = p.gamma_den == 0 || p.gamma_num == 0;
   // loop invariants in registers (no access to the parameter block inside the loop)
   const unsigned long long cost0 = p.uniform_cost_ns[0], cost1 = p.uniform_cost_ns[1];
   const unsigned long long global_ns = p.global_ns, rank_ns = p.rank_ns;
@@ -205,7 +197,7 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
   // A link is only ever charged one cost (its class's), so its budget is a swap count.
   const unsigned long long link_cap0 = p.uniform_link_cap[0], link_cap1 = p.uniform_link_cap[1];
   const uint32_t max_swaps = p.max_swaps, tau = p.tau_tokens;
-  uint32_t my_links[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};   // lane i keeps the links of swaps i, i+32, ...
+  uint32_t my_links[4] = {kNone, kNone, kNone, kNone};            // lane i keeps the links of swaps i, i+32, ...
   unsigned long long global_spent = 0;
   uint32_t n = 0;
   __syncwarp();
@@ -213,8 +205,8 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
     // frontier (lowest index on ties): max of load<<6 | (63 - rank), min of load<<6 | rank
     const uint32_t h0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(63 - lane)) : 0u;
     const uint32_t h1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(31 - lane)) : 0u;
-    const uint32_t l0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(lane)) : 0xffffffffu;
-    const uint32_t l1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(lane + 32)) : 0xffffffffu;
+    const uint32_t l0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(lane)) : kNone;
+    const uint32_t l1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(lane + 32)) : kNone;
     const uint32_t hi_key = __reduce_max_sync(full, h0 > h1 ? h0 : h1);
     const uint32_t lo_key = __reduce_min_sync(full, l0 < l1 ? l0 : l1);
     const int a = 63 - static_cast<int>(hi_key & 63u), b = static_cast<int>(lo_key & 63u);
@@ -222,19 +214,41 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
     const int D = La - Lb;
     // ---- every load of the iteration, before anything depends on one
     const int base_a = a * m, base_b = b * m;
-    uint32_t wa[kPerLane], wb[kPerLane];                           // slot words: count, expert, moved
+    const uint32_t wa = ia < m ? sh.slot_cnt[base_a + ia] : kSlotMoved;   // slot words: count, expert, moved
+    uint32_t wb[kPerLane];
 #pragma unroll
-    for (int t = 0; t < kPerLane; ++t) {
-      wa[t] = sh.slot_cnt[base_a + cand_sa[t]];
-      wb[t] = sh.slot_cnt[base_b + cand_sb[t]];
-    }
+    for (int t = 0; t < kPerLane; ++t) wb[t] = j0 + t < m ? sh.slot_cnt[base_b + j0 + t] : kSlotMoved;
     unsigned long long rs_a = 0, rs_b = 0;
     if (kSide) { rs_a = sh.rank_spent[a]; rs_b = sh.rank_spent[b]; }
     const int node_a = sh.node_of[a], node_b = sh.node_of[b];
-    int m2l = 0;
-    if (lane != a && lane != b && L0 > m2l) m2l = L0;
-    if (lane + 32 != a && lane + 32 != b && L1 > m2l) m2l = L1;
-    const int M2 = static_cast<int>(__reduce_max_sync(full, static_cast<uint32_t>(m2l)));
+    int v_floor = 0;
+    if (flat) {
+      int m2l = 0;
+      if (lane != a && lane != b && L0 > m2l) m2l = L0;
+      if (lane + 32 != a && lane + 32 != b && L1 > m2l) m2l = L1;
+      v_floor = 2 * static_cast<int>(__reduce_max_sync(full, static_cast<uint32_t>(m2l))) - La - Lb;
+    }
+    // ---- candidates of this lane: smallest v, ties -> smallest expert of the light rank
+    uint32_t key[kPerLane];
+#pragma unroll
+    for (int t = 0; t < kPerLane; ++t) {
+      const int dlt = static_cast<int>(wa & kSlotCountMask) - static_cast<int>(wb[t] & kSlotCountMask);   // tokens moved a -> b
+      int v = 2 * dlt - D;
+      v = v < 0 ? -v : v;
+      v = v < v_floor ? v_floor : v;
+      const bool usable = ((wa | wb[t]) >> 31) == 0 && v < D;              // neither expert moved yet
+      key[t] = usable ? static_cast<uint32_t>(v) << 8 | ((wb[t] >> 22) & 0xffu) : kNone;   // v < 2^22
+    }
+    uint32_t best = key[0];
+#pragma unroll
+    for (int t = 1; t < kPerLane; ++t) best = key[t] < best ? key[t] : best;
+    const uint32_t mine = best >> 8;
+    const uint32_t top = __reduce_min_sync(full, mine);
+    uint32_t my_wb = wb[0];
+    int my_jb = j0;
+#pragma unroll
+    for (int t = 1; t < kPerLane; ++t)
+      if (key[t] == best) { my_wb = wb[t]; my_jb = j0 + t; }      // one slot per expert: at most one t matches a valid key
     // ---- budgets: the cost is the same for every pair of this iteration
     const int cls = node_a == node_b ? 0 : 1;
     const unsigned long long c_ns = cls ? cost1 : cost0;
@@ -253,103 +267,27 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
         if (n > 32u * q) used += __popc(__ballot_sync(full, my_links[q] == lkey));    // n is the same in all lanes
       stop = stop || used >= (cls ? link_cap1 : link_cap0);
     }
-    // ---- candidates of this lane: largest benefit, ties -> smallest (expert on a, expert on b)
-    int src, ea, eb, sa, sb;
-    uint32_t wwa, wwb;                                            // slot words of the accepted pair
-    if (k32) {
-      // One 64-bit key per candidate: benefit, then the complement of the pair (so that the
-      // larger key is the better candidate), then the candidate's index in this lane.  The
-      // candidates of a lane are independent of each other; only the maximum chains them.
-      // Written stage by stage over all candidates (differences, bounds, benefits, keys) and reduced
-      // by a tree, so that nothing but the data flow orders the instructions of different candidates.
-      int dl[kPerLane];
-      uint32_t ben[kPerLane];
-      unsigned long long key[kPerLane];
-#pragma unroll
-      for (int t = 0; t < kPerLane; ++t)
-        dl[t] = static_cast<int>(wa[t] & kSlotCountMask) - static_cast<int>(wb[t] & kSlotCountMask);   // tokens moved a -> b
-#pragma unroll
-      for (int t = 0; t < kPerLane; ++t) {
-        int Mn = La - dl[t];                                      // Eq. 6
-        if (Lb + dl[t] > Mn) Mn = Lb + dl[t];                     // Eq. 7
-        if (M2 > Mn) Mn = M2;
-        // gamma_den * (Phi(L) - Phi(L')), variance term 2 dlt (La - Lb - dlt).  It is positive only
-        // for 0 < dlt < D, and inside that range both terms are non-negative.
-        const bool usable = cand_ok[t] && ((wa[t] | wb[t]) >> 31) == 0 && dl[t] > 0 && dl[t] < D;   // neither expert moved yet
-        const uint32_t b32 = gden * static_cast<uint32_t>(La - Mn) +
-                             gnum2 * (static_cast<uint32_t>(dl[t]) * static_cast<uint32_t>(D - dl[t]));
-        ben[t] = usable ? b32 : 0u;
-      }
-#pragma unroll
-      for (int t = 0; t < kPerLane; ++t) {
-        const uint32_t pair = ((wa[t] >> 22) & 0xffu) << 8 | ((wb[t] >> 22) & 0xffu);
-        key[t] = static_cast<unsigned long long>(ben[t]) << 32 |
-                 static_cast<unsigned long long>(0xffffu - pair) << 8 | static_cast<unsigned>(t);
-      }
-#pragma unroll
-      for (int w = kPerLane / 2; w >= 1; w >>= 1)
-#pragma unroll
-        for (int t = 0; t < w; ++t) key[t] = key[t] > key[t + w] ? key[t] : key[t + w];
-      const unsigned long long best_key = key[0];
-      const uint32_t mine = static_cast<uint32_t>(best_key >> 32);
-      const uint32_t top = __reduce_max_sync(full, mine);
-      if (stop || top == 0) break;                                // Algorithm 1 lines 6-7
-      // among the lanes that hold the top benefit: smallest pair, i.e. largest complement; the lane rides along
-      const uint32_t low = static_cast<uint32_t>(best_key);      // complement of the pair << 8 | index
-      const uint32_t win = __reduce_max_sync(full, mine == top ? ((low >> 8) << 5 | static_cast<uint32_t>(31 - lane)) : 0u);
-      src = 31 - static_cast<int>(win & 31u);
-      const uint32_t pair = 0xffffu - (win >> 5);
-      ea = static_cast<int>(pair >> 8);
-      eb = static_cast<int>(pair & 0xffu);
-      // the winning lane's candidate index gives the slots; their words come from shared memory
-      const int t_win = __shfl_sync(full, static_cast<int>(low & 0xffu), src);
-      sa = base_a + sh.cand_a[src + 32 * t_win];
-      sb = base_b + sh.cand_b[src + 32 * t_win];
-      wwa = sh.slot_cnt[sa];
-      wwb = sh.slot_cnt[sb];
-    } else {
-      unsigned long long best_ben = 0;
-      uint32_t best_pair = 0xffffffffu, best_slots = 0, best_wa = 0, best_wb = 0;
-#pragma unroll
-      for (int t = 0; t < kPerLane; ++t) {
-        const int dlt = static_cast<int>(wa[t] & kSlotCountMask) - static_cast<int>(wb[t] & kSlotCountMask);
-        int Mn = La - dlt;
-        if (Lb + dlt > Mn) Mn = Lb + dlt;
-        if (M2 > Mn) Mn = M2;
-        const bool usable = cand_ok[t] && ((wa[t] | wb[t]) >> 31) == 0 && dlt > 0 && dlt < D;
-        const long long ben = static_cast<long long>(gden) * (La - Mn) +
-                              static_cast<long long>(gnum2) * (static_cast<long long>(dlt) * (D - dlt));
-        const unsigned long long ub = usable ? static_cast<unsigned long long>(ben) : 0ull;
-        const uint32_t pair = ((wa[t] >> 22) & 0xffu) << 16 | ((wb[t] >> 22) & 0xffu);
-        if (ub > best_ben || (ub == best_ben && ub > 0 && pair < best_pair)) {
-          best_ben = ub; best_pair = pair; best_wa = wa[t]; best_wb = wb[t];
-          best_slots = static_cast<uint32_t>(base_a + cand_sa[t]) << 16 | static_cast<uint32_t>(base_b + cand_sb[t]);
-        }
-      }
-      const uint32_t top_hi = __reduce_max_sync(full, static_cast<uint32_t>(best_ben >> 32));
-      const uint32_t top_lo = __reduce_max_sync(full, static_cast<uint32_t>(best_ben >> 32) == top_hi ? static_cast<uint32_t>(best_ben) : 0u);
-      const unsigned long long top_ben = static_cast<unsigned long long>(top_hi) << 32 | top_lo;
-      if (stop || top_ben == 0) break;                            // Algorithm 1 lines 6-7
-      const uint32_t win = __reduce_min_sync(full, best_ben == top_ben ? best_pair : 0xffffffffu);
-      src = __ffs(__ballot_sync(full, best_ben == top_ben && best_pair == win)) - 1;
-      ea = static_cast<int>(win >> 16);
-      eb = static_cast<int>(win & 0xffffu);
-      // the lane that holds the accepted pair hands out its slots and slot words
-      const uint32_t slots = __shfl_sync(full, best_slots, src);
-      wwa = __shfl_sync(full, best_wa, src);
-      wwb = __shfl_sync(full, best_wb, src);
-      sa = static_cast<int>(slots >> 16);
-      sb = static_cast<int>(slots & 0xffffu);
+    if (stop || top == kNone >> 8) break;                         // Algorithm 1 lines 6-7
+    // the winner: the only lane with the smallest v, or among several the smallest (expert on a, expert on b)
+    uint32_t holders = __ballot_sync(full, mine == top);
+    if (__popc(holders) > 1) {
+      const uint32_t pair = mine == top ? ((wa >> 22) & 0xffu) << 8 | (best & 0xffu) : kNone;
+      holders = __ballot_sync(full, pair == __reduce_min_sync(full, pair));
     }
+    const int src = __ffs(holders) - 1;
+    const uint32_t wwa = __shfl_sync(full, wa, src), wwb = __shfl_sync(full, my_wb, src);
+    const int slots = __shfl_sync(full, ia << 8 | my_jb, src);
     const int dlt = static_cast<int>(wwa & kSlotCountMask) - static_cast<int>(wwb & kSlotCountMask);
     if (lane == 0) {
-      sh.slot_cnt[sa] = wwb | kSlotMoved; sh.slot_cnt[sb] = wwa | kSlotMoved;   // the two experts trade slots
+      // the two experts trade slots
+      sh.slot_cnt[base_a + (slots >> 8)] = wwb | kSlotMoved;
+      sh.slot_cnt[base_b + (slots & 0xff)] = wwa | kSlotMoved;
       if (kSide) { sh.rank_spent[a] = rs_a + c_ns; sh.rank_spent[b] = rs_b + c_ns; }
       // The accepted swap stays in shared memory until the loop is over (ranks and expert ids
       // are below 256: one word; link_key is otherwise unused on this path): a global store
       // here would be waited for at the warp barrier below, once per iteration.
       sh.link_key[n] = static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 |
-                       static_cast<uint32_t>(ea) << 8 | static_cast<uint32_t>(eb);
+                       ((wwa >> 22) & 0xffu) << 8 | ((wwb >> 22) & 0xffu);
     }
     if (lane == a) L0 -= dlt;
     if (lane + 32 == a) L1 -= dlt;
@@ -528,8 +466,7 @@ __device__ __noinline__ void plan_loop_general(const PlanParams& p, PlanShared& 
 }
 
 // The planner, run by ONE warp (all 32 lanes) once plan_load_placement has filled the
-// placement arrays, sh.cnt holds the count vector and plan_scatter_counts has turned it into
-// counts per slot.  A single warp keeps the rank loads in registers (lane r holds ranks r and
+// placement arrays and plan_put_count has turned the count vector into counts per slot.  A single warp keeps the rank loads in registers (lane r holds ranks r and
 // r + 32) and needs no block barrier.  Writes the swaps, their number and the rank loads
 // before and after; the new placement is written afterwards by plan_write_placement.
 // kGeneral: the instance carries the general loop as well.  The router kernels' fused tail uses
@@ -573,28 +510,19 @@ __device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh
 
   if (!plan_needs_general_loop(p)) {
     int l0 = static_cast<int>(L0), l1 = static_cast<int>(L1);
-    const int mm = m * m;
-    // largest benefit any swap of this call can have (rank loads never exceed the initial maximum)
-    const unsigned long long lmax = __reduce_max_sync(full, static_cast<uint32_t>(s0 > s1 ? s0 : s1));
-    const unsigned long long bound = static_cast<unsigned long long>(p.gamma_den ? p.gamma_den : 1u) * lmax +
-                                     (p.gamma_den ? 2ull * p.gamma_num : 0ull) * ((lmax * lmax) >> 2);
-    const bool narrow = bound < (1ull << 32);
     // can the per-rank or the per-link budget stop a swap that the global budget admits?
     const bool side = (p.rank_ns != FB_BUDGET_OFF && !(p.global_ns != FB_BUDGET_OFF && p.rank_ns >= p.global_ns)) ||
                       (p.link_ns != FB_BUDGET_OFF && !(p.global_ns != FB_BUDGET_OFF && p.link_ns >= p.global_ns));
     uint32_t n_fast;
     if (lane == 0) sh.fast = 1;
-    if (narrow && !side)
-      n_fast = mm <= 32 ? plan_loop_uniform<1, true, false>(p, sh, lane, l0, l1)
-               : mm <= 64 ? plan_loop_uniform<2, true, false>(p, sh, lane, l0, l1)
-               : mm <= 128 ? plan_loop_uniform<4, true, false>(p, sh, lane, l0, l1)
-                           : plan_loop_uniform<8, true, false>(p, sh, lane, l0, l1);
-    else if (narrow)
-      n_fast = mm <= 64 ? plan_loop_uniform<2, true, true>(p, sh, lane, l0, l1)
-                        : plan_loop_uniform<8, true, true>(p, sh, lane, l0, l1);
+    if (!side)
+      n_fast = m <= 4 ? plan_loop_uniform<1, false>(p, sh, lane, l0, l1)
+               : m <= 8 ? plan_loop_uniform<2, false>(p, sh, lane, l0, l1)
+                        : plan_loop_uniform<8, false>(p, sh, lane, l0, l1);
     else
-      n_fast = mm <= 64 ? plan_loop_uniform<2, false, true>(p, sh, lane, l0, l1)
-                        : plan_loop_uniform<8, false, true>(p, sh, lane, l0, l1);
+      n_fast = m <= 4 ? plan_loop_uniform<1, true>(p, sh, lane, l0, l1)
+               : m <= 8 ? plan_loop_uniform<2, true>(p, sh, lane, l0, l1)
+                        : plan_loop_uniform<8, true>(p, sh, lane, l0, l1);
     FB_PLAN_STAMP(20);
     if (lane == 0) *p.n_swaps = static_cast<int32_t>(n_fast);
     if (lane < R) p.load_after[lane] = static_cast<uint32_t>(l0);

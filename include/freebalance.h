@@ -409,25 +409,23 @@ fb_status fb_topk_hits(const int32_t* ids_a, const int32_t* ids_b, int32_t T, in
  * 256-row tile pairs than the limit (or than fit on the GPU at once, fb_max_pairs) runs
  * the persistent kernel, where each block pair walks several tiles (on as few block pairs as
  * the resulting number of rounds needs: 128 tile pairs run on 64 block pairs, not on all 74);
- * results do not depend on the limit.  Honoured for the gate shapes that kernel supports (E a multiple of 32 up
- * to 256; sigmoid gates with 32-expert groups and topk_group <= 4, or softmax gates whose
- * weights are renormalised); other shapes ignore it.  Returns FB_ERR_INVALID_ARG for a
- * negative limit. */
+ * results do not depend on the limit, except that it may switch the k-range split off (see
+ * fb_set_split).  Returns FB_ERR_INVALID_ARG for a negative limit. */
 fb_status fb_set_pair_limit(fb_ctx* ctx, int32_t pairs);
-/* k-range split of the router kernel (on by default).  When a call has fewer 256-row tile pairs
- * than block pairs fit on the GPU (and the persistent kernel is not used), the spare pairs sum
- * the tail of every tile's k-range into partial tiles that the tiles' owners add before their
- * epilogue, so that every SM's tensor core works through the whole main loop (128 tiles leave
- * 20 of 148 SMs idle otherwise; the smaller shapes leave more than half).  The schedule is a
+/* k-range split of the router kernel (on by default).  When a call has so few 256-row tile pairs that
+ * 2, 4 or 8 block pairs per tile pair fit on the GPU at once, that many pairs share a tile: each sums a
+ * piece of the k-range, the partial sums meet through the shared memory of the cluster and each block
+ * selects for its share of the rows.  The schedule is a
  * function of the shape and of the number of pairs only: a call is reproducible, but its logits
  * differ from an unsplit call's in the order of the fp32 additions (both stay within the
  * library's tolerance of the fp64 product), so a token whose k-th and (k+1)-th keys are closer
- * than that rounding may be routed differently by the two.  mode 0 switches the split off, 1 on;
- * owner_bias_kblocks tunes how many k-blocks more than an even share a tile's owner keeps
- * (-1: built-in choice).  FB_ERR_INVALID_ARG for other values. */
+ * than that rounding may be routed differently by the two.  mode 0 switches the split off, 1 on.
+ * owner_bias_kblocks (-1 .. 1024) is accepted and has no effect: the pieces are equal.
+ * FB_ERR_INVALID_ARG for other values. */
 fb_status fb_set_split(fb_ctx* ctx, int32_t mode, int32_t owner_bias_kblocks);
-/* Block pairs of the persistent router kernel that fit on the GPU at once (0 when the
- * configuration does not support that kernel). */
+/* Block pairs of the persistent router kernel that fit on the GPU at once (0 when the gate does not
+ * suit that kernel: E a multiple of 32; sigmoid gates with 32-expert groups and topk_group <= 4, or
+ * softmax gates; other gates walk several tiles in another kernel). */
 int32_t fb_max_pairs(const fb_ctx* ctx);
 /* Text for a status code; never NULL. */
 const char* fb_status_string(fb_status s);

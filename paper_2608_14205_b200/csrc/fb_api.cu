@@ -16,6 +16,7 @@
 #include "fb_quality.cuh"
 #include "fb_router.cuh"
 #include "fb_router_persistent.cuh"
+#include "fb_router_rows.cuh"
 
 namespace {
 
@@ -38,33 +39,32 @@ struct fb_ctx {
   fb_config cfg;
   int device = 0;
   int N = 0;                      // experts padded to a multiple of 16 (UMMA N)
-  int stages[2] = {0, 0};         // pipeline depth for the single-block and the pair kernel
-  int tmem_cols = 0;
-  size_t smem_bytes[2] = {0, 0};
-  int max_tiles = 0;
-  // persistent router kernel (several tiles per block pair): pipeline depth (0 = not usable
-  // for this shape), dynamic shared memory, block pairs that fit on the GPU at once, and
-  // the caller's limit on the pairs to use (0 = none)
+  fb::RouterParams gate;          // the shape- and gate-dependent fields of a launch (copied per call)
+  bool ranking[2] = {false, false};    // the gate suits the ranking kernels [without / with routing weights]
+  // One-tile ranking kernel: pipeline depth and dynamic shared memory
+  int stages = 0;
+  size_t smem_bytes = 0;
+  // Persistent ranking kernel (several tiles per block pair)
   int persist_stages = 0;
   size_t persist_smem = 0;
-  int max_pairs = 0;
-  int pair_limit = 0;
-  int stage_limit = 0;                 // diagnostic: pipeline stages at most (0 = as many as fit)
-  int n_sm = 148;                      // SMs of the device
-  // k-range split of the one-tile pair kernel: block pairs that fit on the GPU at once, the
-  // partial tiles and their flags (one slot per helper item; set by the helper, put back by the
-  // owner), and the caller's switch / tuning value
-  int split_pairs = 0;
-  float* split_partial = nullptr;
-  uint32_t* split_flags = nullptr;
-  int split_mode = 1;                  // 0 off, 1 on
-  int split_bias = -1;                 // extra k-blocks an owner keeps (-1: the built-in choice)
+  // Row-per-warp kernel: instance (log2 of the columns per lane), pipeline depth and dynamic shared memory
+  // with one tile per block pair [0] and with several [1]
+  int rows_kernel = 0;
+  int rows_stages[2] = {0, 0};
+  size_t rows_smem[2] = {0, 0};
+  // clusters of 2 J blocks that fit on the GPU at once, by log2 J (J block pairs share a tile pair)
+  int max_clusters[4] = {0, 0, 0, 0};
+  int max_tiles = 0;
+  int pair_limit = 0;             // the caller's limit on the block pairs to use (0 = none)
+  int stage_limit = 0;            // diagnostic: pipeline stages at most (0 = as many as fit)
+  int n_sm = 148;                 // SMs of the device
+  int split_mode = 1;             // k-range split over the blocks of a cluster: 0 off, 1 on
   EncodeTiledFn encode = nullptr;
   // device scratch
   uint32_t* counts_scratch = nullptr;   // [256], zero between calls
   uint32_t* ticket = nullptr;           // [1],   zero between calls
   int32_t* status = nullptr;            // [1]
-  uint8_t* slice_counts = nullptr;      // [max_tiles][slice_row_bytes(E)]: per-tile histograms for the dispatch index
+  uint8_t* slice_counts = nullptr;      // [max_slices][slice_row_bytes(E)]: per-slice histograms for the dispatch index
   // descriptor cache
   MapEntry x_maps[kMapCache];
   MapEntry w_maps[kMapCache];
@@ -200,32 +200,31 @@ fb_status fill_plan(const fb_ctx* ctx, const fb_budget* b, const int32_t* pi, in
   return FB_OK;
 }
 
-// Kernel instances by (selection kind, logit bias present).
+// Kernel instances of the ranking kernels by (gate, logit bias present), of the row-per-warp kernel by
+// (log2 of the columns per lane, gate).
 using RouterKernelFn = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, fb::RouterParams);
-template <int kCtas>
-static RouterKernelFn router_kernel_fn(int sel, bool lb) {
-  switch (sel * 2 + (lb ? 1 : 0)) {
-    case 0: return fb::fb_router_kernel<kCtas, fb::kSelectGeneral, false>;
-    case 1: return fb::fb_router_kernel<kCtas, fb::kSelectGeneral, true>;
-    case 2: return fb::fb_router_kernel<kCtas, fb::kSelectSigmoidRank, false>;
-    case 3: return fb::fb_router_kernel<kCtas, fb::kSelectSigmoidRank, true>;
-    case 4: return fb::fb_router_kernel<kCtas, fb::kSelectSoftmaxRank, false>;
-    default: return fb::fb_router_kernel<kCtas, fb::kSelectSoftmaxRank, true>;
-  }
-}
-static RouterKernelFn router_split_kernel_fn(int sel, bool lb) {
-  switch (sel * 2 + (lb ? 1 : 0)) {
-    case 0: return fb::fb_router_kernel<2, fb::kSelectGeneral, false, true>;
-    case 1: return fb::fb_router_kernel<2, fb::kSelectGeneral, true, true>;
-    case 2: return fb::fb_router_kernel<2, fb::kSelectSigmoidRank, false, true>;
-    case 3: return fb::fb_router_kernel<2, fb::kSelectSigmoidRank, true, true>;
-    case 4: return fb::fb_router_kernel<2, fb::kSelectSoftmaxRank, false, true>;
-    default: return fb::fb_router_kernel<2, fb::kSelectSoftmaxRank, true, true>;
-  }
+static RouterKernelFn ranking_kernel_fn(bool sigmoid, bool lb) {
+  if (sigmoid) return lb ? fb::fb_router_kernel<true, true> : fb::fb_router_kernel<true, false>;
+  return lb ? fb::fb_router_kernel<false, true> : fb::fb_router_kernel<false, false>;
 }
 static RouterKernelFn persistent_kernel_fn(bool sigmoid, bool lb) {
   if (sigmoid) return lb ? fb::fb_router_persistent_kernel<true, true> : fb::fb_router_persistent_kernel<true, false>;
   return lb ? fb::fb_router_persistent_kernel<false, true> : fb::fb_router_persistent_kernel<false, false>;
+}
+constexpr int kRowsKernels = 5;
+static RouterKernelFn rows_kernel_fn(int log_cpl, bool sigmoid) {
+  switch (2 * log_cpl + (sigmoid ? 1 : 0)) {
+    case 0: return fb::fb_router_rows_kernel<1, false>;
+    case 1: return fb::fb_router_rows_kernel<1, true>;
+    case 2: return fb::fb_router_rows_kernel<2, false>;
+    case 3: return fb::fb_router_rows_kernel<2, true>;
+    case 4: return fb::fb_router_rows_kernel<4, false>;
+    case 5: return fb::fb_router_rows_kernel<4, true>;
+    case 6: return fb::fb_router_rows_kernel<8, false>;
+    case 7: return fb::fb_router_rows_kernel<8, true>;
+    case 8: return fb::fb_router_rows_kernel<16, false>;
+    default: return fb::fb_router_rows_kernel<16, true>;
+  }
 }
 
 // Launch of a small kernel that may start under the end of the stream's previous kernel (it waits for
@@ -251,11 +250,13 @@ fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* cou
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
-// Launch the router kernel in one of its three modes.
+// Launch a router kernel in one of its modes.
 // x2 is the second input of kModeLayer (the normal router input), nullptr otherwise.
+// *pieces_out (optional): block pairs per tile pair, i.e. row slices per tile of the histogram table.
 fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T, int mode,
                         uint32_t* counts_out, int32_t* topk_ids, float* topk_w, float* logits,
-                        const fb::PlanParams* plan, cudaStream_t stream, const void* x2 = nullptr, int probe = 0) {
+                        const fb::PlanParams* plan, cudaStream_t stream, const void* x2 = nullptr, int probe = 0,
+                        int* pieces_out = nullptr) {
   const CUtensorMap *mx = nullptr, *mx2 = nullptr, *mw = nullptr;
   fb_status st = make_map(ctx, ctx->x_maps, &ctx->x_next, x, T, fb::kTileM, &mx);
   if (st != FB_OK) return st;
@@ -266,22 +267,11 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
     st = make_map(ctx, ctx->x_maps, &ctx->x_next, x2, T, fb::kTileM, &mx2);
     if (st != FB_OK) return st;
   }
-  const int tiles = (T + fb::kTileM - 1) / fb::kTileM;
-  const int pair = (tiles > 1 && ctx->stages[1] >= 2) ? 1 : 0;   // a single tile gains nothing from a partner
-  st = make_map(ctx, ctx->w_maps, &ctx->w_next, router->W, ctx->cfg.E,
-                static_cast<uint32_t>(pair ? ctx->N / 2 : ctx->N), &mw);
+  st = make_map(ctx, ctx->w_maps, &ctx->w_next, router->W, ctx->cfg.E, static_cast<uint32_t>(ctx->N / 2), &mw);
   if (st != FB_OK) return st;
-  fb::RouterParams p;
-  memset(&p, 0, sizeof(p));
   const fb_config& c = ctx->cfg;
-  p.T = T; p.d = c.d; p.E = c.E; p.N = ctx->N; p.k = c.k;
-  p.gate = c.gate; p.n_group = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? c.n_group : 1;
-  p.topk_group = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? c.topk_group : 1;
-  p.renorm = c.renorm; p.route_scale = c.route_scale;
-  p.num_kb = (c.d + fb::kBlockK - 1) / fb::kBlockK;
-  p.stages = ctx->stages[pair];
-  if (ctx->stage_limit >= 2 && ctx->stage_limit < p.stages) p.stages = ctx->stage_limit;
-  p.tmem_cols = ctx->tmem_cols;
+  fb::RouterParams p = ctx->gate;
+  p.T = T;
   p.mode = mode;
   p.logit_bias = router->logit_bias;
   p.select_bias = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? router->select_bias : nullptr;
@@ -301,111 +291,85 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   // the router kernel instead.
   const bool plan_wanted = plan != nullptr && (mode == fb::kModePredictPlan || mode == fb::kModeLayer);
   p.fuse_planner = (plan_wanted && !fb::plan_needs_general_loop(*plan)) ? 1 : 0;
-  const int tiles_pad = pair ? (tiles + 1) / 2 * 2 : tiles;       // a pair never straddles the two passes
-  int blocks = mode == fb::kModeLayer ? 2 * tiles_pad : tiles_pad;
-  p.tiles_first = tiles_pad;
-  p.ticket_target = tiles_pad;
-  // More tile pairs than block pairs fit on the GPU (or than the caller allows): the
-  // persistent kernel walks several tiles per block pair and overlaps their epilogues.
-  // selection code of this launch: the ranking selection only if it applies to every block
-  // (in layer mode the normal pass writes weights, the early pass does not)
-  const int sel = fb::select_kind(c.E, ctx->N, c.k, c.gate, p.n_group, p.topk_group,
-                                  topk_w != nullptr && !c.renorm && c.gate == FB_GATE_SOFTMAX_TOPK);
-  bool persistent = false;
-  if (pair && ctx->persist_stages >= 2 && logits == nullptr && probe == 0) {
-    const bool want_sum = topk_w != nullptr && !c.renorm && c.gate == FB_GATE_SOFTMAX_TOPK;
-    const int pairs_avail = ctx->pair_limit > 0 && ctx->pair_limit < ctx->max_pairs ? ctx->pair_limit : ctx->max_pairs;
-    if (fb::persistent_gate_ok(c.E, c.k, c.gate, p.n_group, p.topk_group, want_sum) && blocks / 2 > pairs_avail) {
-      persistent = true;
-      // no more block pairs than the number of rounds needs: 128 tile pairs run as 2 rounds on 64
-      // block pairs just as fast as on 74 (measured), and the other SMs stay free for other streams
-      const int rounds = (blocks / 2 + pairs_avail - 1) / pairs_avail;
-      blocks = 2 * ((blocks / 2 + rounds - 1) / rounds);
-      // every block publishes its counts once: as many tickets as blocks that own a tile of the
-      // counted pass
-      p.ticket_target = blocks < tiles_pad ? blocks : tiles_pad;
-      // room for two accumulator sets (4 N columns) when the 512 tensor-memory columns allow it
-      if (4 * ctx->N <= 512) p.tmem_cols = next_pow2_at_least_32(4 * ctx->N);
-      p.stages = ctx->persist_stages;
-      if (ctx->stage_limit >= 2 && ctx->stage_limit < p.stages) p.stages = ctx->stage_limit;
-    }
+  const int tiles = (T + fb::kTileM - 1) / fb::kTileM;
+  p.tiles_first = (tiles + 1) / 2 * 2;                            // a pair never straddles the two passes
+  const int tile_pairs = (mode == fb::kModeLayer ? 2 : 1) * (p.tiles_first / 2);
+  const int pairs_avail = ctx->pair_limit > 0 && ctx->pair_limit < ctx->max_clusters[0] && probe == 0
+                              ? ctx->pair_limit : ctx->max_clusters[0];
+  // Few tile pairs: as many block pairs per tile pair as fit at once (all clusters of the launch
+  // are resident together) and have at least two k-blocks each.
+  int log_j = 0;
+  if (ctx->split_mode != 0 && probe == 0)
+    for (int l = 1; l <= 3; ++l)
+      if (tile_pairs <= ctx->max_clusters[l] && tile_pairs << l <= pairs_avail && p.num_kb >= 2 << l) log_j = l;
+  const int J = 1 << log_j;
+  p.pieces = J;
+  if (pieces_out) *pieces_out = J;
+  // Which kernel: whole tiles of a gate that the ranking selection handles go there (one tile per pair,
+  // or several where more tile pairs than block pairs fit or than the caller allows); tiles shared by
+  // several pairs and all other gates take the row-per-warp selection (figures: fb_router_rows.cuh).
+  const bool ranking = J == 1 && ctx->ranking[topk_w != nullptr ? 1 : 0];
+  const bool several = J == 1 && probe == 0 && tile_pairs > pairs_avail && !(ranking && logits != nullptr);
+  int clusters = tile_pairs;
+  if (several) {
+    // no more pairs than the number of rounds needs: 128 tile pairs run as 2 rounds on 64
+    // block pairs just as fast as on 74 (measured), and the other SMs stay free for other streams
+    const int rounds = (tile_pairs + pairs_avail - 1) / pairs_avail;
+    clusters = (tile_pairs + rounds - 1) / rounds;
+    // room for two accumulator sets (4 N columns) when the 512 tensor-memory columns allow it
+    if (4 * ctx->N <= 512) p.tmem_cols = next_pow2_at_least_32(4 * ctx->N);
   }
-  // Fewer tile pairs than block pairs fit on the GPU: the spare pairs become helpers that sum
-  // the tail of every tile's k-range (see RouterParams).  The schedule depends on the shape and
-  // on the number of pairs only.
-  bool split = false;
-  if (pair && !persistent && ctx->split_partial != nullptr && ctx->split_mode != 0 && probe == 0) {
-    const int tile_pairs = blocks / 2;                   // over both passes of a layer launch
-    int pairs_avail = ctx->split_pairs;
-    if (ctx->pair_limit > 0 && ctx->pair_limit < pairs_avail) pairs_avail = ctx->pair_limit;
-    const int spare = pairs_avail - tile_pairs;
-    // Worth it only where at least half of the pairs would idle: with 64 tile pairs on 74 block
-    // pairs (the 16k-token DeepSeek-V3 shape) the chip is power bound while the main loop runs -
-    // more busy SMs lower the clock, rows per microsecond rise by 5 % from 128 to 148 SMs - and
-    // helpers add their copy-outs on top (measured: 60 -> 68 us).
-    if (spare >= tile_pairs && p.num_kb >= 32) {
-      int J = spare / tile_pairs;                      // helpers per tile: J pieces each
-      if (J > 3) J = 3;
-      const int helpers = tile_pairs * J;
-      int ko = (p.num_kb + J) / (J + 1);
-      // a helper pays for the copy-out of its partial, the owner for reading it: owners keep a
-      // few k-blocks more than an even share
-      ko += ctx->split_bias >= 0 ? ctx->split_bias : 4;
-      if (ko > p.num_kb - 2 * J) ko = p.num_kb - 2 * J;     // every piece has at least two k-blocks
-      if (ko >= 2) {
-        split = true;
-        p.split_helpers = helpers;
-        p.split_ko = ko;
-        p.split_j = J;
-        p.split_epoch = 1;          // "complete"; the owner that consumed a partial puts the flag back to 0
-        p.split_partial = ctx->split_partial;
-        p.split_flags = ctx->split_flags;
-        blocks += 2 * helpers;
-      }
-    }
+  const int blocks = 2 * J * clusters;
+  // every block publishes its counts once: as many tickets as blocks that own a tile of the counted pass
+  p.ticket_target = blocks < p.tiles_first * J ? blocks : p.tiles_first * J;
+  RouterKernelFn fn;
+  size_t smem;
+  const bool sigmoid = c.gate == FB_GATE_SIGMOID_GROUP_TOPK;
+  if (!ranking) {
+    fn = rows_kernel_fn(ctx->rows_kernel, sigmoid);
+    p.stages = ctx->rows_stages[several ? 1 : 0];
+    smem = ctx->rows_smem[several ? 1 : 0];
+  } else if (several) {
+    fn = persistent_kernel_fn(sigmoid, router->logit_bias != nullptr);
+    p.stages = ctx->persist_stages;
+    smem = ctx->persist_smem;
+  } else {
+    fn = ranking_kernel_fn(sigmoid, router->logit_bias != nullptr);
+    p.stages = ctx->stages;
+    smem = ctx->smem_bytes;
   }
+  if (ctx->stage_limit >= 2 && ctx->stage_limit < p.stages) p.stages = ctx->stage_limit;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
   cfg.blockDim = dim3(fb::kRouterThreads, 1, 1);
-  cfg.dynamicSmemBytes = ctx->smem_bytes[pair];
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  cudaError_t err;
-  if (persistent) cfg.dynamicSmemBytes = ctx->persist_smem;
   if (ctx->ev_before) cudaEventRecord(ctx->ev_before, stream);
-  // Programmatic dependent launch: when the previous kernel of the stream allows it (the
-  // dispatch-index kernel does), this kernel's set-up overlaps that kernel's execution; the
-  // kernel waits for its completion (griddepcontrol.wait) before it reads any global memory.
+  // Programmatic dependent launch: this kernel's set-up overlaps the previous kernel's execution (where
+  // that one allows it, as the library's kernels do); the kernel waits for its completion
+  // (griddepcontrol.wait) before it reads any global memory.
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(2 * J);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (pair) {
-    cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.numAttrs = 2;
-    const bool lb = router->logit_bias != nullptr;
-    err = cudaLaunchKernelEx(&cfg, persistent ? persistent_kernel_fn(c.gate == FB_GATE_SIGMOID_GROUP_TOPK, lb)
-                                   : split    ? router_split_kernel_fn(sel, lb)
-                                              : router_kernel_fn<2>(sel, lb), *mx, *mx2, *mw, p);
-  } else {
-    cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
-    err = cudaLaunchKernelEx(&cfg, router_kernel_fn<1>(sel, router->logit_bias != nullptr), *mx, *mx2, *mw, p);
-  }
+  cfg.numAttrs = 2;
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, fn, *mx, *mx2, *mw, p);
   if (ctx->ev_after) cudaEventRecord(ctx->ev_after, stream);
   ctx->ev_before = ctx->ev_after = nullptr;
   ++ctx->launches;
-  if (persistent) ++ctx->persistent_launches;
+  if (several) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
   if (plan_wanted && !p.fuse_planner) return launch_plan(ctx, *plan, counts_out, stream);
   return FB_OK;
 }
 
-// Dispatch index from the router kernel's top-k ids and per-tile histograms.
-fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, const int32_t* expert_to_slot, const int32_t* topk_ids,
+// Dispatch index from the router kernel's top-k ids and per-slice histograms.
+fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, const int32_t* expert_to_slot, const int32_t* topk_ids,
                                 uint32_t* slot_offsets, uint32_t* rank_offsets, int32_t* perm, int32_t* inv_perm,
                                 uint32_t* rank_load, cudaStream_t stream) {
   const fb_config& c = ctx->cfg;
@@ -413,8 +377,9 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, const int32_t* expert_to
   dp.T = T; dp.k = c.k; dp.E = c.E; dp.R = c.R;
   dp.num_tiles = (T + fb::kDispatchTile - 1) / fb::kDispatchTile;
   dp.topk_ids = topk_ids;
-  dp.slices_per_tile = 1;
-  dp.num_slices = dp.num_tiles;
+  dp.slices_per_tile = slices_per_tile;
+  const int slice_rows = fb::kDispatchTile / slices_per_tile;
+  dp.num_slices = (T + slice_rows - 1) / slice_rows;
   dp.slice_counts = ctx->slice_counts;
   dp.expert_to_slot = expert_to_slot;
   dp.slot_offsets = slot_offsets;
@@ -450,28 +415,66 @@ bool dev_alloc(Tp** p, size_t count) {
 
 }  // namespace
 
-// Shape-dependent launch parameters of the one-tile router kernel (host arithmetic
-// only): padded width, TMEM columns, pipeline depth and dynamic shared
-// memory of the single-block and the pair variant.
+// Shape-dependent launch parameters of the router kernels (host arithmetic only): padded width, TMEM
+// columns, gate layout, pipeline depths and dynamic shared memory.
 static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
-  const fb_config& cfg = ctx->cfg;
-  ctx->N = (cfg.E + 15) / 16 * 16;
-  ctx->tmem_cols = next_pow2_at_least_32(2 * ctx->N)   /* two accumulators */;
-  const size_t budget = static_cast<size_t>(prop.sharedMemPerBlockOptin) - sizeof(fb::RouterShared) - 2048;
-  for (int pair = 0; pair < 2; ++pair) {
-    const size_t stage_bytes = fb::kATileBytes + static_cast<size_t>(ctx->N / (pair + 1)) * fb::kBlockK * 2;
-    int stages = static_cast<int>((budget - 1024) / stage_bytes);
-    if (stages > fb::kMaxStages) stages = fb::kMaxStages;
-    size_t dyn = stages * stage_bytes;
+  const fb_config& c = ctx->cfg;
+  ctx->N = (c.E + 15) / 16 * 16;
+  fb::RouterParams& g = ctx->gate;
+  memset(&g, 0, sizeof(g));
+  g.d = c.d; g.E = c.E; g.N = ctx->N; g.k = c.k;
+  g.gate = c.gate;
+  g.n_group = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? c.n_group : 1;
+  g.topk_group = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? c.topk_group : 1;
+  g.renorm = c.renorm; g.route_scale = c.route_scale;
+  g.num_kb = (c.d + fb::kBlockK - 1) / fb::kBlockK;
+  g.tmem_cols = next_pow2_at_least_32(2 * ctx->N);               // two accumulators
+  const int cpl = fb::gate_layout(c.E, c.gate, c.n_group, c.topk_group, &g);
+  ctx->rows_kernel = 0;
+  while ((1 << ctx->rows_kernel) < cpl) ++ctx->rows_kernel;
+  if (ctx->rows_kernel >= kRowsKernels) return FB_ERR_UNSUPPORTED_SHAPE;   // (no gate within the limits has more columns per lane)
+  const size_t optin = static_cast<size_t>(prop.sharedMemPerBlockOptin) - 2048 - 1024;
+  const size_t stage_bytes = fb::kATileBytes + static_cast<size_t>(ctx->N / 2) * fb::kBlockK * 2;
+  auto depth = [&](size_t bytes) {
+    const int n = static_cast<int>(bytes / stage_bytes);
+    return n > fb::kMaxStages ? fb::kMaxStages : n;
+  };
+  for (int w = 0; w < 2; ++w)
+    ctx->ranking[w] = fb::ranking_gate(c.E, c.k, c.gate, g.n_group, g.topk_group,
+                                       w != 0 && !c.renorm && c.gate == FB_GATE_SOFTMAX_TOPK);
+  if (ctx->ranking[0]) {
+    size_t budget = optin - sizeof(fb::RouterShared);
+    ctx->stages = depth(budget);
+    size_t dyn = ctx->stages * stage_bytes;
     if (dyn < fb::epilogue_scratch_bytes(ctx->N)) dyn = fb::epilogue_scratch_bytes(ctx->N);
-    if (stages < 2 || dyn + 1024 > budget) {
-      if (pair == 0) return FB_ERR_UNSUPPORTED_SHAPE;
-      stages = 0;                                      // pair kernel not usable for this shape
-    }
-    ctx->stages[pair] = stages;
-    ctx->smem_bytes[pair] = dyn + 1024;
+    ctx->smem_bytes = dyn + 1024;
+    if (ctx->stages < 2 || dyn > budget) return FB_ERR_UNSUPPORTED_SHAPE;
+    budget = optin - sizeof(fb::PersistShared);
+    ctx->persist_stages = depth(budget - fb::kPersistScratchBytes);
+    ctx->persist_smem = ctx->persist_stages * stage_bytes + fb::kPersistScratchBytes + 1024;
+    if (ctx->persist_stages < 2) return FB_ERR_UNSUPPORTED_SHAPE;
   }
-  ctx->max_tiles = (cfg.T_max + fb::kTileM - 1) / fb::kTileM;
+  // one tile per pair: the staged logits reuse the ring
+  const size_t budget = optin - sizeof(fb::RowsShared);
+  const size_t full_staging = fb::staging_bytes(fb::kTileM, ctx->N);
+  ctx->rows_stages[0] = depth(budget);
+  size_t dyn = ctx->rows_stages[0] * stage_bytes;
+  if (dyn < full_staging) dyn = full_staging;
+  if (ctx->rows_stages[0] < 2 || dyn > budget) return FB_ERR_UNSUPPORTED_SHAPE;
+  ctx->rows_smem[0] = dyn + 1024;
+  // several tiles per pair: staging of its own behind the ring, as many rows at a time as leave five
+  // stages (128 rows of up to 144 columns, 32 rows of 256)
+  for (int rows = fb::kTileM; rows >= 32; rows /= 2) {
+    const size_t staging = fb::staging_bytes(rows, ctx->N);
+    ctx->rows_stages[1] = depth(budget - staging);
+    dyn = ctx->rows_stages[1] * stage_bytes + staging;
+    if (dyn < full_staging) dyn = full_staging;                  // the last tile stages all rows over the ring
+    ctx->rows_smem[1] = dyn + 1024;
+    g.chunk_rows = rows;
+    if (ctx->rows_stages[1] >= 5) break;
+  }
+  if (ctx->rows_stages[1] < 2) return FB_ERR_UNSUPPORTED_SHAPE;
+  ctx->max_tiles = (c.T_max + fb::kTileM - 1) / fb::kTileM;
   ctx->n_sm = prop.multiProcessorCount;
   return FB_OK;
 }
@@ -490,19 +493,49 @@ static fb_status ensure_kernel_attributes(int device, const cudaDeviceProp& prop
     const int most = static_cast<int>(prop.sharedMemPerBlockOptin) - static_cast<int>(fa.sharedSizeBytes);
     ok = ok && most > 0 &&
          cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
-             cudaSuccess;
+             cudaSuccess &&
+         cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+             cudaSuccess;                                // clusters of 16
   };
-  for (int sel = 0; sel < 3; ++sel)
-    for (int lb = 0; lb < 2; ++lb) {
-      raise(router_kernel_fn<1>(sel, lb != 0));
-      raise(router_kernel_fn<2>(sel, lb != 0));
-      raise(router_split_kernel_fn(sel, lb != 0));
-    }
-  for (int sg = 0; sg < 2; ++sg)
-    for (int lb = 0; lb < 2; ++lb) raise(persistent_kernel_fn(sg != 0, lb != 0));
+  for (int i = 0; i < 4; ++i) {
+    raise(ranking_kernel_fn(i / 2 != 0, i % 2 != 0));
+    raise(persistent_kernel_fn(i / 2 != 0, i % 2 != 0));
+  }
+  for (int i = 0; i < 2 * kRowsKernels; ++i) raise(rows_kernel_fn(i / 2, i % 2 != 0));
   if (!ok) { cudaGetLastError(); return FB_ERR_CUDA; }
   if (device >= 0 && device < 64) done[device] = true;
   return FB_OK;
+}
+
+// How many clusters of 2, 4, 8 and 16 blocks the GPU holds at once.  Counted for the row-per-warp kernel
+// at the largest shared memory of this shape's launches (one block per SM either way).
+static fb_status count_clusters(fb_ctx* ctx) {
+  cudaLaunchConfig_t occ;
+  memset(&occ, 0, sizeof(occ));
+  occ.blockDim = dim3(fb::kRouterThreads, 1, 1);
+  occ.dynamicSmemBytes = ctx->rows_smem[0] > ctx->rows_smem[1] ? ctx->rows_smem[0] : ctx->rows_smem[1];
+  cudaLaunchAttribute cl[1];
+  cl[0].id = cudaLaunchAttributeClusterDimension;
+  occ.attrs = cl;
+  occ.numAttrs = 1;
+  for (int l = 0; l < 4; ++l) {
+    cl[0].val.clusterDim.x = 2u << l; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
+    occ.gridDim = dim3((2u << l) * static_cast<unsigned>(ctx->n_sm), 1, 1);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, rows_kernel_fn(ctx->rows_kernel, ctx->cfg.gate == FB_GATE_SIGMOID_GROUP_TOPK),
+                                       &occ) != cudaSuccess)
+      n = 0;
+    ctx->max_clusters[l] = n;
+  }
+  cudaGetLastError();
+  return ctx->max_clusters[0] >= 1 ? FB_OK : FB_ERR_CUDA;
+}
+
+// Rows of the histogram table: a launch that cuts its tiles into slices has at most one slice per SM
+// (see launch_router), any other one per tile.
+static size_t max_slices(const fb_ctx* ctx) {
+  const size_t tiles = static_cast<size_t>(ctx->max_tiles), sliced = static_cast<size_t>(ctx->n_sm) + 8;
+  return tiles > sliced ? tiles : sliced;
 }
 
 extern "C" {
@@ -553,17 +586,6 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
     if (ss == FB_OK) ss = ensure_kernel_attributes(device, prop);
     if (ss != FB_OK) { delete ctx; return ss; }
   }
-  if (ctx->stages[1] >= 2 && ctx->N % 32 == 0 && ctx->N == cfg->E) {
-    const size_t budget_p = static_cast<size_t>(prop.sharedMemPerBlockOptin) - sizeof(fb::PersistShared) - 2048;
-    const size_t stage_bytes = fb::kATileBytes + static_cast<size_t>(ctx->N / 2) * fb::kBlockK * 2;
-    if (budget_p > 1024 + fb::kPersistScratchBytes + 2 * stage_bytes) {
-      int stages = static_cast<int>((budget_p - 1024 - fb::kPersistScratchBytes) / stage_bytes);
-      if (stages > fb::kMaxStages) stages = fb::kMaxStages;
-      ctx->persist_stages = stages;
-      ctx->persist_smem = stages * stage_bytes + fb::kPersistScratchBytes + 1024;
-    }
-  }
-
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
   if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
@@ -572,54 +594,10 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
     return FB_ERR_CUDA;
   }
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
-  bool ok = true;
-  if (ctx->persist_stages >= 2) {
-    // how many block pairs the GPU holds at once (the grid of the persistent kernel)
-    cudaLaunchConfig_t occ;
-    memset(&occ, 0, sizeof(occ));
-    occ.gridDim = dim3(2 * static_cast<unsigned>(prop.multiProcessorCount), 1, 1);
-    occ.blockDim = dim3(fb::kRouterThreads, 1, 1);
-    occ.dynamicSmemBytes = ctx->persist_smem;
-    cudaLaunchAttribute cl[1];
-    cl[0].id = cudaLaunchAttributeClusterDimension;
-    cl[0].val.clusterDim.x = 2; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
-    occ.attrs = cl;
-    occ.numAttrs = 1;
-    int n_clusters = 0;
-    if (ok && cudaOccupancyMaxActiveClusters(&n_clusters, persistent_kernel_fn(cfg->gate == FB_GATE_SIGMOID_GROUP_TOPK, false),
-                                             &occ) == cudaSuccess &&
-        n_clusters >= 1)
-      ctx->max_pairs = n_clusters;
-    else
-      ctx->persist_stages = 0;                           // not usable here: the one-tile kernel serves every call
-    cudaGetLastError();
-  }
-  if (ctx->stages[1] >= 2) {
-    // block pairs of the one-tile pair kernel that the GPU holds at once: the grid of a split launch
-    cudaLaunchConfig_t occ;
-    memset(&occ, 0, sizeof(occ));
-    occ.gridDim = dim3(2 * static_cast<unsigned>(prop.multiProcessorCount), 1, 1);
-    occ.blockDim = dim3(fb::kRouterThreads, 1, 1);
-    occ.dynamicSmemBytes = ctx->smem_bytes[1];
-    cudaLaunchAttribute cl[1];
-    cl[0].id = cudaLaunchAttributeClusterDimension;
-    cl[0].val.clusterDim.x = 2; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
-    occ.attrs = cl;
-    occ.numAttrs = 1;
-    int n_clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&n_clusters, router_split_kernel_fn(0, false), &occ) == cudaSuccess &&
-        n_clusters >= 2) {
-      ctx->split_pairs = n_clusters;
-      const size_t slots = static_cast<size_t>(n_clusters);          // one partial per helper item, at most
-      ok = ok && dev_alloc(&ctx->split_partial, slots * 2 * ctx->N * fb::kTileM) &&
-           dev_alloc(&ctx->split_flags, slots * 2) &&
-           cudaMemset(ctx->split_flags, 0, slots * 2 * sizeof(uint32_t)) == cudaSuccess;
-    }
-    cudaGetLastError();
-  }
+  bool ok = count_clusters(ctx) == FB_OK;
   ok = ok && dev_alloc(&ctx->counts_scratch, FB_MAX_EXPERTS) && dev_alloc(&ctx->ticket, 1) &&
        dev_alloc(&ctx->status, 1) &&
-       dev_alloc(&ctx->slice_counts, static_cast<size_t>(ctx->max_tiles) * fb::slice_row_bytes(cfg->E));
+       dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E));
   ok = ok && cudaMemset(ctx->counts_scratch, 0, FB_MAX_EXPERTS * sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->ticket, 0, sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess;
@@ -632,8 +610,7 @@ fb_status fb_destroy(fb_ctx* ctx) {
   if (!ctx) return FB_OK;
   DeviceGuard guard(ctx->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {ctx->split_partial, ctx->split_flags,
-                  ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->st_hprev, ctx->st_H,
+  void* ptrs[] = {ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->st_hprev, ctx->st_H,
                   ctx->st_pi, ctx->st_pi_out, ctx->st_counts, ctx->st_swaps, ctx->st_nswaps, ctx->st_load_before,
                   ctx->st_load_after, ctx->st_ids, ctx->st_w, ctx->st_slot_offsets, ctx->st_rank_offsets,
                   ctx->st_perm, ctx->st_inv_perm, ctx->st_rank_load};
@@ -719,10 +696,11 @@ fb_status fb_route_dispatch(fb_ctx* ctx, const fb_router* router, const void* x,
       return FB_ERR_CUDA;
     return FB_OK;
   }
+  int pieces = 1;
   const fb_status st = launch_router(ctx, router, x, T, fb::kModeDispatch, nullptr, topk_ids, topk_w, logits,
-                                     nullptr, stream);
+                                     nullptr, stream, nullptr, 0, &pieces);
   if (st != FB_OK) return st;
-  return launch_dispatch_index(ctx, T, expert_to_slot, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
+  return launch_dispatch_index(ctx, T, pieces, expert_to_slot, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
                                rank_load, stream);
 }
 
@@ -753,9 +731,10 @@ fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
   // one launch for both router passes; the dispatch index needs the new placement and follows
-  st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, nullptr, &pp, stream, H);
+  int pieces = 1;
+  st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, nullptr, &pp, stream, H, 0, &pieces);
   if (st != FB_OK) return st;
-  return launch_dispatch_index(ctx, T, expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
+  return launch_dispatch_index(ctx, T, pieces, expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
                                rank_load, stream);
 }
 
@@ -832,10 +811,6 @@ fb_status fb_device_status(fb_ctx* ctx, int32_t* word, fb_stream stream_) {
   if (cudaMemcpy(word, ctx->status, sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess) return FB_ERR_CUDA;
   if (*word != 0) {
     if (cudaMemset(ctx->status, 0, sizeof(int32_t)) != cudaSuccess) return FB_ERR_CUDA;
-    // a launch that gave up may have left partial-tile flags of the k-range split set: re-arm them
-    if (ctx->split_flags != nullptr &&
-        cudaMemset(ctx->split_flags, 0, static_cast<size_t>(ctx->split_pairs) * 2 * sizeof(uint32_t)) != cudaSuccess)
-      return FB_ERR_CUDA;
   }
   return FB_OK;
 }
@@ -1021,8 +996,7 @@ fb_status fb_topk_hits(const int32_t* ids_a, const int32_t* ids_b, int32_t T, in
 
 fb_status fb_set_split(fb_ctx* ctx, int32_t mode, int32_t owner_bias_kblocks) {
   if (!ctx || (mode != 0 && mode != 1) || owner_bias_kblocks < -1 || owner_bias_kblocks > 1024) return FB_ERR_INVALID_ARG;
-  ctx->split_mode = mode;
-  ctx->split_bias = owner_bias_kblocks;
+  ctx->split_mode = mode;      // (the pieces of a tile's k-range are equal: there is no owner to favour)
   return FB_OK;
 }
 
@@ -1047,8 +1021,7 @@ fb_status fb_time_next_router_launch(fb_ctx* ctx, void* event_before, void* even
 
 fb_status fb_router_floor(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T, int32_t what,
                           fb_stream stream_) {
-  if (!ctx || !router || !router->W || !x || T <= 0 || (what != 1 && what != 2
-       )) return FB_ERR_INVALID_ARG;
+  if (!ctx || !router || !router->W || !x || T <= 0 || (what != 1 && what != 2)) return FB_ERR_INVALID_ARG;
   if (T > ctx->cfg.T_max) return FB_ERR_UNSUPPORTED_SHAPE;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
@@ -1056,7 +1029,7 @@ fb_status fb_router_floor(fb_ctx* ctx, const fb_router* router, const void* x, i
                        static_cast<cudaStream_t>(stream_), nullptr, what);
 }
 
-int32_t fb_max_pairs(const fb_ctx* ctx) { return ctx ? ctx->max_pairs : 0; }
+int32_t fb_max_pairs(const fb_ctx* ctx) { return ctx && ctx->ranking[0] ? ctx->max_clusters[0] : 0; }
 
 fb_status fb_dispatch_slot_counts(fb_ctx* ctx, const uint32_t* slot_offsets, uint32_t* slot_counts, fb_stream stream_) {
   if (!ctx || !slot_offsets || !slot_counts) return FB_ERR_INVALID_ARG;
@@ -1284,7 +1257,9 @@ extern "C" fb_status fb_predict_load_static(const fb_config* cfg, int device, co
     ctx.cfg = *cfg;
     fb_status ss = setup_router_shape(&ctx, prop);
     if (ss == FB_OK) ss = ensure_kernel_attributes(device, prop);
+    if (ss == FB_OK) ss = count_clusters(&ctx);
     if (ss != FB_OK) { ctx.cfg.E = -1; return ss; }
+    ctx.split_mode = 0;                                  // the sums of an unsplit call, whatever the shape
     for (int i = 0; i < kMapCache; ++i) { ctx.x_maps[i] = MapEntry(); ctx.w_maps[i] = MapEntry(); }
   }
   ctx.counts_scratch = st.scratch;

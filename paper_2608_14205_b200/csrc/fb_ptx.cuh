@@ -24,15 +24,9 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // Arrive on the barrier at the same shared-memory offset in another CTA of the cluster.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t cta_rank) {
@@ -119,19 +113,8 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-// 2-D tile load global -> shared (this CTA), completion counted in bytes on `bar`.
-// c0 is the innermost (contiguous) coordinate; c0 * element size must be a multiple of 16.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint32_t bar,
-                                            int32_t c0, int32_t c1, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "l"(policy)
-      : "memory");
-}
-
-// Pair version (two CTAs of a cluster feed one MMA): the data lands in the executing
-// CTA's shared memory, the byte count is reported to `bar`, which may be a barrier of
+// 2-D tile load global -> shared for a pair of CTAs that feed one MMA.  c0 is the innermost (contiguous)
+// coordinate; c0 * element size must be a multiple of 16.  The data lands in the executing CTA's shared memory, the byte count is reported to `bar`, which may be a barrier of
 // the other CTA (a shared::cluster address).  No multicast: each CTA loads its own tiles.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* tmap, uint32_t bar,
                                                  int32_t c0, int32_t c1, uint64_t policy) {
@@ -212,12 +195,7 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
         : "memory");
 }
 
-// Make `bar` (in this CTA) complete once all MMAs issued so far by this thread are done.
-__device__ __forceinline__ void umma_commit_1cta(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-// Pair version: make the barrier at this offset complete in BOTH blocks of the pair once all
+// Make the barrier at this offset complete in BOTH blocks of the pair once all
 // MMAs issued so far by this thread are done.  Two plain commits - one to this block's
 // barrier, one to the partner's (its shared::cluster address) - rather than one commit with a
 // cluster-wide destination mask.
@@ -242,7 +220,7 @@ __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -251,6 +229,59 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)
         "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
+}
+// Four words to shared memory.
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// Words from this block's shared memory.
+__device__ __forceinline__ float ld_shared_float(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+template <int kN>
+__device__ __forceinline__ void ld_shared_floats(uint32_t addr, float (&v)[kN]) {
+  if constexpr (kN == 1) {
+    v[0] = ld_shared_float(addr);
+  } else if constexpr (kN == 2) {
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(addr) : "memory");
+  } else {
+#pragma unroll
+    for (int i = 0; i < kN; i += 4)
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(v[i]), "=f"(v[i + 1]), "=f"(v[i + 2]), "=f"(v[i + 3]) : "r"(addr + 4u * i) : "memory");
+  }
+}
+// Words from the shared memory of a block of the cluster (a shared::cluster address).
+__device__ __forceinline__ float ld_cluster_float(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+template <int kN>
+__device__ __forceinline__ void ld_cluster_floats(uint32_t addr, float (&v)[kN]) {
+  if constexpr (kN == 1) {
+    v[0] = ld_cluster_float(addr);
+  } else if constexpr (kN == 2) {
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(addr) : "memory");
+  } else {
+#pragma unroll
+    for (int i = 0; i < kN; i += 4)
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(v[i]), "=f"(v[i + 1]), "=f"(v[i + 2]), "=f"(v[i + 3]) : "r"(addr + 4u * i) : "memory");
+  }
+}
+// Largest / smallest of a float over the warp.
+__device__ __forceinline__ float redux_max_f32(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float redux_min_f32(float x) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
 }
 // Both 32-bit words to shared memory when pred != 0; a predicated store, not a branch.
 __device__ __forceinline__ void st_shared_v2_if(uint32_t pred, uint32_t addr, uint32_t lo, uint32_t hi) {

@@ -49,20 +49,6 @@ struct PersistShared {
   PlanShared plan;
 };
 
-// Host-side test of the gate shapes this kernel supports (same rule as the ranking
-// selection of fb_router_kernel, without the cases that need the softmax denominator).
-__host__ __device__ inline bool persistent_gate_ok(int E, int k, int gate, int n_group, int topk_group,
-                                                   bool want_sum) {
-  if (E % 32 != 0 || E / 32 > kPersistGroups) return false;
-  if (gate != FB_GATE_SOFTMAX_TOPK)
-    return E / n_group == 32 && topk_group <= kEpiSubs && topk_group * 2 >= k;
-  return (E / 32) * 2 >= k && !want_sum;
-}
-
-__device__ __forceinline__ void ring_advance(int& s, uint32_t& phase, int stages) {
-  if (++s == stages) { s = 0; phase ^= 1u; }
-}
-
 // kSigmoid: sigmoid + bias group-limited gate (true) or softmax gate (false); kLogitBias: a logit
 // bias is given.  One instance per combination keeps code and registers to what it needs.
 template <bool kSigmoid, bool kLogitBias>
@@ -272,7 +258,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           if (two_acc) {                                     // add the odd k-blocks' accumulator
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-              uint32_t r2[32];
+              uint32_t r2[16];
               tmem_ld_32x32b_x16(taddr + N + c * 32 + 16 * h, r2);
               tmem_ld_wait();
 #pragma unroll
@@ -448,7 +434,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       const bool writer = valid && sub == 0;
       if (writer) {
         // softmax gates reach this kernel only with renormalised weights: no denominator needed
-        write_row_outputs(top, p, row, out_ids, out_w, sh.select_bias, 0.0f, 1.0f);
+        write_row_outputs(top, p, row, out_ids, out_w, sh.select_bias);
         // ---------------- histogram (Eq. 5)
 #pragma unroll
         for (int j = 0; j < FB_MAX_TOPK; ++j)

@@ -1,0 +1,798 @@
+// Fused router kernel for calls with few tiles and for gates that the ranking selection does not
+// serve: logits = x W^T (+ b) as in fb_router_kernel, then a WARP per token row for gating and top-k.
+//
+// Work split.  Two blocks of a cluster (a pair) compute a tile pair: 256 token rows x all N = pad16(E)
+// expert columns with one cta_group::2 MMA; each loads its own 128 rows of x and half of the W tile.
+//   * Few tile pairs: a cluster of 2 J blocks (J = 2, 4, 8 pairs) works on ONE tile pair.  Pair j
+//     accumulates the j-th piece of the k-range; the J partial tiles meet through distributed shared
+//     memory, and each block finishes 128 / J of its rows.  Both the stream of operands and the
+//     selection work are then spread over J times as many SMs, and nothing but a cluster barrier lies
+//     between the two.
+//   * More tile pairs than pairs fit on the GPU: every pair walks a strided list of tile pairs, and
+//     the selection of one tile runs while the tensor cores already work on the next one.
+// Warp roles as in fb_router_kernel.
+//
+// Epilogue.  The 16 epilogue warps copy the sums from tensor memory (one row per thread) to shared
+// memory row by row ("staging", rows padded by 16 bytes: conflict-free both ways), and from there on a
+// warp owns a token row: the lanes hold its keys in registers, group scores and bounds are formed by a
+// few shuffles and warp reductions, the keys that can still enter the top-k (about 10 of 256) are
+// compacted into a short list and ranked there.  Any gate fits the same code, no barrier separates the
+// steps, and a tile cut into J row slices keeps the warps busy.  It costs more instructions per row than
+// the ranking selection with one row per thread where that one has whole tiles to itself (16384 rows x 256
+// columns, d = 512, sigmoid groups: 21.6 against 18.1 us per prediction pass; 128 columns, softmax: 16.0
+// against 15.3), so those launches stay there; against the insertion code that other gates had before it
+// is faster throughout (64 experts, sigmoid without groups: 25.9 -> 14.9 us).
+#pragma once
+#include <stddef.h>
+
+#include "fb_router.cuh"
+
+namespace fb {
+
+// How a gate's columns lie over the lanes (host).  Returns the number of columns a lane holds, rounded up
+// to a power of two (the kernel instance), at most 16.
+inline int gate_layout(int E, int gate, int n_group, int topk_group, RouterParams* p) {
+  const bool restricted = gate != FB_GATE_SOFTMAX_TOPK && topk_group < n_group;
+  const int groups = restricted ? n_group : 1, gs = E / groups;
+  int lpg = 1;
+  while (lpg * 2 * groups <= 32) lpg *= 2;
+  const int per_lane = (gs + lpg - 1) / lpg;
+  int cpl = 1;
+  while (cpl < per_lane) cpl *= 2;
+  p->groups = groups;
+  p->group_size = gs;
+  p->keep_groups = restricted ? topk_group : 1;
+  p->lanes_per_group = lpg;
+  // one group, or whole vectors per group: round the lane's share up so that it is one vector load
+  p->vector_load = (groups == 1 || gs % cpl == 0) ? 1 : 0;
+  p->cols_per_lane = p->vector_load ? cpl : per_lane;
+  p->ragged = !(p->vector_load && groups * lpg * cpl == E && groups * lpg == 32) ? 1 : 0;
+  return cpl;
+}
+
+// Staged logits: rows of N + 4 floats.  A warp writes 32 rows of one 16-byte column group at a time, 8
+// rows per wavefront: N is a multiple of 16, so the row stride is 4 or 20 words modulo 32 and those 8 rows
+// hit all 32 banks once.
+__host__ __device__ constexpr int staging_stride(int N) { return N + 4; }
+constexpr int kListStride = kCandCap + 12;     // + the last lane's columns, rounded up (never read); 12 banks apart for two rows
+struct RowScratch {                    // one per epilogue warp
+  alignas(16) float cand_key[2][kListStride];  // keys of two rows' candidates in ascending id order; -inf behind the last one
+  alignas(16) int32_t cand_id[2][kListStride];
+  alignas(16) float win_key[8][FB_MAX_TOPK];   // the rows' top-k in order of rank
+  alignas(16) int32_t win_id[8][FB_MAX_TOPK];
+  float row_sum[8];                            // softmax denominators relative to the row's largest key
+};
+__host__ __device__ constexpr size_t staging_bytes(int rows, int N) {
+  return static_cast<size_t>(rows) * staging_stride(N) * 4 + kEpilogueWarps * sizeof(RowScratch);
+}
+
+struct RowsShared {
+  uint64_t full_bar[kMaxStages];
+  uint64_t empty_bar[kMaxStages];
+  // Accumulator sets: one (2 N of the 512 tensor-memory columns) or, when 4 N <= 512 and a pair walks
+  // several tiles, two that alternate, so that the next tile's MMAs need not wait for the drain.
+  uint64_t accum_bar[2];                     // per set: both issuers' commits, once per use
+  uint64_t tmem_empty_bar[2];                // per set, even block's copy: all epilogue warps of the pair, once per use
+  uint32_t tmem_base;
+  int32_t abort_flag;
+  int32_t is_last;
+  int32_t accum_ok;
+  int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
+  alignas(16) float logit_bias[FB_MAX_EXPERTS];
+  alignas(16) float select_bias[FB_MAX_EXPERTS];
+  alignas(16) uint32_t hist[FB_MAX_EXPERTS];
+  PlanShared plan;
+};
+
+// ---------------------------------------------------------------- selection, one warp per token row
+// What a lane needs to know about its columns.
+struct LaneColumns {
+  int32_t c0, n;                       // first column, number of columns
+  int32_t group;                       // group of its columns (>= groups: an idle lane)
+};
+
+// Plain selection of one row by repeated maximum over keys in shared memory (dropped columns hold
+// -inf): the path of rows with more candidates than the list holds, and of rows with equal keys among
+// the candidates (the lower expert id wins).  Rare; kept out of line.
+__device__ __noinline__ void select_slow(float* keys, int E, int k, float* win_key, int32_t* win_id, int lane) {
+  for (int r = 0; r < k; ++r) {
+    float best = -INFINITY;
+    int at = E;
+    for (int e = lane; e < E; e += 32)
+      if (keys[e] > best) { best = keys[e]; at = e; }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int oa = __shfl_xor_sync(0xffffffffu, at, off);
+      if (ob > best || (ob == best && oa < at)) { best = ob; at = oa; }
+    }
+    if (at >= E) break;                                     // nothing left (keys that are no numbers): the defaults stay
+    if (lane == 0) { win_key[r] = best; win_id[r] = at; keys[at] = -INFINITY; }
+    __syncwarp();
+  }
+}
+
+// A lane's columns of one staged row of this block / of the block with cluster rank `rank` at the same
+// place.  Lanes without columns read valid words all the same; what they read is masked afterwards.
+template <int kCpl>
+__device__ __forceinline__ void load_columns(float (&z)[kCpl], uint32_t addr, const RouterParams& p, int n) {
+  if (kCpl == 1 || p.vector_load) {
+    ld_shared_floats<kCpl>(addr, z);
+  } else {
+#pragma unroll
+    for (int j = 0; j < kCpl; ++j) z[j] = ld_shared_float(addr + 4 * max(0, min(j, n - 1)));
+  }
+}
+template <int kCpl>
+__device__ __forceinline__ void load_columns_of(float (&z)[kCpl], uint32_t addr, uint32_t rank, const RouterParams& p, int n) {
+  const uint32_t remote = map_to_cta(addr, rank);
+  if (kCpl == 1 || p.vector_load) {
+    ld_cluster_floats<kCpl>(remote, z);
+  } else {
+#pragma unroll
+    for (int j = 0; j < kCpl; ++j) z[j] = ld_cluster_float(remote + 4 * max(0, min(j, n - 1)));
+  }
+}
+
+// r += a > b
+__device__ __forceinline__ void count_greater(int& r, float a, float b) {
+  asm("{\n.reg .pred p;\nsetp.gt.f32 p, %1, %2;\n@p add.s32 %0, %0, 1;\n}" : "+r"(r) : "f"(a), "f"(b));
+}
+// key >= bound: key and id to the lists at `slot`, which moves on (predicated, no branch)
+__device__ __forceinline__ void append_candidate(uint32_t& slot, float key, float bound, int id) {
+  constexpr int kIdOffset = static_cast<int>(offsetof(RowScratch, cand_id) - offsetof(RowScratch, cand_key));
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ge.f32 p, %1, %2;\n@p st.shared.f32 [%0], %1;\n@p st.shared.u32 [%0 + %4], %3;\n"
+      "@p add.u32 %0, %0, 4;\n}"
+      : "+r"(slot) : "f"(key), "f"(bound), "r"(id), "n"(kIdOffset) : "memory");
+}
+
+// Softmax denominator of a row relative to its largest key, for weights without renormalisation.
+template <int kCpl>
+__device__ __forceinline__ float row_exp_sum(const float (&key)[kCpl], float lane_max) {
+  const float top = redux_max_f32(lane_max);
+  float s = 0.0f;
+#pragma unroll
+  for (int j = 0; j < kCpl; ++j) s += __expf(key[j] - top);                 // exp(-inf) = 0 for missing columns
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  return s;
+}
+
+// The top-k of two staged rows (row_addr: shared-memory address of the first one's first word in this block;
+// the J blocks whose cluster ranks are first_rank + 2 i hold one partial sum each at the same place) into
+// rows 2 pair and 2 pair + 1 of the scratch's result lists.  row: token index of the first one.
+// Two rows at a time because a row's steps are a chain of short dependent ones.
+template <int kCpl, bool kSigmoid>
+__device__ __forceinline__ void select_two_rows(const RouterParams& p, const LaneColumns& lc, const float (&sb)[kCpl],
+                                                const float* logit_bias_s, uint32_t row_addr, uint32_t first_rank,
+                                                long long row, RowScratch& rs, int pair, int lane) {
+  const uint32_t full = 0xffffffffu;
+  const uint32_t stride = static_cast<uint32_t>(staging_stride(p.N)) * 4u;
+  const bool want_sum = !kSigmoid && p.topk_w != nullptr && !p.renorm;
+  float key[2][kCpl];
+  // ---- logits: the J partial sums in order
+  const uint32_t a0 = row_addr + static_cast<uint32_t>(lc.c0) * 4u;
+  if (p.pieces == 1) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) load_columns<kCpl>(key[u], a0 + u * stride, p, lc.n);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) load_columns_of<kCpl>(key[u], a0 + u * stride, first_rank, p, lc.n);
+#pragma unroll (kCpl >= 8 ? 1 : 3)
+    for (int i = 1; i < p.pieces; ++i) {
+      float t[2][kCpl];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) load_columns_of<kCpl>(t[u], a0 + u * stride, first_rank + 2u * i, p, lc.n);
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int j = 0; j < kCpl; ++j) key[u][j] += t[u][j];
+    }
+  }
+  if (p.logit_bias != nullptr) {
+#pragma unroll
+    for (int j = 0; j < kCpl; ++j) {
+      const float b = logit_bias_s[lc.c0 + max(0, min(j, lc.n - 1))];
+      key[0][j] += b;
+      key[1][j] += b;
+    }
+  }
+  if (p.logits != nullptr) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j)
+        if (j < lc.n && row + u < p.T) p.logits[(row + u) * p.E + lc.c0 + j] = key[u][j];
+  }
+  // ---- selection keys
+  if (kSigmoid) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j) key[u][j] = fb_sigmoid(key[u][j]) + sb[j];
+  }
+  if (p.ragged) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j) key[u][j] = j < lc.n ? key[u][j] : -INFINITY;
+  }
+  // ---- groups: score = sum of the two largest keys (the only key of a one-expert group); the best
+  // keep_groups are kept, a lower-numbered group wins ties
+  float bound[2];                                            // lower bound for the k-th key; +inf in a lane of a dropped group
+  const bool bound_from_groups = p.groups > 1 && p.keep_groups * (p.group_size >= 2 ? 2 : 1) >= p.k;
+  bool kept[2] = {true, true};
+  if (p.groups > 1) {
+    float m1[2], m2[2];                                      // the lane's, then the group's two largest keys
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (kCpl == 1) {
+        m1[u] = key[u][0];
+        m2[u] = -INFINITY;
+      } else {
+        float t1[kCpl / 2 + 1], t2[kCpl / 2 + 1];
+#pragma unroll
+        for (int j = 0; j < kCpl / 2; ++j) {
+          t1[j] = fmaxf(key[u][2 * j], key[u][2 * j + 1]);
+          t2[j] = fminf(key[u][2 * j], key[u][2 * j + 1]);
+        }
+#pragma unroll
+        for (int w = kCpl / 4; w >= 1; w >>= 1)
+#pragma unroll
+          for (int j = 0; j < w; ++j) {
+            t2[j] = fmaxf(fmaxf(fminf(t1[j], t1[j + w]), t2[j]), t2[j + w]);
+            t1[j] = fmaxf(t1[j], t1[j + w]);
+          }
+        m1[u] = t1[0];
+        m2[u] = t2[0];
+      }
+    }
+    for (int off = 1; off < p.lanes_per_group; off <<= 1) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float o1 = __shfl_xor_sync(full, m1[u], off), o2 = __shfl_xor_sync(full, m2[u], off);
+        m2[u] = fmaxf(fmaxf(fminf(m1[u], o1), m2[u]), o2);
+        m1[u] = fmaxf(m1[u], o1);
+      }
+    }
+    if (p.group_size == 1) { m2[0] = m1[0]; m2[1] = m1[1]; }     // the smallest known key of the group
+    float score[2];
+    int rank[2] = {0, 0};
+    const bool in_group = lc.group < p.groups;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) score[u] = in_group ? (p.group_size >= 2 ? m1[u] + m2[u] : m1[u]) : -INFINITY;
+    const int lanes = p.groups * p.lanes_per_group;
+    int src = lane;
+    for (int h = 1; h < p.groups; ++h) {
+      src += p.lanes_per_group;
+      if (src >= lanes) src -= lanes;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) count_greater(rank[u], __shfl_sync(full, score[u], src), score[u]);
+    }
+    const int keep_lanes = p.keep_groups * p.lanes_per_group;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) kept[u] = in_group && rank[u] < p.keep_groups;
+    const uint32_t b0 = __ballot_sync(full, kept[0]), b1 = __ballot_sync(full, kept[1]);
+    if (__popc(b0) != keep_lanes || __popc(b1) != keep_lanes) {
+      // equal scores (or scores that are no numbers): count again, the lower group first
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        int r = 0;
+        for (int g = 0; g < p.groups; ++g) {
+          const float os = __shfl_sync(full, score[u], g * p.lanes_per_group);
+          r += (os > score[u] || (os == score[u] && g < lc.group)) ? 1 : 0;
+        }
+        kept[u] = in_group && r < p.keep_groups;
+      }
+    }
+    // the kept groups' best (two) keys are known keys: if there are at least k, the smallest bounds the k-th
+    if (bound_from_groups) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) bound[u] = redux_min_f32(kept[u] ? m2[u] : INFINITY);
+    }
+  }
+  if (kCpl == 1) {
+    // one key per lane: k rounds of "largest remaining key", the lowest lane (lowest id) on ties
+    if (want_sum) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float s = row_exp_sum<kCpl>(key[u], key[u][0]);
+        if (lane == 0) rs.row_sum[2 * pair + u] = s;
+      }
+    }
+    if (p.groups > 1) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) key[u][0] = kept[u] ? key[u][0] : -INFINITY;
+    }
+    for (int r = 0; r < p.k; ++r) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float top = redux_max_f32(key[u][0]);
+        const uint32_t holders = __ballot_sync(full, key[u][0] == top && top > -INFINITY);
+        if (lane == __ffs(holders) - 1) {
+          rs.win_key[2 * pair + u][r] = top;
+          rs.win_id[2 * pair + u][r] = lc.c0;
+          key[u][0] = -INFINITY;
+        }
+      }
+    }
+    return;
+  }
+  if (!bound_from_groups) {
+    // the k-th largest of the (kept) lanes' largest keys
+    float lane_max[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      lane_max[u] = key[u][0];
+#pragma unroll
+      for (int j = 1; j < kCpl; ++j) lane_max[u] = fmaxf(lane_max[u], key[u][j]);
+      if (p.groups > 1) lane_max[u] = kept[u] ? lane_max[u] : -INFINITY;
+    }
+    if (want_sum) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float s = row_exp_sum<kCpl>(key[u], lane_max[u]);
+        if (lane == 0) rs.row_sum[2 * pair + u] = s;
+      }
+    }
+#pragma unroll 1
+    for (int r = 0; r < p.k; ++r) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        bound[u] = redux_max_f32(lane_max[u]);
+        lane_max[u] = lane_max[u] == bound[u] ? -INFINITY : lane_max[u];
+      }
+    }
+  }
+  // missing columns and dropped groups never qualify
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    bound[u] = fmaxf(bound[u], -3.402823466e38f);
+    if (p.groups > 1) bound[u] = kept[u] ? bound[u] : INFINITY;
+  }
+  // ---- compact the keys at or above the bound, in ascending id order (lanes hold ascending columns):
+  // first every lane's place in the list, then the stores
+  const uint32_t below = (1u << lane) - 1u;
+  const uint32_t list0 = smem_u32(&rs.cand_key[0][0]);
+  int n[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    n[u] = 0;
+#pragma unroll
+    for (int j = 0; j < kCpl; ++j) n[u] += __popc(__ballot_sync(full, key[u][j] >= bound[u]) & below);
+    rs.cand_key[u][lane] = -INFINITY;
+  }
+  __syncwarp();
+  // The last lane starts at most kCandCap entries in and adds at most kCpl: no store leaves the list.
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int last = __shfl_sync(full, n[u], 31);            // candidates before the last lane's
+    if (last <= kListStride - (kCpl > 12 ? kCpl : 12)) {     // (the same for the whole warp)
+      uint32_t slot = list0 + static_cast<uint32_t>(u * kListStride + n[u]) * 4u;
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j) append_candidate(slot, key[u][j], bound[u], lc.c0 + j);
+      n[u] = __shfl_sync(full, static_cast<int>(slot - list0) / 4 - u * kListStride, 31);
+    } else {
+      n[u] = kCandCap + 1;
+    }
+  }
+  __syncwarp();
+  // ---- rank them: lanes 0..15 the first row's, 16..31 the second row's; with more than 16, each lane two
+  const int h = lane >> 4, c = lane & 15;
+  const int most = min(max(n[0], n[1]), kCandCap);
+  const float* list = rs.cand_key[h];
+  uint32_t used = 0;                                         // ranks below k that were found, one bit each
+  const float my0 = list[c];
+  int r0 = 0;
+  if (most <= 16) {
+#pragma unroll 1
+    for (int d = 0; d < most; d += 4) {
+      const float4 o = *reinterpret_cast<const float4*>(list + d);
+      count_greater(r0, o.x, my0); count_greater(r0, o.y, my0); count_greater(r0, o.z, my0); count_greater(r0, o.w, my0);
+    }
+  } else {
+    const float my1 = list[c + 16];
+    int r1 = 0;
+#pragma unroll 1
+    for (int d = 0; d < most; d += 4) {
+      const float4 o = *reinterpret_cast<const float4*>(list + d);
+      count_greater(r0, o.x, my0); count_greater(r0, o.y, my0); count_greater(r0, o.z, my0); count_greater(r0, o.w, my0);
+      count_greater(r1, o.x, my1); count_greater(r1, o.y, my1); count_greater(r1, o.z, my1); count_greater(r1, o.w, my1);
+    }
+    if (my1 > -INFINITY && r1 < p.k) {
+      rs.win_key[2 * pair + h][r1] = my1;
+      rs.win_id[2 * pair + h][r1] = rs.cand_id[h][c + 16];
+      used |= 1u << (8 * h + r1);
+    }
+  }
+  if (my0 > -INFINITY && r0 < p.k) {
+    rs.win_key[2 * pair + h][r0] = my0;
+    rs.win_id[2 * pair + h][r0] = rs.cand_id[h][c];
+    used |= 1u << (8 * h + r0);
+  }
+  // A rank that nobody found means equal keys among the best (or too few candidates): such rows, and
+  // rows whose list overflowed, take the plain path.
+  used = __reduce_or_sync(full, used);
+  const uint32_t want = (1u << p.k) - 1u;
+  if (used != (want | want << 8) || n[0] > kCandCap || n[1] > kCandCap) {
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+      if (((used >> (8 * u)) & 0xffu) == want && (u == 0 ? n[0] : n[1]) <= kCandCap) continue;
+      // scratch: the row's staged words in this block, which nobody else reads (of a shared tile, a block
+      // reads the other blocks' copies of its own slice only)
+      float* keys = reinterpret_cast<float*>(__cvta_shared_to_generic(row_addr + u * stride));
+      __syncwarp();
+      for (int e = lane; e < p.E; e += 32) keys[e] = -INFINITY;
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j)
+        if (j < lc.n && (u == 0 ? kept[0] : kept[1])) keys[lc.c0 + j] = u == 0 ? key[0][j] : key[1][j];
+      __syncwarp();
+      select_slow(keys, p.E, p.k, rs.win_key[2 * pair + u], rs.win_id[2 * pair + u], lane);
+    }
+  }
+}
+
+// Expert ids, routing weights (Eq. 3's top-k with the model's weight rule) and histogram of up to 8 rows,
+// four at a time: lane = (row, rank).
+template <bool kSigmoid>
+__device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& sh, const RowScratch& rs, int n_rows,
+                                            long long row0, int32_t* out_ids, float* out_w, int lane) {
+  const uint32_t full = 0xffffffffu;
+  const int rk = lane & 7;
+  for (int base = 0; base < n_rows; base += 4) {
+    const int i = base + (lane >> 3);
+    const long long row = row0 + i;
+    const bool valid = i < n_rows && row < p.T && rk < p.k;
+    const float key = rs.win_key[i & 7][rk];
+    const int id = valid ? rs.win_id[i & 7][rk] : 0;
+#ifdef FB_DEBUG
+    // what the sanitizer would catch: a chosen expert outside [0, E), a repeated expert
+    {
+      bool bad = id < 0 || id >= p.E;
+      for (int o = 1; o < 8; ++o) {
+        const int other = __shfl_xor_sync(full, valid ? id : -1 - rk, o);
+        bad = bad || (valid && other == id);
+      }
+      if (bad) atomicCAS(p.status, 0, FB_ERR_INTERNAL);
+    }
+#endif
+    if (out_ids != nullptr && valid) out_ids[row * p.k + rk] = id;
+    if (out_w != nullptr) {
+      float w;
+      if (kSigmoid) {
+        w = valid ? key - sh.select_bias[id] : 0.0f;                        // unbiased sigmoid score
+      } else {
+        const float ref = __shfl_sync(full, key, lane & 24);                // row maximum of the keys
+        w = valid ? __expf(key - ref) : 0.0f;
+      }
+      float sum = w;
+      sum += __shfl_xor_sync(full, sum, 1);
+      sum += __shfl_xor_sync(full, sum, 2);
+      sum += __shfl_xor_sync(full, sum, 4);
+      float scale;
+      if (kSigmoid) scale = p.renorm ? p.route_scale / sum : p.route_scale;
+      else scale = 1.0f / (p.renorm ? sum : rs.row_sum[i & 7]);
+      if (valid) out_w[row * p.k + rk] = w * scale;
+    }
+    if (valid) atomicAdd(&sh.hist[id], 1u);
+  }
+}
+
+// kCpl: columns per lane of the selection (gate_layout); kSigmoid: sigmoid + bias gate or softmax gate.
+template <int kCpl, bool kSigmoid>
+__global__ void __launch_bounds__(kRouterThreads, 1)
+fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_x2,
+                      const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ RouterParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ RowsShared sh;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const uint32_t cluster_rank = cluster_ctarank();
+  const uint32_t cta_rank = cluster_rank & 1u;               // which block of its pair
+  const uint32_t lead_rank = cluster_rank & ~1u;             // the pair's even block
+  const int J = p.pieces;
+  const int piece = static_cast<int>(cluster_rank >> 1);
+  const uint32_t stage_bytes = kATileBytes + static_cast<uint32_t>(p.N / 2) * kBlockK * 2;
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzle atoms need 1024-byte alignment
+  volatile int* abort_flag = &sh.abort_flag;
+  FB_STAMP(0, 64);
+
+  // Tile pairs of this cluster: pair_first, pair_first + pair_stride, ...  In kModeLayer the
+  // first pairs_per_pass pairs belong to the early pass, the rest to the normal pass.
+  const int pairs_per_pass = p.tiles_first / 2;
+  const int total_pairs = p.mode == kModeLayer ? 2 * pairs_per_pass : pairs_per_pass;
+  const int pair_first = static_cast<int>(blockIdx.x) / (2 * J);
+  const int pair_stride = static_cast<int>(gridDim.x) / (2 * J);
+  const bool several_tiles = pair_stride < total_pairs;
+  // k-blocks of this pair
+  const int kb0 = p.num_kb * piece / J, n_kb = p.num_kb * (piece + 1) / J - kb0;
+
+  if (threadIdx.x == 0) {
+    sh.abort_flag = 0;
+    sh.is_last = 0;
+    sh.issuer_progress[0] = -1;
+    sh.issuer_progress[1] = -1;
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(smem_u32(&sh.full_bar[s]), 1);
+      mbar_init(smem_u32(&sh.empty_bar[s]), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(smem_u32(&sh.accum_bar[a]), 2);              // one commit per MMA issuer
+      mbar_init(smem_u32(&sh.tmem_empty_bar[a]), 2 * kEpilogueWarps);
+    }
+    fence_mbar_init();
+    prefetch_tensormap(&tmap_x);
+    if (p.mode == kModeLayer) prefetch_tensormap(&tmap_x2);
+    prefetch_tensormap(&tmap_w);
+  }
+  if (warp == 1) {
+    tmem_alloc<2>(smem_u32(&sh.tmem_base), static_cast<uint32_t>(p.tmem_cols));
+    tmem_relinquish<2>();
+  }
+  if (warp >= 2) {
+    const int et = threadIdx.x - 64;
+    for (int e = et; e < FB_MAX_EXPERTS; e += kEpilogueThreads) sh.hist[e] = 0;
+    if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_clear(sh.plan, et, kEpilogueThreads);
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  cluster_arrive(); cluster_wait();          // the other blocks' barriers and tensor memory are ready too
+  tcgen05_fence_after();
+  // (see fb_router_kernel for these two)
+  pdl_wait();
+  pdl_launch_dependents();
+  const uint32_t tmem_base = sh.tmem_base;
+  FB_STAMP(1, 64);
+  bool closing_arrived = false;              // this warp has delivered its arrival for the closing cluster barrier
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ TMA producer
+    if (lane == 0) {
+      const uint64_t pol_x = l2_policy_evict_first();        // x is streamed once
+      const uint64_t pol_w = l2_policy_evict_last();         // W is re-read by every pair
+      int s = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int pt = pair_first; pt < total_pairs && ok; pt += pair_stride) {
+        const bool second_pass = pt >= pairs_per_pass;
+        const int tile = 2 * (second_pass ? pt - pairs_per_pass : pt) + static_cast<int>(cta_rank);
+        const CUtensorMap* xmap = second_pass ? &tmap_x2 : &tmap_x;
+        for (int kb = kb0; kb < kb0 + n_kb; ++kb) {
+          ok = mbar_wait<true>(smem_u32(&sh.empty_bar[s]), phase ^ 1u, abort_flag);
+          if (!ok) break;
+          if (kb == kb0) FB_STAMP(14, 0);
+          if (kb == kb0 + n_kb - 1) FB_STAMP(15, 0);
+          const uint32_t a_dst = smem_base + static_cast<uint32_t>(s) * stage_bytes;
+          // both blocks of the pair report their bytes to the even block's barrier, which expects
+          // the bytes of both
+          const uint32_t full = map_to_cta(smem_u32(&sh.full_bar[s]), lead_rank);
+          if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&sh.full_bar[s]), 2u * stage_bytes);
+          tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, tile * kTileM, pol_x);
+          tma_load_2d_pair(a_dst + kATileBytes, &tmap_w, full, kb * kBlockK,
+                           static_cast<int32_t>(cta_rank) * (p.N / 2), pol_w);
+          ring_advance(s, phase, p.stages);
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1 || warp == kSecondIssuerWarp) {
+    // ------------------------------------------------------------ MMA issuers (even block only)
+    // warp 1: the piece's k-blocks 0, 2, 4, ... into accumulator 0; the last warp: 1, 3, 5, ... into
+    // accumulator 1 (N columns further).
+    if (lane == 0 && cta_rank == 0) {
+      const int first_kb = warp == 1 ? 0 : 1;
+      const uint32_t acc_sets = 4 * p.N <= p.tmem_cols ? 2u : 1u;
+      const uint32_t idesc = umma_idesc_bf16_f32(kTileM * 2, static_cast<uint32_t>(p.N));
+      int s = 0;
+      uint32_t phase = 0;
+      uint32_t ti = 0;                        // this pair's tile counter
+      bool ok = true;
+      int32_t g = 0;                          // ring position: k-blocks of all of this pair's tiles, in order
+      const bool odd_ring = (p.stages & 1) != 0;
+      volatile int32_t* my_progress = &sh.issuer_progress[warp == 1 ? 0 : 1];
+      const volatile int32_t* other_progress = &sh.issuer_progress[warp == 1 ? 1 : 0];
+      for (int pt = pair_first; pt < total_pairs && ok; pt += pair_stride, ++ti) {
+        const uint32_t set = ti % acc_sets, use = ti / acc_sets;
+        const uint32_t acc = tmem_base + set * 2u * static_cast<uint32_t>(p.N) + (warp == 1 ? 0u : static_cast<uint32_t>(p.N));
+        if (use != 0) {
+          // the set's previous contents must have been read out by both blocks
+          ok = mbar_wait<true>(smem_u32(&sh.tmem_empty_bar[set]), (use - 1u) & 1u, abort_flag);
+          if (!ok) break;
+          tcgen05_fence_after();
+        }
+        for (int kb = 0; kb < n_kb; ++kb, ++g) {
+          if ((kb & 1) == first_kb) {
+            if (odd_ring && g >= p.stages) {
+              // whose was the stage's previous use (ring position g - stages)?  Its k-block index
+              // inside its own tile decides, as for every k-block.
+              int kbp = kb - p.stages;
+              while (kbp < 0) kbp += n_kb;
+              if ((kbp & 1) != first_kb) ok = issuer_turn_wait(other_progress, g - p.stages, abort_flag);
+            }
+            ok = ok && mbar_wait<true>(smem_u32(&sh.full_bar[s]), phase, abort_flag);
+            if (!ok) break;
+            if (odd_ring) *my_progress = g;
+            tcgen05_fence_after();
+            if (kb == 0) FB_STAMP(16, 32);
+            const uint32_t a_addr = smem_base + static_cast<uint32_t>(s) * stage_bytes;
+            const uint64_t adesc = umma_smem_desc_sw128(a_addr);
+            const uint64_t bdesc = umma_smem_desc_sw128(a_addr + kATileBytes);
+            if (p.probe != 1) {
+              // advance 16 elements = 32 bytes inside the swizzled row: +2 in the address field
+#pragma unroll
+              for (int kk = 0; kk < kBlockK / kUmmaK; ++kk)
+                umma_bf16<2>(acc, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb != first_kb || kk != 0) ? 1u : 0u);
+            }
+            umma_commit_pair(smem_u32(&sh.empty_bar[s]), cluster_rank);   // frees the stage in both blocks
+          }
+          ring_advance(s, phase, p.stages);
+        }
+        if (warp == 1) FB_STAMP(17, 32);
+        if (ok) umma_commit_pair(smem_u32(&sh.accum_bar[set]), cluster_rank);   // this issuer's accumulator is complete
+      }
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int et = threadIdx.x - 64;                       // 0 .. kEpilogueThreads-1
+    const int ew = warp - 2;
+    const int quarter = warp & 3;                          // TMEM lanes this warp may touch
+    const int sub = ew >> 2;                               // copies every fourth 16-column chunk
+    const uint32_t taddr0 = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+    const uint32_t acc_sets = 4 * p.N <= p.tmem_cols ? 2u : 1u;
+    const int E = p.E, N = p.N;
+    const uint32_t row_stride = static_cast<uint32_t>(staging_stride(N)) * 4u;
+    const bool two_acc = n_kb > 1;
+
+    LaneColumns lc;
+    {
+      lc.group = lane / p.lanes_per_group;
+      const int first = (lane % p.lanes_per_group) * p.cols_per_lane;
+      lc.c0 = lc.group < p.groups ? lc.group * p.group_size + first : 0;
+      lc.n = lc.group < p.groups ? max(0, min(p.cols_per_lane, p.group_size - first)) : 0;
+      if (lc.n == 0) lc.c0 = 0;
+    }
+    // While the main loop runs, stage the biases and the placement for the planner (any block may
+    // turn out to be the last one).
+    for (int e = et; e < FB_MAX_EXPERTS; e += kEpilogueThreads) {
+      sh.logit_bias[e] = (p.logit_bias != nullptr && e < E) ? p.logit_bias[e] : 0.0f;
+      sh.select_bias[e] = (p.select_bias != nullptr && e < E) ? p.select_bias[e] : 0.0f;
+    }
+    float sb[kCpl];
+#pragma unroll
+    for (int j = 0; j < kCpl; ++j)
+      sb[j] = (kSigmoid && p.select_bias != nullptr && j < lc.n) ? p.select_bias[lc.c0 + j] : 0.0f;
+    if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
+
+    uint32_t tiles_done = 0;
+    for (int pt = pair_first; pt < total_pairs; pt += pair_stride) {
+      const bool second_pass = pt >= pairs_per_pass;
+      const int mode = p.mode == kModeLayer ? (second_pass ? kModeDispatch : kModePredictPlan) : p.mode;
+      const int tile = 2 * (second_pass ? pt - pairs_per_pass : pt) + static_cast<int>(cta_rank);
+      // outputs of the normal pass are not written by tiles of the early pass
+      int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_ids;
+      float* const out_w = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_w;
+      const bool last_tile = pt + pair_stride >= total_pairs;
+
+      // one thread polls for the finished accumulators, the others sleep at the barrier
+      const uint32_t set = tiles_done % acc_sets, use = tiles_done / acc_sets;
+      const uint32_t taddr = taddr0 + set * 2u * static_cast<uint32_t>(N);
+      if (et == 0) sh.accum_ok = mbar_wait<true>(smem_u32(&sh.accum_bar[set]), use & 1u, abort_flag) ? 1 : 0;
+      named_bar_sync(kAccumBarrierId, kEpilogueThreads);
+      const bool got = sh.accum_ok != 0 && p.probe == 0;     // a measurement launch ends with its main loop
+      if (sh.accum_ok == 0 && J == 1) break;                 // (blocks that share a tile pair go on to their common barrier)
+      ++tiles_done;
+      tcgen05_fence_after();
+      FB_STAMP(2, 64);
+
+      // The last tile's staging reuses the operand ring, which is idle by then; earlier ones have
+      // their own (smaller) area behind it and go through it a few rows at a time.
+      const int chunk_rows = last_tile ? kTileM : p.chunk_rows;
+      const uint32_t staging = smem_base + (last_tile ? 0u : static_cast<uint32_t>(p.stages) * stage_bytes);
+      RowScratch& rs = reinterpret_cast<RowScratch*>(smem_raw + (staging - smem_u32(smem_raw)) +
+                                                     static_cast<size_t>(chunk_rows) * row_stride)[ew];
+      for (int r0 = 0; r0 < kTileM; r0 += chunk_rows) {
+        if (r0 > 0) named_bar_sync(kPlanBarrierId, kEpilogueThreads);      // the previous rows have been read
+        // ---- tensor memory -> shared memory: thread = row, 16 columns at a time
+        if (quarter * 32 >= r0 && quarter * 32 < r0 + chunk_rows) {
+          if (got) {
+            const uint32_t dst = staging + static_cast<uint32_t>(quarter * 32 - r0 + lane) * row_stride;
+#pragma unroll 1
+            for (int c0 = sub * 16; c0 < N; c0 += kEpiSubs * 16) {
+              uint32_t r[16], r2[16];
+              tmem_ld_32x32b_x16(taddr + c0, r);
+              if (two_acc) tmem_ld_32x32b_x16(taddr + N + c0, r2);
+              tmem_ld_wait();
+              if (two_acc) {                                 // add the odd k-blocks' accumulator
+#pragma unroll
+                for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
+              }
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                st_shared_v4(dst + static_cast<uint32_t>(c0 + 4 * q) * 4u, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+            }
+          }
+          tcgen05_fence_before();
+          __syncwarp();
+          // the issuers may overwrite the accumulators now
+          if (several_tiles && lane == 0) mbar_arrive_cluster(smem_u32(&sh.tmem_empty_bar[set]), lead_rank);
+        }
+        FB_STAMP(3, 64);
+        // ---- this warp's rows of the staged ones
+        int first, count;
+        if (J > 1) {
+          cluster_arrive(); cluster_wait();                  // every block's partial tile is staged
+          const int slice = kTileM / J, per = max(2, slice / kEpilogueWarps);
+          first = piece * slice + ew * per;
+          count = ew * per < slice ? per : 0;
+        } else if (chunk_rows == kTileM) {
+          // the four warps that share a quarter of the rows meet at their own barrier
+          if (last_tile) { cluster_arrive(); closing_arrived = true; }     // done with tensor memory and the partner
+          named_bar_sync(kRowBarrierBase + static_cast<uint32_t>(quarter), kEpiSubs * 32);
+          first = quarter * 32 + sub * 8;
+          count = 8;
+        } else {
+          named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+          const int per = chunk_rows / kEpilogueWarps;
+          first = r0 + ew * per;
+          count = per;
+        }
+        FB_STAMP(4, 64);
+        const long long row0 = static_cast<long long>(tile) * kTileM + first;
+        if (got && count > 0 && row0 < p.T) {
+          // default choice (kept only where keys are not numbers): distinct experts
+          for (int i = lane; i < 8 * FB_MAX_TOPK; i += 32) { rs.win_id[i >> 3][i & 7] = i & 7; rs.win_key[i >> 3][i & 7] = -INFINITY; }
+          __syncwarp();
+#pragma unroll 1
+          for (int i = 0; i < count; i += 2)
+            if (row0 + i < p.T)
+              select_two_rows<kCpl, kSigmoid>(p, lc, sb, sh.logit_bias, staging + static_cast<uint32_t>(first - r0 + i) * row_stride,
+                                              cta_rank, row0 + i, rs, i >> 1, lane);
+          __syncwarp();
+          FB_STAMP(8, 64);
+          finish_rows<kSigmoid>(p, sh, rs, count, row0, out_ids, out_w, lane);
+          FB_STAMP(10, 64);
+        }
+      }
+      if (J > 1) { cluster_arrive(); closing_arrived = true; }   // done with the other blocks' staged rows
+      named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+      if (p.probe != 0) {
+        // measurement launch: nothing is published
+      } else if (mode == kModeDispatch) {
+        const int slice = tile * J + piece;
+        if (static_cast<long long>(slice) * (kTileM / J) < p.T)  // a slice beyond the last token owns no row
+          write_slice_counts(p.slice_counts, slice, E, sh.hist, et);
+        if (several_tiles) {
+          named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+          for (int e = et; e < E; e += kEpilogueThreads) sh.hist[e] = 0;
+        }
+      } else if (pt + pair_stride >= pairs_per_pass) {
+        // The histogram keeps accumulating over this block's tiles of the pass and is published
+        // once, after the last of them (one fence and one ticket per block, not per tile).
+        publish_counts(sh, p, et, warp, lane, mode == kModePredictPlan && p.fuse_planner != 0);
+      }
+      FB_STAMP(12, 64);
+    }
+  }
+
+  // ---------------------------------------------------------------- teardown
+  // Tensor memory may be released, and a block may leave, only when all blocks of the cluster are
+  // done with it: a warp delivers its arrival as soon as its own last access to the others is over, so
+  // the wait normally finds the barrier complete.
+  if (J > 1 && (warp < 2 || warp == kSecondIssuerWarp)) { cluster_arrive(); cluster_wait(); }   // the barrier behind the staging
+  if (!closing_arrived) cluster_arrive();
+  tcgen05_fence_before();
+  __syncthreads();
+  cluster_wait();
+  if (threadIdx.x == 0 && sh.abort_flag) atomicCAS(p.status, 0, FB_ERR_TIMEOUT);
+  if (warp == 1) {
+    tcgen05_fence_after();
+    tmem_dealloc<2>(tmem_base, static_cast<uint32_t>(p.tmem_cols));
+  }
+  FB_STAMP(13, 64);
+}
+
+}  // namespace fb

@@ -723,6 +723,49 @@ def test_dispatch_index_over_table_widths_and_runs_of_tiles(E, k, R, T):
     _run(wl, T, want_logits=False, sample=sample)
 
 
+@pytest.mark.parametrize("kw", [
+    dict(E=16, k=2, R=4),                                             # one column per lane
+    dict(E=33, k=4, R=3, renorm=0),                                   # two, the last lane holds one; softmax denominator
+    dict(E=100, k=6, R=4),                                            # four
+    dict(E=200, k=8, R=8, renorm=0),                                  # eight
+    dict(gate=1, n_group=5, topk_group=2, k=7, E=250, R=5),           # sixteen; bound from the lanes, idle lanes
+    dict(gate=1, n_group=8, topk_group=3, k=6, E=160, R=8),           # groups of 20: five per lane, single loads
+    dict(gate=1, n_group=32, topk_group=4, k=8, E=64, R=8),           # groups of two
+    dict(gate=1, n_group=3, topk_group=3, k=5, E=96, R=6, route_scale=2.5),   # every group kept
+    dict(E=128, k=8, R=8), dict(gate=1, n_group=8, topk_group=4, k=8, E=256, R=32),   # ranking gates, tiles shared by pairs
+])
+@pytest.mark.parametrize("T,limit", [
+    (1, 0), (17, 0), (129, 0),          # one tile pair: eight block pairs share it; slices of 16 rows, the last partly or not filled
+    (1300, 0), (4500, 0),               # four and two pairs per tile in the layer call, more in the separate ones
+    (1300, 2),                          # several tiles per pair: staged a few rows at a time
+])
+def test_row_selection_over_gates_and_shared_tiles(kw, T, limit):
+    # same tolerances as every parity test (bf16 products are exact, sums in fp32)
+    _run(_wl(d=1024, **kw), T, layer=1, with_logit_bias=T in (17, 1300), want_logits=limit == 0, pair_limit=limit)
+
+
+@pytest.mark.parametrize("T", [100, 1300])
+def test_row_selection_breaks_ties_and_survives_overfull_lists(T):
+    # half of the rows have equal keys everywhere (more candidates than a row's list holds), in the others
+    # experts 2 i and 2 i + 1 have equal weights: every choice is decided by the lower id
+    for kw in (dict(E=100, k=5, R=4), dict(gate=1, n_group=10, topk_group=4, k=7, E=200, R=8), dict(E=12, k=5, R=3)):
+        wl = _wl(d=512, **kw)
+        li = I.make_layer(wl, 2, 0, T=T)
+        li.W[1::2] = li.W[0::2]
+        li.h_prev[::2] = 0
+        li.H[::2] = 0
+        if li.select_bias is not None:
+            li.select_bias = torch.zeros(wl.E)
+        ctx = P.make_context(wl, T)
+        bkw = P.budget_kwargs(wl, T)
+        gpu = P.run_gpu_layer(ctx, wl, li, bkw, want_logits=False)
+        P.compare_layer(wl, li, bkw, gpu)
+        assert (gpu["ids"][::2] == np.arange(wl.k)).all()
+        even = gpu["ids"][1::2] % 2 == 0                     # an odd expert is chosen only right after its twin
+        assert (even[:, 1:] | (gpu["ids"][1::2, 1:] == gpu["ids"][1::2, :-1] + 1)).all() and even[:, 0].all()
+        ctx.close()
+
+
 def test_contexts_of_different_shapes_alive_together():
     # Kernel attributes (the dynamic shared-memory ceiling) belong to the kernel, not to a context:
     # a large-shape context must keep working after a small-shape one was created, and the

@@ -1035,10 +1035,10 @@ fb_status fb_dispatch_slot_counts(fb_ctx* ctx, const uint32_t* slot_offsets, uin
   if (!ctx || !slot_offsets || !slot_counts) return FB_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
-  fb::fb_slot_counts_kernel<<<1, FB_MAX_EXPERTS, 0, static_cast<cudaStream_t>(stream_)>>>(slot_offsets, ctx->cfg.E,
-                                                                                          slot_counts);
+  const cudaError_t err = launch_dependent(fb::fb_slot_counts_kernel, 1, FB_MAX_EXPERTS, static_cast<cudaStream_t>(stream_),
+                                           slot_offsets, ctx->cfg.E, slot_counts);
   ++ctx->launches;
-  return cudaGetLastError() == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
 fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int32_t rank,
@@ -1062,10 +1062,10 @@ fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int
   long long blocks = (n + fb::kGlobalizeThreads - 1) / fb::kGlobalizeThreads;
   if (blocks < 1) blocks = 1;
   if (blocks > 4 * ctx->n_sm) blocks = 4 * ctx->n_sm;
-  fb::fb_dispatch_globalize_kernel<<<static_cast<unsigned>(blocks), fb::kGlobalizeThreads, 0,
-                                     static_cast<cudaStream_t>(stream_)>>>(gp);
+  const cudaError_t err = launch_dependent(fb::fb_dispatch_globalize_kernel, static_cast<int>(blocks), fb::kGlobalizeThreads,
+                                           static_cast<cudaStream_t>(stream_), gp);
   ++ctx->launches;
-  return cudaGetLastError() == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
 fb_status fb_attention_begin(fb_ctx* ctx, int32_t layer_id, int32_t attn_type, fb_stream stream_) {

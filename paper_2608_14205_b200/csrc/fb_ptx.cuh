@@ -272,6 +272,10 @@ __device__ __forceinline__ void ld_cluster_floats(uint32_t addr, float (&v)[kN])
                    : "=f"(v[i]), "=f"(v[i + 1]), "=f"(v[i + 2]), "=f"(v[i + 3]) : "r"(addr + 4u * i) : "memory");
   }
 }
+// Integer sum (order does not matter) into a word of a block of the cluster.
+__device__ __forceinline__ void red_add_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 // Largest / smallest of a float over the warp.
 __device__ __forceinline__ float redux_max_f32(float x) {
   float r;

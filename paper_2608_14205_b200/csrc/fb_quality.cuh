@@ -8,6 +8,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/freebalance.h"
+#include "fb_ptx.cuh"
+
 namespace fb {
 
 constexpr int kCosineWarpsPerBlock = 8;
@@ -46,6 +49,8 @@ fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long 
   constexpr int kVec = 16 / static_cast<int>(sizeof(Tin));
   const long long row = static_cast<long long>(blockIdx.x) * kCosineWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_launch_dependents();
+  pdl_wait();
   if (row >= rows) return;
   const long long base = row * n;
   double dot = 0.0, na = 0.0, nb = 0.0;
@@ -74,35 +79,63 @@ fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long 
   if (lane == 0) row_cos[row] = (na > 0.0 && nb > 0.0) ? dot / (sqrt(na) * sqrt(nb)) : 0.0;
 }
 
-// Mean of v[0 .. count) by one block: strided partial sums, then a shared-memory tree.
+// Mean of v[0 .. count) by one block: strided partial sums with eight loads in flight, then warp
+// butterflies; the order of the additions is fixed.
 __global__ void __launch_bounds__(kMeanThreads)
 fb_mean_kernel(const double* __restrict__ v, long long count, double* __restrict__ out) {
-  __shared__ double part[kMeanThreads];
+  __shared__ double part[kMeanThreads / 32];
+  static_assert(kMeanThreads == 1024, "one warp adds the warps' sums");
+  pdl_launch_dependents();
+  pdl_wait();
   double s = 0.0;
-  for (long long i = threadIdx.x; i < count; i += kMeanThreads) s += v[i];
-  part[threadIdx.x] = s;
+#pragma unroll 8
+  for (long long i = threadIdx.x; i < count; i += kMeanThreads) s += __ldcg(v + i);
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = kMeanThreads / 2; w >= 1; w >>= 1) {
-    if (threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    s = part[threadIdx.x];
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (threadIdx.x == 0) *out = count > 0 ? s / static_cast<double>(count) : 0.0;
   }
-  if (threadIdx.x == 0) *out = count > 0 ? part[0] / static_cast<double>(count) : 0.0;
 }
 
-// hits += |ids_a[i, :] intersect ids_b[i, :]| over tokens i (ids within a token are distinct).
-__global__ void __launch_bounds__(256)
+// hits = sum over tokens i of |ids_a[i, :] intersect ids_b[i, :]| (ids within a token are distinct).
+// One cluster: its blocks' sums meet in the first one's shared memory, so nothing has to be cleared
+// before (a memset between the kernels keeps them from overlapping).
+constexpr int kHitsBlocks = 8;
+constexpr int kHitsThreads = 1024;
+__global__ void __cluster_dims__(kHitsBlocks, 1, 1) __launch_bounds__(kHitsThreads)
 fb_topk_hits_kernel(const int32_t* __restrict__ ids_a, const int32_t* __restrict__ ids_b, int T, int k,
                     uint32_t* __restrict__ hits) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ uint32_t block_sum, cluster_sum;
+  if (threadIdx.x == 0) { block_sum = 0; cluster_sum = 0; }
+  __syncthreads();
+  cluster_arrive();
+  pdl_launch_dependents();
+  pdl_wait();
   uint32_t mine = 0;
-  if (i < T) {
-    for (int x = 0; x < k; ++x) {
-      const int32_t e = ids_b[static_cast<long long>(i) * k + x];
-      for (int y = 0; y < k; ++y) mine += ids_a[static_cast<long long>(i) * k + y] == e ? 1u : 0u;
+  for (long long i = static_cast<long long>(blockIdx.x) * kHitsThreads + threadIdx.x; i < T; i += kHitsBlocks * kHitsThreads) {
+    int32_t a[FB_MAX_TOPK];
+#pragma unroll
+    for (int y = 0; y < FB_MAX_TOPK; ++y) a[y] = y < k ? ids_a[i * k + y] : INT32_MIN;
+#pragma unroll
+    for (int x = 0; x < FB_MAX_TOPK; ++x) {
+      const int32_t e = x < k ? ids_b[i * k + x] : INT32_MAX;
+#pragma unroll
+      for (int y = 0; y < FB_MAX_TOPK; ++y) mine += a[y] == e ? 1u : 0u;
     }
   }
   mine = __reduce_add_sync(0xffffffffu, mine);
-  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(hits, mine);      // integer sum: order does not matter
+  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&block_sum, mine);
+  __syncthreads();
+  cluster_wait();
+  if (threadIdx.x == 0) red_add_cluster(map_to_cta(smem_u32(&cluster_sum), 0u), block_sum);
+  cluster_arrive();
+  cluster_wait();
+  if (cluster_ctarank() == 0 && threadIdx.x == 0) *hits = cluster_sum;
 }
 
 // SM clock probe: one thread records (global nanosecond timer, SM cycle counter) pairs, `n` of

@@ -168,8 +168,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream or None
+    if stream is None:                   # torch's current stream without building a Stream object (3 us of a call's 14)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return stream or None

@@ -21,7 +21,7 @@ import numpy as np
 import torch
 
 SLOTS = {0: "block start", 1: "set-up done", 14: "first load issued", 16: "first operands landed",
-         15: "last load issued", 17: "last MMA issued", 2: "accumulators complete", 3: "keys computed",
+         15: "last load issued", 17: "last MMA issued", 2: "accumulators complete", 3: "keys computed / logits staged",
          4: "barrier", 5: "groups chosen", 7: "candidates collected", 8: "candidates ranked", 9: "top-k read back",
          10: "outputs written", 11: "counts published", 18: "planner entered", 19: "rank loads formed",
          20: "greedy loop left", 12: "planner done", 13: "block exit"}
@@ -59,7 +59,7 @@ def main(argv=None):
                            ranks_per_node=wl.ranks_per_node, expert_bytes=wl.expert_bytes)
     i32 = lambda n: torch.zeros(max(1, n), dtype=torch.int32, device=dev)
     counts, pio, sw, ns, lb, la = i32(wl.E), i32(wl.E), i32(4 * 128), i32(1), i32(wl.R), i32(wl.R)
-    blocks_max = 2 * ((T + 127) // 128 + 1) + 64
+    blocks_max = max(2 * ((T + 127) // 128 + 1), 2 * 148)      # short calls: as many blocks as the GPU has SMs
     n = args.launches
     stamps = torch.zeros((n, blocks_max, 64), dtype=torch.int64, device=dev)
 
@@ -94,7 +94,7 @@ def main(argv=None):
     start = ns_t[:, :, 0].min(axis=1, keepdims=True)         # first block start of each launch
     print(f"{args.call} on {wl.name} T={T}: {nblk} blocks, {per_launch_us:.1f} us per launch "
           f"(two events around {n} back-to-back launches)")
-    print(f"{'phase boundary':26s} {'mean':>8s} {'latest':>8s}   (us since the launch's first block start; "
+    print(f"{'phase boundary':32s} {'mean':>8s} {'latest':>8s}   (us since the launch's first block start; "
           f"launches 2..{n})")
     sel = slice(1, None)
     for slot in ORDER:
@@ -105,7 +105,7 @@ def main(argv=None):
         rel = np.where(ok, (t - start[sel]) / 1e3, np.nan)
         mean, latest = float(np.nanmean(rel)), float(np.nanmean(np.nanmax(rel, axis=1)))
         out["phases"][SLOTS[slot]] = {"mean_us": mean, "latest_us": latest, "blocks": int(ok[0].sum())}
-        print(f"{SLOTS[slot]:26s} {mean:8.2f} {latest:8.2f}   [{int(ok[0].sum())} blocks]")
+        print(f"{SLOTS[slot]:32s} {mean:8.2f} {latest:8.2f}   [{int(ok[0].sum())} blocks]")
     end = ns_t[:, :, 13].max(axis=1)
     span = (end - start[:, 0]) / 1e3
     gap = (start[1:, 0] - end[:-1]) / 1e3

@@ -316,8 +316,9 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
     // block pairs just as fast as on 74 (measured), and the other SMs stay free for other streams
     const int rounds = (tile_pairs + pairs_avail - 1) / pairs_avail;
     clusters = (tile_pairs + rounds - 1) / rounds;
-    // room for two accumulator sets (4 N columns) when the 512 tensor-memory columns allow it
-    if (4 * ctx->N <= 512) p.tmem_cols = next_pow2_at_least_32(4 * ctx->N);
+    // two accumulator sets: 512 tensor-memory columns at most
+    p.acc_sets = 2;
+    p.tmem_cols = next_pow2_at_least_32(2 * p.issuers * ctx->N);
   }
   const int blocks = 2 * J * clusters;
   // every block publishes its counts once: as many tickets as blocks that own a tile of the counted pass
@@ -428,7 +429,9 @@ static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
   g.topk_group = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? c.topk_group : 1;
   g.renorm = c.renorm; g.route_scale = c.route_scale;
   g.num_kb = (c.d + fb::kBlockK - 1) / fb::kBlockK;
-  g.tmem_cols = next_pow2_at_least_32(2 * ctx->N);               // two accumulators
+  g.issuers = ctx->N <= 128 ? 2 : 1;                             // the reason is in fb_router.cuh
+  g.acc_sets = 1;
+  g.tmem_cols = next_pow2_at_least_32(g.issuers * ctx->N);
   const int cpl = fb::gate_layout(c.E, c.gate, c.n_group, c.topk_group, &g);
   ctx->rows_kernel = 0;
   while ((1 << ctx->rows_kernel) < cpl) ++ctx->rows_kernel;

@@ -87,6 +87,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// True in one lane of a converged warp.  A role loop runs with all 32 lanes and only its asynchronous
+// instructions under this predicate: its counters, addresses and descriptors are then warp-uniform.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}" : "=r"(pred));
+  return pred != 0;
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // Lets the next kernel of the stream (if it was launched with programmatic stream
 // serialization) start its prologue now instead of after this grid has drained.
@@ -253,6 +261,19 @@ __device__ __forceinline__ void ld_shared_floats(uint32_t addr, float (&v)[kN]) 
                    : "=f"(v[i]), "=f"(v[i + 1]), "=f"(v[i + 2]), "=f"(v[i + 3]) : "r"(addr + 4u * i) : "memory");
   }
 }
+// Two vectors of four words, 512 bytes apart.
+__device__ __forceinline__ void ld_shared_two_vectors(uint32_t addr, float (&v)[8]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[4 * i]), "=f"(v[4 * i + 1]), "=f"(v[4 * i + 2]), "=f"(v[4 * i + 3]) : "r"(addr + 512u * i) : "memory");
+}
+__device__ __forceinline__ void ld_cluster_two_vectors(uint32_t addr, float (&v)[8]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[4 * i]), "=f"(v[4 * i + 1]), "=f"(v[4 * i + 2]), "=f"(v[4 * i + 3]) : "r"(addr + 512u * i) : "memory");
+}
 // Words from the shared memory of a block of the cluster (a shared::cluster address).
 __device__ __forceinline__ float ld_cluster_float(uint32_t addr) {
   float v;
@@ -313,6 +334,10 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
+}
+// Without ordering of memory (the barriers' initialisation is published by fence_mbar_init).
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -5,12 +5,17 @@
 //
 // One block owns 128 token rows and all N = pad16(E) expert columns.
 // Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer for the even k-blocks (owns the
-// TMEM allocation), warp 18 = MMA issuer for the odd k-blocks, warps 2..17 = epilogue.
-// A thread that issues tcgen05.mma gets the next one accepted only ~175 cycles later,
-// whatever the MMA's shape, which is slower than the tensor pipe and than the x stream
-// from HBM; two issuing threads, each accumulating its own k-blocks into its own TMEM
-// accumulator (columns [0, N) and [N, 2N)), remove that limit and keep the summation
-// order fixed.  The epilogue adds the two accumulators.
+// TMEM allocation; issuer of all k-blocks where there is one), warp 18 = MMA issuer for the odd
+// k-blocks, warps 2..17 = epilogue.
+// With N <= 128 there are two issuers, each accumulating its own k-blocks into its own TMEM accumulator
+// (columns [0, N) and [N, 2N)): waiting for a stage, four MMAs and two commits take a warp longer than
+// the tensor pipe needs for narrow tiles (4096 rows x 8 columns, d = 4096: bare main loop 13.6 us with two,
+// 14.9 with one).  The epilogue adds the two accumulators.  Wider tiles keep the pipe busy from one warp
+// (512 cycles per k-block at N = 256; 39.3 us either way for 14 tiles, d = 7168) and need one accumulator.
+// Producer and issuers run their loops with the whole warp and one elected lane for the asynchronous
+// instructions.  Written as "if (lane == 0)" around the loop, counters and descriptors are per-lane
+// values that every such instruction has to fetch first: the loads of 4096 rows, d = 4096, took 17.3
+// instead of 12.2 us, with the MMAs 22.1 instead of 13.6.
 // Epilogue warps:  A warp may only read the 32 TMEM lanes (token rows) selected
 // by warp_id % 4, so the 16 epilogue warps form 4 "row quarters" x 4 "subs"; the subs of
 // a quarter split the expert columns between them in 32-column chunks, one thread per
@@ -87,7 +92,9 @@ struct RouterParams {
   float route_scale;
   int32_t num_kb;                    // ceil(d / 64)
   int32_t stages;
-  int32_t tmem_cols;                 // power of two >= max(32, 2 N): two accumulators
+  int32_t tmem_cols;                 // power of two >= 32 that holds acc_sets sets of N columns per issuer
+  int32_t issuers;                   // MMA issuers, each with an accumulator of its own (see above)
+  int32_t acc_sets;                  // sets of accumulators: 2 where a pair walks several tiles
   int32_t mode;
   int32_t tiles_first;               // kModeLayer: blocks below this index (even) belong to the early pass
   int32_t ticket_target;             // number of blocks that take a ticket (those that publish counts)
@@ -98,6 +105,7 @@ struct RouterParams {
   // g = l / lanes_per_group.  Gates that keep every group have groups == 1.
   int32_t pieces, chunk_rows;
   int32_t groups, group_size, keep_groups, lanes_per_group, cols_per_lane;
+  int32_t two_vectors;               // eight columns per lane, staged as two vectors 128 words apart
   int32_t vector_load;               // a lane's columns are all inside or all outside its group, and contiguous words
   int32_t ragged;                    // some lane holds fewer columns than the kernel instance is made for
   const float* logit_bias;           // [E] or nullptr
@@ -418,6 +426,120 @@ __device__ __forceinline__ void ring_advance(int& s, uint32_t& phase, int stages
   if (++s == stages) { s = 0; phase ^= 1u; }
 }
 
+// The tile pairs of a block pair and its share of their k-blocks: pair_first, pair_first + pair_stride, ...;
+// in kModeLayer the first pairs_per_pass pairs belong to the early pass, the rest to the normal pass.
+struct TileWalk {
+  int pair_first, pair_stride, total_pairs, pairs_per_pass;
+  int kb0, n_kb;
+  uint32_t cluster_rank;
+};
+
+// TMA producer (a whole warp): both blocks of a pair report their bytes to the even block's barrier, which
+// expects the bytes of both.
+__device__ __forceinline__ void produce_operands(const RouterParams& p, const CUtensorMap* map_x, const CUtensorMap* map_x2,
+                                                 const CUtensorMap* map_w, const TileWalk& w, uint32_t smem_base,
+                                                 uint32_t stage_bytes, uint64_t* full_bar, uint64_t* empty_bar,
+                                                 volatile int* abort_flag) {
+  const uint64_t pol_x = l2_policy_evict_first();            // x is streamed once
+  const uint64_t pol_w = l2_policy_evict_last();             // W is re-read by every pair
+  const bool leader = elect_one();
+  const uint32_t cta_rank = w.cluster_rank & 1u;
+  const int stages = p.stages, w_row = static_cast<int>(cta_rank) * (p.N / 2);
+  int s = 0;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int pt = w.pair_first; pt < w.total_pairs && ok; pt += w.pair_stride) {
+    const bool second_pass = pt >= w.pairs_per_pass;
+    const int row = (2 * (second_pass ? pt - w.pairs_per_pass : pt) + static_cast<int>(cta_rank)) * kTileM;
+    const CUtensorMap* xmap = second_pass ? map_x2 : map_x;
+    for (int kb = w.kb0; kb < w.kb0 + w.n_kb; ++kb) {
+      ok = __all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&empty_bar[s]), phase ^ 1u, abort_flag));
+      if (!ok) break;
+      if (kb == w.kb0) FB_STAMP(14, 0);
+      if (kb == w.kb0 + w.n_kb - 1) FB_STAMP(15, 0);
+      if (leader) {
+        const uint32_t a_dst = smem_base + static_cast<uint32_t>(s) * stage_bytes;
+        const uint32_t full = map_to_cta(smem_u32(&full_bar[s]), w.cluster_rank & ~1u);
+        if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&full_bar[s]), 2u * stage_bytes);
+        tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, row, pol_x);
+        tma_load_2d_pair(a_dst + kATileBytes, map_w, full, kb * kBlockK, w_row, pol_w);
+      }
+      __syncwarp();
+      ring_advance(s, phase, stages);
+    }
+  }
+}
+
+// MMA issuer (a whole warp of the pair's even block): issuer 0 takes the k-blocks 0, 2, 4, ... of every
+// tile, issuer 1 the others; a single issuer takes all.  accum_bar[set] completes when the tile is done,
+// tmem_empty_bar[set] (several tiles only) when its accumulators have been read out.
+__device__ __forceinline__ void issue_mmas(const RouterParams& p, const TileWalk& w, int issuer, uint32_t tmem_base,
+                                           uint32_t smem_base, uint32_t stage_bytes, uint64_t* full_bar, uint64_t* empty_bar,
+                                           uint64_t* accum_bar, uint64_t* tmem_empty_bar, int32_t* progress,
+                                           volatile int* abort_flag) {
+  const bool leader = elect_one();
+  const int stages = p.stages, step = p.issuers;
+  const uint32_t idesc = umma_idesc_bf16_f32(kTileM * 2, static_cast<uint32_t>(p.N));
+  const bool odd_ring = step == 2 && (stages & 1) != 0;
+  volatile int32_t* my_progress = progress + issuer;
+  const volatile int32_t* other_progress = progress + (issuer ^ 1);
+  int s0 = 0;                                  // stage and phase of the tile's first k-block
+  uint32_t phase0 = 0;
+  int32_t g0 = 0;                              // its ring position: k-blocks of all of this pair's tiles, in order
+  uint32_t set = 0, use = 0;
+  bool ok = true;
+  for (int pt = w.pair_first; pt < w.total_pairs && ok; pt += w.pair_stride) {
+    const uint32_t acc = tmem_base + (set * static_cast<uint32_t>(step) + static_cast<uint32_t>(issuer)) * static_cast<uint32_t>(p.N);
+    if (use != 0) {
+      // the set's previous contents must have been read out by both blocks
+      ok = __all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&tmem_empty_bar[set]), (use - 1u) & 1u, abort_flag));
+      if (!ok) break;
+      tcgen05_fence_after();
+    }
+    int s = s0 + issuer;
+    uint32_t phase = phase0;
+    if (s >= stages) { s -= stages; phase ^= 1u; }
+    for (int kb = issuer; kb < w.n_kb; kb += step) {
+      if (odd_ring && g0 + kb >= stages) {
+        // whose was the stage's previous use (ring position g0 + kb - stages)?  Its k-block index
+        // inside its own tile decides, as for every k-block.
+        int kbp = kb - stages;
+        while (kbp < 0) kbp += w.n_kb;
+        if ((kbp & 1) != issuer)
+          ok = __all_sync(0xffffffffu, issuer_turn_wait(other_progress, g0 + kb - stages, abort_flag));
+      }
+      ok = ok && __all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&full_bar[s]), phase, abort_flag));
+      if (!ok) break;
+      if (odd_ring && leader) *my_progress = g0 + kb;
+      tcgen05_fence_after();
+      if (kb == 0) FB_STAMP(16, 32);
+      const uint32_t a_addr = smem_base + static_cast<uint32_t>(s) * stage_bytes;
+      const uint64_t adesc = umma_smem_desc_sw128(a_addr);
+      const uint64_t bdesc = umma_smem_desc_sw128(a_addr + kATileBytes);
+      if (leader) {
+        if (p.probe != 1) {
+          // advance 16 elements = 32 bytes inside the swizzled row: +2 in the address field
+#pragma unroll
+          for (int kk = 0; kk < kBlockK / kUmmaK; ++kk)
+            umma_bf16<2>(acc, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb != issuer || kk != 0) ? 1u : 0u);
+        }
+        umma_commit_pair(smem_u32(&empty_bar[s]), w.cluster_rank);   // frees the stage in both blocks when these retire
+      }
+      __syncwarp();
+      s += step;
+      if (s >= stages) { s -= stages; phase ^= 1u; }
+    }
+    if (issuer == 0) FB_STAMP(17, 32);
+    if (ok && leader) umma_commit_pair(smem_u32(&accum_bar[set]), w.cluster_rank);   // this issuer's accumulator is complete
+    __syncwarp();
+    g0 += w.n_kb;
+    s0 += w.n_kb % stages;
+    phase0 ^= static_cast<uint32_t>(w.n_kb / stages) & 1u;
+    if (s0 >= stages) { s0 -= stages; phase0 ^= 1u; }
+    if (++set == static_cast<uint32_t>(p.acc_sets)) { set = 0; ++use; }
+  }
+}
+
 // One tile pair per block pair.  Launched in clusters of two; the pair shares one 256 x N MMA
 // (tcgen05 cta_group::2).  Each block loads its own 128 rows of x and half of the W tile.  The even
 // block of the pair issues the MMAs and owns the "full" barriers; both blocks get their stage-free and
@@ -432,14 +554,14 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   extern __shared__ uint8_t smem_raw[];
   __shared__ RouterShared sh;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);      // warp-uniform for the compiler as well
   const int lane = threadIdx.x & 31;
   // kModeLayer: which pass this block belongs to, its tile there and its input
   const int owner_block = static_cast<int>(blockIdx.x);
   const bool second_pass = p.mode == kModeLayer && owner_block >= p.tiles_first;
   const int mode = p.mode == kModeLayer ? (second_pass ? kModeDispatch : kModePredictPlan) : p.mode;
   const int tile = second_pass ? owner_block - p.tiles_first : owner_block;
-  const int kb_end = p.num_kb;
+  const bool two_acc = p.issuers == 2 && p.num_kb > 1;
   const CUtensorMap* xmap = second_pass ? &tmap_x2 : &tmap_x;
   // outputs of the normal pass are not written by blocks of the early pass
   int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_ids;
@@ -460,7 +582,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       mbar_init(smem_u32(&sh.full_bar[s]), 1);
       mbar_init(smem_u32(&sh.empty_bar[s]), 1);
     }
-    mbar_init(smem_u32(&sh.accum_bar), 2);                 // one commit per MMA issuer
+    mbar_init(smem_u32(&sh.accum_bar), static_cast<uint32_t>(p.issuers));      // one commit per MMA issuer
     fence_mbar_init();
     prefetch_tensormap(xmap);
     prefetch_tensormap(&tmap_w);
@@ -479,7 +601,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   }
   tcgen05_fence_before();
   __syncthreads();
-  cluster_arrive(); cluster_wait();          // the partner's barriers and TMEM are ready too
+  cluster_arrive_relaxed(); cluster_wait();  // the partner's barriers and TMEM are ready too
   tcgen05_fence_after();
   // Everything above touched only this block's own state and the call's parameters; from here on
   // the kernel reads memory that earlier work of the stream may have written.
@@ -494,77 +616,27 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   const uint32_t tmem_base = sh.tmem_base;
   FB_STAMP(1, 64);
 
+  TileWalk walk;
+  walk.pair_first = static_cast<int>(blockIdx.x) / 2;
+  walk.pair_stride = walk.total_pairs = static_cast<int>(gridDim.x) / 2;       // one tile pair per block pair
+  walk.pairs_per_pass = p.tiles_first / 2;
+  walk.kb0 = 0;
+  walk.n_kb = p.num_kb;
+  walk.cluster_rank = cta_rank;
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const uint64_t pol_x = l2_policy_evict_first();   // x is streamed once
-      const uint64_t pol_w = l2_policy_evict_last();    // W is re-read by every block
-      for (int kb = 0; kb < kb_end; ++kb) {
-        const int s = kb % p.stages;
-        const uint32_t phase = static_cast<uint32_t>(kb / p.stages) & 1u;
-        if (!mbar_wait<true>(smem_u32(&sh.empty_bar[s]), phase ^ 1u, abort_flag)) break;
-        if (kb == 0) FB_STAMP(14, 0);
-        if (kb == kb_end - 1) FB_STAMP(15, 0);
-        const uint32_t a_dst = smem_base + static_cast<uint32_t>(s) * stage_bytes;
-        // both blocks report their bytes to the even block's barrier, which expects
-        // the bytes of the whole pair
-        const uint32_t full = map_to_cta(smem_u32(&sh.full_bar[s]), 0u);
-        if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&sh.full_bar[s]), 2u * stage_bytes);
-        tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, tile * kTileM, pol_x);
-        tma_load_2d_pair(a_dst + kATileBytes, &tmap_w, full, kb * kBlockK,
-                         static_cast<int32_t>(cta_rank) * (p.N / 2), pol_w);
-      }
-    }
-    __syncwarp();
+    produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
     cluster_arrive();          // this warp is done with the pair's shared state (see the teardown)
   } else if (warp == 1 || warp == kSecondIssuerWarp) {
-    // ------------------------------------------------------------ MMA issuers
-    // warp 1: k-blocks 0, 2, 4, ... into accumulator 0; the last warp: 1, 3, 5, ... into
-    // accumulator 1 (N columns further).  In a pair only the even block issues.
-    if (lane == 0 && cta_rank == 0) {
-      const int first_kb = warp == 1 ? 0 : 1;
-      const uint32_t acc = tmem_base + (warp == 1 ? 0u : static_cast<uint32_t>(p.N));
-      const uint32_t idesc = umma_idesc_bf16_f32(kTileM * 2, static_cast<uint32_t>(p.N));
-      bool ok = true;
-      const bool odd_ring = (p.stages & 1) != 0;
-      volatile int32_t* my_progress = &sh.issuer_progress[warp == 1 ? 0 : 1];
-      const volatile int32_t* other_progress = &sh.issuer_progress[warp == 1 ? 1 : 0];
-      for (int kb = first_kb; kb < kb_end && ok; kb += 2) {
-        const int s = kb % p.stages;
-        const uint32_t phase = static_cast<uint32_t>(kb / p.stages) & 1u;
-        // an odd ring: the stage's previous use (k-block kb - stages) was the other issuer's
-        if (odd_ring && kb >= p.stages) ok = issuer_turn_wait(other_progress, kb - p.stages, abort_flag);
-        ok = ok && mbar_wait<true>(smem_u32(&sh.full_bar[s]), phase, abort_flag);
-        if (!ok) break;
-        if (odd_ring) *my_progress = kb;
-        tcgen05_fence_after();
-        if (kb == 0) FB_STAMP(16, 32);
-        const uint32_t a_addr = smem_base + static_cast<uint32_t>(s) * stage_bytes;
-        const uint64_t adesc = umma_smem_desc_sw128(a_addr);
-        const uint64_t bdesc = umma_smem_desc_sw128(a_addr + kATileBytes);
-        if (p.probe != 1) {
-#pragma unroll
-          for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {
-            // advance 16 elements = 32 bytes inside the swizzled row: +2 in the address field
-            umma_bf16<2>(acc, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb != first_kb || kk != 0) ? 1u : 0u);
-          }
-        }
-        // frees the stage in both blocks when these MMAs retire
-        umma_commit_pair(smem_u32(&sh.empty_bar[s]), cta_rank);
-      }
-      if (warp == 1) FB_STAMP(17, 32);
-      // this issuer's accumulator is complete
-      umma_commit_pair(smem_u32(&sh.accum_bar), cta_rank);
-    }
+    // MMA issuers: in a pair only the even block issues
+    if (cta_rank == 0 && (warp == 1 || p.issuers == 2))
+      issue_mmas(p, walk, warp == 1 ? 0 : 1, tmem_base, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, &sh.accum_bar,
+                 nullptr, sh.issuer_progress, abort_flag);
     if (warp == 1) {
-    // One thread polls for the finished accumulator on behalf of the 16 epilogue warps,
-    // which sleep at a hardware barrier meanwhile (no issue slots, no power).
-    if (lane == 0) {
-      bool ok = mbar_wait<true>(smem_u32(&sh.accum_bar), 0u, abort_flag);
-      sh.accum_ok = ok ? 1 : 0;
-    }
-    __syncwarp();
-    named_bar_arrive(kAccumBarrierId, kEpilogueThreads + 32);
+      // One thread polls for the finished accumulator on behalf of the 16 epilogue warps,
+      // which sleep at a hardware barrier meanwhile (no issue slots, no power).
+      if (lane == 0) sh.accum_ok = mbar_wait<true>(smem_u32(&sh.accum_bar), 0u, abort_flag) ? 1 : 0;
+      __syncwarp();
+      named_bar_arrive(kAccumBarrierId, kEpilogueThreads + 32);
     }
     __syncwarp();
     cluster_arrive();
@@ -614,9 +686,9 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
           // both accumulators' loads in flight at once, one wait
           uint32_t r2[32];
           tmem_ld_32x32b_x32(taddr + c0, r);
-          if (kb_end > 1) tmem_ld_32x32b_x32(taddr + N + c0, r2);
+          if (two_acc) tmem_ld_32x32b_x32(taddr + N + c0, r2);
           tmem_ld_wait();
-          if (kb_end > 1) {
+          if (two_acc) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
           }

@@ -4,19 +4,18 @@
 // next one.
 //
 // What makes the overlap possible
+//   * two accumulator sets alternate from tile to tile (256 columns fit twice since one issuer with one
+//     accumulator keeps the tensor pipe busy at that width);
 //   * the epilogue warps copy their share of the finished accumulators from tensor memory
-//     into registers (64 columns per thread), hand tensor memory back to the MMA issuers
-//     at once, and do all gating / selection work from registers;
+//     into registers (64 columns per thread) and do all gating / selection work from registers;
 //   * the epilogue's shared-memory scratch (group scores, candidate lists) has its own
 //     44 KB behind the pipeline stages instead of reusing them.
 // Restricted to the gates the ranking selection handles (DeepSeek-V3-like sigmoid gates with
 // 32-expert groups, softmax gates over whole 32-column chunks); everything else, and
-// every call that fits one tile per block, runs fb_router_kernel.  Arithmetic, summation
-// order (even k-blocks in accumulator 0, odd ones in accumulator 1) and tie-breaking are
-// those of fb_router_kernel, so both kernels give identical results.
+// every call that fits one tile per block, runs one of the other kernels.  Arithmetic, summation
+// order and tie-breaking are those of fb_router_kernel, so both kernels give identical results.
 //
-// Warp roles as in fb_router_kernel: warp 0 TMA producer, warps 1 and 18 MMA issuers (even
-// block of the pair only), warps 2..17 epilogue (4 row quarters x 4 column shares).
+// Warp roles as in fb_router_kernel.
 #pragma once
 #include "fb_router.cuh"
 
@@ -32,8 +31,8 @@ static_assert(kPersistGroups == kBoundRows, "the three tables of best keys lie o
 struct PersistShared {
   uint64_t full_bar[kMaxStages];
   uint64_t empty_bar[kMaxStages];
-  // Accumulator sets: one (2 N of the 512 tensor-memory columns each) or, when 4 N <= 512, two that
-  // alternate from tile to tile, so that the next tile's MMAs need not wait for the drain.
+  // Two accumulator sets (of N columns per issuer) that alternate from tile to tile, so that the next
+  // tile's MMAs need not wait for the drain.
   uint64_t accum_bar[2];                     // per set: both issuers' commits, once per use
   uint64_t tmem_empty_bar[2];                // per set, even block's copy: all epilogue warps of the pair, once per use
   uint32_t tmem_base;
@@ -58,7 +57,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   extern __shared__ uint8_t smem_raw[];
   __shared__ PersistShared sh;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);      // warp-uniform for the compiler as well
   const int lane = threadIdx.x & 31;
   const uint32_t cta_rank = cluster_ctarank();
   const uint32_t b_tile_bytes = static_cast<uint32_t>(p.N / 2) * kBlockK * 2;
@@ -84,7 +83,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       mbar_init(smem_u32(&sh.empty_bar[s]), 1);
     }
     for (int a = 0; a < 2; ++a) {
-      mbar_init(smem_u32(&sh.accum_bar[a]), 2);
+      mbar_init(smem_u32(&sh.accum_bar[a]), static_cast<uint32_t>(p.issuers));
       mbar_init(smem_u32(&sh.tmem_empty_bar[a]), 2 * (kEpilogueThreads / 32));
     }
     fence_mbar_init();
@@ -106,7 +105,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   }
   tcgen05_fence_before();
   __syncthreads();
-  cluster_arrive(); cluster_wait();          // the partner's barriers and tensor memory are ready too
+  cluster_arrive_relaxed(); cluster_wait();  // the partner's barriers and tensor memory are ready too
   tcgen05_fence_after();
   // Everything above touched only this block's own state and the call's parameters; from here on
   // the kernel reads memory that earlier work of the stream may have written.
@@ -120,81 +119,20 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   pdl_launch_dependents();
   const uint32_t tmem_base = sh.tmem_base;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const uint64_t pol_x = l2_policy_evict_first();
-      const uint64_t pol_w = l2_policy_evict_last();
-      int s = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int pt = pair_first; pt < total_pairs && ok; pt += pair_stride) {
-        const bool second_pass = pt >= pairs_per_pass;
-        const int tile = 2 * (second_pass ? pt - pairs_per_pass : pt) + static_cast<int>(cta_rank);
-        const CUtensorMap* xmap = second_pass ? &tmap_x2 : &tmap_x;
-        for (int kb = 0; kb < p.num_kb; ++kb) {
-          ok = mbar_wait<true>(smem_u32(&sh.empty_bar[s]), phase ^ 1u, abort_flag);
-          if (!ok) break;
-          const uint32_t a_dst = smem_base + static_cast<uint32_t>(s) * stage_bytes;
-          // both blocks report their bytes to the even block's barrier
-          const uint32_t full = map_to_cta(smem_u32(&sh.full_bar[s]), 0u);
-          if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&sh.full_bar[s]), 2u * stage_bytes);
-          tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, tile * kTileM, pol_x);
-          tma_load_2d_pair(a_dst + kATileBytes, &tmap_w, full, kb * kBlockK,
-                           static_cast<int32_t>(cta_rank) * (p.N / 2), pol_w);
-          ring_advance(s, phase, p.stages);
-        }
-      }
-    }
-  } else if (warp == 1 || warp == kSecondIssuerWarp) {
-    // ------------------------------------------------------------ MMA issuers (even block only)
-    if (lane == 0 && cta_rank == 0) {
-      const int first_kb = warp == 1 ? 0 : 1;
-      const uint32_t acc_sets = 4 * p.N <= p.tmem_cols ? 2u : 1u;
-      const uint32_t idesc = umma_idesc_bf16_f32(kTileM * 2, static_cast<uint32_t>(p.N));
-      int s = 0;
-      uint32_t phase = 0;
-      uint32_t ti = 0;                        // this block pair's tile counter
-      bool ok = true;
-      int32_t g = 0;                          // ring position: k-blocks of all of this pair's tiles, in order
-      const bool odd_ring = (p.stages & 1) != 0;
-      volatile int32_t* my_progress = &sh.issuer_progress[warp == 1 ? 0 : 1];
-      const volatile int32_t* other_progress = &sh.issuer_progress[warp == 1 ? 1 : 0];
-      for (int pt = pair_first; pt < total_pairs && ok; pt += pair_stride, ++ti) {
-        const uint32_t set = ti % acc_sets, use = ti / acc_sets;
-        const uint32_t acc = tmem_base + set * 2u * static_cast<uint32_t>(p.N) + (warp == 1 ? 0u : static_cast<uint32_t>(p.N));
-        if (use != 0) {
-          // the set's previous contents must have been read out by both blocks
-          ok = mbar_wait<true>(smem_u32(&sh.tmem_empty_bar[set]), (use - 1u) & 1u, abort_flag);
-          if (!ok) break;
-          tcgen05_fence_after();
-        }
-        for (int kb = 0; kb < p.num_kb; ++kb, ++g) {
-          if ((kb & 1) == first_kb) {
-            if (odd_ring && g >= p.stages) {
-              // whose was the stage's previous use (ring position g - stages)?  Its k-block index
-              // inside its own tile decides, as for every k-block.
-              int kbp = kb - p.stages;
-              while (kbp < 0) kbp += p.num_kb;
-              if ((kbp & 1) != first_kb) ok = issuer_turn_wait(other_progress, g - p.stages, abort_flag);
-            }
-            ok = ok && mbar_wait<true>(smem_u32(&sh.full_bar[s]), phase, abort_flag);
-            if (!ok) break;
-            if (odd_ring) *my_progress = g;
-            tcgen05_fence_after();
-            const uint32_t a_addr = smem_base + static_cast<uint32_t>(s) * stage_bytes;
-            const uint64_t adesc = umma_smem_desc_sw128(a_addr);
-            const uint64_t bdesc = umma_smem_desc_sw128(a_addr + kATileBytes);
-#pragma unroll
-            for (int kk = 0; kk < kBlockK / kUmmaK; ++kk)
-              umma_bf16<2>(acc, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb != first_kb || kk != 0) ? 1u : 0u);
-            umma_commit_pair(smem_u32(&sh.empty_bar[s]), cta_rank);   // frees the stage in both blocks
-          }
-          ring_advance(s, phase, p.stages);
-        }
-        if (ok) umma_commit_pair(smem_u32(&sh.accum_bar[set]), cta_rank);   // this issuer's accumulator is complete
-      }
-    }
+  if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
+    TileWalk walk;
+    walk.pair_first = pair_first;
+    walk.pair_stride = pair_stride;
+    walk.total_pairs = total_pairs;
+    walk.pairs_per_pass = pairs_per_pass;
+    walk.kb0 = 0;
+    walk.n_kb = p.num_kb;
+    walk.cluster_rank = cta_rank;
+    if (warp == 0)
+      produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
+    else if (cta_rank == 0 && (warp == 1 || p.issuers == 2))
+      issue_mmas(p, walk, warp == 1 ? 0 : 1, tmem_base, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, sh.accum_bar,
+                 sh.tmem_empty_bar, sh.issuer_progress, abort_flag);
   } else {
     // ------------------------------------------------------------ epilogue
     const int et = threadIdx.x - 64;                       // 0 .. kEpilogueThreads-1
@@ -202,12 +140,12 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     const int sub = (warp - 2) >> 2;                       // owns chunks sub and sub + 4
     const int row_in_tile = quarter * 32 + lane;
     const uint32_t taddr0 = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-    const uint32_t acc_sets = 4 * p.N <= p.tmem_cols ? 2u : 1u;
+    const uint32_t acc_sets = static_cast<uint32_t>(p.acc_sets), set_cols = static_cast<uint32_t>(p.issuers * p.N);
     const int E = p.E, N = p.N, k = p.k;
     constexpr bool sigmoid_gate = kSigmoid;
     const int n_chunks = E >> 5;                           // E is a multiple of 32 here
     constexpr bool has_lb = kLogitBias;
-    const bool two_acc = p.num_kb > 1;
+    const bool two_acc = p.issuers == 2 && p.num_kb > 1;
     // scratch behind the pipeline stages
     float* gscore_s = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)) +
                                                static_cast<size_t>(p.stages) * stage_bytes);   // [8][128]
@@ -239,7 +177,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
 
       // one thread polls for the finished accumulators, the others sleep at the barrier
       const uint32_t set = tiles_done % acc_sets, use = tiles_done / acc_sets;
-      const uint32_t taddr = taddr0 + set * 2u * static_cast<uint32_t>(N);
+      const uint32_t taddr = taddr0 + set * set_cols;
       if (et == 0) sh.accum_ok = mbar_wait<true>(smem_u32(&sh.accum_bar[set]), use & 1u, abort_flag) ? 1 : 0;
       named_bar_sync(kAccumBarrierId, kEpilogueThreads);
       if (sh.accum_ok == 0) break;

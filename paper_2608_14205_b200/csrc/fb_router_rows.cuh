@@ -46,6 +46,7 @@ inline int gate_layout(int E, int gate, int n_group, int topk_group, RouterParam
   // one group, or whole vectors per group: round the lane's share up so that it is one vector load
   p->vector_load = (groups == 1 || gs % cpl == 0) ? 1 : 0;
   p->cols_per_lane = p->vector_load ? cpl : per_lane;
+  p->two_vectors = (cpl == 8 && p->vector_load && (groups == 1 || lpg * 8 == gs)) ? 1 : 0;   // lane = column / 8
   p->ragged = !(p->vector_load && groups * lpg * cpl == E && groups * lpg == 32) ? 1 : 0;
   return cpl;
 }
@@ -53,7 +54,11 @@ inline int gate_layout(int E, int gate, int n_group, int topk_group, RouterParam
 // Staged logits: rows of N + 4 floats.  A warp writes 32 rows of one 16-byte column group at a time, 8
 // rows per wavefront: N is a multiple of 16, so the row stride is 4 or 20 words modulo 32 and those 8 rows
 // hit all 32 banks once.
-__host__ __device__ constexpr int staging_stride(int N) { return N + 4; }
+// Rows of more than 128 columns are padded to 256: lanes with eight columns each hold two vectors, which
+// are stored 128 words apart (all lanes' first vectors, then all second ones), so that a warp's loads are
+// contiguous - for rows of other blocks, read over the cluster's network, 512-byte pieces instead of
+// 16-byte ones (1733 tokens, 256 experts, four pairs per tile: the selection took 13 us with the latter).
+__host__ __device__ constexpr int staging_stride(int N) { return (N > 128 ? 256 : N) + 4; }
 constexpr int kListStride = kCandCap + 12;     // + the last lane's columns, rounded up (never read); 12 banks apart for two rows
 struct RowScratch {                    // one per epilogue warp
   alignas(16) float cand_key[2][kListStride];  // keys of two rows' candidates in ascending id order; -inf behind the last one
@@ -69,8 +74,8 @@ __host__ __device__ constexpr size_t staging_bytes(int rows, int N) {
 struct RowsShared {
   uint64_t full_bar[kMaxStages];
   uint64_t empty_bar[kMaxStages];
-  // Accumulator sets: one (2 N of the 512 tensor-memory columns) or, when 4 N <= 512 and a pair walks
-  // several tiles, two that alternate, so that the next tile's MMAs need not wait for the drain.
+  // Accumulator sets (of N columns per issuer): one, or two that alternate where a pair walks several
+  // tiles, so that the next tile's MMAs need not wait for the drain.
   uint64_t accum_bar[2];                     // per set: both issuers' commits, once per use
   uint64_t tmem_empty_bar[2];                // per set, even block's copy: all epilogue warps of the pair, once per use
   uint32_t tmem_base;
@@ -88,6 +93,7 @@ struct RowsShared {
 // What a lane needs to know about its columns.
 struct LaneColumns {
   int32_t c0, n;                       // first column, number of columns
+  int32_t word;                        // where they start in a staged row
   int32_t group;                       // group of its columns (>= groups: an idle lane)
 };
 
@@ -116,6 +122,9 @@ __device__ __noinline__ void select_slow(float* keys, int E, int k, float* win_k
 // place.  Lanes without columns read valid words all the same; what they read is masked afterwards.
 template <int kCpl>
 __device__ __forceinline__ void load_columns(float (&z)[kCpl], uint32_t addr, const RouterParams& p, int n) {
+  if constexpr (kCpl == 8) {
+    if (p.two_vectors) { ld_shared_two_vectors(addr, z); return; }
+  }
   if (kCpl == 1 || p.vector_load) {
     ld_shared_floats<kCpl>(addr, z);
   } else {
@@ -126,6 +135,9 @@ __device__ __forceinline__ void load_columns(float (&z)[kCpl], uint32_t addr, co
 template <int kCpl>
 __device__ __forceinline__ void load_columns_of(float (&z)[kCpl], uint32_t addr, uint32_t rank, const RouterParams& p, int n) {
   const uint32_t remote = map_to_cta(addr, rank);
+  if constexpr (kCpl == 8) {
+    if (p.two_vectors) { ld_cluster_two_vectors(remote, z); return; }
+  }
   if (kCpl == 1 || p.vector_load) {
     ld_cluster_floats<kCpl>(remote, z);
   } else {
@@ -172,7 +184,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
   const bool want_sum = !kSigmoid && p.topk_w != nullptr && !p.renorm;
   float key[2][kCpl];
   // ---- logits: the J partial sums in order
-  const uint32_t a0 = row_addr + static_cast<uint32_t>(lc.c0) * 4u;
+  const uint32_t a0 = row_addr + static_cast<uint32_t>(lc.word) * 4u;
   if (p.pieces == 1) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) load_columns<kCpl>(key[u], a0 + u * stride, p, lc.n);
@@ -488,7 +500,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   extern __shared__ uint8_t smem_raw[];
   __shared__ RowsShared sh;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);      // warp-uniform for the compiler as well
   const int lane = threadIdx.x & 31;
   const uint32_t cluster_rank = cluster_ctarank();
   const uint32_t cta_rank = cluster_rank & 1u;               // which block of its pair
@@ -520,7 +532,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       mbar_init(smem_u32(&sh.empty_bar[s]), 1);
     }
     for (int a = 0; a < 2; ++a) {
-      mbar_init(smem_u32(&sh.accum_bar[a]), 2);              // one commit per MMA issuer
+      mbar_init(smem_u32(&sh.accum_bar[a]), static_cast<uint32_t>(p.issuers));   // one commit per MMA issuer
       mbar_init(smem_u32(&sh.tmem_empty_bar[a]), 2 * kEpilogueWarps);
     }
     fence_mbar_init();
@@ -539,7 +551,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   }
   tcgen05_fence_before();
   __syncthreads();
-  cluster_arrive(); cluster_wait();          // the other blocks' barriers and tensor memory are ready too
+  cluster_arrive_relaxed(); cluster_wait();  // the other blocks' barriers and tensor memory are ready too
   tcgen05_fence_after();
   // (see fb_router_kernel for these two)
   pdl_wait();
@@ -548,92 +560,20 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   FB_STAMP(1, 64);
   bool closing_arrived = false;              // this warp has delivered its arrival for the closing cluster barrier
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const uint64_t pol_x = l2_policy_evict_first();        // x is streamed once
-      const uint64_t pol_w = l2_policy_evict_last();         // W is re-read by every pair
-      int s = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int pt = pair_first; pt < total_pairs && ok; pt += pair_stride) {
-        const bool second_pass = pt >= pairs_per_pass;
-        const int tile = 2 * (second_pass ? pt - pairs_per_pass : pt) + static_cast<int>(cta_rank);
-        const CUtensorMap* xmap = second_pass ? &tmap_x2 : &tmap_x;
-        for (int kb = kb0; kb < kb0 + n_kb; ++kb) {
-          ok = mbar_wait<true>(smem_u32(&sh.empty_bar[s]), phase ^ 1u, abort_flag);
-          if (!ok) break;
-          if (kb == kb0) FB_STAMP(14, 0);
-          if (kb == kb0 + n_kb - 1) FB_STAMP(15, 0);
-          const uint32_t a_dst = smem_base + static_cast<uint32_t>(s) * stage_bytes;
-          // both blocks of the pair report their bytes to the even block's barrier, which expects
-          // the bytes of both
-          const uint32_t full = map_to_cta(smem_u32(&sh.full_bar[s]), lead_rank);
-          if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&sh.full_bar[s]), 2u * stage_bytes);
-          tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, tile * kTileM, pol_x);
-          tma_load_2d_pair(a_dst + kATileBytes, &tmap_w, full, kb * kBlockK,
-                           static_cast<int32_t>(cta_rank) * (p.N / 2), pol_w);
-          ring_advance(s, phase, p.stages);
-        }
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1 || warp == kSecondIssuerWarp) {
-    // ------------------------------------------------------------ MMA issuers (even block only)
-    // warp 1: the piece's k-blocks 0, 2, 4, ... into accumulator 0; the last warp: 1, 3, 5, ... into
-    // accumulator 1 (N columns further).
-    if (lane == 0 && cta_rank == 0) {
-      const int first_kb = warp == 1 ? 0 : 1;
-      const uint32_t acc_sets = 4 * p.N <= p.tmem_cols ? 2u : 1u;
-      const uint32_t idesc = umma_idesc_bf16_f32(kTileM * 2, static_cast<uint32_t>(p.N));
-      int s = 0;
-      uint32_t phase = 0;
-      uint32_t ti = 0;                        // this pair's tile counter
-      bool ok = true;
-      int32_t g = 0;                          // ring position: k-blocks of all of this pair's tiles, in order
-      const bool odd_ring = (p.stages & 1) != 0;
-      volatile int32_t* my_progress = &sh.issuer_progress[warp == 1 ? 0 : 1];
-      const volatile int32_t* other_progress = &sh.issuer_progress[warp == 1 ? 1 : 0];
-      for (int pt = pair_first; pt < total_pairs && ok; pt += pair_stride, ++ti) {
-        const uint32_t set = ti % acc_sets, use = ti / acc_sets;
-        const uint32_t acc = tmem_base + set * 2u * static_cast<uint32_t>(p.N) + (warp == 1 ? 0u : static_cast<uint32_t>(p.N));
-        if (use != 0) {
-          // the set's previous contents must have been read out by both blocks
-          ok = mbar_wait<true>(smem_u32(&sh.tmem_empty_bar[set]), (use - 1u) & 1u, abort_flag);
-          if (!ok) break;
-          tcgen05_fence_after();
-        }
-        for (int kb = 0; kb < n_kb; ++kb, ++g) {
-          if ((kb & 1) == first_kb) {
-            if (odd_ring && g >= p.stages) {
-              // whose was the stage's previous use (ring position g - stages)?  Its k-block index
-              // inside its own tile decides, as for every k-block.
-              int kbp = kb - p.stages;
-              while (kbp < 0) kbp += n_kb;
-              if ((kbp & 1) != first_kb) ok = issuer_turn_wait(other_progress, g - p.stages, abort_flag);
-            }
-            ok = ok && mbar_wait<true>(smem_u32(&sh.full_bar[s]), phase, abort_flag);
-            if (!ok) break;
-            if (odd_ring) *my_progress = g;
-            tcgen05_fence_after();
-            if (kb == 0) FB_STAMP(16, 32);
-            const uint32_t a_addr = smem_base + static_cast<uint32_t>(s) * stage_bytes;
-            const uint64_t adesc = umma_smem_desc_sw128(a_addr);
-            const uint64_t bdesc = umma_smem_desc_sw128(a_addr + kATileBytes);
-            if (p.probe != 1) {
-              // advance 16 elements = 32 bytes inside the swizzled row: +2 in the address field
-#pragma unroll
-              for (int kk = 0; kk < kBlockK / kUmmaK; ++kk)
-                umma_bf16<2>(acc, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb != first_kb || kk != 0) ? 1u : 0u);
-            }
-            umma_commit_pair(smem_u32(&sh.empty_bar[s]), cluster_rank);   // frees the stage in both blocks
-          }
-          ring_advance(s, phase, p.stages);
-        }
-        if (warp == 1) FB_STAMP(17, 32);
-        if (ok) umma_commit_pair(smem_u32(&sh.accum_bar[set]), cluster_rank);   // this issuer's accumulator is complete
-      }
-    }
+  if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
+    TileWalk walk;
+    walk.pair_first = pair_first;
+    walk.pair_stride = pair_stride;
+    walk.total_pairs = total_pairs;
+    walk.pairs_per_pass = pairs_per_pass;
+    walk.kb0 = kb0;
+    walk.n_kb = n_kb;
+    walk.cluster_rank = cluster_rank;
+    if (warp == 0)
+      produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
+    else if (cta_rank == 0 && (warp == 1 || p.issuers == 2))
+      issue_mmas(p, walk, warp == 1 ? 0 : 1, tmem_base, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, sh.accum_bar,
+                 sh.tmem_empty_bar, sh.issuer_progress, abort_flag);
     __syncwarp();
   } else {
     // ------------------------------------------------------------ epilogue
@@ -642,10 +582,10 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
     const int quarter = warp & 3;                          // TMEM lanes this warp may touch
     const int sub = ew >> 2;                               // copies every fourth 16-column chunk
     const uint32_t taddr0 = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-    const uint32_t acc_sets = 4 * p.N <= p.tmem_cols ? 2u : 1u;
+    const uint32_t acc_sets = static_cast<uint32_t>(p.acc_sets), set_cols = static_cast<uint32_t>(p.issuers * p.N);
     const int E = p.E, N = p.N;
     const uint32_t row_stride = static_cast<uint32_t>(staging_stride(N)) * 4u;
-    const bool two_acc = n_kb > 1;
+    const bool two_acc = p.issuers == 2 && n_kb > 1;
 
     LaneColumns lc;
     {
@@ -654,6 +594,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       lc.c0 = lc.group < p.groups ? lc.group * p.group_size + first : 0;
       lc.n = lc.group < p.groups ? max(0, min(p.cols_per_lane, p.group_size - first)) : 0;
       if (lc.n == 0) lc.c0 = 0;
+      lc.word = p.two_vectors ? 4 * lane : lc.c0;
     }
     // While the main loop runs, stage the biases and the placement for the planner (any block may
     // turn out to be the last one).
@@ -679,7 +620,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 
       // one thread polls for the finished accumulators, the others sleep at the barrier
       const uint32_t set = tiles_done % acc_sets, use = tiles_done / acc_sets;
-      const uint32_t taddr = taddr0 + set * 2u * static_cast<uint32_t>(N);
+      const uint32_t taddr = taddr0 + set * set_cols;
       if (et == 0) sh.accum_ok = mbar_wait<true>(smem_u32(&sh.accum_bar[set]), use & 1u, abort_flag) ? 1 : 0;
       named_bar_sync(kAccumBarrierId, kEpilogueThreads);
       const bool got = sh.accum_ok != 0 && p.probe == 0;     // a measurement launch ends with its main loop
@@ -712,7 +653,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
               }
 #pragma unroll
               for (int q = 0; q < 4; ++q)
-                st_shared_v4(dst + static_cast<uint32_t>(c0 + 4 * q) * 4u, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                st_shared_v4(dst + static_cast<uint32_t>(p.two_vectors ? (q & 1) * 128 + (c0 + 4 * q) / 8 * 4 : c0 + 4 * q) * 4u, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
             }
           }
           tcgen05_fence_before();

@@ -64,6 +64,7 @@ struct fb_ctx {
   uint32_t* counts_scratch = nullptr;   // [256], zero between calls
   uint32_t* ticket = nullptr;           // [1],   zero between calls
   int32_t* status = nullptr;            // [1]
+  uint8_t* early_counts = nullptr;      // the same for the early pass of a layer call whose plan is made with the index
   uint8_t* slice_counts = nullptr;      // [max_slices][slice_row_bytes(E)]: per-slice histograms for the dispatch index
   // descriptor cache
   MapEntry x_maps[kMapCache];
@@ -253,10 +254,11 @@ fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* cou
 // Launch a router kernel in one of its modes.
 // x2 is the second input of kModeLayer (the normal router input), nullptr otherwise.
 // *pieces_out (optional): block pairs per tile pair, i.e. row slices per tile of the histogram table.
+// *deferred_out (layer calls): the dispatch-index kernel has to count and plan.
 fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T, int mode,
                         uint32_t* counts_out, int32_t* topk_ids, float* topk_w, float* logits,
                         const fb::PlanParams* plan, cudaStream_t stream, const void* x2 = nullptr, int probe = 0,
-                        int* pieces_out = nullptr) {
+                        int* pieces_out = nullptr, bool* deferred_out = nullptr) {
   const CUtensorMap *mx = nullptr, *mx2 = nullptr, *mw = nullptr;
   fb_status st = make_map(ctx, ctx->x_maps, &ctx->x_next, x, T, fb::kTileM, &mx);
   if (st != FB_OK) return st;
@@ -310,6 +312,15 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   // several pairs and all other gates take the row-per-warp selection (figures: fb_router_rows.cuh).
   const bool ranking = J == 1 && ctx->ranking[topk_w != nullptr ? 1 : 0];
   const bool several = J == 1 && probe == 0 && tile_pairs > pairs_avail && !(ranking && logits != nullptr);
+  // Both passes of the layer at the same time: nothing could hide the planner behind the second pass, so
+  // the dispatch-index kernel counts and plans (see fb_dispatch_kernel).  With several tiles per pair the
+  // early pass is done long before the normal one and its last block plans meanwhile.
+  p.defer_counts = (mode == fb::kModeLayer && !several && p.fuse_planner && deferred_out != nullptr) ? 1 : 0;
+  if (p.defer_counts) {
+    p.fuse_planner = 0;
+    p.early_counts = ctx->early_counts;
+    *deferred_out = true;
+  }
   int clusters = tile_pairs;
   if (several) {
     // no more pairs than the number of rounds needs: 128 tile pairs run as 2 rounds on 64
@@ -365,16 +376,20 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   ++ctx->launches;
   if (several) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
-  if (plan_wanted && !p.fuse_planner) return launch_plan(ctx, *plan, counts_out, stream);
+  if (plan_wanted && !p.fuse_planner && !p.defer_counts) return launch_plan(ctx, *plan, counts_out, stream);
   return FB_OK;
 }
 
-// Dispatch index from the router kernel's top-k ids and per-slice histograms.
-fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, const int32_t* expert_to_slot, const int32_t* topk_ids,
+// Dispatch index from the router kernel's top-k ids and per-slice histograms.  plan: also the count vector and
+// the plan, from the early pass's histograms (one tile per block only; expert_to_slot is then the placement
+// before the plan, and the index is made under the one after it).
+fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, const fb::PlanParams* plan,
+                                uint32_t* counts_out, const int32_t* expert_to_slot, const int32_t* topk_ids,
                                 uint32_t* slot_offsets, uint32_t* rank_offsets, int32_t* perm, int32_t* inv_perm,
                                 uint32_t* rank_load, cudaStream_t stream) {
   const fb_config& c = ctx->cfg;
   fb::DispatchParams dp;
+  memset(&dp, 0, sizeof(dp));
   dp.T = T; dp.k = c.k; dp.E = c.E; dp.R = c.R;
   dp.num_tiles = (T + fb::kDispatchTile - 1) / fb::kDispatchTile;
   dp.topk_ids = topk_ids;
@@ -382,6 +397,9 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   const int slice_rows = fb::kDispatchTile / slices_per_tile;
   dp.num_slices = (T + slice_rows - 1) / slice_rows;
   dp.slice_counts = ctx->slice_counts;
+  dp.early_counts = ctx->early_counts;
+  dp.counts_out = counts_out;
+  if (plan) dp.plan = *plan;
   dp.expert_to_slot = expert_to_slot;
   dp.slot_offsets = slot_offsets;
   dp.rank_offsets = rank_offsets;
@@ -391,9 +409,11 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   dp.status = ctx->status;
   // one block per SM at most: more tiles than that are walked in runs (every block reads the whole
   // histogram table once, so more blocks would only read it more often)
-  const int dispatch_blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;
-  const cudaError_t err = launch_dependent(dispatch_blocks < dp.num_tiles ? fb::fb_dispatch_kernel<true> : fb::fb_dispatch_kernel<false>,
-                                           dispatch_blocks, fb::kDispatchThreads, stream, dp);
+  const int blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;
+  const cudaError_t err = launch_dependent(blocks < dp.num_tiles ? fb::fb_dispatch_runs_kernel
+                                           : plan != nullptr     ? fb::fb_dispatch_kernel<true>
+                                                                 : fb::fb_dispatch_kernel<false>,
+                                           blocks, fb::kDispatchThreads, stream, dp);
   ++ctx->launches;
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
@@ -600,7 +620,8 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
   bool ok = count_clusters(ctx) == FB_OK;
   ok = ok && dev_alloc(&ctx->counts_scratch, FB_MAX_EXPERTS) && dev_alloc(&ctx->ticket, 1) &&
        dev_alloc(&ctx->status, 1) &&
-       dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E));
+       dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E)) &&
+       dev_alloc(&ctx->early_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E));
   ok = ok && cudaMemset(ctx->counts_scratch, 0, FB_MAX_EXPERTS * sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->ticket, 0, sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess;
@@ -613,7 +634,7 @@ fb_status fb_destroy(fb_ctx* ctx) {
   if (!ctx) return FB_OK;
   DeviceGuard guard(ctx->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->st_hprev, ctx->st_H,
+  void* ptrs[] = {ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->early_counts, ctx->st_hprev, ctx->st_H,
                   ctx->st_pi, ctx->st_pi_out, ctx->st_counts, ctx->st_swaps, ctx->st_nswaps, ctx->st_load_before,
                   ctx->st_load_after, ctx->st_ids, ctx->st_w, ctx->st_slot_offsets, ctx->st_rank_offsets,
                   ctx->st_perm, ctx->st_inv_perm, ctx->st_rank_load};
@@ -703,7 +724,7 @@ fb_status fb_route_dispatch(fb_ctx* ctx, const fb_router* router, const void* x,
   const fb_status st = launch_router(ctx, router, x, T, fb::kModeDispatch, nullptr, topk_ids, topk_w, logits,
                                      nullptr, stream, nullptr, 0, &pieces);
   if (st != FB_OK) return st;
-  return launch_dispatch_index(ctx, T, pieces, expert_to_slot, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
+  return launch_dispatch_index(ctx, T, pieces, nullptr, nullptr, expert_to_slot, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
                                rank_load, stream);
 }
 
@@ -735,9 +756,11 @@ fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev
   if (!guard.ok) return FB_ERR_CUDA;
   // one launch for both router passes; the dispatch index needs the new placement and follows
   int pieces = 1;
-  st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, nullptr, &pp, stream, H, 0, &pieces);
+  bool deferred = false;
+  st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, nullptr, &pp, stream, H, 0, &pieces,
+                     &deferred);
   if (st != FB_OK) return st;
-  return launch_dispatch_index(ctx, T, pieces, expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
+  return launch_dispatch_index(ctx, T, pieces, deferred ? &pp : nullptr, counts, deferred ? expert_to_slot : expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
                                rank_load, stream);
 }
 

@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include "../../include/freebalance.h"
+#include "fb_planner.cuh"
 #include "fb_ptx.cuh"
 
 namespace fb {
@@ -45,6 +46,11 @@ struct DispatchParams {
   int32_t* inv_perm;               // [T*k]
   uint32_t* rank_load;             // [R]
   int32_t* status;
+  // fb_dispatch_kernel<true>: the histogram table of the early pass, the count vector and the plan that
+  // are formed from it, and whose output placement the index is made under
+  const uint8_t* early_counts;     // [num_slices][slice_row_bytes(E)]
+  uint32_t* counts_out;            // [E]
+  PlanParams plan;
 };
 
 // Four bytes as two pairs of 16-bit counters.
@@ -53,13 +59,222 @@ __device__ __forceinline__ void add_bytes(uint32_t& even, uint32_t& odd, uint32_
   odd += (w >> 8) & 0x00ff00ffu;
 }
 
-// kRuns: a block walks several tiles (more tiles than SMs).  The instance for one tile per block carries
-// none of that: in a launch of a few microseconds the instructions themselves have to be fetched, and
-// the code for runs costs it 1 us (512 tokens, 8 experts: layer step 21.1 -> 20.1 us without it).
-template <bool kRuns>
+// What a thread holds of one 16-byte unit's column sums, and the sums over a warp: word i of a unit holds
+// bytes (4 (i / 2) + (i & 1)) and that + 2 as 16-bit counters.
+struct UnitSums {
+  uint32_t all[8], earlier[8];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) all[i] = earlier[i] = 0;
+  }
+  __device__ __forceinline__ void add(const uint4& v, bool is_earlier) {
+    const uint32_t keep = is_earlier ? 0xffffffffu : 0u;
+    add_bytes(all[0], all[1], v.x); add_bytes(all[2], all[3], v.y);
+    add_bytes(all[4], all[5], v.z); add_bytes(all[6], all[7], v.w);
+    add_bytes(earlier[0], earlier[1], v.x & keep); add_bytes(earlier[2], earlier[3], v.y & keep);
+    add_bytes(earlier[4], earlier[5], v.z & keep); add_bytes(earlier[6], earlier[7], v.w & keep);
+  }
+  // Adds up the warp's threads and leaves the result in part[0 = all, 1 = earlier][i * U + unit]; U units
+  // per row, lane l of the warp holds unit (l + first) % U (nothing if !holds).  The whole warp calls it.
+  __device__ __forceinline__ void to_warp(uint32_t (*part)[FB_MAX_EXPERTS / 2], int U, int unit, int lane, bool holds) {
+    if ((U & (U - 1)) == 0) {                      // units of a warp repeat every U lanes
+      for (int off = U; off < 32; off <<= 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          all[i] += __shfl_xor_sync(0xffffffffu, all[i], off);
+          earlier[i] += __shfl_xor_sync(0xffffffffu, earlier[i], off);
+        }
+      }
+      if (lane < U) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { part[0][i * U + lane] = all[i]; part[1][i * U + lane] = earlier[i]; }
+      }
+    } else {
+      // a unit count that does not divide a warp (E = 160, say): shared-memory adds
+      for (int i = lane; i < 8 * U; i += 32) { part[0][i] = 0; part[1][i] = 0; }
+      __syncwarp();
+      if (holds) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (all[i]) atomicAdd(&part[0][i * U + unit], all[i]);
+          if (earlier[i]) atomicAdd(&part[1][i * U + unit], earlier[i]);
+        }
+      }
+    }
+  }
+};
+
+template <bool kFirst, class A, class B> struct Choose { using type = A; };
+template <class A, class B> struct Choose<false, A, B> { using type = B; };
+
+// Rows of a tile below `row` among those marked in m (128 bits).
+__device__ __forceinline__ uint32_t rows_before(const uint4& m, int row) {
+  const int w = row >> 5;
+  const uint32_t low = (1u << (row & 31)) - 1u;
+  return __popc(m.x & (w > 0 ? 0xffffffffu : low)) + __popc(m.y & (w > 1 ? 0xffffffffu : (w == 1 ? low : 0u))) +
+         __popc(m.z & (w > 2 ? 0xffffffffu : (w == 2 ? low : 0u))) + __popc(m.w & (w == 3 ? low : 0u));
+}
+
+// Exclusive scan of value(s) over slots 0 .. E-1 by one warp, 8 slots per lane; out(s, prefix) gets the
+// prefixes, the total is returned in lane 31.
+template <class Value, class Out>
+__device__ __forceinline__ uint32_t warp_scan_slots(int E, int lane, Value value, Out out) {
+  uint32_t v[8], run = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { v[i] = run; run += (lane * 8 + i < E) ? value(lane * 8 + i) : 0u; }
+  uint32_t incl = run;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += o;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (lane * 8 + i < E) out(lane * 8 + i, incl - run + v[i]);
+  return incl;
+}
+
+__device__ __forceinline__ void write_offsets(const DispatchParams& p, const uint32_t* offs, int t) {
+  const int m = p.E / p.R;
+  for (int s = t; s <= p.E; s += kDispatchThreads) p.slot_offsets[s] = offs[s];
+  for (int r = t; r <= p.R; r += kDispatchThreads) p.rank_offsets[r] = offs[r * m];
+  for (int r = t; r < p.R; r += kDispatchThreads) p.rank_load[r] = offs[(r + 1) * m] - offs[r * m];
+}
+
+// One tile per block (at most as many tiles as SMs).  The work per expert does not depend on the
+// placement; the slots come in with one scan at the end.
+// kPlan: the swap planner runs in here as well, in every block (its decisions are integer and reproducible,
+// so no block waits for another; block 0 writes the outputs).  Used where a layer launch runs both passes at
+// the same time: counting through global memory, electing the last block of the early pass and planning in
+// it were 3 to 5 us at the end of the router kernel with every other SM idle; here the planner works beside
+// the loads of the index.  Layer steps: 512 tokens x 8 experts 15.3 -> 13.6 us, 40 x 128 20.1 -> 19.3,
+// 1733 x 256 36.0 -> 35.2, 8192 x 128 32.0 -> 31.5.
+template <bool kPlan>
 __global__ void __launch_bounds__(kDispatchThreads, 1)
 fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
-  constexpr int kBatch = kRuns ? kDispatchBatch : 1;
+  // threads [0, 512) add up the table of the normal pass, [512, 1024) that of the early pass (kPlan)
+  constexpr int kSumThreads = kPlan ? kDispatchThreads / 2 : kDispatchThreads;
+  constexpr int kSumWarps = kSumThreads / 32;
+  struct Empty {};
+  __shared__ int32_t expert_at[FB_MAX_EXPERTS];    // slot -> expert
+  __shared__ uint32_t base[FB_MAX_EXPERTS];        // expert: assignments in earlier tiles; then the tile's first position
+  __shared__ uint32_t total[FB_MAX_EXPERTS];       // expert: assignments in all tiles
+  __shared__ uint32_t offs[FB_MAX_EXPERTS + 1];    // exclusive prefix of total over slots
+  __shared__ uint4 mask[FB_MAX_EXPERTS];           // rows of the tile that chose the expert
+  __shared__ uint32_t part[kDispatchWarps][2][FB_MAX_EXPERTS / 2];
+  __shared__ typename Choose<kPlan, PlanShared, Empty>::type plan;
+  __shared__ int32_t bad;
+
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int E = p.E, k = p.k;
+  const int tile = static_cast<int>(blockIdx.x);
+  // The next router kernel of the stream may set itself up while this grid runs (it waits for
+  // this grid's completion before it reads anything).
+  pdl_launch_dependents();
+  if (t == 0) bad = 0;
+  if (t < FB_MAX_EXPERTS) { expert_at[t] = -1; mask[t] = make_uint4(0, 0, 0, 0); }
+  if constexpr (kPlan) plan_clear(plan, t, kDispatchThreads);
+  // Thread t owns assignment t of the tile: row t / k, choice t % k (exact for t < 8192, k <= 8).
+  const int row = (t * ((65536 + k - 1) / k)) >> 16;
+  const long long flat = static_cast<long long>(tile) * kDispatchTile * k + t;
+  const long long n_assign = static_cast<long long>(p.T) * k;
+  const int row_bytes = slice_row_bytes(E), U = row_bytes >> 4;
+  const int P = kSumThreads / U, st = t % kSumThreads;
+  const int unit = st % U, slice0 = st / U;
+  const uint8_t* table = t < kSumThreads ? p.slice_counts : p.early_counts;
+  const int first_slice = tile * p.slices_per_tile;
+  __syncthreads();
+  pdl_wait();                                    // from here on: what the router kernel wrote
+  // ---- everything the block needs from global memory, before anything depends on it
+  const int my_slot = t < E ? p.expert_to_slot[t] : 0;
+  int e = (t < kDispatchTile * k && flat < n_assign) ? p.topk_ids[flat] : -1;
+  UnitSums sums;
+  sums.clear();
+  if (slice0 < P) {
+#pragma unroll 4
+    for (int s = slice0; s < p.num_slices; s += P)
+      sums.add(__ldg(reinterpret_cast<const uint4*>(table + static_cast<size_t>(s) * row_bytes) + unit), s < first_slice);
+  }
+  if (t < kDispatchTile * k && flat < n_assign) {
+#ifdef FB_DEBUG
+    if (e < 0 || e >= E) atomicCAS(p.status, 0, FB_ERR_INTERNAL);       // an expert id outside [0, E)
+#endif
+    if (e < 0 || e >= E) e = 0;
+    atomicOr(reinterpret_cast<uint32_t*>(&mask[e]) + (row >> 5), 1u << (row & 31));
+  }
+  const int warps = min(kSumWarps, (min(P, p.num_slices) * U + 31) >> 5);
+  if (warp % kSumWarps < warps) sums.to_warp(part[warp], U, unit, lane, slice0 < P);
+  if (t < E) {
+    if constexpr (kPlan) {
+      plan_place(p.plan, plan, t, my_slot);
+    } else {
+      if (my_slot < 0 || my_slot >= E || atomicExch(&expert_at[my_slot], t) != -1) bad = 1;
+    }
+  }
+  if constexpr (kPlan) plan_place_ranks(p.plan, plan, t, kDispatchThreads);
+  __syncthreads();
+  if (st < 8 * U) {
+    uint32_t all0 = 0, all1 = 0, bef0 = 0, bef1 = 0;
+    const int w0 = warp - warp % kSumWarps;
+    for (int w = w0; w < w0 + warps; ++w) {
+      const uint32_t a = part[w][0][st], b = part[w][1][st];
+      all0 += a & 0xffffu; all1 += a >> 16;
+      bef0 += b & 0xffffu; bef1 += b >> 16;
+    }
+    const int un = st % U, i = st / U;
+    const int e0 = 16 * un + 4 * (i >> 1) + (i & 1), e1 = e0 + 2;
+    if (t < kSumThreads) {
+      if (e0 < E) { total[e0] = all0; base[e0] = bef0; }
+      if (e1 < E) { total[e1] = all1; base[e1] = bef1; }
+    } else if constexpr (kPlan) {
+      if (e0 < E) { plan_put_count(plan, e0, all0); if (tile == 0) p.counts_out[e0] = all0; }
+      if (e1 < E) { plan_put_count(plan, e1, all1); if (tile == 0) p.counts_out[e1] = all1; }
+    }
+  }
+  __syncthreads();
+  uint32_t ahead = 0;
+  if (warp == 0) {
+    if constexpr (kPlan) {
+      plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
+      __syncwarp();
+      if (plan.bad && lane == 0) bad = 1;
+      for (int s = lane; s < E; s += 32)
+        expert_at[s] = plan.bad_range ? plan.expert_at[s] : static_cast<int32_t>((plan.slot_cnt[s] >> 22) & 0xffu);
+      __syncwarp();
+    }
+    const bool usable = kPlan ? *static_cast<volatile int32_t*>(&bad) == 0 : bad == 0;
+    if (usable) {
+      const uint32_t sum = warp_scan_slots(
+          E, lane, [&](int s) { return total[expert_at[s]]; },
+          [&](int s, uint32_t prefix) { offs[s] = prefix; base[expert_at[s]] += prefix; });
+      if (lane == 31) offs[E] = sum;
+    }
+  }
+  if (e >= 0) ahead = rows_before(mask[e], row);
+  __syncthreads();
+  if constexpr (kPlan)
+    if (tile == 0) plan_write_placement(p.plan, plan, t, kDispatchThreads);
+  if (bad) {                                    // not a bijection: report, write no index
+    if (!kPlan && t == 0 && tile == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
+    return;
+  }
+  if (tile == 0) write_offsets(p, offs, t);
+  if (e >= 0) {
+    const long long pos = static_cast<long long>(base[e]) + ahead;
+#ifdef FB_DEBUG
+    if (pos < 0 || pos >= n_assign) atomicCAS(p.status, 0, FB_ERR_INTERNAL);   // a position outside [0, T k)
+#endif
+    if (pos < n_assign) {
+      p.perm[pos] = static_cast<int32_t>(flat);
+      p.inv_perm[flat] = static_cast<int32_t>(pos);
+    }
+  }
+}
+
+// A run of consecutive tiles per block (more tiles than SMs).
+__global__ void __launch_bounds__(kDispatchThreads, 1)
+fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
+  constexpr int kBatch = kDispatchBatch;
   __shared__ int32_t slot_of[FB_MAX_EXPERTS];
   __shared__ int32_t owner[FB_MAX_EXPERTS];
   __shared__ uint32_t gbase[FB_MAX_EXPERTS];       // position of the slot's first assignment of this batch of tiles
@@ -114,53 +329,21 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   const int unit = t % U, slice0 = t / U;
   const int first_slice = tile_begin * p.slices_per_tile;
   const int chunk = 15 * (U < 16 ? 1 : 16);      // slices per thread and flush: 15 * 128 * 32 < 2^16, 240 * 128 * 2 < 2^16
-  const bool shuffle = (U & (U - 1)) == 0;       // units of a warp repeat every U lanes
   const bool active_part = slice0 < P;
   uint32_t sum_all0 = 0, sum_all1 = 0, sum_bef0 = 0, sum_bef1 = 0;      // thread w < row_bytes / 2: experts 2 w, 2 w + 1
   for (int s_base = 0; s_base < p.num_slices; s_base += chunk * P) {
-    uint32_t acc[16];                            // [all, earlier][8 words: even / odd bytes of the four words]
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0;
+    UnitSums sums;
+    sums.clear();
     const int s_end = min(p.num_slices, s_base + chunk * P);
     if (active_part) {
 #pragma unroll 4
-      for (int s = s_base + slice0; s < s_end; s += P) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p.slice_counts + static_cast<size_t>(s) * row_bytes) + unit);
-        const uint32_t keep = s < first_slice ? 0xffffffffu : 0u;
-        add_bytes(acc[0], acc[1], v.x); add_bytes(acc[2], acc[3], v.y);
-        add_bytes(acc[4], acc[5], v.z); add_bytes(acc[6], acc[7], v.w);
-        add_bytes(acc[8], acc[9], v.x & keep); add_bytes(acc[10], acc[11], v.y & keep);
-        add_bytes(acc[12], acc[13], v.z & keep); add_bytes(acc[14], acc[15], v.w & keep);
-      }
+      for (int s = s_base + slice0; s < s_end; s += P)
+        sums.add(__ldg(reinterpret_cast<const uint4*>(p.slice_counts + static_cast<size_t>(s) * row_bytes) + unit), s < first_slice);
     }
     const int span = min(P, s_end - s_base);     // threads of slices beyond it hold nothing
     const int warps = min(kDispatchWarps, (span * U + 31) >> 5);
     if (s_base > 0) __syncthreads();             // the previous flush has been read
-    if (shuffle) {
-      if (warp < warps) {
-        for (int off = U; off < 32; off <<= 1) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
-        }
-        if (lane < U) {
-          // word i of a unit holds bytes (4 (i / 2) + (i & 1)) and that + 2: stored as 16-bit pairs in that order
-#pragma unroll
-          for (int i = 0; i < 8; ++i) { u.part[warp][0][i * U + lane] = acc[i]; u.part[warp][1][i * U + lane] = acc[8 + i]; }
-        }
-      }
-    } else {
-      // a unit count that does not divide a warp (E = 160, say): shared-memory adds, one table row per set
-      if (warp < warps)
-        for (int i = lane; i < 8 * U; i += 32) { u.part[warp][0][i] = 0; u.part[warp][1][i] = 0; }
-      __syncwarp();
-      if (warp < warps && active_part) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (acc[i]) atomicAdd(&u.part[warp][0][i * U + unit], acc[i]);
-          if (acc[8 + i]) atomicAdd(&u.part[warp][1][i * U + unit], acc[8 + i]);
-        }
-      }
-    }
+    if (warp < warps) sums.to_warp(u.part[warp], U, unit, lane, active_part);
     __syncthreads();
     if (t < 8 * U) {
       for (int w = 0; w < warps; ++w) {
@@ -188,23 +371,12 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     if (e1 < E) { total[slot_of[e1]] = sum_all1; gbase[slot_of[e1]] = sum_bef1; }
   }
   static_assert(kDispatchThreads == kDispatchBatch * FB_MAX_EXPERTS, "one mask per thread");
-  if (t < kBatch * FB_MAX_EXPERTS) u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
+  u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
   __syncthreads();
-  // Exclusive scan of total[] over slots into offs[], by one warp, 8 slots per lane.
+  // Exclusive scan of total[] over slots into offs[], by one warp
   auto scan = [&]() {
-    uint32_t v[8], run = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { v[i] = run; run += (lane * 8 + i < E) ? total[lane * 8 + i] : 0u; }
-    uint32_t incl = run;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += o;
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (lane * 8 + i < E) offs[lane * 8 + i] = incl - run + v[i];
-    if (lane == 31) offs[E] = incl;
+    const uint32_t sum = warp_scan_slots(E, lane, [&](int s) { return total[s]; }, [&](int s, uint32_t prefix) { offs[s] = prefix; });
+    if (lane == 31) offs[E] = sum;
   };
   auto mark_rows = [&]() {
 #pragma unroll
@@ -217,18 +389,13 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   if (warp == 0) scan();
   mark_rows();
   __syncthreads();
-  if (blockIdx.x == 0) {
-    const int m = E / p.R;
-    for (int s = t; s <= E; s += kDispatchThreads) p.slot_offsets[s] = offs[s];
-    for (int r = t; r <= p.R; r += kDispatchThreads) p.rank_offsets[r] = offs[r * m];
-    for (int r = t; r < p.R; r += kDispatchThreads) p.rank_load[r] = offs[(r + 1) * m] - offs[r * m];
-  }
+  if (blockIdx.x == 0) write_offsets(p, offs, t);
   if (t < E) gbase[t] += offs[t];
   // Up to four tiles at a time.  With more than one, their assignments are first put into slot
   // order in shared memory, so that perm is written in runs (4-byte stores to as many sectors as
   // threads took 4 us of the 18 us at 131072 tokens); a single tile has runs of a few entries only and writes directly.
   for (int tile0 = tile_begin; tile0 < tile_end; tile0 += kBatch) {
-    const bool several = kRuns && tile_end - tile0 > 1;         // (the same for the whole block)
+    const bool several = tile_end - tile0 > 1;                  // (the same for the whole block)
     if (several && t < E) {
       uint32_t run = 0;
 #pragma unroll
@@ -246,18 +413,12 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     }
     int next_ids[kBatch];
 #pragma unroll
-    for (int i = 0; i < kBatch; ++i) next_ids[i] = kRuns ? load_id(tile0 + kBatch + i) : -1;
+    for (int i = 0; i < kBatch; ++i) next_ids[i] = load_id(tile0 + kBatch + i);
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) {
       if (ids[i] < 0) continue;
       const int my_slot = slot_of[ids[i]];
-      const uint4 m = u.b.mask[i][my_slot];
-      const int w = row >> 5;
-      const uint32_t low = (1u << (row & 31)) - 1u;
-      uint32_t ahead = __popc(m.x & (w > 0 ? 0xffffffffu : low)) +
-                       __popc(m.y & (w > 1 ? 0xffffffffu : (w == 1 ? low : 0u))) +
-                       __popc(m.z & (w > 2 ? 0xffffffffu : (w == 2 ? low : 0u))) +
-                       __popc(m.w & (w == 3 ? low : 0u));
+      uint32_t ahead = rows_before(u.b.mask[i][my_slot], row);
       if (several) ahead += ahead_of[i][my_slot];
       const long long pos = static_cast<long long>(gbase[my_slot]) + ahead;
       const long long flat = static_cast<long long>(tile0 + i) * kDispatchTile * k + t;
@@ -286,7 +447,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
         p.perm[pos] = static_cast<int32_t>((tile0 + static_cast<int>((v >> 10) & 3u)) * kDispatchTile * k + static_cast<int>(v & 1023u));
     }
     if (tile0 + kBatch >= tile_end) break;
-    u.b.mask[(t / FB_MAX_EXPERTS) % kBatch][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
+    u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     if (t < E) gbase[t] += total[t];
 #pragma unroll

@@ -109,24 +109,23 @@ __device__ __forceinline__ unsigned long long plan_cost_ns(const PlanParams& p, 
   return c < 1 ? 1 : c;
 }
 
-// Load the placement into shared memory, invert it and check that it is a bijection.
-// Called by `nthreads` threads (t = 0..nthreads-1); the caller synchronises afterwards.
+// Expert e's slot under the placement as given: into shared memory, inverted, checked to be a bijection.
 // sh.bad must have been cleared and sh.expert_at filled with -1 beforehand.
-__device__ __forceinline__ void plan_load_placement(const PlanParams& p, PlanShared& sh, int t, int nthreads) {
-  for (int e = t; e < p.E; e += nthreads) {
-    const int s = p.expert_to_slot[e];
-    sh.slot_of[e] = s;
-    sh.moved[e] = 0;
-    if (s < 0 || s >= p.E) sh.bad = 1;
-    else if (atomicExch(&sh.expert_at[s], e) != -1) sh.bad = 1;
-  }
-  const int m = p.E / p.R;
-  for (int e = t; e < p.E; e += nthreads) {
-    const int s = sh.slot_of[e];
-    sh.rank_of[e] = static_cast<uint8_t>((s >= 0 && s < p.E) ? s / m : 0);
-  }
+__device__ __forceinline__ void plan_place(const PlanParams& p, PlanShared& sh, int e, int s) {
+  const bool inside = s >= 0 && s < p.E;
+  sh.slot_of[e] = s;
+  sh.moved[e] = 0;
+  sh.rank_of[e] = static_cast<uint8_t>(inside ? s / (p.E / p.R) : 0);
+  if (!inside || atomicExch(&sh.expert_at[s], e) != -1) sh.bad = 1;
+}
+__device__ __forceinline__ void plan_place_ranks(const PlanParams& p, PlanShared& sh, int t, int nthreads) {
   for (int r = t; r < p.R; r += nthreads)
     sh.node_of[r] = static_cast<uint8_t>(p.ranks_per_node > 0 ? r / p.ranks_per_node : 0);
+}
+// The whole placement, by `nthreads` threads (t = 0..nthreads-1); the caller synchronises afterwards.
+__device__ __forceinline__ void plan_load_placement(const PlanParams& p, PlanShared& sh, int t, int nthreads) {
+  for (int e = t; e < p.E; e += nthreads) plan_place(p, sh, e, p.expert_to_slot[e]);
+  plan_place_ranks(p, sh, t, nthreads);
 }
 __device__ __forceinline__ void plan_clear(PlanShared& sh, int t, int nthreads) {
   if (t == 0) { sh.bad = 0; sh.bad_range = 0; sh.fast = 0; }
@@ -182,7 +181,7 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 // books at all.
 template <int kPerLane, bool kSide>
 __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanShared& sh, int lane,
-                                                      int& L0, int& L1) {
+                                                      int& L0, int& L1, bool write) {
   const int R = p.R, m = p.E / R;
   const uint32_t full = 0xffffffffu;
   constexpr uint32_t kNone = 0xffffffffu;
@@ -301,7 +300,7 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
     ++n;
     __syncwarp();                                                 // the next iteration reads what lane 0 wrote
   }
-  for (uint32_t i = lane; i < n; i += 32) {                       // the plan, in order of acceptance
+  for (uint32_t i = lane; write && i < n; i += 32) {              // the plan, in order of acceptance
     const uint32_t w = sh.link_key[i];
     fb_swap sw;
     sw.src_rank = static_cast<int32_t>(w >> 24); sw.dst_rank = static_cast<int32_t>((w >> 16) & 0xffu);
@@ -473,8 +472,11 @@ __device__ __noinline__ void plan_loop_general(const PlanParams& p, PlanShared& 
 // the instance without it (the host launches the stand-alone planner kernel behind the router
 // kernel when a plan needs the general loop - see plan_needs_general_loop): the general loop's
 // registers and code would otherwise weigh on every router kernel.
+// write: whether this warp's results go to global memory (several blocks may replay a plan, see the
+// dispatch index); only for instances without the general loop.
 template <bool kGeneral>
-__device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh, int lane, int* status) {
+__device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh, int lane, int* status,
+                                             bool write = true) {
   const int E = p.E, R = p.R, m = E / R;
   const uint32_t full = 0xffffffffu;
   __syncwarp();
@@ -486,23 +488,23 @@ __device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh
   int bad = sh.bad ? 1 : ((sh.bad_range || total > FB_MAX_COUNT_SUM) ? 2 : 0);
   if (bad) {
     // Unusable input: report it, keep the placement as given, empty plan.
-    if (lane == 0) {
+    if (lane == 0 && write) {
       atomicCAS(status, 0, bad == 1 ? FB_ERR_BAD_PLACEMENT : FB_ERR_RANGE);
       *p.n_swaps = 0;
-      sh.bad_range = 1;                          // plan_write_placement copies the input placement
     }
-    for (int r = lane; r < R; r += 32) { p.load_before[r] = 0; p.load_after[r] = 0; }
+    if (lane == 0) sh.bad_range = 1;             // plan_write_placement copies the input placement
+    for (int r = lane; write && r < R; r += 32) { p.load_before[r] = 0; p.load_after[r] = 0; }
     return;
   }
   long long L0 = -1, L1 = -1;                  // -1 marks "no such rank"
   if (lane < R) {
     L0 = static_cast<long long>(s0);
-    p.load_before[lane] = static_cast<uint32_t>(s0);
+    if (write) p.load_before[lane] = static_cast<uint32_t>(s0);
     sh.rank_spent[lane] = 0;
   }
   if (lane + 32 < R) {
     L1 = static_cast<long long>(s1);
-    p.load_before[lane + 32] = static_cast<uint32_t>(s1);
+    if (write) p.load_before[lane + 32] = static_cast<uint32_t>(s1);
     sh.rank_spent[lane + 32] = 0;
   }
   __syncwarp();
@@ -516,17 +518,17 @@ __device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh
     uint32_t n_fast;
     if (lane == 0) sh.fast = 1;
     if (!side)
-      n_fast = m <= 4 ? plan_loop_uniform<1, false>(p, sh, lane, l0, l1)
-               : m <= 8 ? plan_loop_uniform<2, false>(p, sh, lane, l0, l1)
-                        : plan_loop_uniform<8, false>(p, sh, lane, l0, l1);
+      n_fast = m <= 4 ? plan_loop_uniform<1, false>(p, sh, lane, l0, l1, write)
+               : m <= 8 ? plan_loop_uniform<2, false>(p, sh, lane, l0, l1, write)
+                        : plan_loop_uniform<8, false>(p, sh, lane, l0, l1, write);
     else
-      n_fast = m <= 4 ? plan_loop_uniform<1, true>(p, sh, lane, l0, l1)
-               : m <= 8 ? plan_loop_uniform<2, true>(p, sh, lane, l0, l1)
-                        : plan_loop_uniform<8, true>(p, sh, lane, l0, l1);
+      n_fast = m <= 4 ? plan_loop_uniform<1, true>(p, sh, lane, l0, l1, write)
+               : m <= 8 ? plan_loop_uniform<2, true>(p, sh, lane, l0, l1, write)
+                        : plan_loop_uniform<8, true>(p, sh, lane, l0, l1, write);
     FB_PLAN_STAMP(20);
-    if (lane == 0) *p.n_swaps = static_cast<int32_t>(n_fast);
-    if (lane < R) p.load_after[lane] = static_cast<uint32_t>(l0);
-    if (lane + 32 < R) p.load_after[lane + 32] = static_cast<uint32_t>(l1);
+    if (lane == 0 && write) *p.n_swaps = static_cast<int32_t>(n_fast);
+    if (lane < R && write) p.load_after[lane] = static_cast<uint32_t>(l0);
+    if (lane + 32 < R && write) p.load_after[lane + 32] = static_cast<uint32_t>(l1);
     return;
   }
   if constexpr (kGeneral) {

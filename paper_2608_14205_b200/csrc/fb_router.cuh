@@ -99,6 +99,8 @@ struct RouterParams {
   int32_t tiles_first;               // kModeLayer: blocks below this index (even) belong to the early pass
   int32_t ticket_target;             // number of blocks that take a ticket (those that publish counts)
   int32_t fuse_planner;              // prediction modes: the block that finishes last runs the planner
+  int32_t defer_counts;              // kModeLayer: the early pass leaves its histograms in early_counts and the
+                                     // dispatch-index kernel counts and plans (fb_dispatch_kernel<true>)
   // fb_router_rows_kernel only: J block pairs per tile pair (cluster size / 2), the rows staged at a time
   // while the operand ring is busy with the next tile, and the column layout of a row over the lanes of a
   // warp: lane l holds columns g group_size + (l % lanes_per_group) cols_per_lane + j of group
@@ -118,6 +120,7 @@ struct RouterParams {
   float* topk_w;                     // [T][k] or nullptr
   float* logits;                     // [T][E] or nullptr
   uint8_t* slice_counts;             // [tiles * pieces][slice_row_bytes(E)] (dispatch mode)
+  uint8_t* early_counts;             // the same table for the early pass (defer_counts)
   unsigned long long* stamps;        // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
   int32_t probe;                     // measurement aid: 1 = operands are loaded but no MMA is issued and nothing
                                      // follows the main loop; 2 = with the MMAs, still nothing after them
@@ -597,7 +600,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       sh.hist[e] = 0;
       if (e < kTileM) sh.cand_count[e] = 0;
     }
-    if (mode == kModePredictPlan) plan_clear(sh.plan, et, kEpilogueThreads);
+    if (mode == kModePredictPlan && !p.defer_counts) plan_clear(sh.plan, et, kEpilogueThreads);
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -657,7 +660,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       sh.logit_bias[e] = (p.logit_bias != nullptr && e < p.E) ? p.logit_bias[e] : 0.0f;
       sh.select_bias[e] = (p.select_bias != nullptr && e < p.E) ? p.select_bias[e] : 0.0f;
     }
-    if (mode == kModePredictPlan) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
+    if (mode == kModePredictPlan && !p.defer_counts) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
     named_bar_sync(kAccumBarrierId, kEpilogueThreads + 32);
     const bool got = sh.accum_ok != 0 && p.probe == 0;     // a measurement launch ends with its main loop
     tcgen05_fence_after();
@@ -879,9 +882,9 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       FB_STAMP(10, 64);
     }
     named_bar_sync(kPlanBarrierId, kEpilogueThreads);
-    if (mode == kModeDispatch) {
+    if (mode == kModeDispatch || p.defer_counts) {
       if (static_cast<long long>(tile) * kTileM < p.T)       // the padding block of an odd pair owns no tile
-        write_slice_counts(p.slice_counts, tile, E, sh.hist, et);
+        write_slice_counts(mode == kModeDispatch ? p.slice_counts : p.early_counts, tile, E, sh.hist, et);
     } else if (p.probe == 0) {
       publish_counts(sh, p, et, warp, lane, mode == kModePredictPlan && p.fuse_planner != 0);
     }

@@ -547,7 +547,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   if (warp >= 2) {
     const int et = threadIdx.x - 64;
     for (int e = et; e < FB_MAX_EXPERTS; e += kEpilogueThreads) sh.hist[e] = 0;
-    if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_clear(sh.plan, et, kEpilogueThreads);
+    if ((p.mode == kModePredictPlan || p.mode == kModeLayer) && !p.defer_counts) plan_clear(sh.plan, et, kEpilogueThreads);
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -606,7 +606,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 #pragma unroll
     for (int j = 0; j < kCpl; ++j)
       sb[j] = (kSigmoid && p.select_bias != nullptr && j < lc.n) ? p.select_bias[lc.c0 + j] : 0.0f;
-    if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
+    if ((p.mode == kModePredictPlan || p.mode == kModeLayer) && !p.defer_counts) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
 
     uint32_t tiles_done = 0;
     for (int pt = pair_first; pt < total_pairs; pt += pair_stride) {
@@ -702,10 +702,10 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
       if (p.probe != 0) {
         // measurement launch: nothing is published
-      } else if (mode == kModeDispatch) {
+      } else if (mode == kModeDispatch || p.defer_counts) {
         const int slice = tile * J + piece;
         if (static_cast<long long>(slice) * (kTileM / J) < p.T)  // a slice beyond the last token owns no row
-          write_slice_counts(p.slice_counts, slice, E, sh.hist, et);
+          write_slice_counts(mode == kModeDispatch ? p.slice_counts : p.early_counts, slice, E, sh.hist, et);
         if (several_tiles) {
           named_bar_sync(kPlanBarrierId, kEpilogueThreads);
           for (int e = et; e < E; e += kEpilogueThreads) sh.hist[e] = 0;

@@ -187,6 +187,16 @@ fb_status fill_plan(const fb_ctx* ctx, const fb_budget* b, const int32_t* pi, in
     if (b->expert_bytes_table == nullptr && pp->uniform_cost_ns[c] == 0) return FB_ERR_INVALID_ARG;
     pp->uniform_link_cap[c] = pp->uniform_cost_ns[c] ? b->link_ns / pp->uniform_cost_ns[c] : 0;
   }
+  // Swaps the global budget carries when every swap costs the same, and whether the planner's uniform loop
+  // has to keep books.  With one cost class a rank or a link is never charged more than the whole plan, so
+  // a side budget that starts at or above the global one (the usual case: all three start at the same B) can
+  // never stop a swap the global budget admits.
+  pp->swap_cap = b->max_swaps;
+  if (b->global_ns != FB_BUDGET_OFF && pp->uniform_cost_ns[0] != 0 && b->global_ns / pp->uniform_cost_ns[0] < pp->swap_cap)
+    pp->swap_cap = static_cast<uint32_t>(b->global_ns / pp->uniform_cost_ns[0]);
+  auto binds = [&](uint64_t side) { return side != FB_BUDGET_OFF && !(b->global_ns != FB_BUDGET_OFF && side >= b->global_ns); };
+  const bool one_node = b->ranks_per_node <= 0 || b->ranks_per_node >= pp->R;
+  pp->books = (!one_node || binds(b->rank_ns) || binds(b->link_ns)) ? 1 : 0;
   if (b->mode != FB_PLAN_LOOP && b->mode != FB_PLAN_SWEEP && b->mode != FB_PLAN_WIDE) return FB_ERR_INVALID_ARG;
   pp->mode = b->mode;
   pp->frontier_width = b->frontier_width;

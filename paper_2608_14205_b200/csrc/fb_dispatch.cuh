@@ -238,15 +238,17 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
       plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
       __syncwarp();
       if (plan.bad && lane == 0) bad = 1;
-      for (int s = lane; s < E; s += 32)
-        expert_at[s] = plan.bad_range ? plan.expert_at[s] : static_cast<int32_t>((plan.slot_cnt[s] >> 22) & 0xffu);
       __syncwarp();
     }
     const bool usable = kPlan ? *static_cast<volatile int32_t*>(&bad) == 0 : bad == 0;
+    auto expert_in = [&](int s) -> int {
+      if constexpr (kPlan) return plan.bad_range ? plan.expert_at[s] : static_cast<int>(plan.slot_cnt[s] & 0xffu);
+      else return expert_at[s];
+    };
     if (usable) {
       const uint32_t sum = warp_scan_slots(
-          E, lane, [&](int s) { return total[expert_at[s]]; },
-          [&](int s, uint32_t prefix) { offs[s] = prefix; base[expert_at[s]] += prefix; });
+          E, lane, [&](int s) { return total[expert_in(s)]; },
+          [&](int s, uint32_t prefix) { offs[s] = prefix; base[expert_in(s)] += prefix; });
       if (lane == 31) offs[E] = sum;
     }
   }

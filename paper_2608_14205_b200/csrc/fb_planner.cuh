@@ -24,6 +24,9 @@ struct PlanParams {
   uint64_t fs_per_byte[2];
   uint64_t uniform_cost_ns[2];          // Eq. 9 evaluated on the host for the uniform expert size
   uint64_t uniform_link_cap[2];         // link_ns / uniform_cost_ns: swaps one link can carry (host)
+  uint32_t swap_cap;                    // max_swaps, or fewer if the global budget carries fewer (one cost class only; host)
+  int32_t books;                        // the uniform loop has to keep books: two cost classes, or a per-rank or
+                                        // per-link budget that can stop a swap the global one admits (host)
   int32_t ranks_per_node;
   int32_t mode;                         // fb_plan_mode
   int32_t frontier_width;               // FB_PLAN_WIDE: ranks taken from each end of the load order (1..4)
@@ -67,9 +70,9 @@ struct PlanShared {
   int32_t slot_of[FB_MAX_EXPERTS];       // expert -> slot (current placement)
   int32_t expert_at[FB_MAX_EXPERTS];     // slot -> expert
   uint8_t moved[FB_MAX_EXPERTS];
-  // fast loop: one word per slot - bits 0..21 the count of the expert placed there, bits 22..29
-  // that expert's id, bit 31 set once the expert has moved
-  uint32_t slot_cnt[FB_MAX_EXPERTS];
+  // fast loop: one word per slot - the expert placed there in bits 0..7, its count above (kSlotMoved once
+  // the expert has moved)
+  alignas(16) uint32_t slot_cnt[FB_MAX_EXPERTS];
   uint8_t rank_of[FB_MAX_EXPERTS];       // expert -> rank under the placement as given
   uint8_t node_of[FB_MAX_RANKS];         // rank -> node (all 0 when every rank is in one node)
   uint32_t load[FB_MAX_RANKS];           // rank loads under the placement as given
@@ -81,9 +84,9 @@ struct PlanShared {
   int32_t fast;                          // the fast loop ran: the placement is in slot_cnt, not in expert_at
 };
 
-constexpr uint32_t kSlotCountMask = (1u << 22) - 1;
-constexpr uint32_t kSlotMoved = 1u << 31;
-static_assert(FB_MAX_COUNT_SUM <= kSlotCountMask && FB_MAX_EXPERTS <= 256, "slot word layout");
+constexpr uint32_t kSlotMoved = 1u << 23;       // as a count
+static_assert(FB_MAX_COUNT_SUM <= kSlotMoved / 4 && FB_MAX_EXPERTS <= 256, "slot word layout");
+__device__ __forceinline__ uint32_t slot_word(uint32_t count, int expert) { return count << 8 | static_cast<uint32_t>(expert); }
 
 // true if x is a better choice than y: larger benefit / cost, compared exactly as
 // cross products in 128 bits; equal ratios -> smaller (a, b, ea, eb).
@@ -140,7 +143,7 @@ __device__ __forceinline__ void plan_put_count(PlanShared& sh, int e, uint32_t c
   sh.cnt[e] = c;
   if (c > FB_MAX_COUNT_SUM) { sh.bad_range = 1; return; }
   if (sh.bad) return;
-  sh.slot_cnt[sh.slot_of[e]] = c | static_cast<uint32_t>(e) << 22;
+  sh.slot_cnt[sh.slot_of[e]] = slot_word(c, e);
   atomicAdd(&sh.load[sh.rank_of[e]], c);
 }
 
@@ -151,7 +154,7 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
   if (sh.bad || sh.bad_range) {
     for (int e = t; e < p.E; e += nthreads) p.expert_to_slot_out[e] = p.expert_to_slot[e];
   } else if (sh.fast) {
-    for (int sl = t; sl < p.E; sl += nthreads) p.expert_to_slot_out[(sh.slot_cnt[sl] >> 22) & 0xffu] = sl;
+    for (int sl = t; sl < p.E; sl += nthreads) p.expert_to_slot_out[sh.slot_cnt[sl] & 0xffu] = sl;
   } else {
     for (int sl = t; sl < p.E; sl += nthreads) p.expert_to_slot_out[sh.expert_at[sl]] = sl;
   }
@@ -168,138 +171,137 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 // (M2: largest load of the other ranks) falls with v - strictly when gamma_num > 0; when it is 0, it is
 // constant up to v = 2 M2 - La - Lb.  A pair is useful exactly if v < D (0 < d < D), and with
 // gamma_num = 0 also M2 < La, which the same comparison tests.  The best pair is therefore the one
-// with the smallest v (clamped from below when gamma_num = 0), ties to the smallest pair: 32-bit
-// keys and one warp minimum, no products and no bound on the benefits.  (Benefits formed and
-// compared per candidate took 0.41 us per swap with 8 experts per rank and 0.75 us with 16; now 0.25 and 0.3.)
-// L0 / L1: this lane's rank loads (ranks lane and lane + 32, -1 if absent).
+// with the smallest v (clamped from below when gamma_num = 0), ties to the smallest pair.
+// A moved expert counts as 2^23 tokens: paired with an unmoved one v is beyond any D, with a moved one it is
+// D, so no candidate has to be tested - only the smallest v is, against D.
+//
 // Lane l tries expert slot l / g of the heavy rank with kPerLane slots of the light one, g lanes per
-// heavy slot (kPerLane g >= m).
-// kSide: the per-rank or the per-link budget can bind.  With a uniform cost per link class
-// a rank or a link is never charged more than the whole plan, so a side budget that starts at
-// or above the global one (the usual case: all three start at the same B) can never stop a
-// swap the global budget admits; the instance without them keeps no per-rank or per-link
-// books at all.
-template <int kPerLane, bool kSide>
+// heavy slot; slots beyond m repeat the last one (the same pair twice changes nothing).  A lane keeps the
+// packed (load, rank) keys of its two ranks, so an iteration is: two warp reductions for the frontier, the
+// slot words, the smallest v of the lane, one reduction for v, one for the pair (the lane rides along), one
+// shuffle for the moved tokens.
+// kBooks: two cost classes, or per-rank or per-link budgets that can bind.  Otherwise the budgets allow
+// a fixed number of swaps (swap_cap) and the loop keeps no books at all.
+template <int kPerLane, bool kBooks>
 __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanShared& sh, int lane,
                                                       int& L0, int& L1, bool write) {
   const int R = p.R, m = p.E / R;
   const uint32_t full = 0xffffffffu;
   constexpr uint32_t kNone = 0xffffffffu;
   constexpr int g = kPerLane == 8 ? 2 : (kPerLane == 2 ? 4 : 8);     // m <= 16, <= 8, <= 4
-  const int ia = lane / g, j0 = (lane % g) * kPerLane;
+  const int ia = min(lane / g, m - 1), j0 = (lane % g) * kPerLane;
+  const bool whole = m == g * kPerLane;                           // the lane's light slots are contiguous and exist
   const bool flat = p.gamma_den == 0 || p.gamma_num == 0;
-  // loop invariants in registers (no access to the parameter block inside the loop)
-  const unsigned long long cost0 = p.uniform_cost_ns[0], cost1 = p.uniform_cost_ns[1];
-  const unsigned long long global_ns = p.global_ns, rank_ns = p.rank_ns;
-  const bool global_on = global_ns != FB_BUDGET_OFF;
-  const bool rank_on = kSide && rank_ns != FB_BUDGET_OFF, link_on = kSide && p.link_ns != FB_BUDGET_OFF;
-  // A link is only ever charged one cost (its class's), so its budget is a swap count.
-  const unsigned long long link_cap0 = p.uniform_link_cap[0], link_cap1 = p.uniform_link_cap[1];
-  const uint32_t max_swaps = p.max_swaps, tau = p.tau_tokens;
+  const uint32_t tau = p.tau_tokens, max_swaps = kBooks ? p.max_swaps : p.swap_cap;
+  // frontier keys (lowest index on ties): max of load << 6 | (63 - rank), min of load << 6 | rank
+  uint32_t h0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(63 - lane)) : 0u;
+  uint32_t h1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(31 - lane)) : 0u;
+  uint32_t l0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(lane)) : kNone;
+  uint32_t l1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(lane + 32)) : kNone;
+  // books
   uint32_t my_links[4] = {kNone, kNone, kNone, kNone};            // lane i keeps the links of swaps i, i+32, ...
   unsigned long long global_spent = 0;
   uint32_t n = 0;
   __syncwarp();
   while (n < max_swaps) {
-    // frontier (lowest index on ties): max of load<<6 | (63 - rank), min of load<<6 | rank
-    const uint32_t h0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(63 - lane)) : 0u;
-    const uint32_t h1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(31 - lane)) : 0u;
-    const uint32_t l0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(lane)) : kNone;
-    const uint32_t l1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(lane + 32)) : kNone;
-    const uint32_t hi_key = __reduce_max_sync(full, h0 > h1 ? h0 : h1);
-    const uint32_t lo_key = __reduce_min_sync(full, l0 < l1 ? l0 : l1);
+    const uint32_t hi_key = __reduce_max_sync(full, max(h0, h1));
+    const uint32_t lo_key = __reduce_min_sync(full, min(l0, l1));
     const int a = 63 - static_cast<int>(hi_key & 63u), b = static_cast<int>(lo_key & 63u);
     const int La = static_cast<int>(hi_key >> 6), Lb = static_cast<int>(lo_key >> 6);
     const int D = La - Lb;
-    // ---- every load of the iteration, before anything depends on one
     const int base_a = a * m, base_b = b * m;
-    const uint32_t wa = ia < m ? sh.slot_cnt[base_a + ia] : kSlotMoved;   // slot words: count, expert, moved
+    const uint32_t wa = sh.slot_cnt[base_a + ia];                 // slot words: count, expert
     uint32_t wb[kPerLane];
+    if (kPerLane == 8 && whole) {
+      const uint4 q0 = *reinterpret_cast<const uint4*>(&sh.slot_cnt[base_b + j0]);
+      const uint4 q1 = *reinterpret_cast<const uint4*>(&sh.slot_cnt[base_b + j0 + 4]);
+      wb[0] = q0.x; wb[1 % kPerLane] = q0.y; wb[2 % kPerLane] = q0.z; wb[3 % kPerLane] = q0.w;
+      wb[4 % kPerLane] = q1.x; wb[5 % kPerLane] = q1.y; wb[6 % kPerLane] = q1.z; wb[7 % kPerLane] = q1.w;
+    } else {
 #pragma unroll
-    for (int t = 0; t < kPerLane; ++t) wb[t] = j0 + t < m ? sh.slot_cnt[base_b + j0 + t] : kSlotMoved;
-    unsigned long long rs_a = 0, rs_b = 0;
-    if (kSide) { rs_a = sh.rank_spent[a]; rs_b = sh.rank_spent[b]; }
-    const int node_a = sh.node_of[a], node_b = sh.node_of[b];
+      for (int t = 0; t < kPerLane; ++t) wb[t] = sh.slot_cnt[base_b + min(j0 + t, m - 1)];
+    }
+    if (static_cast<uint32_t>(D) <= tau) break;                   // (the same in all lanes)
+    unsigned long long c_ns = 0, rs_a = 0, rs_b = 0;
+    uint32_t lkey = 0;
+    if (kBooks) {
+      // the cost is the same for every pair of this iteration
+      rs_a = sh.rank_spent[a]; rs_b = sh.rank_spent[b];
+      const int node_a = sh.node_of[a], node_b = sh.node_of[b];
+      const int cls = node_a == node_b ? 0 : 1;
+      c_ns = p.uniform_cost_ns[cls];
+      // link: the unordered rank pair inside a node, the unordered node pair across nodes
+      const int ka = cls ? node_a : a, kb = cls ? node_b : b;
+      lkey = static_cast<uint32_t>(cls) << 16 | static_cast<uint32_t>(ka < kb ? ka : kb) << 8 |
+             static_cast<uint32_t>(ka < kb ? kb : ka);
+      bool stop = p.global_ns != FB_BUDGET_OFF && (c_ns > p.global_ns || global_spent > p.global_ns - c_ns);
+      const unsigned long long rs = rs_a > rs_b ? rs_a : rs_b;
+      stop = stop || (p.rank_ns != FB_BUDGET_OFF && (c_ns > p.rank_ns || rs > p.rank_ns - c_ns));
+      if (p.link_ns != FB_BUDGET_OFF) {
+        // A link is only ever charged one cost (its class's), so its budget is a swap count.
+        uint32_t used = 0;                                       // swaps already charged to this link
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (n > 32u * q) used += __popc(__ballot_sync(full, my_links[q] == lkey));    // n is the same in all lanes
+        stop = stop || used >= p.uniform_link_cap[cls];
+      }
+      if (stop) break;
+    }
     int v_floor = 0;
     if (flat) {
-      int m2l = 0;
-      if (lane != a && lane != b && L0 > m2l) m2l = L0;
-      if (lane + 32 != a && lane + 32 != b && L1 > m2l) m2l = L1;
-      v_floor = 2 * static_cast<int>(__reduce_max_sync(full, static_cast<uint32_t>(m2l))) - La - Lb;
+      const uint32_t m2 = max(lane != a && lane != b ? h0 >> 6 : 0u, lane + 32 != a && lane + 32 != b ? h1 >> 6 : 0u);
+      v_floor = 2 * static_cast<int>(__reduce_max_sync(full, m2)) - La - Lb;
     }
-    // ---- candidates of this lane: smallest v, ties -> smallest expert of the light rank
+    // ---- smallest v of this lane, ties -> smallest expert of the light rank
+    const int x = 2 * static_cast<int>(wa >> 8) - D;
     uint32_t key[kPerLane];
 #pragma unroll
     for (int t = 0; t < kPerLane; ++t) {
-      const int dlt = static_cast<int>(wa & kSlotCountMask) - static_cast<int>(wb[t] & kSlotCountMask);   // tokens moved a -> b
-      int v = 2 * dlt - D;
-      v = v < 0 ? -v : v;
-      v = v < v_floor ? v_floor : v;
-      const bool usable = ((wa | wb[t]) >> 31) == 0 && v < D;              // neither expert moved yet
-      key[t] = usable ? static_cast<uint32_t>(v) << 8 | ((wb[t] >> 22) & 0xffu) : kNone;   // v < 2^22
+      const int v = max(abs(x - 2 * static_cast<int>(wb[t] >> 8)), v_floor);
+      key[t] = static_cast<uint32_t>(min(v, (1 << 24) - 1)) << 8 | (wb[t] & 0xffu);
     }
     uint32_t best = key[0];
 #pragma unroll
-    for (int t = 1; t < kPerLane; ++t) best = key[t] < best ? key[t] : best;
+    for (int t = 1; t < kPerLane; ++t) best = min(best, key[t]);
     const uint32_t mine = best >> 8;
     const uint32_t top = __reduce_min_sync(full, mine);
-    uint32_t my_wb = wb[0];
-    int my_jb = j0;
+    int jb = 0, delta = 0;
 #pragma unroll
-    for (int t = 1; t < kPerLane; ++t)
-      if (key[t] == best) { my_wb = wb[t]; my_jb = j0 + t; }      // one slot per expert: at most one t matches a valid key
-    // ---- budgets: the cost is the same for every pair of this iteration
-    const int cls = node_a == node_b ? 0 : 1;
-    const unsigned long long c_ns = cls ? cost1 : cost0;
-    // link: the unordered rank pair inside a node, the unordered node pair across nodes
-    const int ka = cls ? node_a : a, kb = cls ? node_b : b;
-    const uint32_t lkey = static_cast<uint32_t>(cls) << 16 | static_cast<uint32_t>(ka < kb ? ka : kb) << 8 |
-                          static_cast<uint32_t>(ka < kb ? kb : ka);
-    bool stop = static_cast<uint32_t>(D) <= tau;
-    stop = stop || (global_on && (c_ns > global_ns || global_spent > global_ns - c_ns));
-    const unsigned long long rs = rs_a > rs_b ? rs_a : rs_b;
-    stop = stop || (rank_on && (c_ns > rank_ns || rs > rank_ns - c_ns));
-    if (link_on) {
-      uint32_t used = 0;                                         // swaps already charged to this link
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (n > 32u * q) used += __popc(__ballot_sync(full, my_links[q] == lkey));    // n is the same in all lanes
-      stop = stop || used >= (cls ? link_cap1 : link_cap0);
-    }
-    if (stop || top == kNone >> 8) break;                         // Algorithm 1 lines 6-7
-    // the winner: the only lane with the smallest v, or among several the smallest (expert on a, expert on b)
-    uint32_t holders = __ballot_sync(full, mine == top);
-    if (__popc(holders) > 1) {
-      const uint32_t pair = mine == top ? ((wa >> 22) & 0xffu) << 8 | (best & 0xffu) : kNone;
-      holders = __ballot_sync(full, pair == __reduce_min_sync(full, pair));
-    }
-    const int src = __ffs(holders) - 1;
-    const uint32_t wwa = __shfl_sync(full, wa, src), wwb = __shfl_sync(full, my_wb, src);
-    const int slots = __shfl_sync(full, ia << 8 | my_jb, src);
-    const int dlt = static_cast<int>(wwa & kSlotCountMask) - static_cast<int>(wwb & kSlotCountMask);
-    if (lane == 0) {
+    for (int t = kPerLane - 1; t >= 0; --t)
+      if (key[t] == best) { jb = t; delta = static_cast<int>(wa >> 8) - static_cast<int>(wb[t] >> 8); }   // tokens moved a -> b
+    if (top >= static_cast<uint32_t>(D)) break;                   // Algorithm 1 lines 6-7
+    const uint32_t win = __reduce_min_sync(
+        full, mine == top ? (wa & 0xffu) << 13 | (best & 0xffu) << 5 | static_cast<uint32_t>(lane) : kNone);
+    const int src = static_cast<int>(win & 31u);
+    const int dlt = __shfl_sync(full, delta, src);
+    if (lane == src) {
       // the two experts trade slots
-      sh.slot_cnt[base_a + (slots >> 8)] = wwb | kSlotMoved;
-      sh.slot_cnt[base_b + (slots & 0xff)] = wwa | kSlotMoved;
-      if (kSide) { sh.rank_spent[a] = rs_a + c_ns; sh.rank_spent[b] = rs_b + c_ns; }
+      sh.slot_cnt[base_a + ia] = slot_word(kSlotMoved, static_cast<int>(best & 0xffu));
+      sh.slot_cnt[base_b + min(j0 + jb, m - 1)] = slot_word(kSlotMoved, static_cast<int>(wa & 0xffu));
+      if (kBooks) { sh.rank_spent[a] = rs_a + c_ns; sh.rank_spent[b] = rs_b + c_ns; }
       // The accepted swap stays in shared memory until the loop is over (ranks and expert ids
       // are below 256: one word; link_key is otherwise unused on this path): a global store
       // here would be waited for at the warp barrier below, once per iteration.
-      sh.link_key[n] = static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 |
-                       ((wwa >> 22) & 0xffu) << 8 | ((wwb >> 22) & 0xffu);
+      sh.link_key[n] = static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 | (win >> 5);
     }
-    if (lane == a) L0 -= dlt;
-    if (lane + 32 == a) L1 -= dlt;
-    if (lane == b) L0 += dlt;
-    if (lane + 32 == b) L1 += dlt;
-    if (kSide && static_cast<int>(n & 31u) == lane) {
+    const uint32_t moved = static_cast<uint32_t>(dlt) << 6;
+    if (lane == a) { h0 -= moved; l0 -= moved; }
+    if (lane + 32 == a) { h1 -= moved; l1 -= moved; }
+    if (lane == b) { h0 += moved; l0 += moved; }
+    if (lane + 32 == b) { h1 += moved; l1 += moved; }
+    if (kBooks) {
+      if (static_cast<int>(n & 31u) == lane) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) if (static_cast<int>(n >> 5) == q) my_links[q] = lkey;
+        for (int q = 0; q < 4; ++q) if (static_cast<int>(n >> 5) == q) my_links[q] = lkey;
+      }
+      global_spent += c_ns;
     }
-    global_spent += c_ns;
     ++n;
-    __syncwarp();                                                 // the next iteration reads what lane 0 wrote
+    __syncwarp();                                                 // the next iteration reads what the winner wrote
   }
+  if (L0 >= 0) L0 = static_cast<int>(h0 >> 6);
+  if (L1 >= 0) L1 = static_cast<int>(h1 >> 6);
+  __syncwarp();
   for (uint32_t i = lane; write && i < n; i += 32) {              // the plan, in order of acceptance
     const uint32_t w = sh.link_key[i];
     fb_swap sw;
@@ -512,12 +514,9 @@ __device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh
 
   if (!plan_needs_general_loop(p)) {
     int l0 = static_cast<int>(L0), l1 = static_cast<int>(L1);
-    // can the per-rank or the per-link budget stop a swap that the global budget admits?
-    const bool side = (p.rank_ns != FB_BUDGET_OFF && !(p.global_ns != FB_BUDGET_OFF && p.rank_ns >= p.global_ns)) ||
-                      (p.link_ns != FB_BUDGET_OFF && !(p.global_ns != FB_BUDGET_OFF && p.link_ns >= p.global_ns));
     uint32_t n_fast;
     if (lane == 0) sh.fast = 1;
-    if (!side)
+    if (!p.books)
       n_fast = m <= 4 ? plan_loop_uniform<1, false>(p, sh, lane, l0, l1, write)
                : m <= 8 ? plan_loop_uniform<2, false>(p, sh, lane, l0, l1, write)
                         : plan_loop_uniform<8, false>(p, sh, lane, l0, l1, write);

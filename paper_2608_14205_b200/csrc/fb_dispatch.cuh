@@ -161,6 +161,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   __shared__ uint32_t total[FB_MAX_EXPERTS];       // expert: assignments in all tiles
   __shared__ uint32_t offs[FB_MAX_EXPERTS + 1];    // exclusive prefix of total over slots
   __shared__ uint4 mask[FB_MAX_EXPERTS];           // rows of the tile that chose the expert
+  __shared__ uint32_t warp_sum[FB_MAX_EXPERTS / 32];
   __shared__ uint32_t part[kDispatchWarps][2][FB_MAX_EXPERTS / 2];
   __shared__ typename Choose<kPlan, PlanShared, Empty>::type plan;
   __shared__ int32_t bad;
@@ -232,31 +233,41 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     }
   }
   __syncthreads();
-  uint32_t ahead = 0;
-  if (warp == 0) {
-    if constexpr (kPlan) {
-      plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
-      __syncwarp();
-      if (plan.bad && lane == 0) bad = 1;
-      __syncwarp();
+  if constexpr (kPlan)
+    if (warp == 0) plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
+  const uint32_t ahead = e >= 0 ? rows_before(mask[e], row) : 0u;
+  if constexpr (kPlan) __syncthreads();
+  // Exclusive prefix over the slots, thread t for slot t (by one warp with 8 slots per lane it took 1 us)
+  bool usable = bad == 0;
+  if constexpr (kPlan) usable = plan.bad == 0;
+  uint32_t count = 0, incl = 0;
+  int expert = 0;
+  if (warp < FB_MAX_EXPERTS / 32 && usable) {
+    if (t < E) {
+      if constexpr (kPlan) expert = plan.bad_range ? plan.expert_at[t] : static_cast<int>(plan.slot_cnt[t] & 0xffu);
+      else expert = expert_at[t];
+      count = total[expert];
     }
-    const bool usable = kPlan ? *static_cast<volatile int32_t*>(&bad) == 0 : bad == 0;
-    auto expert_in = [&](int s) -> int {
-      if constexpr (kPlan) return plan.bad_range ? plan.expert_at[s] : static_cast<int>(plan.slot_cnt[s] & 0xffu);
-      else return expert_at[s];
-    };
-    if (usable) {
-      const uint32_t sum = warp_scan_slots(
-          E, lane, [&](int s) { return total[expert_in(s)]; },
-          [&](int s, uint32_t prefix) { offs[s] = prefix; base[expert_in(s)] += prefix; });
-      if (lane == 31) offs[E] = sum;
+    incl = count;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
     }
+    if (lane == 31) warp_sum[warp] = incl;
   }
-  if (e >= 0) ahead = rows_before(mask[e], row);
+  __syncthreads();
+  if (t < E && usable) {
+#pragma unroll
+    for (int w = 0; w < FB_MAX_EXPERTS / 32; ++w) incl += w < warp ? warp_sum[w] : 0u;
+    offs[t] = incl - count;
+    base[expert] += incl - count;
+    if (t == E - 1) offs[E] = incl;
+  }
   __syncthreads();
   if constexpr (kPlan)
     if (tile == 0) plan_write_placement(p.plan, plan, t, kDispatchThreads);
-  if (bad) {                                    // not a bijection: report, write no index
+  if (!usable) {                                // not a bijection: report (the planner has), write no index
     if (!kPlan && t == 0 && tile == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
     return;
   }

@@ -304,28 +304,47 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
       for (int u = 0; u < 2; ++u) bound[u] = redux_min_f32(kept[u] ? m2[u] : INFINITY);
     }
   }
-  if (kCpl == 1) {
-    // one key per lane: k rounds of "largest remaining key", the lowest lane (lowest id) on ties
-    if (want_sum) {
+  if (kCpl <= 4) {
+    // Few keys per lane: k rounds of "largest remaining key"; the lowest lane, and in it the lowest column,
+    // has the lowest id on ties.  (Compacting the keys above a bound and ranking them, as below, takes
+    // k reductions for the bound alone: layer step 40 tokens x 128 experts 18.5 us that way and 17.3 this way,
+    // 5003 x 64 25.4 and 24.6, prediction and plan 2729 x 60 16.0 and 14.3.)
+    float lane_max[2];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const float s = row_exp_sum<kCpl>(key[u], key[u][0]);
+    for (int u = 0; u < 2; ++u) {
+      if (p.groups > 1) {
+#pragma unroll
+        for (int j = 0; j < kCpl; ++j) key[u][j] = kept[u] ? key[u][j] : -INFINITY;
+      }
+      lane_max[u] = key[u][0];
+#pragma unroll
+      for (int j = 1; j < kCpl; ++j) lane_max[u] = fmaxf(lane_max[u], key[u][j]);
+      if (want_sum) {
+        const float s = row_exp_sum<kCpl>(key[u], lane_max[u]);
         if (lane == 0) rs.row_sum[2 * pair + u] = s;
       }
     }
-    if (p.groups > 1) {
-#pragma unroll
-      for (int u = 0; u < 2; ++u) key[u][0] = kept[u] ? key[u][0] : -INFINITY;
-    }
+#pragma unroll 1
     for (int r = 0; r < p.k; ++r) {
+      float top[2];
+      uint32_t holders[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) top[u] = redux_max_f32(lane_max[u]);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) holders[u] = __ballot_sync(full, lane_max[u] == top[u] && top[u] > -INFINITY);
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const float top = redux_max_f32(key[u][0]);
-        const uint32_t holders = __ballot_sync(full, key[u][0] == top && top > -INFINITY);
-        if (lane == __ffs(holders) - 1) {
-          rs.win_key[2 * pair + u][r] = top;
-          rs.win_id[2 * pair + u][r] = lc.c0;
-          key[u][0] = -INFINITY;
+        if (lane == __ffs(holders[u]) - 1) {
+          int at = 0;
+#pragma unroll
+          for (int j = kCpl - 1; j >= 0; --j) at = key[u][j] == top[u] ? j : at;
+          rs.win_key[2 * pair + u][r] = top[u];
+          rs.win_id[2 * pair + u][r] = lc.c0 + at;
+#pragma unroll
+          for (int j = 0; j < kCpl; ++j) key[u][j] = j == at ? -INFINITY : key[u][j];
+          lane_max[u] = key[u][0];
+#pragma unroll
+          for (int j = 1; j < kCpl; ++j) lane_max[u] = fmaxf(lane_max[u], key[u][j]);
         }
       }
     }

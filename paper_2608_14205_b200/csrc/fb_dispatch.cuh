@@ -115,23 +115,27 @@ __device__ __forceinline__ uint32_t rows_before(const uint4& m, int row) {
          __popc(m.z & (w > 2 ? 0xffffffffu : (w == 2 ? low : 0u))) + __popc(m.w & (w == 3 ? low : 0u));
 }
 
-// Exclusive scan of value(s) over slots 0 .. E-1 by one warp, 8 slots per lane; out(s, prefix) gets the
-// prefixes, the total is returned in lane 31.
-template <class Value, class Out>
-__device__ __forceinline__ uint32_t warp_scan_slots(int E, int lane, Value value, Out out) {
-  uint32_t v[8], run = 0;
+// Exclusive prefix of `count` over the slots, thread t for slot t (0 beyond the last); the whole block calls
+// it.  Returns the prefix; *all receives the total in thread E - 1.  warp_sum: 8 words that nobody else uses
+// until the next barrier.  (By one warp with 8 slots per lane it took 1 us.)
+__device__ __forceinline__ uint32_t block_prefix(uint32_t count, uint32_t* warp_sum, int t, uint32_t* all) {
+  const int warp = t >> 5, lane = t & 31;
+  uint32_t incl = count;
+  if (warp < FB_MAX_EXPERTS / 32) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) { v[i] = run; run += (lane * 8 + i < E) ? value(lane * 8 + i) : 0u; }
-  uint32_t incl = run;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += o;
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
   }
+  __syncthreads();
+  if (warp < FB_MAX_EXPERTS / 32) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (lane * 8 + i < E) out(lane * 8 + i, incl - run + v[i]);
-  return incl;
+    for (int w = 0; w < FB_MAX_EXPERTS / 32; ++w) incl += w < warp ? warp_sum[w] : 0u;
+  }
+  *all = incl;
+  return incl - count;
 }
 
 __device__ __forceinline__ void write_offsets(const DispatchParams& p, const uint32_t* offs, int t) {
@@ -237,32 +241,20 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     if (warp == 0) plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
   const uint32_t ahead = e >= 0 ? rows_before(mask[e], row) : 0u;
   if constexpr (kPlan) __syncthreads();
-  // Exclusive prefix over the slots, thread t for slot t (by one warp with 8 slots per lane it took 1 us)
   bool usable = bad == 0;
   if constexpr (kPlan) usable = plan.bad == 0;
-  uint32_t count = 0, incl = 0;
+  uint32_t count = 0, all = 0;
   int expert = 0;
-  if (warp < FB_MAX_EXPERTS / 32 && usable) {
-    if (t < E) {
-      if constexpr (kPlan) expert = plan.bad_range ? plan.expert_at[t] : static_cast<int>(plan.slot_cnt[t] & 0xffu);
-      else expert = expert_at[t];
-      count = total[expert];
-    }
-    incl = count;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += o;
-    }
-    if (lane == 31) warp_sum[warp] = incl;
-  }
-  __syncthreads();
   if (t < E && usable) {
-#pragma unroll
-    for (int w = 0; w < FB_MAX_EXPERTS / 32; ++w) incl += w < warp ? warp_sum[w] : 0u;
-    offs[t] = incl - count;
-    base[expert] += incl - count;
-    if (t == E - 1) offs[E] = incl;
+    if constexpr (kPlan) expert = plan.bad_range ? plan.expert_at[t] : static_cast<int>(plan.slot_cnt[t] & 0xffu);
+    else expert = expert_at[t];
+    count = total[expert];
+  }
+  const uint32_t first = block_prefix(count, warp_sum, t, &all);
+  if (t < E && usable) {
+    offs[t] = first;
+    base[expert] += first;
+    if (t == E - 1) offs[E] = all;
   }
   __syncthreads();
   if constexpr (kPlan)
@@ -291,7 +283,8 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
   __shared__ int32_t slot_of[FB_MAX_EXPERTS];
   __shared__ int32_t owner[FB_MAX_EXPERTS];
   __shared__ uint32_t gbase[FB_MAX_EXPERTS];       // position of the slot's first assignment of this batch of tiles
-  __shared__ uint32_t total[FB_MAX_EXPERTS];       // assignments to this slot in all tiles; later: in this batch
+  __shared__ uint32_t total[FB_MAX_EXPERTS];       // assignments to this slot in all tiles
+  __shared__ uint32_t warp_sum[FB_MAX_EXPERTS / 32];
   __shared__ uint32_t offs[FB_MAX_EXPERTS + 1];    // exclusive prefix of total over slots; later: of the batch's counts
   __shared__ uint16_t ahead_of[kBatch][FB_MAX_EXPERTS];   // the batch's assignments to this slot in earlier tiles
   // The per-warp sums of the histogram table are read before the tile loop starts and share their
@@ -386,11 +379,6 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
   static_assert(kDispatchThreads == kDispatchBatch * FB_MAX_EXPERTS, "one mask per thread");
   u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
   __syncthreads();
-  // Exclusive scan of total[] over slots into offs[], by one warp
-  auto scan = [&]() {
-    const uint32_t sum = warp_scan_slots(E, lane, [&](int s) { return total[s]; }, [&](int s, uint32_t prefix) { offs[s] = prefix; });
-    if (lane == 31) offs[E] = sum;
-  };
   auto mark_rows = [&]() {
 #pragma unroll
     for (int i = 0; i < kBatch; ++i)
@@ -399,29 +387,39 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
         atomicOr(m + (row >> 5), 1u << (row & 31));
       }
   };
-  if (warp == 0) scan();
   mark_rows();
-  __syncthreads();
-  if (blockIdx.x == 0) write_offsets(p, offs, t);
-  if (t < E) gbase[t] += offs[t];
+  uint32_t all = 0;
+  const uint32_t first = block_prefix(t < E ? total[t] : 0u, warp_sum, t, &all);
+  if (t < E) {
+    offs[t] = first;
+    gbase[t] += first;
+    if (t == E - 1) offs[E] = all;
+  }
+  if (blockIdx.x == 0) {
+    __syncthreads();
+    write_offsets(p, offs, t);
+  }
   // Up to four tiles at a time.  With more than one, their assignments are first put into slot
   // order in shared memory, so that perm is written in runs (4-byte stores to as many sectors as
   // threads took 4 us of the 18 us at 131072 tokens); a single tile has runs of a few entries only and writes directly.
   for (int tile0 = tile_begin; tile0 < tile_end; tile0 += kBatch) {
     const bool several = tile_end - tile0 > 1;                  // (the same for the whole block)
-    if (several && t < E) {
-      uint32_t run = 0;
-#pragma unroll
-      for (int i = 0; i < kBatch; ++i) {
-        ahead_of[i][t] = static_cast<uint16_t>(run);
-        const uint4 m = u.b.mask[i][t];
-        run += __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
-      }
-      total[t] = run;
-    }
-    __syncthreads();
+    __syncthreads();                                            // the masks are complete, the offsets written
+    uint32_t run = 0;
     if (several) {
-      if (warp == 0) scan();
+      if (t < E) {
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          ahead_of[i][t] = static_cast<uint16_t>(run);
+          const uint4 m = u.b.mask[i][t];
+          run += __popc(m.x) + __popc(m.y) + __popc(m.z) + __popc(m.w);
+        }
+      }
+      const uint32_t at = block_prefix(run, warp_sum, t, &all);
+      if (t < E) {
+        offs[t] = at;
+        if (t == E - 1) offs[E] = all;
+      }
       __syncthreads();
     }
     int next_ids[kBatch];
@@ -462,7 +460,7 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
     if (tile0 + kBatch >= tile_end) break;
     u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
     __syncthreads();
-    if (t < E) gbase[t] += total[t];
+    if (t < E) gbase[t] += run;
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) ids[i] = next_ids[i];
     mark_rows();

@@ -43,11 +43,11 @@ inline int gate_layout(int E, int gate, int n_group, int topk_group, RouterParam
   p->group_size = gs;
   p->keep_groups = restricted ? topk_group : 1;
   p->lanes_per_group = lpg;
-  // one group, or whole vectors per group: round the lane's share up so that it is one vector load
-  p->vector_load = (groups == 1 || gs % cpl == 0) ? 1 : 0;
+  // one group, or groups that start on a vector: round the lane's share up so that it is whole vectors
+  p->vector_load = (groups == 1 || gs % (cpl < 4 ? cpl : 4) == 0) ? 1 : 0;
   p->cols_per_lane = p->vector_load ? cpl : per_lane;
-  p->two_vectors = (cpl == 8 && p->vector_load && (groups == 1 || lpg * 8 == gs)) ? 1 : 0;   // lane = column / 8
-  p->ragged = !(p->vector_load && groups * lpg * cpl == E && groups * lpg == 32) ? 1 : 0;
+  p->two_vectors = (cpl == 8 && p->vector_load) ? 1 : 0;
+  p->ragged = groups * lpg * cpl != E || groups * lpg != 32 ? 1 : 0;
   return cpl;
 }
 
@@ -83,6 +83,7 @@ struct RowsShared {
   int32_t is_last;
   int32_t accum_ok;
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
+  uint16_t quad_word[FB_MAX_EXPERTS / 4];    // where columns 4 q .. 4 q + 3 lie in a staged row
   alignas(16) float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];
   alignas(16) uint32_t hist[FB_MAX_EXPERTS];
@@ -621,6 +622,12 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       sh.logit_bias[e] = (p.logit_bias != nullptr && e < E) ? p.logit_bias[e] : 0.0f;
       sh.select_bias[e] = (p.select_bias != nullptr && e < E) ? p.select_bias[e] : 0.0f;
     }
+    for (int q = et; q < FB_MAX_EXPERTS / 4; q += kEpilogueThreads) {
+      // (a quad lies in one group and one lane where rows are stored as two vectors per lane; groups start on
+      // a quad there; padding columns go behind the lanes' words)
+      const int in = 4 * q % p.group_size, of_lane = 4 * q / p.group_size * p.lanes_per_group + in / 8;
+      sh.quad_word[q] = static_cast<uint16_t>(!p.two_vectors ? 4 * q : 4 * q < E ? in / 4 % 2 * 128 + of_lane * 4 : 256);
+    }
     float sb[kCpl];
 #pragma unroll
     for (int j = 0; j < kCpl; ++j)
@@ -672,7 +679,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
               }
 #pragma unroll
               for (int q = 0; q < 4; ++q)
-                st_shared_v4(dst + static_cast<uint32_t>(p.two_vectors ? (q & 1) * 128 + (c0 + 4 * q) / 8 * 4 : c0 + 4 * q) * 4u, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                st_shared_v4(dst + static_cast<uint32_t>(sh.quad_word[c0 / 4 + q]) * 4u, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
             }
           }
           tcgen05_fence_before();

@@ -727,7 +727,7 @@ def test_dispatch_index_over_table_widths_and_runs_of_tiles(E, k, R, T):
     dict(E=16, k=2, R=4),                                             # one column per lane
     dict(E=33, k=4, R=3, renorm=0),                                   # two, the last lane holds one; softmax denominator
     dict(E=100, k=6, R=4),                                            # four
-    dict(E=200, k=8, R=8, renorm=0),                                  # eight
+    dict(E=200, k=8, R=8, renorm=0), dict(E=250, k=8, R=5),           # eight; the last lane's second vector is padding
     dict(gate=1, n_group=5, topk_group=2, k=7, E=250, R=5),           # sixteen; bound from the lanes, idle lanes
     dict(gate=1, n_group=8, topk_group=3, k=6, E=160, R=8),           # groups of 20: five per lane, single loads
     dict(gate=1, n_group=32, topk_group=4, k=8, E=64, R=8),           # groups of two

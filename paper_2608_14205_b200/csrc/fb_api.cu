@@ -299,7 +299,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.probe = probe;
   if (plan) p.plan = *plan;
   // The fused tail serves the common plans; a plan that needs the general loop (per-expert sizes,
-  // more than 16 experts per rank, a planner variant) gets the stand-alone planner kernel behind
+  // a planner variant) gets the stand-alone planner kernel behind
   // the router kernel instead.
   const bool plan_wanted = plan != nullptr && (mode == fb::kModePredictPlan || mode == fb::kModeLayer);
   p.fuse_planner = (plan_wanted && !fb::plan_needs_general_loop(*plan)) ? 1 : 0;

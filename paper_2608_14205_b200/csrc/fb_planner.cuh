@@ -161,7 +161,7 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 }
 
 // Greedy loop specialised for the common case: one cost per link class (no per-expert
-// size table) and at most 256 candidate pairs per iteration (m <= 16).  One warp runs alone here,
+// size table).  m experts per rank, m * m candidate pairs per iteration.  One warp runs alone here,
 // so what counts is the length of the dependent instruction chain of an iteration.
 //
 // All pairs of an iteration have the same cost, so the largest benefit / cost is the largest
@@ -176,7 +176,9 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 // D, so no candidate has to be tested - only the smallest v is, against D.
 //
 // Lane l tries expert slot l / g of the heavy rank with kPerLane slots of the light one, g lanes per
-// heavy slot; slots beyond m repeat the last one (the same pair twice changes nothing).  A lane keeps the
+// heavy slot; slots beyond m repeat the last one (the same pair twice changes nothing).  kPerLane == 0: more
+// than 16 experts per rank, lane l takes the heavy slots l, l + 32, ... with every light one (20 experts per
+// rank, 4 tokens: layer step 63 us with the general loop below, 22 with this one).  A lane keeps the
 // packed (load, rank) keys of its two ranks, so an iteration is: two warp reductions for the frontier, the
 // slot words, the smallest v of the lane, one reduction for v, one for the pair (the lane rides along), one
 // shuffle for the moved tokens.
@@ -188,9 +190,10 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
   const int R = p.R, m = p.E / R;
   const uint32_t full = 0xffffffffu;
   constexpr uint32_t kNone = 0xffffffffu;
+  constexpr int kNarrow = kPerLane == 0 ? 1 : kPerLane;
   constexpr int g = kPerLane == 8 ? 2 : (kPerLane == 2 ? 4 : 8);     // m <= 16, <= 8, <= 4
-  const int ia = min(lane / g, m - 1), j0 = (lane % g) * kPerLane;
-  const bool whole = m == g * kPerLane;                           // the lane's light slots are contiguous and exist
+  const int ia = min(lane / g, m - 1), j0 = (lane % g) * kNarrow;
+  const bool whole = m == g * kNarrow;                            // the lane's light slots are contiguous and exist
   const bool flat = p.gamma_den == 0 || p.gamma_num == 0;
   const uint32_t tau = p.tau_tokens, max_swaps = kBooks ? p.max_swaps : p.swap_cap;
   // frontier keys (lowest index on ties): max of load << 6 | (63 - rank), min of load << 6 | rank
@@ -210,16 +213,19 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
     const int La = static_cast<int>(hi_key >> 6), Lb = static_cast<int>(lo_key >> 6);
     const int D = La - Lb;
     const int base_a = a * m, base_b = b * m;
-    const uint32_t wa = sh.slot_cnt[base_a + ia];                 // slot words: count, expert
-    uint32_t wb[kPerLane];
-    if (kPerLane == 8 && whole) {
-      const uint4 q0 = *reinterpret_cast<const uint4*>(&sh.slot_cnt[base_b + j0]);
-      const uint4 q1 = *reinterpret_cast<const uint4*>(&sh.slot_cnt[base_b + j0 + 4]);
-      wb[0] = q0.x; wb[1 % kPerLane] = q0.y; wb[2 % kPerLane] = q0.z; wb[3 % kPerLane] = q0.w;
-      wb[4 % kPerLane] = q1.x; wb[5 % kPerLane] = q1.y; wb[6 % kPerLane] = q1.z; wb[7 % kPerLane] = q1.w;
-    } else {
+    uint32_t wa = 0, wb[kNarrow];                                 // slot words: count, expert
+    if constexpr (kPerLane != 0) {
+      wa = sh.slot_cnt[base_a + ia];
+      if (kPerLane == 8 && whole) {
 #pragma unroll
-      for (int t = 0; t < kPerLane; ++t) wb[t] = sh.slot_cnt[base_b + min(j0 + t, m - 1)];
+        for (int t = 0; t < kNarrow; t += 4) {
+          const uint4 q = *reinterpret_cast<const uint4*>(&sh.slot_cnt[base_b + j0 + t]);
+          wb[t] = q.x; wb[(t + 1) % kNarrow] = q.y; wb[(t + 2) % kNarrow] = q.z; wb[(t + 3) % kNarrow] = q.w;
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < kNarrow; ++t) wb[t] = sh.slot_cnt[base_b + min(j0 + t, m - 1)];
+      }
     }
     if (static_cast<uint32_t>(D) <= tau) break;                   // (the same in all lanes)
     unsigned long long c_ns = 0, rs_a = 0, rs_b = 0;
@@ -252,32 +258,55 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
       const uint32_t m2 = max(lane != a && lane != b ? h0 >> 6 : 0u, lane + 32 != a && lane + 32 != b ? h1 >> 6 : 0u);
       v_floor = 2 * static_cast<int>(__reduce_max_sync(full, m2)) - La - Lb;
     }
-    // ---- smallest v of this lane, ties -> smallest expert of the light rank
-    const int x = 2 * static_cast<int>(wa >> 8) - D;
-    uint32_t key[kPerLane];
+    // ---- smallest v of this lane, ties -> smallest pair; where its experts are, and the tokens moved a -> b
+    uint32_t mine = (1u << 24) - 1, pair = 0;
+    int sa = 0, sb = 0, delta = 0;
+    if constexpr (kPerLane != 0) {
+      const int x = 2 * static_cast<int>(wa >> 8) - D;
+      uint32_t key[kNarrow];
 #pragma unroll
-    for (int t = 0; t < kPerLane; ++t) {
-      const int v = max(abs(x - 2 * static_cast<int>(wb[t] >> 8)), v_floor);
-      key[t] = static_cast<uint32_t>(min(v, (1 << 24) - 1)) << 8 | (wb[t] & 0xffu);
+      for (int t = 0; t < kNarrow; ++t) {
+        const int v = max(abs(x - 2 * static_cast<int>(wb[t] >> 8)), v_floor);
+        key[t] = static_cast<uint32_t>(min(v, (1 << 24) - 1)) << 8 | (wb[t] & 0xffu);
+      }
+      uint32_t best = key[0];
+#pragma unroll
+      for (int t = 1; t < kNarrow; ++t) best = min(best, key[t]);
+      mine = best >> 8;
+      pair = (wa & 0xffu) << 8 | (best & 0xffu);
+      sa = base_a + ia;
+#pragma unroll
+      for (int t = kNarrow - 1; t >= 0; --t)
+        if (key[t] == best) { sb = base_b + min(j0 + t, m - 1); delta = static_cast<int>(wa >> 8) - static_cast<int>(wb[t] >> 8); }
+    } else {
+      for (int i = lane; i < m; i += 32) {
+        const uint32_t wi = sh.slot_cnt[base_a + i];
+        const int x = 2 * static_cast<int>(wi >> 8) - D;
+        for (int jj = 0; jj < m; jj += 8) {
+          uint32_t wj[8];
+#pragma unroll
+          for (int t = 0; t < 8; ++t) wj[t] = sh.slot_cnt[base_b + min(jj + t, m - 1)];
+#pragma unroll
+          for (int t = 0; t < 8; ++t) {
+            const uint32_t v = static_cast<uint32_t>(min(max(abs(x - 2 * static_cast<int>(wj[t] >> 8)), v_floor), (1 << 24) - 1));
+            const uint32_t pr = (wi & 0xffu) << 8 | (wj[t] & 0xffu);
+            if (v < mine || (v == mine && pr < pair)) {
+              mine = v; pair = pr; sa = base_a + i; sb = base_b + min(jj + t, m - 1);
+              delta = static_cast<int>(wi >> 8) - static_cast<int>(wj[t] >> 8);
+            }
+          }
+        }
+      }
     }
-    uint32_t best = key[0];
-#pragma unroll
-    for (int t = 1; t < kPerLane; ++t) best = min(best, key[t]);
-    const uint32_t mine = best >> 8;
     const uint32_t top = __reduce_min_sync(full, mine);
-    int jb = 0, delta = 0;
-#pragma unroll
-    for (int t = kPerLane - 1; t >= 0; --t)
-      if (key[t] == best) { jb = t; delta = static_cast<int>(wa >> 8) - static_cast<int>(wb[t] >> 8); }   // tokens moved a -> b
     if (top >= static_cast<uint32_t>(D)) break;                   // Algorithm 1 lines 6-7
-    const uint32_t win = __reduce_min_sync(
-        full, mine == top ? (wa & 0xffu) << 13 | (best & 0xffu) << 5 | static_cast<uint32_t>(lane) : kNone);
+    const uint32_t win = __reduce_min_sync(full, mine == top ? pair << 5 | static_cast<uint32_t>(lane) : kNone);
     const int src = static_cast<int>(win & 31u);
     const int dlt = __shfl_sync(full, delta, src);
     if (lane == src) {
       // the two experts trade slots
-      sh.slot_cnt[base_a + ia] = slot_word(kSlotMoved, static_cast<int>(best & 0xffu));
-      sh.slot_cnt[base_b + min(j0 + jb, m - 1)] = slot_word(kSlotMoved, static_cast<int>(wa & 0xffu));
+      sh.slot_cnt[sa] = slot_word(kSlotMoved, static_cast<int>(pair & 0xffu));
+      sh.slot_cnt[sb] = slot_word(kSlotMoved, static_cast<int>(pair >> 8));
       if (kBooks) { sh.rank_spent[a] = rs_a + c_ns; sh.rank_spent[b] = rs_b + c_ns; }
       // The accepted swap stays in shared memory until the loop is over (ranks and expert ids
       // are below 256: one word; link_key is otherwise unused on this path): a global store
@@ -314,11 +343,10 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
 
 // Which plans the fast loop cannot serve (host and device agree on this test).
 __host__ __device__ inline bool plan_needs_general_loop(const PlanParams& p) {
-  return p.expert_bytes_table != nullptr || p.E / p.R > 16 || p.mode != FB_PLAN_LOOP;
+  return p.expert_bytes_table != nullptr || p.mode != FB_PLAN_LOOP;
 }
 
-// The general greedy loop: per-expert sizes, more than 16 experts per rank, or a planner
-// variant (the one-pass sweep of the ordering paragraph, a widened frontier).  Plain and slow;
+// The general greedy loop: per-expert sizes or a planner variant (the one-pass sweep of the ordering paragraph, a widened frontier).  Plain and slow;
 // a function of its own so that its registers and spills stay out of the common path.
 // L0 / L1: this lane's rank loads (ranks lane and lane + 32, -1 if absent).
 __device__ __noinline__ void plan_loop_general(const PlanParams& p, PlanShared& sh, int lane, long long L0,
@@ -519,11 +547,13 @@ __device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh
     if (!p.books)
       n_fast = m <= 4 ? plan_loop_uniform<1, false>(p, sh, lane, l0, l1, write)
                : m <= 8 ? plan_loop_uniform<2, false>(p, sh, lane, l0, l1, write)
-                        : plan_loop_uniform<8, false>(p, sh, lane, l0, l1, write);
+               : m <= 16 ? plan_loop_uniform<8, false>(p, sh, lane, l0, l1, write)
+                         : plan_loop_uniform<0, false>(p, sh, lane, l0, l1, write);
     else
       n_fast = m <= 4 ? plan_loop_uniform<1, true>(p, sh, lane, l0, l1, write)
                : m <= 8 ? plan_loop_uniform<2, true>(p, sh, lane, l0, l1, write)
-                        : plan_loop_uniform<8, true>(p, sh, lane, l0, l1, write);
+               : m <= 16 ? plan_loop_uniform<8, true>(p, sh, lane, l0, l1, write)
+                         : plan_loop_uniform<0, true>(p, sh, lane, l0, l1, write);
     FB_PLAN_STAMP(20);
     if (lane == 0 && write) *p.n_swaps = static_cast<int32_t>(n_fast);
     if (lane < R && write) p.load_after[lane] = static_cast<uint32_t>(l0);

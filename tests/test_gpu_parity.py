@@ -454,6 +454,14 @@ def test_random_shapes(seed):
     _run(wl, T, layer=seed, with_logit_bias=bool(rng.integers(0, 2)))
 
 
+@pytest.mark.parametrize("E,R", [(160, 8), (256, 8), (256, 4), (256, 2), (198, 6), (66, 2), (17, 1)])
+@pytest.mark.parametrize("bud", [dict(), dict(gamma_num=0), dict(ranks_per_node=2, alpha_ns=(100, 900), fs_per_byte=(2000, 9000),
+                                                                  expert_bytes=100_000, global_ns=6000, rank_ns=3000, link_ns=2500)])
+def test_planner_with_many_experts_per_rank(E, R, bud):
+    # more than 16 experts per rank, in the separate call and in the layer step (whole numbers: exact)
+    _run(_wl(E=E, k=4, R=R, d=64, max_swaps=12), 700, placement=I.random_placement(E, seed=R), **bud)
+
+
 # ------------------------------------------------------------------ persistent router kernel (several tiles per block pair)
 @pytest.mark.parametrize("name,T,limit,d,lb", [
     ("dsv3", 777, 1, None, False), ("dsv3", 1500, 2, None, False), ("dsv3", 2049, 3, None, True),

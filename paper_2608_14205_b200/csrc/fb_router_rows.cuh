@@ -173,30 +173,35 @@ __device__ __forceinline__ float row_exp_sum(const float (&key)[kCpl], float lan
 }
 
 // The top-k of two staged rows (row_addr: shared-memory address of the first one's first word in this block;
-// the J blocks whose cluster ranks are first_rank + 2 i hold one partial sum each at the same place) into
+// the J blocks of the cluster whose ranks have my_rank's parity hold one partial sum each at the same place) into
 // rows 2 pair and 2 pair + 1 of the scratch's result lists.  row: token index of the first one.
 // Two rows at a time because a row's steps are a chain of short dependent ones.
 template <int kCpl, bool kSigmoid>
 __device__ __forceinline__ void select_two_rows(const RouterParams& p, const LaneColumns& lc, const float (&sb)[kCpl],
-                                                const float* logit_bias_s, uint32_t row_addr, uint32_t first_rank,
+                                                const float* logit_bias_s, uint32_t row_addr, uint32_t my_rank,
                                                 long long row, RowScratch& rs, int pair, int lane) {
   const uint32_t full = 0xffffffffu;
   const uint32_t stride = static_cast<uint32_t>(staging_stride(p.N)) * 4u;
   const bool want_sum = !kSigmoid && p.topk_w != nullptr && !p.renorm;
   float key[2][kCpl];
-  // ---- logits: the J partial sums in order
+  // ---- logits: the J partial sums, beginning with this block's own.  Which one is added when depends on the
+  // row's place in its tile only.  (With all blocks beginning at the same one, its outgoing 16 bytes per
+  // cycle served the whole cluster: 475 tokens, 256 experts, eight pairs per tile 25.3 us for prediction and plan
+  // and 22.2 in turn.)
   const uint32_t a0 = row_addr + static_cast<uint32_t>(lc.word) * 4u;
   if (p.pieces == 1) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) load_columns<kCpl>(key[u], a0 + u * stride, p, lc.n);
   } else {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) load_columns_of<kCpl>(key[u], a0 + u * stride, first_rank, p, lc.n);
+    for (int u = 0; u < 2; ++u) load_columns<kCpl>(key[u], a0 + u * stride, p, lc.n);
+    uint32_t from = my_rank;
 #pragma unroll (kCpl >= 8 ? 1 : 3)
     for (int i = 1; i < p.pieces; ++i) {
       float t[2][kCpl];
+      from = from + 2 < 2u * p.pieces ? from + 2 : from + 2 - 2u * p.pieces;
 #pragma unroll
-      for (int u = 0; u < 2; ++u) load_columns_of<kCpl>(t[u], a0 + u * stride, first_rank + 2u * i, p, lc.n);
+      for (int u = 0; u < 2; ++u) load_columns_of<kCpl>(t[u], a0 + u * stride, from, p, lc.n);
 #pragma unroll
       for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -717,7 +722,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
           for (int i = 0; i < count; i += 2)
             if (row0 + i < p.T)
               select_two_rows<kCpl, kSigmoid>(p, lc, sb, sh.logit_bias, staging + static_cast<uint32_t>(first - r0 + i) * row_stride,
-                                              cta_rank, row0 + i, rs, i >> 1, lane);
+                                              cluster_rank, row0 + i, rs, i >> 1, lane);
           __syncwarp();
           FB_STAMP(8, 64);
           finish_rows<kSigmoid>(p, sh, rs, count, row0, out_ids, out_w, lane);

@@ -403,6 +403,14 @@ fb_status fb_row_cosine_mean(const void* a, const void* b, int64_t rows, int32_t
 fb_status fb_topk_hits(const int32_t* ids_a, const int32_t* ids_b, int32_t T, int32_t k, uint32_t* hits_out,
                        fb_stream stream);
 
+/* The three figures of one layer of one step in two launches: metrics_out[0] the mean cosine of h_prev and H
+ * (bf16 [T][d]), [1] that of the logits z_early and z (f32 [T][E]), [2] the number of recovered assignments
+ * (ids_early, ids: [T][k]) as a double.  Same definitions and precision as the two calls above; row_scratch:
+ * double [3 T].  All pointers are device pointers.  T = 0 gives 0, 0, 0. */
+fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* z_early, const float* z,
+                                const int32_t* ids_early, const int32_t* ids, int32_t T, int32_t d, int32_t E, int32_t k,
+                                double* row_scratch, double* metrics_out, fb_stream stream);
+
 /* Limit on the SM pairs the router kernel may occupy (0 = no limit, the default).  The
  * prediction pass is meant to run beside the previous layer's attention (stage 1 of the
  * method is hidden behind it), so a caller may want to leave SMs free.  A call with more

@@ -59,7 +59,7 @@ EXPORTS = ["fb_create", "fb_destroy", "fb_budget_ns", "fb_swap_cost_ns", "fb_pre
            "fb_apply_swaps_staged", "fb_fit_cost_model", "fb_calibrate_exchange", "fb_selftest_wait_timeout",
            "fb_set_stamp_buffer", "fb_clock_probe", "fb_attention_begin", "fb_attention_end", "fb_layer_budget_ns",
            "fb_attention_set_time_ns", "fb_attention_reset", "fb_dispatch_slot_counts", "fb_dispatch_globalize",
-           "fb_standin_attention", "fb_set_split"]
+           "fb_standin_attention", "fb_set_split", "fb_prediction_quality"]
 
 _lib = None
 
@@ -133,6 +133,8 @@ def lib() -> ctypes.CDLL:
     L.fb_selftest_wait_timeout.restype = ctypes.c_int
     L.fb_row_cosine_mean.argtypes = [vp, vp, ctypes.c_int64, i32, i32, vp, vp, vp]
     L.fb_row_cosine_mean.restype = ctypes.c_int
+    L.fb_prediction_quality.argtypes = [vp] * 6 + [i32] * 4 + [vp] * 3
+    L.fb_prediction_quality.restype = ctypes.c_int
     L.fb_topk_hits.argtypes = [vp, vp, i32, i32, vp, vp]
     L.fb_apply_swaps.argtypes = [vp, u64, i32, vp, vp, vp, i32, vp, vp]
     L.fb_apply_swaps.restype = ctypes.c_int
@@ -253,6 +255,16 @@ def fb_apply_swaps(slot_weights: torch.Tensor, expert_bytes: int, E: int, expert
 def fb_topk_hits(ids_a: torch.Tensor, ids_b: torch.Tensor, T: int, k: int, hits_out: torch.Tensor,
                  stream=None) -> None:
     _check(lib().fb_topk_hits(_ptr(ids_a), _ptr(ids_b), T, k, _ptr(hits_out), _stream(stream)), "fb_topk_hits")
+
+
+def fb_prediction_quality(h_prev, H, z_early, z, ids_early, ids, T: int, d: int, E: int, k: int, row_scratch,
+                          metrics_out, stream=None) -> None:
+    """Mean hidden-state cosine, mean logit cosine and recovered assignments into metrics_out (float64 [3])."""
+    assert h_prev.dtype == H.dtype == torch.bfloat16 and z_early.dtype == z.dtype == torch.float32
+    assert row_scratch.dtype == metrics_out.dtype == torch.float64
+    _check(lib().fb_prediction_quality(_ptr(h_prev), _ptr(H), _ptr(z_early), _ptr(z), _ptr(ids_early), _ptr(ids), T, d,
+                                       E, k, _ptr(row_scratch), _ptr(metrics_out), _stream(stream)),
+           "fb_prediction_quality")
 
 
 def fb_predict_load_static(cfg: FbConfig, device: int, router: FbRouter, x, T: int, counts, topk_ids=None,

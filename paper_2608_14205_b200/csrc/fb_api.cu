@@ -1033,6 +1033,30 @@ fb_status fb_topk_hits(const int32_t* ids_a, const int32_t* ids_b, int32_t T, in
                  cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
+fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* z_early, const float* z,
+                                const int32_t* ids_early, const int32_t* ids, int32_t T, int32_t d, int32_t E, int32_t k,
+                                double* row_scratch, double* metrics_out, fb_stream stream_) {
+  if (T < 0 || d <= 0 || E <= 0 || k < 1 || k > FB_MAX_TOPK || !metrics_out) return FB_ERR_INVALID_ARG;
+  if (T > 0 && (!h_prev || !H || !z_early || !z || !ids_early || !ids || !row_scratch)) return FB_ERR_INVALID_ARG;
+  cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+  fb::QualityParams qp;
+  qp.h_prev = static_cast<const __nv_bfloat16*>(h_prev);
+  qp.h = static_cast<const __nv_bfloat16*>(H);
+  qp.z_early = z_early;
+  qp.z = z;
+  qp.ids_early = ids_early;
+  qp.ids = ids;
+  qp.T = T; qp.d = d; qp.E = E; qp.k = k;
+  qp.rows = row_scratch;
+  qp.out = metrics_out;
+  cudaError_t err = cudaSuccess;
+  if (T > 0)
+    err = launch_dependent(fb::fb_quality_rows_kernel, (T + fb::kCosineWarpsPerBlock - 1) / fb::kCosineWarpsPerBlock,
+                           32 * fb::kCosineWarpsPerBlock, stream, qp);
+  if (err == cudaSuccess) err = launch_dependent(fb::fb_quality_sums_kernel, fb::kQualityBlocks, fb::kMeanThreads, stream, qp);
+  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+}
+
 fb_status fb_set_split(fb_ctx* ctx, int32_t mode, int32_t owner_bias_kblocks) {
   if (!ctx || (mode != 0 && mode != 1) || owner_bias_kblocks < -1 || owner_bias_kblocks > 1024) return FB_ERR_INVALID_ARG;
   ctx->split_mode = mode;      // (the pieces of a tile's k-range are equal: there is no owner to favour)

@@ -280,6 +280,11 @@ __device__ __forceinline__ float ld_cluster_float(uint32_t addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
   return v;
 }
+__device__ __forceinline__ double ld_cluster_double(uint32_t addr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
 template <int kN>
 __device__ __forceinline__ void ld_cluster_floats(uint32_t addr, float (&v)[kN]) {
   if constexpr (kN == 1) {

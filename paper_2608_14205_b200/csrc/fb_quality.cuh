@@ -38,20 +38,13 @@ __device__ __forceinline__ int unpack16(const float* p, long long i, double (&v)
   return 4;
 }
 
-// One warp per row.  Rows whose start and length allow it are read 16 bytes per lane and
+// Cosine of two rows by one warp.  Rows whose start and length allow it are read 16 bytes per lane and
 // step (kVec elements); otherwise lane l takes elements l, l + 32, ...  Either way a lane
 // adds its elements in ascending order and the three partial sums are combined by a
 // butterfly, which gives every lane the same total.
 template <class Tin>
-__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock)
-fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long long rows, int n,
-                     double* __restrict__ row_cos) {
+__device__ __forceinline__ double row_cosine(const Tin* __restrict__ a, const Tin* __restrict__ b, long long row, int n, int lane) {
   constexpr int kVec = 16 / static_cast<int>(sizeof(Tin));
-  const long long row = static_cast<long long>(blockIdx.x) * kCosineWarpsPerBlock + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  pdl_launch_dependents();
-  pdl_wait();
-  if (row >= rows) return;
   const long long base = row * n;
   double dot = 0.0, na = 0.0, nb = 0.0;
   const bool wide = n % kVec == 0 && reinterpret_cast<uintptr_t>(a) % 16 == 0 && reinterpret_cast<uintptr_t>(b) % 16 == 0;
@@ -76,7 +69,94 @@ fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long 
     na += __shfl_xor_sync(0xffffffffu, na, off);
     nb += __shfl_xor_sync(0xffffffffu, nb, off);
   }
-  if (lane == 0) row_cos[row] = (na > 0.0 && nb > 0.0) ? dot / (sqrt(na) * sqrt(nb)) : 0.0;
+  return (na > 0.0 && nb > 0.0) ? dot / (sqrt(na) * sqrt(nb)) : 0.0;
+}
+
+// One warp per row.
+template <class Tin>
+__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock)
+fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long long rows, int n,
+                     double* __restrict__ row_cos) {
+  const long long row = static_cast<long long>(blockIdx.x) * kCosineWarpsPerBlock + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  pdl_launch_dependents();
+  pdl_wait();
+  if (row >= rows) return;
+  const double c = row_cosine(a, b, row, n, lane);
+  if (lane == 0) row_cos[row] = c;
+}
+
+// The three quality figures of a step, row by row, in one launch: the hidden-state cosine, the logit cosine
+// and the number of recovered assignments into rows[0 .. T), [T .. 2 T), [2 T .. 3 T).  Bound by the fp64
+// conversions of the hidden states (15 us for 2 x 8192 x 2048 bf16 values); as five launches behind one
+// another the three figures took 31 us, most of it with the GPU nearly empty.
+struct QualityParams {
+  const __nv_bfloat16 *h_prev, *h;       // [T][d]
+  const float *z_early, *z;              // [T][E]
+  const int32_t *ids_early, *ids;        // [T][k]
+  long long T;
+  int32_t d, E, k;
+  double* rows;                          // [3][T]
+  double* out;                           // [3]: mean, mean, sum
+};
+__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock)
+fb_quality_rows_kernel(const __grid_constant__ QualityParams p) {
+  const long long row = static_cast<long long>(blockIdx.x) * kCosineWarpsPerBlock + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  pdl_launch_dependents();
+  pdl_wait();
+  if (row >= p.T) return;
+  const int32_t mine = lane < p.k ? p.ids[row * p.k + lane] : INT32_MAX;
+  const int32_t early = lane < p.k ? p.ids_early[row * p.k + lane] : INT32_MIN;
+  uint32_t hits = 0;
+#pragma unroll
+  for (int y = 0; y < FB_MAX_TOPK; ++y) hits += __popc(__ballot_sync(0xffffffffu, mine == __shfl_sync(0xffffffffu, early, y)));
+  const double cz = row_cosine(p.z_early, p.z, row, p.E, lane);
+  const double ch = row_cosine(p.h_prev, p.h, row, p.d, lane);
+  if (lane == 0) {
+    p.rows[row] = ch;
+    p.rows[p.T + row] = cz;
+    p.rows[2 * p.T + row] = static_cast<double>(hits);
+  }
+}
+// Sums of the three columns by one cluster, in a fixed order.
+constexpr int kQualityBlocks = 8;
+__global__ void __cluster_dims__(kQualityBlocks, 1, 1) __launch_bounds__(kMeanThreads)
+fb_quality_sums_kernel(const __grid_constant__ QualityParams p) {
+  __shared__ double part[3][kMeanThreads / 32];
+  __shared__ double sums[3];
+  const int t = threadIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
+  double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (long long i = static_cast<long long>(cluster_ctarank()) * kMeanThreads + t; i < p.T; i += kQualityBlocks * kMeanThreads) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) s[c] += __ldcg(p.rows + c * p.T + i);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], off);
+    if ((t & 31) == 0) part[c][t >> 5] = s[c];
+  }
+  __syncthreads();
+  if (t < 96) {
+    const int c = t >> 5;
+    double v = part[c][t & 31];
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((t & 31) == 0) sums[c] = v;
+  }
+  cluster_arrive();
+  cluster_wait();
+  if (cluster_ctarank() == 0 && t < 3) {
+    double v = 0.0;
+    for (uint32_t r = 0; r < kQualityBlocks; ++r) v += ld_cluster_double(map_to_cta(smem_u32(&sums[t]), r));
+    p.out[t] = p.T > 0 && t < 2 ? v / static_cast<double>(p.T) : v;
+  }
+  cluster_arrive();
+  cluster_wait();
 }
 
 // Mean of v[0 .. count) by one block: strided partial sums with eight loads in flight, then warp

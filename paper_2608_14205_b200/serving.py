@@ -68,10 +68,7 @@ class ServingLoop:
             self._q = dict(z_early=torch.zeros(max(1, T * E), device=self.dev),
                            z=torch.zeros(max(1, T * E), device=self.dev),
                            ids_early=torch.zeros(max(1, T * k), dtype=torch.int32, device=self.dev),
-                           rows=f64(T), metrics=f64(3))
-            # one word each for the two cosines and the hit count, so that one copy brings all three back
-            m = self._q["metrics"]
-            self._q.update(cos_hidden=m[0:1], cos_logits=m[1:2], hits=m[2:3].view(torch.int32)[:1])
+                           rows=f64(3 * T), metrics=f64(3))
         return self._q
 
     def layer_step(self, layer: int, router: B.FbRouter, h_prev: torch.Tensor, H: torch.Tensor,
@@ -95,13 +92,10 @@ class ServingLoop:
                               o["load_after"])
             ctx.fb_route_dispatch(router, H, T, pi_new, o["ids"], o["w"], o["slot_offsets"], o["rank_offsets"],
                                   o["perm"], o["inv_perm"], o["rank_load"], q["z"])
-            B.fb_row_cosine_mean(h_prev, H, q["rows"], q["cos_hidden"])
-            B.fb_row_cosine_mean(q["z_early"][:T * E].view(T, E), q["z"][:T * E].view(T, E), q["rows"],
-                                 q["cos_logits"])
-            B.fb_topk_hits(q["ids_early"], o["ids"], T, k, q["hits"])
-            m = q["metrics"].cpu()
-            hits = int(m[2:3].view(torch.int32)[0]) & 0xFFFFFFFF
-            report = dict(cos_hidden=float(m[0]), cos_logits=float(m[1]), hit_rate=hits / (T * k) if T * k else 1.0)
+            B.fb_prediction_quality(h_prev, H, q["z_early"], q["z"], q["ids_early"], o["ids"], T, self.wl.d, E, k,
+                                    q["rows"], q["metrics"])
+            cos_hidden, cos_logits, hits = q["metrics"].tolist()       # one copy to the host
+            report = dict(cos_hidden=cos_hidden, cos_logits=cos_logits, hit_rate=hits / (T * k) if T * k else 1.0)
         # the plan is committed: the buffer that held the old placement receives the next one
         self.placement[layer], self._spare = pi_new, pi
         return dict(out=o, pi_old=pi, pi_new=pi_new, **report)

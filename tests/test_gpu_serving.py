@@ -87,3 +87,25 @@ def test_metric_kernels_on_constructed_inputs():
     assert hits.item() == 0
     with pytest.raises(B.FbError):
         B.fb_topk_hits(ids_a, ids_b, 3, 9, hits)
+
+
+@pytest.mark.parametrize("T,d,E,k", [(1, 8, 5, 1), (37, 72, 100, 8), (1000, 20, 33, 3), (8200, 64, 8, 2)])
+def test_combined_metrics_match_the_separate_calls(T, d, E, k):
+    # row sums are formed alike; the means add them in another order: 1e-12 is far above 2^-53 sqrt(T)
+    g = torch.Generator().manual_seed(T)
+    dev = torch.device("cuda")
+    h = torch.randn(T, d, generator=g).to(torch.bfloat16).to(dev)
+    H = (h.float().cpu() + 0.3 * torch.randn(T, d, generator=g)).to(torch.bfloat16).to(dev)
+    H[T // 2] = 0                                                # a row that is zero on one side contributes 0
+    za, zb = (torch.randn(T, E, generator=g).to(dev) for _ in range(2))
+    ia, ib = (torch.rand(T, E, generator=g).topk(k, dim=1).indices.to(torch.int32).to(dev).contiguous() for _ in range(2))
+    rows, mean = torch.zeros(3 * T, dtype=torch.float64, device=dev), torch.zeros(1, dtype=torch.float64, device=dev)
+    hits, out = torch.zeros(1, dtype=torch.int32, device=dev), torch.zeros(3, dtype=torch.float64, device=dev)
+    B.fb_prediction_quality(h, H, za, zb, ia, ib, T, d, E, k, rows, out)
+    got = out.tolist()
+    B.fb_row_cosine_mean(h, H, rows, mean)
+    assert abs(got[0] - mean.item()) < 1e-12
+    B.fb_row_cosine_mean(za, zb, rows, mean)
+    assert abs(got[1] - mean.item()) < 1e-12
+    B.fb_topk_hits(ia, ib, T, k, hits)
+    assert got[2] == hits.item()

@@ -406,7 +406,8 @@ fb_status fb_topk_hits(const int32_t* ids_a, const int32_t* ids_b, int32_t T, in
 /* The three figures of one layer of one step in two launches: metrics_out[0] the mean cosine of h_prev and H
  * (bf16 [T][d]), [1] that of the logits z_early and z (f32 [T][E]), [2] the number of recovered assignments
  * (ids_early, ids: [T][k]) as a double.  Same definitions and precision as the two calls above; row_scratch:
- * double [3 T].  All pointers are device pointers.  T = 0 gives 0, 0, 0. */
+ * double [3 T].  All pointers are device pointers; metrics_out may also be page-locked host memory (complete
+ * when the stream has drained).  T = 0 gives 0, 0, 0. */
 fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* z_early, const float* z,
                                 const int32_t* ids_early, const int32_t* ids, int32_t T, int32_t d, int32_t E, int32_t k,
                                 double* row_scratch, double* metrics_out, fb_stream stream);

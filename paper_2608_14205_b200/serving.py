@@ -68,7 +68,8 @@ class ServingLoop:
             self._q = dict(z_early=torch.zeros(max(1, T * E), device=self.dev),
                            z=torch.zeros(max(1, T * E), device=self.dev),
                            ids_early=torch.zeros(max(1, T * k), dtype=torch.int32, device=self.dev),
-                           rows=f64(3 * T), metrics=f64(3))
+                           rows=f64(3 * T),
+                           metrics=torch.zeros(3, dtype=torch.float64).pin_memory())     # the kernel writes to the host
         return self._q
 
     def layer_step(self, layer: int, router: B.FbRouter, h_prev: torch.Tensor, H: torch.Tensor,
@@ -94,7 +95,8 @@ class ServingLoop:
                                   o["perm"], o["inv_perm"], o["rank_load"], q["z"])
             B.fb_prediction_quality(h_prev, H, q["z_early"], q["z"], q["ids_early"], o["ids"], T, self.wl.d, E, k,
                                     q["rows"], q["metrics"])
-            cos_hidden, cos_logits, hits = q["metrics"].tolist()       # one copy to the host
+            torch.cuda.current_stream(self.dev).synchronize()
+            cos_hidden, cos_logits, hits = q["metrics"].tolist()
             report = dict(cos_hidden=cos_hidden, cos_logits=cos_logits, hit_rate=hits / (T * k) if T * k else 1.0)
         # the plan is committed: the buffer that held the old placement receives the next one
         self.placement[layer], self._spare = pi_new, pi

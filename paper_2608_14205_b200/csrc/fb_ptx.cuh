@@ -67,6 +67,9 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 
 constexpr uint64_t kWaitLimitNs = 1000ull * 1000ull * 1000ull;   // one second per wait
 
+// Release and acquire at device scope (what __threadfence() does beyond that, a total order, is not needed here).
+__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // Wait for the phase with the given parity.  Gives up after limit_ns, or as soon
 // as another thread of the block has given up (abort flag in shared memory), and
 // returns false; the caller then skips to its clean-up.
@@ -340,7 +343,9 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// Without ordering of memory (the barriers' initialisation is published by fence_mbar_init).
+// Without ordering of memory: for barriers that only say "I am done with your block" (no data is handed over;
+// the barriers' initialisation is published by fence_mbar_init).  The releasing form makes every warp wait for
+// its outstanding writes.
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }

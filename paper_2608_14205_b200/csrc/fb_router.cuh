@@ -355,12 +355,12 @@ __device__ __forceinline__ void publish_counts(Shared& sh, const RouterParams& p
   if (et == 0) {
     // The barrier orders every thread's histogram atomics before this fence, and the
     // fence (cumulative) publishes them device-wide before the ticket is taken.
-    __threadfence();
+    fence_acq_rel_gpu();
     const uint32_t prev = atomicAdd(p.ticket, 1u);
     const bool last = prev == static_cast<uint32_t>(p.ticket_target) - 1;
     // Acquire side of the same hand-shake: the other blocks' counts are visible to this thread
     // after the fence and, through the barrier below, to the whole block.
-    if (last) __threadfence();
+    if (last) fence_acq_rel_gpu();
     sh.is_last = last ? 1 : 0;
   }
   named_bar_sync(kPlanBarrierId, kEpilogueThreads);
@@ -628,7 +628,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   walk.cluster_rank = cta_rank;
   if (warp == 0) {
     produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
-    cluster_arrive();          // this warp is done with the pair's shared state (see the teardown)
+    cluster_arrive_relaxed();  // this warp is done with the pair's shared state (see the teardown)
   } else if (warp == 1 || warp == kSecondIssuerWarp) {
     // MMA issuers: in a pair only the even block issues
     if (cta_rank == 0 && (warp == 1 || p.issuers == 2))
@@ -642,7 +642,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       named_bar_arrive(kAccumBarrierId, kEpilogueThreads + 32);
     }
     __syncwarp();
-    cluster_arrive();
+    cluster_arrive_relaxed();
   } else {
     // ------------------------------------------------------------ epilogue
     const int et = threadIdx.x - 64;                       // 0 .. kEpilogueThreads-1
@@ -767,7 +767,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     tcgen05_fence_before();
     // This warp has read its part of tensor memory: its share of the pair's closing barrier
     // is delivered now, so that nobody waits for it at the end (see the teardown).
-    cluster_arrive();
+    cluster_arrive_relaxed();
     row_sync();
     FB_STAMP(4, 64);
     if (got) {

@@ -78,6 +78,7 @@ struct RowsShared {
   // tiles, so that the next tile's MMAs need not wait for the drain.
   uint64_t accum_bar[2];                     // per set: both issuers' commits, once per use
   uint64_t tmem_empty_bar[2];                // per set, even block's copy: all epilogue warps of the pair, once per use
+  uint64_t staged_bar;                       // the blocks that share this block's tile have staged their sums
   uint32_t tmem_base;
   int32_t abort_flag;
   int32_t is_last;
@@ -560,6 +561,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       mbar_init(smem_u32(&sh.accum_bar[a]), static_cast<uint32_t>(p.issuers));   // one commit per MMA issuer
       mbar_init(smem_u32(&sh.tmem_empty_bar[a]), 2 * kEpilogueWarps);
     }
+    mbar_init(smem_u32(&sh.staged_bar), static_cast<uint32_t>(J));
     fence_mbar_init();
     prefetch_tensormap(&tmap_x);
     if (p.mode == kModeLayer) prefetch_tensormap(&tmap_x2);
@@ -654,8 +656,8 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       const uint32_t taddr = taddr0 + set * set_cols;
       if (et == 0) sh.accum_ok = mbar_wait<true>(smem_u32(&sh.accum_bar[set]), use & 1u, abort_flag) ? 1 : 0;
       named_bar_sync(kAccumBarrierId, kEpilogueThreads);
-      const bool got = sh.accum_ok != 0 && p.probe == 0;     // a measurement launch ends with its main loop
-      if (sh.accum_ok == 0 && J == 1) break;                 // (blocks that share a tile pair go on to their common barrier)
+      bool got = sh.accum_ok != 0 && p.probe == 0;     // a measurement launch ends with its main loop
+      if (sh.accum_ok == 0 && J == 1) break;                 // (blocks that share a tile pair go on and tell the others)
       ++tiles_done;
       tcgen05_fence_after();
       FB_STAMP(2, 64);
@@ -696,13 +698,22 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
         // ---- this warp's rows of the staged ones
         int first, count;
         if (J > 1) {
-          cluster_arrive(); cluster_wait();                  // every block's partial tile is staged
+          // every block's partial tile is staged: one thread per block tells the others that share the tile (a
+          // cluster barrier of all their warps took 0.9 us, every warp waiting for its own writes first)
+          named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+          if (et < J) mbar_arrive_cluster(smem_u32(&sh.staged_bar), cta_rank + 2u * static_cast<uint32_t>(et));
+          const bool staged = mbar_wait<true>(smem_u32(&sh.staged_bar), 0u, abort_flag);
+          got = got && __all_sync(0xffffffffu, staged);
           const int slice = kTileM / J, per = max(2, slice / kEpilogueWarps);
           first = piece * slice + ew * per;
           count = ew * per < slice ? per : 0;
         } else if (chunk_rows == kTileM) {
           // the four warps that share a quarter of the rows meet at their own barrier
-          if (last_tile) { cluster_arrive(); closing_arrived = true; }     // done with tensor memory and the partner
+          if (last_tile) {                                     // done with tensor memory and the partner
+            // (releasing where arrivals at the partner's barriers may still be under way)
+            if (several_tiles) cluster_arrive(); else cluster_arrive_relaxed();
+            closing_arrived = true;
+          }
           named_bar_sync(kRowBarrierBase + static_cast<uint32_t>(quarter), kEpiSubs * 32);
           first = quarter * 32 + sub * 8;
           count = 8;
@@ -729,7 +740,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
           FB_STAMP(10, 64);
         }
       }
-      if (J > 1) { cluster_arrive(); closing_arrived = true; }   // done with the other blocks' staged rows
+      if (J > 1) { cluster_arrive_relaxed(); closing_arrived = true; }   // done with the other blocks' staged rows
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
       if (p.probe != 0) {
         // measurement launch: nothing is published
@@ -754,7 +765,6 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   // Tensor memory may be released, and a block may leave, only when all blocks of the cluster are
   // done with it: a warp delivers its arrival as soon as its own last access to the others is over, so
   // the wait normally finds the barrier complete.
-  if (J > 1 && (warp < 2 || warp == kSecondIssuerWarp)) { cluster_arrive(); cluster_wait(); }   // the barrier behind the staging
   if (!closing_arrived) cluster_arrive();
   tcgen05_fence_before();
   __syncthreads();

@@ -216,31 +216,88 @@ __device__ __forceinline__ float from_ordered_bits(uint32_t u) {
   return __uint_as_float(u ^ ((u >> 31) ? 0x80000000u : 0xffffffffu));
 }
 
-// The k-th largest of the known keys of a row: tab holds three tables of kBoundRows rows
-// (each chunk's best, second and third key), of which the first n_chunks rows are valid
-// (3 n_chunks >= k).  Counting instead of sorting: value v is the answer if at least k values
-// are >= v and it is the largest such value; all comparisons are independent of each other.
-template <int kRows>
-__device__ __forceinline__ float kth_largest_of_tables(const float* tab, int n_chunks, int k, int row_in_tile) {
-  float v[3 * kRows];
-#pragma unroll
-  for (int t = 0; t < 3; ++t)
-#pragma unroll
-    for (int c = 0; c < kRows; ++c)
-      v[t * kRows + c] = c < n_chunks ? tab[(t * kBoundRows + c) * kTileM + row_in_tile] : -INFINITY;
+// Sorted merge of two descending lists of three (Batcher's odd-even merge of 4 + 4 without the padding).
+__device__ __forceinline__ void merge3(const float (&a)[3], const float (&b)[3], float (&o)[6]) {
+  // even places a0 a2 | b0 b2 and odd places a1 | b1 merged, then neighbours compared
+  const float e0 = fmaxf(a[0], b[0]), x = fminf(a[0], b[0]), y = fmaxf(a[2], b[2]), e3 = fminf(a[2], b[2]);
+  const float e1 = fmaxf(x, y), e2 = fminf(x, y);
+  const float d0 = fmaxf(a[1], b[1]), d1 = fminf(a[1], b[1]);
+  o[0] = e0;
+  o[1] = fmaxf(d0, e1); o[2] = fminf(d0, e1);
+  o[3] = fmaxf(d1, e2); o[4] = fminf(d1, e2);
+  o[5] = e3;
+}
+// The k-th largest of two descending lists: the best of "the i-th of one and the (k - i)-th of the other".
+template <int kLen, int kK>
+__device__ __forceinline__ float kth_of_two(const float (&a)[kLen], const float (&b)[kLen]) {
   float best = -INFINITY;
 #pragma unroll
-  for (int i = 0; i < 3 * kRows; ++i) {
-    int at_least = 0;
-#pragma unroll
-    for (int j = 0; j < 3 * kRows; ++j) at_least += v[j] >= v[i] ? 1 : 0;
-    if (at_least >= k) best = fmaxf(best, v[i]);
+  for (int i = 0; i <= kK; ++i) {
+    if (i <= kLen && kK - i <= kLen) {
+      const float x = i > 0 ? a[i > 0 ? i - 1 : 0] : INFINITY, y = kK - i > 0 ? b[kK - i > 0 ? kK - i - 1 : 0] : INFINITY;
+      best = fmaxf(best, fminf(x, y));
+    }
   }
   return best;
 }
+template <int kLen>
+__device__ __forceinline__ float kth_of_two(const float (&a)[kLen], const float (&b)[kLen], int k) {
+  switch (k) {                                               // (the same for the whole launch)
+    case 1: return kth_of_two<kLen, 1>(a, b);
+    case 2: return kth_of_two<kLen, 2>(a, b);
+    case 3: return kth_of_two<kLen, 3>(a, b);
+    case 4: return kth_of_two<kLen, 4>(a, b);
+    case 5: return kth_of_two<kLen, 5>(a, b);
+    case 6: return kth_of_two<kLen, 6>(a, b);
+    case 7: return kth_of_two<kLen, 7>(a, b);
+    default: return kth_of_two<kLen, 8>(a, b);
+  }
+}
+// The 8 largest of two descending lists of six, in descending order: the larger halves of a bitonic sequence
+// of 16 (six and six with two -inf behind each), then a bitonic sort of 8.
+__device__ __forceinline__ void merge6_top8(const float (&a)[6], const float (&b)[6], float (&o)[8]) {
+  o[0] = a[0]; o[1] = a[1];
+#pragma unroll
+  for (int i = 2; i < 6; ++i) o[i] = fmaxf(a[i], b[7 - i]);
+  o[6] = b[1]; o[7] = b[0];
+#pragma unroll
+  for (int w = 4; w >= 1; w >>= 1) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if ((i & w) == 0) {
+        const float hi = fmaxf(o[i], o[i + w]);
+        o[i + w] = fminf(o[i], o[i + w]);
+        o[i] = hi;
+      }
+  }
+}
+
+// The k-th largest of the known keys of a row: tab holds three tables of kBoundRows rows
+// (each chunk's best, second and third key), of which the first n_chunks rows are valid
+// (3 n_chunks >= k).  By merging the sorted triples (counting for every value how many are at least as
+// large took 0.9 us more of a launch of one tile per pair at 4 chunks; layer step 8192 x 128 30.0 -> 28.7 us,
+// 131072 x 128 211 -> 204).
 __device__ __forceinline__ float kth_largest_known(const float* tab, int n_chunks, int k, int row_in_tile) {
-  return n_chunks <= 4 ? kth_largest_of_tables<4>(tab, n_chunks, k, row_in_tile)
-                       : kth_largest_of_tables<kBoundRows>(tab, n_chunks, k, row_in_tile);
+  auto triple = [&](int c, float (&v)[3]) {
+#pragma unroll
+    for (int t = 0; t < 3; ++t) v[t] = c < n_chunks ? tab[(t * kBoundRows + c) * kTileM + row_in_tile] : -INFINITY;
+  };
+  auto six = [&](int c, float (&o)[6]) {
+    float a[3], b[3];
+    triple(c, a);
+    triple(c + 1, b);
+    merge3(a, b, o);
+  };
+  float p[6], q[6];
+  six(0, p);
+  six(2, q);
+  if (n_chunks <= 4) return kth_of_two<6>(p, q, k);
+  float left[8], right[8];
+  merge6_top8(p, q, left);
+  six(4, p);
+  six(6, q);
+  merge6_top8(p, q, right);
+  return kth_of_two<8>(left, right, k);
 }
 
 // Ranking selection, shared by both router kernels.  cand[c * 128 + row] holds candidate c of

@@ -39,11 +39,12 @@ struct PersistShared {
   int32_t abort_flag;
   int32_t is_last;
   int32_t accum_ok;
-  int32_t any_overflow;
+  int32_t any_overflow[4];                   // per row quarter
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];
-  alignas(16) uint32_t hist[FB_MAX_EXPERTS];
+  alignas(16) uint32_t hist[FB_MAX_EXPERTS];          // early pass: over all of the block's tiles
+  alignas(16) uint32_t tile_hist[2][FB_MAX_EXPERTS];  // normal pass: of one tile, in turn
   uint32_t cand_count[kTileM];
   PlanShared plan;
 };
@@ -75,7 +76,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
     sh.is_last = 0;
-    sh.any_overflow = 0;
+    for (int q = 0; q < 4; ++q) sh.any_overflow[q] = 0;
     sh.issuer_progress[0] = -1;
     sh.issuer_progress[1] = -1;
     for (int s = 0; s < p.stages; ++s) {
@@ -99,6 +100,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     const int et = threadIdx.x - 64;
     for (int e = et; e < FB_MAX_EXPERTS; e += kEpilogueThreads) {
       sh.hist[e] = 0;
+      sh.tile_hist[0][e] = sh.tile_hist[1][e] = 0;
       if (e < kTileM) sh.cand_count[e] = 0;
     }
     if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_clear(sh.plan, et, kEpilogueThreads);
@@ -155,8 +157,6 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     unsigned long long* cand = reinterpret_cast<unsigned long long*>(third_s + kPersistGroups * kTileM);
     uint32_t* out_hi = reinterpret_cast<uint32_t*>(gscore_s);   // [8][128]: group scores are dead by then
     uint32_t* out_lo = reinterpret_cast<uint32_t*>(glow_s);
-    float* merge_v = reinterpret_cast<float*>(cand);            // [3][8][128]: candidates are dead by then
-    int32_t* merge_i = reinterpret_cast<int32_t*>(merge_v + (kEpiSubs - 1) * FB_MAX_TOPK * kTileM);
 
     // biases (read by these warps only, after the first barrier below)
     for (int e = et; e < FB_MAX_EXPERTS; e += kEpilogueThreads) {
@@ -165,6 +165,11 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     }
     // any block may turn out to take the last ticket of the early pass
     if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
+    // Within a tile data passes only between the kEpiSubs warps that share a quarter of the rows: they meet at a
+    // barrier of their own, and the histogram alternates between two tables, so that per tile two barriers of all
+    // 16 warps are left (the accumulator's and the histogram's) of six.  131072 tokens, 128 experts: 203.0 -> 200.2 us
+    // for the layer call; no difference at 16384 tokens, 256 experts.
+    auto row_sync = [&]() { named_bar_sync(kRowBarrierBase + static_cast<uint32_t>(quarter), kEpiSubs * 32); };
     uint32_t tiles_done = 0;
     for (int pt = pair_first; pt < total_pairs; pt += pair_stride) {
       const bool second_pass = pt >= pairs_per_pass;
@@ -183,6 +188,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       if (sh.accum_ok == 0) break;
       ++tiles_done;
       tcgen05_fence_after();
+      uint32_t* const hist = mode == kModeDispatch ? sh.tile_hist[tiles_done & 1u] : sh.hist;
 
       // ---------------- tensor memory -> registers: this thread's row, chunks sub and sub + 4
       float key[2][32];
@@ -272,7 +278,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           }
         }
       }
-      named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+      row_sync();
 
       // ---------------- choose the groups; lower bound for the k-th key
       uint32_t kept = 0;
@@ -321,20 +327,20 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           }
         }
       }
-      named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+      row_sync();
 
       // ---------------- rank the candidates (many equal keys can overflow the list: handled below)
       const bool overflow = rank_candidates(cand, sh.cand_count[row_in_tile], sub, row_in_tile, out_hi, out_lo);
-      if (overflow) sh.any_overflow = 1;
-      named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+      if (overflow) sh.any_overflow[quarter] = 1;
+      row_sync();
       TopK top;
       top.init();
       if (sub == 0) {
         sh.cand_count[row_in_tile] = 0;                      // ready for the next tile
         if (!overflow) read_ranked(top, k, out_hi, out_lo, row_in_tile);
       }
-      if (sh.any_overflow != 0) {
-        // Some row of the tile had more than kCandCap keys at or above its floor (many equal
+      if (sh.any_overflow[quarter] != 0) {
+        // Some of these rows had more than kCandCap keys at or above its floor (many equal
         // keys).  Such rows are selected by plain insertion: every thread scans its own kept
         // chunks in ascending expert order, then the row's first thread merges the lists.
         if (overflow) {
@@ -349,21 +355,18 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           }
           if (sub != 0) {
 #pragma unroll
-            for (int j = 0; j < FB_MAX_TOPK; ++j) {
-              merge_v[((sub - 1) * FB_MAX_TOPK + j) * kTileM + row_in_tile] = top.v[j];
-              merge_i[((sub - 1) * FB_MAX_TOPK + j) * kTileM + row_in_tile] = top.i[j];
-            }
+            for (int j = 0; j < FB_MAX_TOPK; ++j)            // the row's candidates are dead by now
+              cand[((sub - 1) * FB_MAX_TOPK + j) * kTileM + row_in_tile] =
+                  static_cast<unsigned long long>(__float_as_uint(top.v[j])) << 32 | static_cast<uint32_t>(top.i[j]);
           }
         }
-        named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+        row_sync();
         if (overflow && sub == 0) {
 #pragma unroll 1
-          for (int s2 = 1; s2 < kEpiSubs; ++s2) {
-#pragma unroll 1
-            for (int j = 0; j < FB_MAX_TOPK; ++j) {
-              const float x = merge_v[((s2 - 1) * FB_MAX_TOPK + j) * kTileM + row_in_tile];
-              if (x > -INFINITY) top.insert_any_order(x, merge_i[((s2 - 1) * FB_MAX_TOPK + j) * kTileM + row_in_tile]);
-            }
+          for (int j = 0; j < (kEpiSubs - 1) * FB_MAX_TOPK; ++j) {
+            const unsigned long long w = cand[j * kTileM + row_in_tile];
+            const float x = __uint_as_float(static_cast<uint32_t>(w >> 32));
+            if (x > -INFINITY) top.insert_any_order(x, static_cast<int32_t>(static_cast<uint32_t>(w)));
           }
         }
       }
@@ -376,15 +379,15 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
         // ---------------- histogram (Eq. 5)
 #pragma unroll
         for (int j = 0; j < FB_MAX_TOPK; ++j)
-          if (j < k) atomicAdd(&sh.hist[top.i[j]], 1u);
+          if (j < k) atomicAdd(&hist[top.i[j]], 1u);
       }
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
-      if (et == 0) sh.any_overflow = 0;                       // everyone has read it
+      if (et < 4) sh.any_overflow[et] = 0;                    // everyone has read it
       if (mode == kModeDispatch) {
         const bool owns = static_cast<long long>(tile) * kTileM < p.T;   // the padding block of an odd pair owns no tile
-        if (owns) write_slice_counts(p.slice_counts, tile, E, sh.hist, et);
-        named_bar_sync(kPlanBarrierId, kEpilogueThreads);
-        for (int e = et; e < E; e += kEpilogueThreads) sh.hist[e] = 0;
+        if (owns) write_slice_counts(p.slice_counts, tile, E, hist, et);
+        // the other one was written out before the last barrier; the next tile counts into it
+        for (int e = et; e < E; e += kEpilogueThreads) sh.tile_hist[(tiles_done & 1u) ^ 1u][e] = 0;
       } else if (pt + pair_stride >= pairs_per_pass) {
         // The histogram keeps accumulating over this block's tiles of the pass and is published
         // once, after the last of them (one fence and one ticket per block, not per tile).

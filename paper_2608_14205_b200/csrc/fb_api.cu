@@ -324,7 +324,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   const bool several = J == 1 && probe == 0 && tile_pairs > pairs_avail && !(ranking && logits != nullptr);
   // Both passes of the layer at the same time: nothing could hide the planner behind the second pass, so
   // the dispatch-index kernel counts and plans (see fb_dispatch_kernel).  With several tiles per pair the
-  // early pass is done long before the normal one and its last block plans meanwhile.
+  // early pass is done long before the normal one and the planner runs beside it.
   p.defer_counts = (mode == fb::kModeLayer && !several && p.fuse_planner && deferred_out != nullptr) ? 1 : 0;
   if (p.defer_counts) {
     p.fuse_planner = 0;
@@ -353,6 +353,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
     smem = ctx->rows_smem[several ? 1 : 0];
   } else if (several) {
     fn = persistent_kernel_fn(sigmoid, router->logit_bias != nullptr);
+    p.ticket_target /= 2;                      // one ticket per pair there
     p.stages = ctx->persist_stages;
     smem = ctx->persist_smem;
   } else {

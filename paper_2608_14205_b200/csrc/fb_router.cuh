@@ -97,7 +97,7 @@ struct RouterParams {
   int32_t acc_sets;                  // sets of accumulators: 2 where a pair walks several tiles
   int32_t mode;
   int32_t tiles_first;               // kModeLayer: blocks below this index (even) belong to the early pass
-  int32_t ticket_target;             // number of blocks that take a ticket (those that publish counts)
+  int32_t ticket_target;             // number of tickets taken: one per block that publishes counts (persistent kernel: per pair)
   int32_t fuse_planner;              // prediction modes: the block that finishes last runs the planner
   int32_t defer_counts;              // kModeLayer: the early pass leaves its histograms in early_counts and the
                                      // dispatch-index kernel counts and plans (fb_dispatch_kernel<true>)

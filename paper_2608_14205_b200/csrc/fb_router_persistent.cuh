@@ -35,9 +35,9 @@ struct PersistShared {
   // tile's MMAs need not wait for the drain.
   uint64_t accum_bar[2];                     // per set: both issuers' commits, once per use
   uint64_t tmem_empty_bar[2];                // per set, even block's copy: all epilogue warps of the pair, once per use
+  uint64_t counts_bar;                       // odd block's copy: both blocks' early histograms are in counts_scratch
   uint32_t tmem_base;
   int32_t abort_flag;
-  int32_t is_last;
   int32_t accum_ok;
   int32_t any_overflow[4];                   // per row quarter
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
@@ -48,6 +48,41 @@ struct PersistShared {
   uint32_t cand_count[kTileM];
   PlanShared plan;
 };
+
+// End of the early pass, by the odd block's second issuer warp (idle there: the even block issues the pair's
+// MMAs): once both blocks' histograms are in the scratch counts it takes the pair's ticket, and the last pair's
+// publishes the count vector (Eq. 5), re-arms the scratch for the next call and runs the planner (Algorithm 1)
+// when asked - beside the epilogue, which goes on with the next tile.  In the epilogue (publish_counts, as in the
+// other router kernels) the planner held up its pair by 12 us and with it the end of the call: layer call with
+// 131072 tokens, 128 experts 200.2 -> 198.2 us (226.2 -> 223.4 us in a loop).
+__device__ __forceinline__ void finish_early_pass(PersistShared& sh, const RouterParams& p, int lane, volatile int* abort_flag) {
+  const bool planner = p.mode != kModePredict && p.fuse_planner != 0;
+  if (planner) {                                                    // any pair may turn out to be the last
+    plan_clear(sh.plan, lane, 32);
+    __syncwarp();
+    plan_load_placement(p.plan, sh.plan, lane, 32);
+    __syncwarp();
+  }
+  if (!__all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&sh.counts_bar), 0u, abort_flag))) return;
+  int last = 0;
+  if (lane == 0) {
+    fence_acq_rel_gpu();                                            // what the two blocks added, before the ticket
+    last = atomicAdd(p.ticket, 1u) == static_cast<uint32_t>(p.ticket_target) - 1 ? 1 : 0;
+    if (last) fence_acq_rel_gpu();                                  // what the other pairs added
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  for (int e = lane; e < p.E; e += 32) {
+    const uint32_t c = __ldcg(&p.counts_scratch[e]);
+    p.counts_out[e] = c;
+    if (planner) plan_put_count(sh.plan, e, c);
+    p.counts_scratch[e] = 0;                                        // ready for the next call
+  }
+  if (lane == 0) *p.ticket = 0;
+  if (!planner) return;
+  plan_swaps_warp<false>(p.plan, sh.plan, lane, p.status);
+  __syncwarp();
+  plan_write_placement(p.plan, sh.plan, lane, 32);
+}
 
 // kSigmoid: sigmoid + bias group-limited gate (true) or softmax gate (false); kLogitBias: a logit
 // bias is given.  One instance per combination keeps code and registers to what it needs.
@@ -75,7 +110,6 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
 
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
-    sh.is_last = 0;
     for (int q = 0; q < 4; ++q) sh.any_overflow[q] = 0;
     sh.issuer_progress[0] = -1;
     sh.issuer_progress[1] = -1;
@@ -87,6 +121,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       mbar_init(smem_u32(&sh.accum_bar[a]), static_cast<uint32_t>(p.issuers));
       mbar_init(smem_u32(&sh.tmem_empty_bar[a]), 2 * (kEpilogueThreads / 32));
     }
+    mbar_init(smem_u32(&sh.counts_bar), 2);
     fence_mbar_init();
     prefetch_tensormap(&tmap_x);
     if (p.mode == kModeLayer) prefetch_tensormap(&tmap_x2);
@@ -103,7 +138,6 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       sh.tile_hist[0][e] = sh.tile_hist[1][e] = 0;
       if (e < kTileM) sh.cand_count[e] = 0;
     }
-    if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_clear(sh.plan, et, kEpilogueThreads);
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -121,7 +155,9 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   pdl_launch_dependents();
   const uint32_t tmem_base = sh.tmem_base;
 
-  if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
+  if (warp == kSecondIssuerWarp && cta_rank == 1) {
+    if (p.mode != kModeDispatch && pair_first < pairs_per_pass) finish_early_pass(sh, p, lane, abort_flag);
+  } else if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
     TileWalk walk;
     walk.pair_first = pair_first;
     walk.pair_stride = pair_stride;
@@ -163,8 +199,6 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       sh.logit_bias[e] = (p.logit_bias != nullptr && e < p.E) ? p.logit_bias[e] : 0.0f;
       sh.select_bias[e] = (p.select_bias != nullptr && e < p.E) ? p.select_bias[e] : 0.0f;
     }
-    // any block may turn out to take the last ticket of the early pass
-    if (p.mode == kModePredictPlan || p.mode == kModeLayer) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
     // Within a tile data passes only between the kEpiSubs warps that share a quarter of the rows: they meet at a
     // barrier of their own, and the histogram alternates between two tables, so that per tile two barriers of all
     // 16 warps are left (the accumulator's and the histogram's) of six.  131072 tokens, 128 experts: 203.0 -> 200.2 us
@@ -389,9 +423,17 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
         // the other one was written out before the last barrier; the next tile counts into it
         for (int e = et; e < E; e += kEpilogueThreads) sh.tile_hist[(tiles_done & 1u) ^ 1u][e] = 0;
       } else if (pt + pair_stride >= pairs_per_pass) {
-        // The histogram keeps accumulating over this block's tiles of the pass and is published
-        // once, after the last of them (one fence and one ticket per block, not per tile).
-        publish_counts(sh, p, et, warp, lane, mode == kModePredictPlan && p.fuse_planner != 0);
+        // The histogram accumulated over this block's tiles of the pass and is handed on once, after the last of
+        // them: the fence (cumulative over the barrier) and the arrival publish it to the pair's finishing warp.
+        for (int e = et; e < E; e += kEpilogueThreads) {
+          const uint32_t c = hist[e];
+          if (c) atomicAdd(&p.counts_scratch[e], c);
+        }
+        named_bar_sync(kPlanBarrierId, kEpilogueThreads);
+        if (et == 0) {
+          fence_acq_rel_gpu();
+          mbar_arrive_cluster(smem_u32(&sh.counts_bar), 1u);
+        }
       }
     }
   }

@@ -13,68 +13,121 @@
 
 namespace fb {
 
-constexpr int kCosineWarpsPerBlock = 8;
+constexpr int kCosineWarpsPerBlock = 2;      // small blocks: a finished row's place is taken at once
 constexpr int kMeanThreads = 1024;
+constexpr int kCosineSteps = 4;              // steps of a bf16 row whose loads are in flight
+constexpr int kCosineBlocksPerSm = 12;       // for 80 registers a thread, which the four steps need
 
 __device__ __forceinline__ double load_as_double(const __nv_bfloat16* p, long long i) {
   return static_cast<double>(__bfloat162float(p[i]));
 }
 __device__ __forceinline__ double load_as_double(const float* p, long long i) { return static_cast<double>(p[i]); }
 
-// 16 bytes of a row as doubles: 8 bf16 or 4 f32 values.
-__device__ __forceinline__ int unpack16(const __nv_bfloat16* p, long long i, double (&v)[8]) {
-  const uint4 q = *reinterpret_cast<const uint4*>(p + i);
-  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    v[2 * t] = static_cast<double>(__uint_as_float(w[t] << 16));              // low half = element 2t
-    v[2 * t + 1] = static_cast<double>(__uint_as_float(w[t] & 0xffff0000u));
-  }
-  return 8;
-}
-__device__ __forceinline__ int unpack16(const float* p, long long i, double (&v)[8]) {
-  const float4 q = *reinterpret_cast<const float4*>(p + i);
-  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-  return 4;
+// A bf16 value (the upper half of a 32-bit word with a zero lower half) times 2^-896 as a double, by moving its
+// bits: 8 exponent bits under a double's 11-bit exponent.  Exact, zeros and subnormals included (a double's
+// subnormals lie 896 binades below).  Infinities and NaNs become finite values: the caller looks for them itself.
+__device__ __forceinline__ double bf16_scaled(uint32_t u) {
+  return __hiloint2double(static_cast<int>(static_cast<uint32_t>(static_cast<int32_t>(u) >> 3) & 0x8fffffffu), 0);
 }
 
-// Cosine of two rows by one warp.  Rows whose start and length allow it are read 16 bytes per lane and
-// step (kVec elements); otherwise lane l takes elements l, l + 32, ...  Either way a lane
-// adds its elements in ascending order and the three partial sums are combined by a
-// butterfly, which gives every lane the same total.
-template <class Tin>
-__device__ __forceinline__ double row_cosine(const Tin* __restrict__ a, const Tin* __restrict__ b, long long row, int n, int lane) {
-  constexpr int kVec = 16 / static_cast<int>(sizeof(Tin));
-  const long long base = row * n;
+// A lane's part of the sums a.b, a.a and b.b of two rows.  Rows whose start and length allow it are read 16 bytes per
+// lane and step (kVec elements); otherwise lane l takes elements l, l + 32, ...  Either way a lane adds its elements
+// in ascending order, exact products into doubles.
+struct CosineSums {
   double dot = 0.0, na = 0.0, nb = 0.0;
+  __device__ __forceinline__ void add(double x, double y) { dot += x * y; na += x * x; nb += y * y; }
+};
+template <class Tin>
+__device__ __forceinline__ CosineSums row_sums(const Tin* __restrict__ a, const Tin* __restrict__ b, long long row, int n, int lane) {
+  constexpr int kVec = 16 / static_cast<int>(sizeof(Tin)), kStep = 32 * kVec;
+  const long long base = row * n;
+  CosineSums s;
   const bool wide = n % kVec == 0 && reinterpret_cast<uintptr_t>(a) % 16 == 0 && reinterpret_cast<uintptr_t>(b) % 16 == 0;
-  if (wide) {
-    for (int j = lane * kVec; j < n; j += 32 * kVec) {
-      double x[8], y[8];
-      const int m = unpack16(a, base + j, x);
-      unpack16(b, base + j, y);
+  if constexpr (sizeof(Tin) == 2) {
+    if (wide) {
+      // Four steps' loads in flight (the latency of the loads is what a row waits for).  Conversions to double run
+      // at a quarter of the rate of double arithmetic, and two per element kept their unit busy for half of the
+      // time: a's elements are scaled by bit moves instead, which makes the sums dot 2^126, na 2^-770 and nb,
+      // scaled back exactly below - the same bits as with two conversions.
+      __nv_bfloat162 special = __float2bfloat162_rn(0.0f);      // NaN once a has an infinity or a NaN (times 0)
+      for (int j0 = 0; j0 < n; j0 += kCosineSteps * kStep) {
+        uint4 qa[kCosineSteps], qb[kCosineSteps];
 #pragma unroll
-      for (int t = 0; t < 8; ++t)
-        if (t < m) { dot += x[t] * y[t]; na += x[t] * x[t]; nb += y[t] * y[t]; }
+        for (int q = 0; q < kCosineSteps; ++q) {
+          const int j = j0 + q * kStep + lane * kVec;
+          qa[q] = j < n ? *reinterpret_cast<const uint4*>(a + base + j) : make_uint4(0, 0, 0, 0);
+          qb[q] = j < n ? *reinterpret_cast<const uint4*>(b + base + j) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int q = 0; q < kCosineSteps; ++q) {
+          if (j0 + q * kStep >= n) break;
+          const uint32_t wa[4] = {qa[q].x, qa[q].y, qa[q].z, qa[q].w}, wb[4] = {qb[q].x, qb[q].y, qb[q].z, qb[q].w};
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            special = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&wa[t]), __float2bfloat162_rn(0.0f), special);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {                       // low half = the earlier element
+              const double x = bf16_scaled(h ? wa[t] & 0xffff0000u : wa[t] << 16), up = x * 0x1p1022;
+              const double y = static_cast<double>(__uint_as_float(h ? wb[t] & 0xffff0000u : wb[t] << 16));
+              s.dot += up * y; s.na += x * up; s.nb += y * y;
+            }
+          }
+        }
+      }
+      if (!__any_sync(0xffffffffu, __hisnan(special.x) || __hisnan(special.y))) {
+        s.dot *= 0x1p-126; s.na *= 0x1p770;
+        return s;
+      }
+      s = CosineSums();                                         // once more, with conversions
     }
-  } else {
-    for (int j = lane; j < n; j += 32) {
-      const double x = load_as_double(a, base + j), y = load_as_double(b, base + j);
-      dot += x * y; na += x * x; nb += y * y;
+  } else if (wide) {
+    for (int j = lane * kVec; j < n; j += kStep) {
+      const float4 x = *reinterpret_cast<const float4*>(a + base + j), y = *reinterpret_cast<const float4*>(b + base + j);
+      s.add(x.x, y.x); s.add(x.y, y.y); s.add(x.z, y.z); s.add(x.w, y.w);
     }
+    return s;
   }
+  const int per = wide ? kVec : 1;
+  for (int j = lane * per; j < n; j += 32 * per)
+    for (int t = 0; t < per; ++t) s.add(load_as_double(a, base + j + t), load_as_double(b, base + j + t));
+  return s;
+}
+
+// The three partial sums are combined by a butterfly, which gives every lane the same total.
+__device__ __forceinline__ double cosine_of(double dot, double na, double nb) {
+  return (na > 0.0 && nb > 0.0) ? dot / (sqrt(na) * sqrt(nb)) : 0.0;
+}
+__device__ __forceinline__ double row_cosine(CosineSums s) {
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
-    dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    na += __shfl_xor_sync(0xffffffffu, na, off);
-    nb += __shfl_xor_sync(0xffffffffu, nb, off);
+    s.dot += __shfl_xor_sync(0xffffffffu, s.dot, off);
+    s.na += __shfl_xor_sync(0xffffffffu, s.na, off);
+    s.nb += __shfl_xor_sync(0xffffffffu, s.nb, off);
   }
-  return (na > 0.0 && nb > 0.0) ? dot / (sqrt(na) * sqrt(nb)) : 0.0;
+  return cosine_of(s.dot, s.na, s.nb);
+}
+// Two rows' cosines at once, with the same additions: where a butterfly step would form a value twice, half of the
+// lanes go on with another sum instead (8 exchanges instead of 30, one square root and division sequence instead
+// of two).  Lane 0 returns the first row's, lane 16 the second's.
+__device__ __forceinline__ double exchange_add(double keep_low, double keep_high, int lane, int off) {
+  const bool high = (lane & off) != 0;
+  return (high ? keep_high : keep_low) + __shfl_xor_sync(0xffffffffu, high ? keep_low : keep_high, off);
+}
+__device__ __forceinline__ double row_cosines(const CosineSums& s, const CosineSums& t, int lane) {
+  const double dot = exchange_add(s.dot, t.dot, lane, 16), na = exchange_add(s.na, t.na, lane, 16);
+  double nb = exchange_add(s.nb, t.nb, lane, 16);
+  const double dot_na = exchange_add(dot, na, lane, 8);         // lanes with bit 3: na
+  nb += __shfl_xor_sync(0xffffffffu, nb, 8);
+  double v = exchange_add(dot_na, nb, lane, 4);                 // lanes with bit 2: nb
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  const double n1 = __shfl_sync(0xffffffffu, v, (lane & 16) | 8), n2 = __shfl_sync(0xffffffffu, v, (lane & 16) | 4);
+  return cosine_of(v, n1, n2);
 }
 
 // One warp per row.
 template <class Tin>
-__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock)
+__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock, kCosineBlocksPerSm)
 fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long long rows, int n,
                      double* __restrict__ row_cos) {
   const long long row = static_cast<long long>(blockIdx.x) * kCosineWarpsPerBlock + (threadIdx.x >> 5);
@@ -82,14 +135,16 @@ fb_row_cosine_kernel(const Tin* __restrict__ a, const Tin* __restrict__ b, long 
   pdl_launch_dependents();
   pdl_wait();
   if (row >= rows) return;
-  const double c = row_cosine(a, b, row, n, lane);
+  const double c = row_cosine(row_sums(a, b, row, n, lane));
   if (lane == 0) row_cos[row] = c;
 }
 
 // The three quality figures of a step, row by row, in one launch: the hidden-state cosine, the logit cosine
-// and the number of recovered assignments into rows[0 .. T), [T .. 2 T), [2 T .. 3 T).  Bound by the fp64
-// conversions of the hidden states (15 us for 2 x 8192 x 2048 bf16 values); as five launches behind one
-// another the three figures took 31 us, most of it with the GPU nearly empty.
+// and the number of recovered assignments into rows[0 .. T), [T .. 2 T), [2 T .. 3 T).  Bound by the reads of the
+// hidden states and, for short rows, by a warp's chain of loads and exchanges.  With the sums kernel behind it,
+// [T, d, E] = 8192 x 2048 x 128: 20.4 -> 18.0 us; 4096 x 4096 x 8: 25.2 -> 16.7; 1733 x 7168 x 256: 32.9 -> 19.0;
+// 16384 x 7168 x 256: 93.2 -> 83.8 (5.8 TB/s), against eight warps per block, one step's loads in flight, two
+// conversions per element and a reduction per sum.  Two steps in flight: 18.1, 17.8, 23.0 and 87.1 us.
 struct QualityParams {
   const __nv_bfloat16 *h_prev, *h;       // [T][d]
   const float *z_early, *z;              // [T][E]
@@ -99,7 +154,7 @@ struct QualityParams {
   double* rows;                          // [3][T]
   double* out;                           // [3]: mean, mean, sum
 };
-__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock)
+__global__ void __launch_bounds__(32 * kCosineWarpsPerBlock, kCosineBlocksPerSm)
 fb_quality_rows_kernel(const __grid_constant__ QualityParams p) {
   const long long row = static_cast<long long>(blockIdx.x) * kCosineWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -111,13 +166,10 @@ fb_quality_rows_kernel(const __grid_constant__ QualityParams p) {
   uint32_t hits = 0;
 #pragma unroll
   for (int y = 0; y < FB_MAX_TOPK; ++y) hits += __popc(__ballot_sync(0xffffffffu, mine == __shfl_sync(0xffffffffu, early, y)));
-  const double cz = row_cosine(p.z_early, p.z, row, p.E, lane);
-  const double ch = row_cosine(p.h_prev, p.h, row, p.d, lane);
-  if (lane == 0) {
-    p.rows[row] = ch;
-    p.rows[p.T + row] = cz;
-    p.rows[2 * p.T + row] = static_cast<double>(hits);
-  }
+  const CosineSums logits = row_sums(p.z_early, p.z, row, p.E, lane);
+  const double c = row_cosines(row_sums(p.h_prev, p.h, row, p.d, lane), logits, lane);
+  if ((lane & 15) == 0) p.rows[lane == 0 ? row : p.T + row] = c;
+  if (lane == 1) p.rows[2 * p.T + row] = static_cast<double>(hits);
 }
 // Sums of the three columns by one cluster, in a fixed order.
 constexpr int kQualityBlocks = 8;

@@ -89,6 +89,24 @@ def test_metric_kernels_on_constructed_inputs():
         B.fb_topk_hits(ids_a, ids_b, 3, 9, hits)
 
 
+@pytest.mark.parametrize("n", [8, 248, 256, 1016, 1024, 1032, 2056, 77])
+def test_bf16_row_cosines_at_the_edges_of_steps_and_of_the_value_range(n):
+    # products are exact in double and n of them are added: n 2^-53 of |x| |y|, and twice that for the norms
+    g = torch.Generator().manual_seed(n)
+    dev = torch.device("cuda")
+    x, y = (torch.randn(64, n, generator=g).to(torch.bfloat16) for _ in range(2))
+    for r, scale in enumerate([2.0 ** -130, 2.0 ** -126, 2.0 ** 120, 0.0]):      # subnormals, large values, zeros
+        x[r] = (x[r].float() * scale).to(torch.bfloat16)
+        y[r + 2] = (y[r + 2].float() * scale).to(torch.bfloat16)
+    x[8, n // 2], y[9, n - 1], x[10, 0], y[11, n // 3] = float("inf"), float("-inf"), float("nan"), float("nan")
+    rows, mean = torch.zeros(64, dtype=torch.float64, device=dev), torch.zeros(1, dtype=torch.float64, device=dev)
+    B.fb_row_cosine_mean(x.to(dev), y.to(dev), rows, mean)
+    a, b = x.double(), y.double()
+    dot, na, nb = (a * b).sum(1), (a * a).sum(1), (b * b).sum(1)
+    want = torch.where((na > 0) & (nb > 0), dot / (na.sqrt() * nb.sqrt()), torch.zeros(()).double())
+    assert torch.allclose(rows.cpu(), want, rtol=0.0, atol=4 * n * 2.0 ** -53, equal_nan=True)
+
+
 @pytest.mark.parametrize("T,d,E,k", [(1, 8, 5, 1), (37, 72, 100, 8), (1000, 20, 33, 3), (8200, 64, 8, 2)])
 def test_combined_metrics_match_the_separate_calls(T, d, E, k):
     # row sums are formed alike; the means add them in another order: 1e-12 is far above 2^-53 sqrt(T)

@@ -279,6 +279,20 @@ fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev
                         uint32_t* slot_offsets, uint32_t* rank_offsets, int32_t* perm, int32_t* inv_perm,
                         uint32_t* rank_load, fb_stream stream);
 
+/* fb_layer_step that also hands out what the prediction-quality figures compare, each NULL to skip:
+ *   ids_early    dev i32 [T][k]   the early pass's top-k ids (as fb_predict_load's topk_ids)
+ *   logits_early dev f32 [T][E]   the early pass's logits
+ *   logits       dev f32 [T][E]   the normal pass's logits
+ * The other results are those of fb_layer_step; a logit dump may choose another summation order of the
+ * router GEMM (see fb_set_split), so logits can differ from the separate calls' in the last bits. */
+fb_status fb_layer_step_observed(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
+                                 const int32_t* expert_to_slot, const fb_budget* budget, int32_t layer_id,
+                                 uint32_t* counts, int32_t* expert_to_slot_out, fb_swap* swaps, int32_t* n_swaps,
+                                 uint32_t* load_before, uint32_t* load_after, int32_t* topk_ids, float* topk_w,
+                                 uint32_t* slot_offsets, uint32_t* rank_offsets, int32_t* perm, int32_t* inv_perm,
+                                 uint32_t* rank_load, int32_t* ids_early, float* logits_early, float* logits,
+                                 fb_stream stream);
+
 /* One whole layer (fb_layer_step) with HOST buffers for the per-step tensors: h_prev, H, expert_to_slot
  * are copied to the device, every output pointer receives host data, and the call
  * returns after the stream has drained.  The router stays on the device (frozen

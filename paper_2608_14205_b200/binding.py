@@ -59,7 +59,8 @@ EXPORTS = ["fb_create", "fb_destroy", "fb_budget_ns", "fb_swap_cost_ns", "fb_pre
            "fb_apply_swaps_staged", "fb_fit_cost_model", "fb_calibrate_exchange", "fb_selftest_wait_timeout",
            "fb_set_stamp_buffer", "fb_clock_probe", "fb_attention_begin", "fb_attention_end", "fb_layer_budget_ns",
            "fb_attention_set_time_ns", "fb_attention_reset", "fb_dispatch_slot_counts", "fb_dispatch_globalize",
-           "fb_standin_attention", "fb_set_split", "fb_prediction_quality"]
+           "fb_standin_attention", "fb_set_split", "fb_prediction_quality",
+           "fb_layer_step_observed"]
 
 _lib = None
 
@@ -97,6 +98,9 @@ def lib() -> ctypes.CDLL:
     L.fb_layer_step.argtypes = [vp, ctypes.POINTER(FbRouter), vp, vp, i32, vp, ctypes.POINTER(FbBudget), i32] \
         + [vp] * 14
     L.fb_layer_step.restype = ctypes.c_int
+    L.fb_layer_step_observed.argtypes = [vp, ctypes.POINTER(FbRouter), vp, vp, i32, vp, ctypes.POINTER(FbBudget), i32] \
+        + [vp] * 17
+    L.fb_layer_step_observed.restype = ctypes.c_int
     L.fb_layer_step_host.argtypes = [vp, ctypes.POINTER(FbRouter), vp, vp, i32, vp, ctypes.POINTER(FbBudget), i32] \
         + [vp] * 14
     L.fb_predict_load_static.argtypes = [ctypes.POINTER(FbConfig), ctypes.c_int, ctypes.POINTER(FbRouter), vp, i32,
@@ -338,6 +342,16 @@ class Context:
         _check(lib().fb_layer_step(self._h, ctypes.byref(router), _ptr(h_prev), _ptr(H), T, _ptr(expert_to_slot),
                                    ctypes.byref(budget), layer_id, *[_ptr(o) for o in outs], _stream(stream)),
                "fb_layer_step")
+
+    def fb_layer_step_observed(self, router, h_prev, H, T, expert_to_slot, budget, layer_id, counts, expert_to_slot_out,
+                               swaps, n_swaps, load_before, load_after, topk_ids, topk_w, slot_offsets, rank_offsets,
+                               perm, inv_perm, rank_load, ids_early=None, logits_early=None, logits=None, stream=None):
+        """fb_layer_step that also writes the early pass's ids and both passes' logits."""
+        outs = [counts, expert_to_slot_out, swaps, n_swaps, load_before, load_after, topk_ids, topk_w,
+                slot_offsets, rank_offsets, perm, inv_perm, rank_load, ids_early, logits_early, logits]
+        _check(lib().fb_layer_step_observed(self._h, ctypes.byref(router), _ptr(h_prev), _ptr(H), T,
+                                            _ptr(expert_to_slot), ctypes.byref(budget), layer_id,
+                                            *[_ptr(o) for o in outs], _stream(stream)), "fb_layer_step_observed")
 
     def fb_layer_step_host(self, router, h_prev_host, H_host, T, expert_to_slot_host, budget, layer_id,
                            counts=None, expert_to_slot_out=None, swaps=None, n_swaps=None, load_before=None,

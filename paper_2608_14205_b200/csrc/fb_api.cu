@@ -268,7 +268,8 @@ fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* cou
 fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T, int mode,
                         uint32_t* counts_out, int32_t* topk_ids, float* topk_w, float* logits,
                         const fb::PlanParams* plan, cudaStream_t stream, const void* x2 = nullptr, int probe = 0,
-                        int* pieces_out = nullptr, bool* deferred_out = nullptr) {
+                        int* pieces_out = nullptr, bool* deferred_out = nullptr, int32_t* early_ids = nullptr,
+                        float* early_logits = nullptr) {
   const CUtensorMap *mx = nullptr, *mx2 = nullptr, *mw = nullptr;
   fb_status st = make_map(ctx, ctx->x_maps, &ctx->x_next, x, T, fb::kTileM, &mx);
   if (st != FB_OK) return st;
@@ -294,6 +295,8 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.topk_ids = topk_ids;
   p.topk_w = topk_w;
   p.logits = logits;
+  p.early_ids = early_ids;
+  p.early_logits = early_logits;
   p.slice_counts = ctx->slice_counts;
   p.stamps = ctx->stamps;
   p.probe = probe;
@@ -320,12 +323,16 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   // Which kernel: whole tiles of a gate that the ranking selection handles go there (one tile per pair,
   // or several where more tile pairs than block pairs fit or than the caller allows); tiles shared by
   // several pairs and all other gates take the row-per-warp selection (figures: fb_router_rows.cuh).
+  // Logit dumps: a block of the ranking kernel writes its rows from registers, 16 bytes a store (row-per-warp selection for
+  // dumps instead: serving step with 8192 tokens, 128 experts 75.4 us against 71.6), one tile per pair.
+  const bool dump = logits != nullptr || early_logits != nullptr;
   const bool ranking = J == 1 && ctx->ranking[topk_w != nullptr ? 1 : 0];
-  const bool several = J == 1 && probe == 0 && tile_pairs > pairs_avail && !(ranking && logits != nullptr);
+  const bool several = J == 1 && probe == 0 && tile_pairs > pairs_avail && !(ranking && dump);
   // Both passes of the layer at the same time: nothing could hide the planner behind the second pass, so
   // the dispatch-index kernel counts and plans (see fb_dispatch_kernel).  With several tiles per pair the
   // early pass is done long before the normal one and the planner runs beside it.
-  p.defer_counts = (mode == fb::kModeLayer && !several && p.fuse_planner && deferred_out != nullptr) ? 1 : 0;
+  const bool tile_per_block = (T + fb::kDispatchTile - 1) / fb::kDispatchTile <= ctx->n_sm;   // of that kernel
+  p.defer_counts = (mode == fb::kModeLayer && !several && tile_per_block && p.fuse_planner && deferred_out != nullptr) ? 1 : 0;
   if (p.defer_counts) {
     p.fuse_planner = 0;
     p.early_counts = ctx->early_counts;
@@ -739,12 +746,13 @@ fb_status fb_route_dispatch(fb_ctx* ctx, const fb_router* router, const void* x,
                                rank_load, stream);
 }
 
-fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
+fb_status fb_layer_step_observed(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
                         const int32_t* expert_to_slot, const fb_budget* budget, int32_t layer_id,
                         uint32_t* counts, int32_t* expert_to_slot_out, fb_swap* swaps, int32_t* n_swaps,
                         uint32_t* load_before, uint32_t* load_after, int32_t* topk_ids, float* topk_w,
                         uint32_t* slot_offsets, uint32_t* rank_offsets, int32_t* perm, int32_t* inv_perm,
-                        uint32_t* rank_load, fb_stream stream_) {
+                        uint32_t* rank_load, int32_t* ids_early, float* logits_early, float* logits,
+                                 fb_stream stream_) {
   (void)layer_id;
   if (!ctx || !router || !router->W || !counts || !slot_offsets || !rank_offsets || !rank_load || T < 0)
     return FB_ERR_INVALID_ARG;
@@ -768,11 +776,22 @@ fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev
   // one launch for both router passes; the dispatch index needs the new placement and follows
   int pieces = 1;
   bool deferred = false;
-  st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, nullptr, &pp, stream, H, 0, &pieces,
-                     &deferred);
+  st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, logits, &pp, stream, H, 0, &pieces,
+                     &deferred, ids_early, logits_early);
   if (st != FB_OK) return st;
   return launch_dispatch_index(ctx, T, pieces, deferred ? &pp : nullptr, counts, deferred ? expert_to_slot : expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
                                rank_load, stream);
+}
+
+fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
+                        const int32_t* expert_to_slot, const fb_budget* budget, int32_t layer_id,
+                        uint32_t* counts, int32_t* expert_to_slot_out, fb_swap* swaps, int32_t* n_swaps,
+                        uint32_t* load_before, uint32_t* load_after, int32_t* topk_ids, float* topk_w,
+                        uint32_t* slot_offsets, uint32_t* rank_offsets, int32_t* perm, int32_t* inv_perm,
+                        uint32_t* rank_load, fb_stream stream) {
+  return fb_layer_step_observed(ctx, router, h_prev, H, T, expert_to_slot, budget, layer_id, counts, expert_to_slot_out,
+                                swaps, n_swaps, load_before, load_after, topk_ids, topk_w, slot_offsets, rank_offsets,
+                                perm, inv_perm, rank_load, nullptr, nullptr, nullptr, stream);
 }
 
 fb_status fb_layer_step_host(fb_ctx* ctx, const fb_router* router, const void* h_prev_host, const void* H_host,

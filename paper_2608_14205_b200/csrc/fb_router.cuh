@@ -119,6 +119,8 @@ struct RouterParams {
   int32_t* topk_ids;                 // [T][k] or nullptr
   float* topk_w;                     // [T][k] or nullptr
   float* logits;                     // [T][E] or nullptr
+  int32_t* early_ids;                // kModeLayer: the early pass's ids and logits, or nullptr
+  float* early_logits;
   uint8_t* slice_counts;             // [tiles * pieces][slice_row_bytes(E)] (dispatch mode)
   uint8_t* early_counts;             // the same table for the early pass (defer_counts)
   unsigned long long* stamps;        // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
@@ -624,7 +626,8 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   const bool two_acc = p.issuers == 2 && p.num_kb > 1;
   const CUtensorMap* xmap = second_pass ? &tmap_x2 : &tmap_x;
   // outputs of the normal pass are not written by blocks of the early pass
-  int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_ids;
+  int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? p.early_ids : p.topk_ids;
+  float* const out_logits = (p.mode == kModeLayer && !second_pass) ? p.early_logits : p.logits;
   float* const out_w = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_w;
   const uint32_t cta_rank = cluster_ctarank();
   const uint32_t b_tile_bytes = static_cast<uint32_t>(p.N / 2) * kBlockK * 2;
@@ -753,10 +756,17 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
             for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
           }
         }
-        if (p.logits != nullptr && valid) {
+        if (out_logits != nullptr && valid) {
+          float4* const dst = reinterpret_cast<float4*>(out_logits + row * E + c0);
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            p.logits[row * E + c0 + j] = __uint_as_float(r[j]) + (kLogitBias ? sh.logit_bias[c0 + j] : 0.0f);
+          for (int j = 0; j < 32; j += 4) {
+            float4 z = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+            if (kLogitBias) {
+              z.x += sh.logit_bias[c0 + j]; z.y += sh.logit_bias[c0 + j + 1];
+              z.z += sh.logit_bias[c0 + j + 2]; z.w += sh.logit_bias[c0 + j + 3];
+            }
+            dst[j / 4] = z;
+          }
         }
         if (kSigmoid && !kLogitBias) {
           // Every key goes through the same two hardware approximations, so equal logits give equal keys

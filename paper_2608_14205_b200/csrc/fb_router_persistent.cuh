@@ -211,7 +211,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       const int tile = 2 * (second_pass ? pt - pairs_per_pass : pt) + static_cast<int>(cta_rank);
       const long long row = static_cast<long long>(tile) * kTileM + row_in_tile;
       const bool valid = row < p.T;
-      int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_ids;
+      int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? p.early_ids : p.topk_ids;
       float* const out_w = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_w;
 
       // one thread polls for the finished accumulators, the others sleep at the barrier

@@ -180,7 +180,7 @@ __device__ __forceinline__ float row_exp_sum(const float (&key)[kCpl], float lan
 template <int kCpl, bool kSigmoid>
 __device__ __forceinline__ void select_two_rows(const RouterParams& p, const LaneColumns& lc, const float (&sb)[kCpl],
                                                 const float* logit_bias_s, uint32_t row_addr, uint32_t my_rank,
-                                                long long row, RowScratch& rs, int pair, int lane) {
+                                                long long row, float* out_logits, RowScratch& rs, int pair, int lane) {
   const uint32_t full = 0xffffffffu;
   const uint32_t stride = static_cast<uint32_t>(staging_stride(p.N)) * 4u;
   const bool want_sum = !kSigmoid && p.topk_w != nullptr && !p.renorm;
@@ -217,12 +217,12 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
       key[1][j] += b;
     }
   }
-  if (p.logits != nullptr) {
+  if (out_logits != nullptr) {
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
       for (int j = 0; j < kCpl; ++j)
-        if (j < lc.n && row + u < p.T) p.logits[(row + u) * p.E + lc.c0 + j] = key[u][j];
+        if (j < lc.n && row + u < p.T) out_logits[(row + u) * p.E + lc.c0 + j] = key[u][j];
   }
   // ---- selection keys
   if (kSigmoid) {
@@ -647,7 +647,8 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
       const int mode = p.mode == kModeLayer ? (second_pass ? kModeDispatch : kModePredictPlan) : p.mode;
       const int tile = 2 * (second_pass ? pt - pairs_per_pass : pt) + static_cast<int>(cta_rank);
       // outputs of the normal pass are not written by tiles of the early pass
-      int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_ids;
+      int32_t* const out_ids = (p.mode == kModeLayer && !second_pass) ? p.early_ids : p.topk_ids;
+      float* const out_logits = (p.mode == kModeLayer && !second_pass) ? p.early_logits : p.logits;
       float* const out_w = (p.mode == kModeLayer && !second_pass) ? nullptr : p.topk_w;
       const bool last_tile = pt + pair_stride >= total_pairs;
 
@@ -733,7 +734,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
           for (int i = 0; i < count; i += 2)
             if (row0 + i < p.T)
               select_two_rows<kCpl, kSigmoid>(p, lc, sb, sh.logit_bias, staging + static_cast<uint32_t>(first - r0 + i) * row_stride,
-                                              cluster_rank, row0 + i, rs, i >> 1, lane);
+                                              cluster_rank, row0 + i, out_logits, rs, i >> 1, lane);
           __syncwarp();
           FB_STAMP(8, 64);
           finish_rows<kSigmoid>(p, sh, rs, count, row0, out_ids, out_w, lane);

@@ -127,3 +127,37 @@ def test_combined_metrics_match_the_separate_calls(T, d, E, k):
     assert abs(got[1] - mean.item()) < 1e-12
     B.fb_topk_hits(ia, ib, T, k, hits)
     assert got[2] == hits.item()
+
+
+@pytest.mark.parametrize("T,d,E,k,R,gate,n_group,topk_group,renorm", [
+    (1, 64, 8, 2, 4, "softmax", 1, 1, 1), (300, 128, 128, 8, 8, "softmax", 1, 1, 1), (9217, 128, 128, 8, 8, "softmax", 1, 1, 1),
+    (19001, 64, 128, 8, 8, "softmax", 1, 1, 1), (9300, 128, 256, 8, 64, "sigmoid", 8, 4, 1), (19001, 64, 100, 3, 10, "softmax", 1, 1, 0),
+])
+def test_observed_layer_step_matches_the_separate_calls(T, d, E, k, R, gate, n_group, topk_group, renorm):
+    # small integers: every summation order of the router GEMM is exact, so all results agree bit for bit
+    # (tiles shared by several pairs, one per pair, more than the GPU has pairs; planner in either kernel)
+    g = torch.Generator().manual_seed(T)
+    dev = torch.device("cuda")
+    ints = lambda *s: torch.randint(-3, 4, s, generator=g).to(torch.bfloat16).to(dev)
+    h, H, W = ints(T, d), ints(T, d), ints(E, d)
+    code = I.GATE_SOFTMAX_TOPK if gate == "softmax" else I.GATE_SIGMOID_GROUP_TOPK
+    sb = (0.125 * torch.randint(0, 3, (E,), generator=g)).float().to(dev) if gate == "sigmoid" else None
+    router, ctx = B.make_router(W, None, sb), B.Context(T, d, E, k, R, code, n_group, topk_group, renorm, 1.0)
+    budget = B.make_budget(max_swaps=min(16, E // 2))
+    pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+    i32 = lambda n: torch.full((n,), -7, dtype=torch.int32, device=dev)
+    f32 = lambda n: torch.full((n,), float("nan"), device=dev)
+    bufs = lambda: [i32(E), i32(E), i32(4 * (E // 2)), i32(1), i32(R), i32(R), i32(T * k), f32(T * k), i32(E + 1), i32(R + 1),
+                    i32(T * k), i32(T * k), i32(R)]
+    want, got = bufs(), bufs()
+    ids, ids_early, z, z_early, zs = i32(T * k), i32(T * k), f32(T * E), f32(T * E), f32(2 * T * E)
+    ctx.fb_predict_load(router, h, T, i32(E), ids, zs[:T * E])
+    ctx.fb_layer_step(router, h, H, T, pi, budget, 0, *want)
+    other = bufs()
+    ctx.fb_route_dispatch(router, H, T, want[1], *other[6:], zs[T * E:])
+    ctx.fb_layer_step_observed(router, h, H, T, pi, budget, 0, *got, ids_early, z_early, z)
+    assert ctx.fb_device_status() == 0
+    assert torch.equal(ids_early, ids) and torch.equal(torch.cat([z_early, z]), zs)
+    for a, b in zip(got, want):
+        assert torch.equal(a.nan_to_num(), b.nan_to_num())
+    ctx.close()

@@ -436,7 +436,7 @@ fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* 
  * fb_set_split).  Returns FB_ERR_INVALID_ARG for a negative limit. */
 fb_status fb_set_pair_limit(fb_ctx* ctx, int32_t pairs);
 /* k-range split of the router kernel (on by default).  When a call has so few 256-row tile pairs that
- * 2, 4 or 8 block pairs per tile pair fit on the GPU at once, that many pairs share a tile: each sums a
+ * 2 to 8 block pairs per tile pair fit on the GPU at once, that many pairs share a tile: each sums a
  * piece of the k-range, the partial sums meet through the shared memory of the cluster and each block
  * selects for its share of the rows.  The schedule is a
  * function of the shape and of the number of pairs only: a call is reproducible, but its logits

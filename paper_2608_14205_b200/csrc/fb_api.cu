@@ -52,8 +52,8 @@ struct fb_ctx {
   int rows_kernel = 0;
   int rows_stages[2] = {0, 0};
   size_t rows_smem[2] = {0, 0};
-  // clusters of 2 J blocks that fit on the GPU at once, by log2 J (J block pairs share a tile pair)
-  int max_clusters[4] = {0, 0, 0, 0};
+  // [j]: clusters of 2 j blocks that fit on the GPU at once (j block pairs share a tile pair)
+  int max_clusters[fb::kMaxPieces + 1] = {};
   int max_tiles = 0;
   int pair_limit = 0;             // the caller's limit on the block pairs to use (0 = none)
   int stage_limit = 0;            // diagnostic: pipeline stages at most (0 = as many as fit)
@@ -309,15 +309,21 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   const int tiles = (T + fb::kTileM - 1) / fb::kTileM;
   p.tiles_first = (tiles + 1) / 2 * 2;                            // a pair never straddles the two passes
   const int tile_pairs = (mode == fb::kModeLayer ? 2 : 1) * (p.tiles_first / 2);
-  const int pairs_avail = ctx->pair_limit > 0 && ctx->pair_limit < ctx->max_clusters[0] && probe == 0
-                              ? ctx->pair_limit : ctx->max_clusters[0];
+  const int pairs_avail = ctx->pair_limit > 0 && ctx->pair_limit < ctx->max_clusters[1] && probe == 0
+                              ? ctx->pair_limit : ctx->max_clusters[1];
   // Few tile pairs: as many block pairs per tile pair as fit at once (all clusters of the launch
-  // are resident together) and have at least two k-blocks each.
-  int log_j = 0;
+  // are resident together) and have at least two k-blocks each.  Numbers that are not powers of two only
+  // where they shorten a pair's piece by three k-blocks or more: prediction and plan of 4300 x 7168 with 256 experts
+  // takes 37.7 us with two pairs and 31.9 with three, of 2048 x 4096 with 8 experts 12.41 with four (16 k-blocks
+  // each) and 12.03 with five (13); but a layer call of 900 x 2048 with 128 experts 19.85 with four (8 k-blocks
+  // each) and 20.02 with five (7).
+  int J = 1, power = 1;
   if (ctx->split_mode != 0 && probe == 0)
-    for (int l = 1; l <= 3; ++l)
-      if (tile_pairs <= ctx->max_clusters[l] && tile_pairs << l <= pairs_avail && p.num_kb >= 2 << l) log_j = l;
-  const int J = 1 << log_j;
+    for (int j = 2; j <= fb::kMaxPieces; ++j) {
+      if (tile_pairs > ctx->max_clusters[j] || tile_pairs * j > pairs_avail || p.num_kb < 2 * j) continue;
+      if ((j & (j - 1)) == 0) J = power = j;
+      else if ((p.num_kb + power - 1) / power - (p.num_kb + j - 1) / j >= 3) J = j;
+    }
   p.pieces = J;
   if (pieces_out) *pieces_out = J;
   // Which kernel: whole tiles of a gate that the ranking selection handles go there (one tile per pair,
@@ -412,8 +418,8 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   dp.num_tiles = (T + fb::kDispatchTile - 1) / fb::kDispatchTile;
   dp.topk_ids = topk_ids;
   dp.slices_per_tile = slices_per_tile;
-  const int slice_rows = fb::kDispatchTile / slices_per_tile;
-  dp.num_slices = (T + slice_rows - 1) / slice_rows;
+  const int rows = fb::slice_rows(slices_per_tile);
+  dp.num_slices = T / fb::kDispatchTile * slices_per_tile + (T % fb::kDispatchTile + rows - 1) / rows;
   dp.slice_counts = ctx->slice_counts;
   dp.early_counts = ctx->early_counts;
   dp.counts_out = counts_out;
@@ -548,7 +554,7 @@ static fb_status ensure_kernel_attributes(int device, const cudaDeviceProp& prop
   return FB_OK;
 }
 
-// How many clusters of 2, 4, 8 and 16 blocks the GPU holds at once.  Counted for the row-per-warp kernel
+// How many clusters of 2, 4, .. 16 blocks the GPU holds at once.  Counted for the row-per-warp kernel
 // at the largest shared memory of this shape's launches (one block per SM either way).
 static fb_status count_clusters(fb_ctx* ctx) {
   cudaLaunchConfig_t occ;
@@ -559,17 +565,17 @@ static fb_status count_clusters(fb_ctx* ctx) {
   cl[0].id = cudaLaunchAttributeClusterDimension;
   occ.attrs = cl;
   occ.numAttrs = 1;
-  for (int l = 0; l < 4; ++l) {
-    cl[0].val.clusterDim.x = 2u << l; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
-    occ.gridDim = dim3((2u << l) * static_cast<unsigned>(ctx->n_sm), 1, 1);
+  for (int j = 1; j <= fb::kMaxPieces; ++j) {
+    cl[0].val.clusterDim.x = 2u * j; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
+    occ.gridDim = dim3(2u * j * static_cast<unsigned>(ctx->n_sm), 1, 1);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, rows_kernel_fn(ctx->rows_kernel, ctx->cfg.gate == FB_GATE_SIGMOID_GROUP_TOPK),
                                        &occ) != cudaSuccess)
       n = 0;
-    ctx->max_clusters[l] = n;
+    ctx->max_clusters[j] = n;
   }
   cudaGetLastError();
-  return ctx->max_clusters[0] >= 1 ? FB_OK : FB_ERR_CUDA;
+  return ctx->max_clusters[1] >= 1 ? FB_OK : FB_ERR_CUDA;
 }
 
 // Rows of the histogram table: a launch that cuts its tiles into slices has at most one slice per SM
@@ -1112,7 +1118,7 @@ fb_status fb_router_floor(fb_ctx* ctx, const fb_router* router, const void* x, i
                        static_cast<cudaStream_t>(stream_), nullptr, what);
 }
 
-int32_t fb_max_pairs(const fb_ctx* ctx) { return ctx && ctx->ranking[0] ? ctx->max_clusters[0] : 0; }
+int32_t fb_max_pairs(const fb_ctx* ctx) { return ctx && ctx->ranking[0] ? ctx->max_clusters[1] : 0; }
 
 fb_status fb_dispatch_slot_counts(fb_ctx* ctx, const uint32_t* slot_offsets, uint32_t* slot_counts, fb_stream stream_) {
   if (!ctx || !slot_offsets || !slot_counts) return FB_ERR_INVALID_ARG;

@@ -4,7 +4,7 @@
 // position - so the result is unique and reproducible.
 //
 // Input: the router kernel's top-k ids and its per-slice expert histogram
-// slice_counts[slice][e] (slice = 128 / slices_per_tile consecutive tokens, one byte per expert: a
+// slice_counts[slice][e] (slices_per_tile slices of slice_rows tokens per tile, one byte per expert: a
 // token names an expert at most once, so a count is at most 128).  One block per 128-token tile,
 // or per run of consecutive tiles when there are more tiles than blocks.
 //
@@ -29,6 +29,9 @@ namespace fb {
 constexpr int kDispatchThreads = 1024;
 constexpr int kDispatchTile = 128;       // must equal the router kernel's tile height
 constexpr int kDispatchWarps = kDispatchThreads / 32;
+// Rows of a tile that one of `pieces` blocks finishes: even (rows are selected two at a time), the last block has
+// the rest.
+__host__ __device__ constexpr int slice_rows(int pieces) { return (kDispatchTile + 2 * pieces - 1) / (2 * pieces) * 2; }
 constexpr int kDispatchBatch = 4;        // tiles a block works on at a time
 static_assert(kDispatchTile * FB_MAX_TOPK == kDispatchThreads, "one thread per assignment of a tile");
 // Bytes of one row of the histogram table: 16-byte units, so that a thread reads 16 experts at once.

@@ -74,6 +74,7 @@ constexpr int kEpilogueWarps = kEpilogueThreads / 32;
 constexpr int kRouterThreads = 64 + kEpilogueThreads + 32;
 constexpr int kSecondIssuerWarp = kRouterThreads / 32 - 1;
 constexpr int kATileBytes = kTileM * kBlockK * 2;
+constexpr int kMaxPieces = 8;                // block pairs that share a tile pair: clusters of 16 blocks
 constexpr uint32_t kAccumBarrierId = 2;      // named barrier: accumulator finished (MMA warp -> epilogue warps)
 constexpr uint32_t kRowBarrierBase = 3;      // named barriers 3..6: the kEpiSubs warps that share one quarter of the rows
 

@@ -3,9 +3,9 @@
 //
 // Work split.  Two blocks of a cluster (a pair) compute a tile pair: 256 token rows x all N = pad16(E)
 // expert columns with one cta_group::2 MMA; each loads its own 128 rows of x and half of the W tile.
-//   * Few tile pairs: a cluster of 2 J blocks (J = 2, 4, 8 pairs) works on ONE tile pair.  Pair j
+//   * Few tile pairs: a cluster of 2 J blocks (J = 2 .. 8 pairs) works on ONE tile pair.  Pair j
 //     accumulates the j-th piece of the k-range; the J partial tiles meet through distributed shared
-//     memory, and each block finishes 128 / J of its rows.  Both the stream of operands and the
+//     memory, and each block finishes about 128 / J of its rows.  Both the stream of operands and the
 //     selection work are then spread over J times as many SMs, and nothing but a cluster barrier lies
 //     between the two.
 //   * More tile pairs than pairs fit on the GPU: every pair walks a strided list of tile pairs, and
@@ -705,9 +705,10 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
           if (et < J) mbar_arrive_cluster(smem_u32(&sh.staged_bar), cta_rank + 2u * static_cast<uint32_t>(et));
           const bool staged = mbar_wait<true>(smem_u32(&sh.staged_bar), 0u, abort_flag);
           got = got && __all_sync(0xffffffffu, staged);
-          const int slice = kTileM / J, per = max(2, slice / kEpilogueWarps);
+          const int slice = slice_rows(J), mine = min(slice, kTileM - piece * slice);
+          const int per = (slice + 2 * kEpilogueWarps - 1) / (2 * kEpilogueWarps) * 2;
           first = piece * slice + ew * per;
-          count = ew * per < slice ? per : 0;
+          count = max(0, min(per, mine - ew * per));
         } else if (chunk_rows == kTileM) {
           // the four warps that share a quarter of the rows meet at their own barrier
           if (last_tile) {                                     // done with tensor memory and the partner
@@ -747,7 +748,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
         // measurement launch: nothing is published
       } else if (mode == kModeDispatch || p.defer_counts) {
         const int slice = tile * J + piece;
-        if (static_cast<long long>(slice) * (kTileM / J) < p.T)  // a slice beyond the last token owns no row
+        if (static_cast<long long>(tile) * kTileM + piece * slice_rows(J) < p.T)  // (one beyond the last token owns no row)
           write_slice_counts(mode == kModeDispatch ? p.slice_counts : p.early_counts, slice, E, sh.hist, et);
         if (several_tiles) {
           named_bar_sync(kPlanBarrierId, kEpilogueThreads);

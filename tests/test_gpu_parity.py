@@ -774,6 +774,38 @@ def test_row_selection_breaks_ties_and_survives_overfull_lists(T):
         ctx.close()
 
 
+@pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
+def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
+    # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles
+    dev = torch.device("cuda")
+    for kw in (dict(E=100, k=5, R=4, gate=0, n_group=1, topk_group=1), dict(E=256, k=8, R=8, gate=1, n_group=8, topk_group=4)):
+        E, k, R, d = kw["E"], kw["k"], kw["R"], 7168
+        for T in (1, 43, 45, 128, 151, 256, 300, 900):
+            g = torch.Generator().manual_seed(T + pieces)
+            x, W = (torch.randint(-2, 3, s, generator=g).to(torch.bfloat16).to(dev) for s in ((T, d), (E, d)))
+            sb = (torch.randint(0, 4, (E,), generator=g) / 8.0).to(dev) if kw["gate"] else None
+            router = B.make_router(W, None, sb)
+            ctx = B.Context(T, d, E, k, R, kw["gate"], kw["n_group"], kw["topk_group"], 1, 1.0)
+            pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+            tile_pairs = (T + 255) // 256
+            results = []
+            for split in (1, 0):
+                ctx.fb_set_split(split)
+                ctx.fb_set_pair_limit(tile_pairs * pieces)
+                i32 = lambda n: torch.full((n,), -7, dtype=torch.int32, device=dev)
+                counts, early, ids, perm, inv = i32(E), i32(T * k), i32(T * k), i32(T * k), i32(T * k)
+                so, ro, rl, w = i32(E + 1), i32(R + 1), i32(R), torch.full((T * k,), -7.0, device=dev)
+                z = torch.full((T * E,), -7.0, device=dev)
+                ctx.fb_predict_load(router, x, T, counts, early, z)
+                ctx.fb_route_dispatch(router, x, T, pi, ids, w, so, ro, perm, inv, rl)
+                assert ctx.fb_device_status() == 0
+                results.append((counts, early, ids, perm, inv, so, ro, rl, z, w))
+            for a, b in zip(results[0][:-1], results[1][:-1]):
+                assert torch.equal(a, b), (kw, T)
+            assert torch.allclose(results[0][-1], results[1][-1], rtol=0, atol=1e-6)    # weights <= 1: a few ulp
+            ctx.close()
+
+
 def test_contexts_of_different_shapes_alive_together():
     # Kernel attributes (the dynamic shared-memory ceiling) belong to the kernel, not to a context:
     # a large-shape context must keep working after a small-shape one was created, and the

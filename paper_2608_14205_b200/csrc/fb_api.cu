@@ -748,8 +748,8 @@ fb_status fb_route_dispatch(fb_ctx* ctx, const fb_router* router, const void* x,
   const fb_status st = launch_router(ctx, router, x, T, fb::kModeDispatch, nullptr, topk_ids, topk_w, logits,
                                      nullptr, stream, nullptr, 0, &pieces);
   if (st != FB_OK) return st;
-  return launch_dispatch_index(ctx, T, pieces, nullptr, nullptr, expert_to_slot, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
-                               rank_load, stream);
+  return launch_dispatch_index(ctx, T, pieces, nullptr, nullptr, expert_to_slot, topk_ids, slot_offsets, rank_offsets,
+                               perm, inv_perm, rank_load, stream);
 }
 
 fb_status fb_layer_step_observed(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
@@ -785,8 +785,9 @@ fb_status fb_layer_step_observed(fb_ctx* ctx, const fb_router* router, const voi
   st = launch_router(ctx, router, h_prev, T, fb::kModeLayer, counts, topk_ids, topk_w, logits, &pp, stream, H, 0, &pieces,
                      &deferred, ids_early, logits_early);
   if (st != FB_OK) return st;
-  return launch_dispatch_index(ctx, T, pieces, deferred ? &pp : nullptr, counts, deferred ? expert_to_slot : expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm, inv_perm,
-                               rank_load, stream);
+  return launch_dispatch_index(ctx, T, pieces, deferred ? &pp : nullptr, counts,
+                               deferred ? expert_to_slot : expert_to_slot_out, topk_ids, slot_offsets, rank_offsets, perm,
+                               inv_perm, rank_load, stream);
 }
 
 fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,

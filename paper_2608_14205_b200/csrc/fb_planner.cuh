@@ -495,8 +495,8 @@ __device__ __noinline__ void plan_loop_general(const PlanParams& p, PlanShared& 
 }
 
 // The planner, run by ONE warp (all 32 lanes) once plan_load_placement has filled the
-// placement arrays and plan_put_count has turned the count vector into counts per slot.  A single warp keeps the rank loads in registers (lane r holds ranks r and
-// r + 32) and needs no block barrier.  Writes the swaps, their number and the rank loads
+// placement arrays and plan_put_count has turned the count vector into counts per slot.  A single
+// warp keeps the rank loads in registers (lane r holds ranks r and r + 32) and needs no block barrier.  Writes the swaps, their number and the rank loads
 // before and after; the new placement is written afterwards by plan_write_placement.
 // kGeneral: the instance carries the general loop as well.  The router kernels' fused tail uses
 // the instance without it (the host launches the stand-alone planner kernel behind the router

@@ -35,6 +35,15 @@ fb_status fb_time_next_router_launch(fb_ctx* ctx, void* event_before, void* even
  * serves the same issuer). */
 fb_status fb_set_stage_limit(fb_ctx* ctx, int32_t stages);
 
+/* Where a row's logits lie in shared memory between the router GEMM and the row-per-warp
+ * selection, for a gate: *row_words receives the words from one row to the next, stored_at[c]
+ * the word of the row that column c is stored at (c below E rounded up to 16; -1 beyond),
+ * read_at[c] the word that the lane which holds expert c reads it from (-1 where no lane
+ * does: c >= E).  Both arrays: host i32 [FB_MAX_EXPERTS].  Host arithmetic only, no device;
+ * the kernels and this call share it.  Errors as fb_create; a NULL pointer:
+ * FB_ERR_INVALID_ARG. */
+fb_status fb_staged_row_layout(const fb_config* cfg, int32_t* row_words, int32_t* stored_at, int32_t* read_at);
+
 /* Floor of the one-tile router kernel's main loop.  Launches that kernel for x exactly as
  * fb_predict_load would (same grid, block pairs, pipeline stages and tensor maps; never the
  * persistent kernel, never the k-range split), but with what = 1 the operands are only loaded

@@ -60,7 +60,7 @@ EXPORTS = ["fb_create", "fb_destroy", "fb_budget_ns", "fb_swap_cost_ns", "fb_pre
            "fb_set_stamp_buffer", "fb_clock_probe", "fb_attention_begin", "fb_attention_end", "fb_layer_budget_ns",
            "fb_attention_set_time_ns", "fb_attention_reset", "fb_dispatch_slot_counts", "fb_dispatch_globalize",
            "fb_standin_attention", "fb_set_split", "fb_prediction_quality",
-           "fb_layer_step_observed"]
+           "fb_layer_step_observed", "fb_staged_row_layout"]
 
 _lib = None
 
@@ -107,6 +107,8 @@ def lib() -> ctypes.CDLL:
                                          vp, vp, vp, vp]
     L.fb_predict_load_static.restype = ctypes.c_int
     L.fb_device_status.argtypes = [vp, ctypes.POINTER(i32), vp]
+    L.fb_staged_row_layout.argtypes = [ctypes.POINTER(FbConfig)] + [vp] * 3
+    L.fb_staged_row_layout.restype = ctypes.c_int
     L.fb_set_stage_limit.argtypes = [vp, i32]
     L.fb_set_stage_limit.restype = ctypes.c_int
     L.fb_set_pair_limit.argtypes = [vp, i32]

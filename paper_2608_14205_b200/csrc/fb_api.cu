@@ -1090,6 +1090,27 @@ fb_status fb_set_split(fb_ctx* ctx, int32_t mode, int32_t owner_bias_kblocks) {
   return FB_OK;
 }
 
+fb_status fb_staged_row_layout(const fb_config* cfg, int32_t* row_words, int32_t* stored_at, int32_t* read_at) {
+  if (!cfg || !row_words || !stored_at || !read_at) return FB_ERR_INVALID_ARG;
+  const fb_status cs = check_config(*cfg);
+  if (cs != FB_OK) return cs;
+  fb::RouterParams g;
+  memset(&g, 0, sizeof(g));
+  g.E = cfg->E;
+  g.N = (cfg->E + 15) / 16 * 16;
+  fb::gate_layout(cfg->E, cfg->gate, cfg->n_group, cfg->topk_group, &g);
+  *row_words = fb::staging_stride(g.N);
+  for (int c = 0; c < FB_MAX_EXPERTS; ++c) {
+    stored_at[c] = c < g.N ? fb::quad_word(g, c / 4) + c % 4 : -1;
+    read_at[c] = -1;
+  }
+  for (int lane = 0; lane < 32; ++lane) {
+    const fb::LaneColumns lc = fb::lane_columns(g, lane);
+    for (int j = 0; j < lc.n; ++j) read_at[lc.c0 + j] = lc.word + (g.two_vectors ? j / 4 * 128 + j % 4 : j);
+  }
+  return FB_OK;
+}
+
 fb_status fb_set_stage_limit(fb_ctx* ctx, int32_t stages) {
   if (!ctx || stages < 0 || stages == 1) return FB_ERR_INVALID_ARG;
   ctx->stage_limit = stages;

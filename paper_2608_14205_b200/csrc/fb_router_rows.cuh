@@ -46,7 +46,7 @@ inline int gate_layout(int E, int gate, int n_group, int topk_group, RouterParam
   // one group, or groups that start on a vector: round the lane's share up so that it is whole vectors
   p->vector_load = (groups == 1 || gs % (cpl < 4 ? cpl : 4) == 0) ? 1 : 0;
   p->cols_per_lane = p->vector_load ? cpl : per_lane;
-  p->two_vectors = (cpl == 8 && p->vector_load) ? 1 : 0;
+  p->two_vectors = (cpl == 8 && p->vector_load && E > 128) ? 1 : 0;      // (only rows above 128 columns are padded to 256 words)
   p->ragged = groups * lpg * cpl != E || groups * lpg != 32 ? 1 : 0;
   return cpl;
 }
@@ -71,6 +71,29 @@ __host__ __device__ constexpr size_t staging_bytes(int rows, int N) {
   return static_cast<size_t>(rows) * staging_stride(N) * 4 + kEpilogueWarps * sizeof(RowScratch);
 }
 
+// What a lane needs to know about its columns.
+struct LaneColumns {
+  int32_t c0, n;                       // first column, number of columns
+  int32_t word;                        // where they start in a staged row
+  int32_t group;                       // group of its columns (>= groups: an idle lane)
+};
+__host__ __device__ inline LaneColumns lane_columns(const RouterParams& p, int lane) {
+  LaneColumns lc;
+  lc.group = lane / p.lanes_per_group;
+  const int first = lane % p.lanes_per_group * p.cols_per_lane, left = p.group_size - first;
+  lc.n = lc.group >= p.groups || left <= 0 ? 0 : (left < p.cols_per_lane ? left : p.cols_per_lane);
+  lc.c0 = lc.n == 0 ? 0 : lc.group * p.group_size + first;
+  lc.word = p.two_vectors ? 4 * lane : lc.c0;
+  return lc;
+}
+// Where columns 4 q .. 4 q + 3 lie in a staged row.  (A quad lies in one group and one lane where rows are stored
+// as two vectors per lane; groups start on a quad there; padding columns go behind the lanes' words.)
+__host__ __device__ inline int quad_word(const RouterParams& p, int q) {
+  if (!p.two_vectors) return 4 * q;
+  const int in = 4 * q % p.group_size, of_lane = 4 * q / p.group_size * p.lanes_per_group + in / 8;
+  return 4 * q < p.E ? in / 4 % 2 * 128 + of_lane * 4 : 256;
+}
+
 struct RowsShared {
   uint64_t full_bar[kMaxStages];
   uint64_t empty_bar[kMaxStages];
@@ -92,13 +115,6 @@ struct RowsShared {
 };
 
 // ---------------------------------------------------------------- selection, one warp per token row
-// What a lane needs to know about its columns.
-struct LaneColumns {
-  int32_t c0, n;                       // first column, number of columns
-  int32_t word;                        // where they start in a staged row
-  int32_t group;                       // group of its columns (>= groups: an idle lane)
-};
-
 // Plain selection of one row by repeated maximum over keys in shared memory (dropped columns hold
 // -inf): the path of rows with more candidates than the list holds, and of rows with equal keys among
 // the candidates (the lower expert id wins).  Rare; kept out of line.
@@ -614,27 +630,14 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
     const uint32_t row_stride = static_cast<uint32_t>(staging_stride(N)) * 4u;
     const bool two_acc = p.issuers == 2 && n_kb > 1;
 
-    LaneColumns lc;
-    {
-      lc.group = lane / p.lanes_per_group;
-      const int first = (lane % p.lanes_per_group) * p.cols_per_lane;
-      lc.c0 = lc.group < p.groups ? lc.group * p.group_size + first : 0;
-      lc.n = lc.group < p.groups ? max(0, min(p.cols_per_lane, p.group_size - first)) : 0;
-      if (lc.n == 0) lc.c0 = 0;
-      lc.word = p.two_vectors ? 4 * lane : lc.c0;
-    }
+    const LaneColumns lc = lane_columns(p, lane);
     // While the main loop runs, stage the biases and the placement for the planner (any block may
     // turn out to be the last one).
     for (int e = et; e < FB_MAX_EXPERTS; e += kEpilogueThreads) {
       sh.logit_bias[e] = (p.logit_bias != nullptr && e < E) ? p.logit_bias[e] : 0.0f;
       sh.select_bias[e] = (p.select_bias != nullptr && e < E) ? p.select_bias[e] : 0.0f;
     }
-    for (int q = et; q < FB_MAX_EXPERTS / 4; q += kEpilogueThreads) {
-      // (a quad lies in one group and one lane where rows are stored as two vectors per lane; groups start on
-      // a quad there; padding columns go behind the lanes' words)
-      const int in = 4 * q % p.group_size, of_lane = 4 * q / p.group_size * p.lanes_per_group + in / 8;
-      sh.quad_word[q] = static_cast<uint16_t>(!p.two_vectors ? 4 * q : 4 * q < E ? in / 4 % 2 * 128 + of_lane * 4 : 256);
-    }
+    for (int q = et; q < FB_MAX_EXPERTS / 4; q += kEpilogueThreads) sh.quad_word[q] = static_cast<uint16_t>(quad_word(p, q));
     float sb[kCpl];
 #pragma unroll
     for (int j = 0; j < kCpl; ++j)

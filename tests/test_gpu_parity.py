@@ -752,6 +752,21 @@ def test_row_selection_over_gates_and_shared_tiles(kw, T, limit):
     _run(_wl(d=1024, **kw), T, layer=1, with_logit_bias=T in (17, 1300), want_logits=limit == 0, pair_limit=limit)
 
 
+@pytest.mark.parametrize("kw", [
+    # eight columns per lane in rows of at most 128 columns (groups of 20, 24, 36, 12, 40 over 4, 4, 8, 2, 8 lanes)
+    dict(n_group=5, topk_group=3, k=7, E=100, R=5), dict(n_group=5, topk_group=2, k=8, E=120, R=5),
+    dict(n_group=6, topk_group=3, k=6, E=120, R=8), dict(n_group=3, topk_group=1, k=8, E=108, R=6),
+    dict(n_group=9, topk_group=4, k=8, E=108, R=9), dict(n_group=10, topk_group=2, k=3, E=120, R=8),
+    dict(n_group=3, topk_group=2, k=5, E=120, R=8),
+    # groups that are no whole vectors, word by word: 22 columns over 2 lanes, 19 over 4, 3 over 2, 5 over 2
+    dict(n_group=9, topk_group=3, k=8, E=198, R=9), dict(n_group=6, topk_group=4, k=8, E=114, R=6),
+    dict(n_group=16, topk_group=5, k=8, E=48, R=8), dict(n_group=16, topk_group=2, k=6, E=80, R=8),
+])
+@pytest.mark.parametrize("T,limit", [(129, 0), (700, 1)])        # tiles shared by eight pairs; three tile pairs on one pair
+def test_row_selection_of_restricted_gates_at_every_lane_layout(kw, T, limit):
+    _run(_wl(d=1024, gate=1, route_scale=2.5, **kw), T, layer=1, with_logit_bias=limit == 0, want_logits=limit == 0, pair_limit=limit)
+
+
 @pytest.mark.parametrize("T", [100, 1300])
 def test_row_selection_breaks_ties_and_survives_overfull_lists(T):
     # half of the rows have equal keys everywhere (more candidates than a row's list holds), in the others

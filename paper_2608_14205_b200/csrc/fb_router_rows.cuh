@@ -436,7 +436,10 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
   const int h = lane >> 4, c = lane & 15;
   const int most = min(max(n[0], n[1]), kCandCap);
   const float* list = rs.cand_key[h];
-  uint32_t used = 0;                                         // ranks below k that were found, one bit each
+  // Ranks below k that were found: the sum of 2^rank per row in 13 bits each (at most 32 of at most 2^7), and how
+  // many of both rows together above them.
+  uint32_t found = 0;
+  const uint32_t one = 1u << (13 * h), count_one = 1u << 26;
   const float my0 = list[c];
   int r0 = 0;
   if (most <= 16) {
@@ -457,22 +460,24 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
     if (my1 > -INFINITY && r1 < p.k) {
       rs.win_key[2 * pair + h][r1] = my1;
       rs.win_id[2 * pair + h][r1] = rs.cand_id[h][c + 16];
-      used |= 1u << (8 * h + r1);
+      found += (one << r1) + count_one;
     }
   }
   if (my0 > -INFINITY && r0 < p.k) {
     rs.win_key[2 * pair + h][r0] = my0;
     rs.win_id[2 * pair + h][r0] = rs.cand_id[h][c];
-    used |= 1u << (8 * h + r0);
+    found += (one << r0) + count_one;
   }
-  // A rank that nobody found means equal keys among the best (or too few candidates): such rows, and
-  // rows whose list overflowed, take the plain path.
-  used = __reduce_or_sync(full, used);
+  // Anything but every rank found once means equal keys among the best (or too few candidates): such rows, and rows
+  // whose list overflowed, take the plain path.  Equal keys share a rank: within the best k they leave a later one
+  // out and lower the sum of 2^rank, at the end of the list they raise the number found - two sums of 2^k - 1 and
+  // 2 k in all mean no ties (a test for missing ranks alone would leave it to the order of conflicting stores which
+  // of two equal keys at the last rank wins).
+  found = __reduce_add_sync(full, found);
   const uint32_t want = (1u << p.k) - 1u;
-  if (used != (want | want << 8) || n[0] > kCandCap || n[1] > kCandCap) {
+  if (found != (want | want << 13) + 2u * static_cast<uint32_t>(p.k) * count_one || n[0] > kCandCap || n[1] > kCandCap) {
 #pragma unroll 1
     for (int u = 0; u < 2; ++u) {
-      if (((used >> (8 * u)) & 0xffu) == want && (u == 0 ? n[0] : n[1]) <= kCandCap) continue;
       // scratch: the row's staged words in this block, which nobody else reads (of a shared tile, a block
       // reads the other blocks' copies of its own slice only)
       float* keys = reinterpret_cast<float*>(__cvta_shared_to_generic(row_addr + u * stride));

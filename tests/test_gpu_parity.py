@@ -789,6 +789,44 @@ def test_row_selection_breaks_ties_and_survives_overfull_lists(T):
         ctx.close()
 
 
+@pytest.mark.parametrize("E,kw", [
+    (256, dict(gate=0, n_group=1, topk_group=1)), (200, dict(gate=0, n_group=1, topk_group=1)),      # eight columns per lane
+    (256, dict(gate=1, n_group=8, topk_group=4)), (250, dict(gate=1, n_group=5, topk_group=2)),      # bound from the groups; sixteen
+])
+@pytest.mark.parametrize("distance", [1, 3, 9, 40])
+def test_ties_at_the_last_rank_go_to_the_lowest_ids(E, kw, distance):
+    # small integers: exact logits.  Experts come in runs of copies `distance` apart, so that for some k the k-th
+    # and the (k + 1)-th key are equal, in the same lane, in neighbouring ones and far apart
+    dev = torch.device("cuda")
+    T, d = 300, 512                                              # two tile pairs shared by several SM pairs: a warp per row
+    g = torch.Generator().manual_seed(E + distance)
+    x, W = (torch.randint(-3, 4, s, generator=g).float() for s in ((T, d), (E, d)))
+    e = torch.arange(E)
+    for copies in (2, 3, 5):
+        Wc = W[e - (e // distance) % copies * distance]
+        z = (x.double() @ Wc.double().T).numpy()
+        key = z if kw["gate"] == 0 else None
+        router = B.make_router(Wc.to(torch.bfloat16).to(dev), None, None)
+        for k in range(1, 9):
+            ctx = B.Context(T, d, E, k, 2, kw["gate"], kw["n_group"], kw["topk_group"], 1, 1.0)
+            counts, ids = torch.zeros(E, dtype=torch.int32, device=dev), torch.zeros(T * k, dtype=torch.int32, device=dev)
+            ctx.fb_predict_load(router, x.to(torch.bfloat16).to(dev), T, counts, ids)
+            assert ctx.fb_device_status() == 0
+            got = ids.cpu().numpy().reshape(T, k)
+            if key is not None:
+                assert np.array_equal(got, np.argsort(-key, axis=1, kind="stable")[:, :k]), (copies, k)
+            else:
+                # an expert is chosen only if every copy of it with a lower id (in the same group) is
+                gs = E // kw["n_group"]
+                for t in range(T):
+                    chosen = set(got[t].tolist())
+                    assert len(chosen) == k
+                    for c in chosen:
+                        for lower in range(c - distance, c - distance * ((c // distance) % copies) - 1, -distance):
+                            assert lower in chosen or lower // gs != c // gs, (copies, k, t)
+            ctx.close()
+
+
 @pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
 def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
     # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles

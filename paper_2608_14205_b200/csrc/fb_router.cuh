@@ -342,7 +342,8 @@ __device__ __forceinline__ bool rank_candidates(const unsigned long long* cand, 
   return overflow;
 }
 
-// The row's top-k list as rank_candidates left it.
+// The row's top-k list as rank_candidates left it; ranks that no candidate took hold whatever was there before
+// (see fill_missing_ranks).
 __device__ __forceinline__ void read_ranked(TopK& top, int k, const uint32_t* out_hi, const uint32_t* out_lo,
                                             int row_in_tile) {
 #pragma unroll
@@ -352,6 +353,31 @@ __device__ __forceinline__ void read_ranked(TopK& top, int k, const uint32_t* ou
       top.i[j] = static_cast<int32_t>(~out_lo[j * kTileM + row_in_tile]);
     }
   }
+}
+
+// The row's first `have` ranks are known.  Where that is fewer than k - the other keys are -inf or no numbers - the
+// others get the lowest expert ids the row has not named yet: every id is below E, and as no row names an expert
+// twice a tile's histogram bin stays within its byte (write_slice_counts).
+__device__ __forceinline__ void fill_missing_ranks(TopK& top, uint32_t have, int k) {
+  if (have >= static_cast<uint32_t>(k)) return;
+  uint32_t taken = 0;
+#pragma unroll
+  for (int j = 0; j < FB_MAX_TOPK; ++j)
+    if (j < static_cast<int>(have) && top.i[j] < FB_MAX_TOPK) taken |= 1u << top.i[j];
+#pragma unroll
+  for (int j = 0; j < FB_MAX_TOPK; ++j)
+    if (j >= static_cast<int>(have) && j < k) {
+      top.v[j] = -INFINITY;
+      top.i[j] = __ffs(~taken) - 1;
+      taken |= 1u << top.i[j];
+    }
+}
+// Ranks that insertion into an empty list has taken (it takes keys above -inf only).
+__device__ __forceinline__ uint32_t ranks_taken(const TopK& top) {
+  uint32_t n = 0;
+#pragma unroll
+  for (int j = 0; j < FB_MAX_TOPK; ++j) n += top.v[j] > -INFINITY ? 1u : 0u;
+  return n;
 }
 
 // Expert ids and routing weights of one token (Eq. 3's top-k with the model's weight rule).
@@ -864,7 +890,8 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         if (sub + kEpiSubs < n_chunks) my_groups[1] = sub + kEpiSubs;
       }
       FB_STAMP(5, 64);
-      // ---------------- collect the keys >= floor (at least k keys qualify: the bound is one of k known keys)
+      // ---------------- collect the keys >= floor (at least k keys qualify: the bound is one of k known keys; fewer
+      // only where keys are no numbers)
 #pragma unroll 1
       for (int gi = 0; gi < 2; ++gi) {
         if (my_groups[gi] < 0) continue;                  // no such group: true for the whole warp at once
@@ -891,16 +918,20 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     row_sync();
     FB_STAMP(7, 64);
     bool overflow = false;
-    if (got) overflow = rank_candidates(cand, sh.cand_count[row_in_tile], sub, row_in_tile, out_hi, out_lo);
+    uint32_t n_cand = 0;
+    if (got) {
+      n_cand = sh.cand_count[row_in_tile];
+      overflow = rank_candidates(cand, n_cand, sub, row_in_tile, out_hi, out_lo);
+    }
     row_sync();
     FB_STAMP(8, 64);
     if (got && sub == 0) {
       TopK top;
       top.init();
       if (!overflow) read_ranked(top, k, out_hi, out_lo, row_in_tile);
-      if (__any_sync(0xffffffffu, overflow)) {
+      if (__any_sync(0xffffffffu, overflow || n_cand < static_cast<uint32_t>(k))) {
         // More than kCandCap keys reached the floor (many equal keys): plain scan of the
-        // kept groups for the rows concerned.
+        // kept groups for the rows concerned.  Or fewer than k did (keys that are no numbers).
         if (overflow && !kSigmoid) {
           top.init();
           for (int e = 0; e < E; ++e) {
@@ -937,6 +968,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
             }
           }
         }
+        fill_missing_ranks(top, overflow ? ranks_taken(top) : n_cand, k);
       }
       FB_STAMP(9, 64);
       if (valid) {

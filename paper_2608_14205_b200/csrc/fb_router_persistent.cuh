@@ -39,7 +39,7 @@ struct PersistShared {
   uint32_t tmem_base;
   int32_t abort_flag;
   int32_t accum_ok;
-  int32_t any_overflow[4];                   // per row quarter
+  int32_t any_unranked[4];                   // per row quarter: some row has too many or too few candidates
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];
@@ -110,7 +110,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
 
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
-    for (int q = 0; q < 4; ++q) sh.any_overflow[q] = 0;
+    for (int q = 0; q < 4; ++q) sh.any_unranked[q] = 0;
     sh.issuer_progress[0] = -1;
     sh.issuer_progress[1] = -1;
     for (int s = 0; s < p.stages; ++s) {
@@ -338,7 +338,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
         kept = (1u << n_chunks) - 1u;
       }
       // ---------------- collect the keys >= floor of this thread's kept chunks (the bound is one of
-      // k known keys of the row, so at least k keys qualify)
+      // k known keys of the row, so at least k keys qualify; fewer only where keys are no numbers)
 #pragma unroll
       for (int ci = 0; ci < 2; ++ci) {
         const int c = sub + kEpiSubs * ci;
@@ -364,8 +364,9 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       row_sync();
 
       // ---------------- rank the candidates (many equal keys can overflow the list: handled below)
-      const bool overflow = rank_candidates(cand, sh.cand_count[row_in_tile], sub, row_in_tile, out_hi, out_lo);
-      if (overflow) sh.any_overflow[quarter] = 1;
+      const uint32_t n_cand = sh.cand_count[row_in_tile];
+      const bool overflow = rank_candidates(cand, n_cand, sub, row_in_tile, out_hi, out_lo);
+      if (overflow || n_cand < static_cast<uint32_t>(k)) sh.any_unranked[quarter] = 1;
       row_sync();
       TopK top;
       top.init();
@@ -373,7 +374,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
         sh.cand_count[row_in_tile] = 0;                      // ready for the next tile
         if (!overflow) read_ranked(top, k, out_hi, out_lo, row_in_tile);
       }
-      if (sh.any_overflow[quarter] != 0) {
+      if (sh.any_unranked[quarter] != 0) {
         // Some of these rows had more than kCandCap keys at or above its floor (many equal
         // keys).  Such rows are selected by plain insertion: every thread scans its own kept
         // chunks in ascending expert order, then the row's first thread merges the lists.
@@ -403,6 +404,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
             if (x > -INFINITY) top.insert_any_order(x, static_cast<int32_t>(static_cast<uint32_t>(w)));
           }
         }
+        if (sub == 0) fill_missing_ranks(top, overflow ? ranks_taken(top) : n_cand, k);   // fewer than k: no numbers
       }
 
       // ---------------- outputs per row
@@ -416,7 +418,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           if (j < k) atomicAdd(&hist[top.i[j]], 1u);
       }
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
-      if (et < 4) sh.any_overflow[et] = 0;                    // everyone has read it
+      if (et < 4) sh.any_unranked[et] = 0;                    // everyone has read it
       if (mode == kModeDispatch) {
         const bool owns = static_cast<long long>(tile) * kTileM < p.T;   // the padding block of an odd pair owns no tile
         if (owns) write_slice_counts(p.slice_counts, tile, E, hist, et);

@@ -115,6 +115,20 @@ struct RowsShared {
 };
 
 // ---------------------------------------------------------------- selection, one warp per token row
+// The ranks that no key took (key still -inf: a row with fewer than k keys above -inf, the others being -inf or no
+// numbers) get the lowest expert ids the row has not named yet, so that a row never names an expert twice.  By one
+// lane; at most 8 ids are taken, so the lowest free one is below 8 and below E.
+__device__ __noinline__ void fill_missing_ranks(const float* win_key, int32_t* win_id, int k) {
+  uint32_t taken = 0;
+  for (int r = 0; r < k; ++r)
+    if (win_key[r] > -INFINITY && win_id[r] < FB_MAX_TOPK) taken |= 1u << win_id[r];
+  for (int r = 0; r < k; ++r)
+    if (!(win_key[r] > -INFINITY)) {
+      win_id[r] = __ffs(~taken) - 1;
+      taken |= 1u << win_id[r];
+    }
+}
+
 // Plain selection of one row by repeated maximum over keys in shared memory (dropped columns hold
 // -inf): the path of rows with more candidates than the list holds, and of rows with equal keys among
 // the candidates (the lower expert id wins).  Rare; kept out of line.
@@ -130,7 +144,7 @@ __device__ __noinline__ void select_slow(float* keys, int E, int k, float* win_k
       const int oa = __shfl_xor_sync(0xffffffffu, at, off);
       if (ob > best || (ob == best && oa < at)) { best = ob; at = oa; }
     }
-    if (at >= E) break;                                     // nothing left (keys that are no numbers): the defaults stay
+    if (at >= E) break;                                     // nothing left (see fill_missing_ranks)
     if (lane == 0) { win_key[r] = best; win_id[r] = at; keys[at] = -INFINITY; }
     __syncwarp();
   }
@@ -496,7 +510,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
 // Expert ids, routing weights (Eq. 3's top-k with the model's weight rule) and histogram of up to 8 rows,
 // four at a time: lane = (row, rank).
 template <bool kSigmoid>
-__device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& sh, const RowScratch& rs, int n_rows,
+__device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& sh, RowScratch& rs, int n_rows,
                                             long long row0, int32_t* out_ids, float* out_w, int lane) {
   const uint32_t full = 0xffffffffu;
   const int rk = lane & 7;
@@ -505,6 +519,10 @@ __device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& s
     const long long row = row0 + i;
     const bool valid = i < n_rows && row < p.T && rk < p.k;
     const float key = rs.win_key[i & 7][rk];
+    if (__any_sync(full, valid && !(key > -INFINITY))) {                    // a row ran out of keys
+      if (valid && rk == 0) fill_missing_ranks(rs.win_key[i & 7], rs.win_id[i & 7], p.k);
+      __syncwarp();
+    }
     const int id = valid ? rs.win_id[i & 7][rk] : 0;
 #ifdef FB_DEBUG
     // what the sanitizer would catch: a chosen expert outside [0, E), a repeated expert
@@ -736,8 +754,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
         FB_STAMP(4, 64);
         const long long row0 = static_cast<long long>(tile) * kTileM + first;
         if (got && count > 0 && row0 < p.T) {
-          // default choice (kept only where keys are not numbers): distinct experts
-          for (int i = lane; i < 8 * FB_MAX_TOPK; i += 32) { rs.win_id[i >> 3][i & 7] = i & 7; rs.win_key[i >> 3][i & 7] = -INFINITY; }
+          for (int i = lane; i < 8 * FB_MAX_TOPK; i += 32) rs.win_key[i >> 3][i & 7] = -INFINITY;   // no rank is taken yet
           __syncwarp();
 #pragma unroll 1
           for (int i = 0; i < count; i += 2)

@@ -827,6 +827,83 @@ def test_ties_at_the_last_rank_go_to_the_lowest_ids(E, kw, distance):
             ctx.close()
 
 
+@pytest.mark.parametrize("kw,d", [
+    (dict(E=128, gate=0, n_group=1, topk_group=1, renorm=1), 256),
+    (dict(E=100, gate=0, n_group=1, topk_group=1, renorm=0), 256), (dict(E=200, gate=1, n_group=10, topk_group=3, renorm=1), 256),
+])
+@pytest.mark.parametrize("split,limit", [(1, 0), (0, 0), (0, 1)])    # shared tiles; one tile per pair; several per pair
+def test_rows_without_numbers_stay_inside_and_leave_the_others_alone(kw, d, split, limit):
+    # a NaN or an infinity in a token's hidden state: its experts are unspecified, but distinct and in range, the
+    # index holds them, and every other token comes out as without it
+    dev = torch.device("cuda")
+    T, k, R, E = 700, 8, 4, kw["E"]
+    g = torch.Generator().manual_seed(E)
+    clean = torch.randn(T, d, generator=g).to(torch.bfloat16)
+    W = torch.randn(E, d, generator=g).to(torch.bfloat16).to(dev)
+    sb = (torch.rand(E, generator=g) - 0.5).to(dev) if kw["gate"] else None
+    router = B.make_router(W, None, sb)
+    odd_rows = torch.arange(3, T, 7)
+    odd = clean.clone()
+    odd[odd_rows, 5] = torch.tensor([float("nan"), float("inf"), float("-inf")]).repeat(len(odd_rows))[:len(odd_rows)].to(torch.bfloat16)
+    odd[130:260] = float("nan")                                      # a whole tile and its neighbours' edges
+    same = torch.ones(T, dtype=torch.bool)
+    same[odd_rows] = False
+    same[130:260] = False
+    pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+    budget = B.make_budget(max_swaps=4, global_ns=O.U64_OFF, rank_ns=O.U64_OFF, link_ns=O.U64_OFF, tau_tokens=0, gamma_num=1,
+                           gamma_den=64, alpha_ns=(1, 1), fs_per_byte=(1, 1), ranks_per_node=0, expert_bytes=16)
+    ids, w = {}, {}
+    for name, x in (("clean", clean), ("odd", odd)):
+        ctx = B.Context(T, d, E, k, R, kw["gate"], kw["n_group"], kw["topk_group"], kw["renorm"], 1.0)
+        ctx.fb_set_split(split)
+        ctx.fb_set_pair_limit(limit)
+        out = P.GuardedOutputs(dev)
+        i32 = out.i32
+        counts, early = i32(E), i32(T * k)
+        ctx.fb_predict_load(router, x.to(dev), T, counts, early)
+        l_counts, pi_out, swaps, n, lb, la = i32(E), i32(E), i32(16), i32(1), i32(R), i32(R)
+        so, ro, rl, perm, inv, got, weights = i32(E + 1), i32(R + 1), i32(R), i32(T * k), i32(T * k), i32(T * k), out.f32(T * k)
+        ctx.fb_layer_step(router, x.to(dev), x.to(dev).clone(), T, pi, budget, 0, l_counts, pi_out, swaps, n, lb, la, got, weights,
+                          so, ro, perm, inv, rl)
+        assert ctx.fb_device_status() == 0
+        out.check()
+        ids[name], w[name] = got.cpu().numpy().reshape(T, k), weights.cpu().view(T, k)
+        assert ids[name].min() >= 0 and ids[name].max() < E
+        assert (np.diff(np.sort(ids[name], axis=1), axis=1) > 0).all()
+        assert counts.cpu().tolist() == O.expert_histogram(early.cpu().numpy().reshape(T, k), E).tolist()
+        assert l_counts.cpu().tolist() == O.expert_histogram(ids[name], E).tolist()      # both passes saw the same rows
+        want = O.dispatch_index(ids[name], pi_out.cpu().tolist(), R)
+        for a, b in zip((so, ro, perm, inv, rl), want):
+            assert a.cpu().tolist() == b.tolist()
+        ctx.close()
+    assert np.array_equal(ids["clean"][same], ids["odd"][same])
+    assert torch.equal(w["clean"][same], w["odd"][same])
+
+
+@pytest.mark.parametrize("E", [24, 100, 128, 256])
+@pytest.mark.parametrize("split,limit", [(1, 0), (0, 0), (0, 1)])
+def test_experts_masked_out_come_last_lowest_id_first(E, split, limit):
+    # a logit bias of -inf leaves three experts: they come first, the masked ones follow in order of their ids
+    dev = torch.device("cuda")
+    T, k, d = 700, 6, 128
+    g = torch.Generator().manual_seed(E)
+    x, W = (torch.randint(-3, 4, s, generator=g).float() for s in ((T, d), (E, d)))
+    bias = torch.full((E,), float("-inf"))
+    bias[[1, E // 2, E - 1]] = 0.0
+    z = (x.double() @ W.double().T + bias.double()).numpy()
+    router = B.make_router(W.to(torch.bfloat16).to(dev), bias.to(dev), None)
+    ctx = B.Context(T, d, E, k, 2)
+    ctx.fb_set_split(split)
+    ctx.fb_set_pair_limit(limit)
+    counts, ids = torch.zeros(E, dtype=torch.int32, device=dev), torch.zeros(T * k, dtype=torch.int32, device=dev)
+    ctx.fb_predict_load(router, x.to(torch.bfloat16).to(dev), T, counts, ids)
+    assert ctx.fb_device_status() == 0
+    got = ids.cpu().numpy().reshape(T, k)
+    assert np.array_equal(got, np.argsort(-z, axis=1, kind="stable")[:, :k])
+    assert counts.cpu().tolist() == O.expert_histogram(got, E).tolist()
+    ctx.close()
+
+
 @pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
 def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
     # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles

@@ -194,6 +194,11 @@ __host__ __device__ inline bool ranking_gate(int E, int k, int gate, int n_group
   return E % 32 == 0 && E / 32 <= kBoundRows && (E / 32) * 2 >= k && !want_sum;
 }
 
+// A group's score from its two best keys.  A sum that is no number counts as -inf: the ranks of the scores are then a
+// permutation for every row, so that each of the best topk_group ranks has exactly one group - the warps that scan one
+// group per row go through their collective steps together whatever the rows hold.
+__device__ __forceinline__ float group_score(float best, float second) { return fmaxf(best + second, -INFINITY); }
+
 struct RouterShared {
   uint64_t full_bar[kMaxStages];
   uint64_t empty_bar[kMaxStages];
@@ -831,7 +836,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
               a1[j] = hi;
             }
           }
-          gscore_s[c * kTileM + row_in_tile] = a1[0] + a2[0];
+          gscore_s[c * kTileM + row_in_tile] = group_score(a1[0], a2[0]);
           glow_s[c * kTileM + row_in_tile] = a2[0];
         } else {
           // the chunk's three best keys (sorted) feed the bound
@@ -951,7 +956,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
               a1 = fmaxf(a1, x);
             }
 #pragma unroll
-            for (int h = 0; h < 8; ++h) if (h == g) sc[h] = a1 + a2;
+            for (int h = 0; h < 8; ++h) if (h == g) sc[h] = group_score(a1, a2);
           }
           top.init();
 #pragma unroll

@@ -305,7 +305,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           }
           glow_s[c * kTileM + row_in_tile] = m2[0];
           if (sigmoid_gate) {
-            gscore_s[c * kTileM + row_in_tile] = m1[0] + m2[0];   // group score (gs == 32)
+            gscore_s[c * kTileM + row_in_tile] = group_score(m1[0], m2[0]);   // gs == 32
           } else {
             gscore_s[c * kTileM + row_in_tile] = m1[0];
             third_s[c * kTileM + row_in_tile] = m3[0];

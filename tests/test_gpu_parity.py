@@ -828,7 +828,7 @@ def test_ties_at_the_last_rank_go_to_the_lowest_ids(E, kw, distance):
 
 
 @pytest.mark.parametrize("kw,d", [
-    (dict(E=128, gate=0, n_group=1, topk_group=1, renorm=1), 256),
+    (dict(E=128, gate=0, n_group=1, topk_group=1, renorm=1), 256), (dict(E=256, gate=1, n_group=8, topk_group=4, renorm=1), 256),
     (dict(E=100, gate=0, n_group=1, topk_group=1, renorm=0), 256), (dict(E=200, gate=1, n_group=10, topk_group=3, renorm=1), 256),
 ])
 @pytest.mark.parametrize("split,limit", [(1, 0), (0, 0), (0, 1)])    # shared tiles; one tile per pair; several per pair

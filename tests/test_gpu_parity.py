@@ -904,6 +904,33 @@ def test_experts_masked_out_come_last_lowest_id_first(E, split, limit):
     ctx.close()
 
 
+@pytest.mark.parametrize("kw", [dict(E=128, gate=0, n_group=1, topk_group=1), dict(E=256, gate=1, n_group=8, topk_group=4)])
+def test_logit_dumps_at_any_word(kw):
+    # one tile per pair, a gate of the ranking kernel: it stores 16 bytes at a time, the dump need not start on 16
+    dev = torch.device("cuda")
+    T, d, k, R, E = 300, 512, 6, 4, kw["E"]
+    g = torch.Generator().manual_seed(E)
+    x, W = (torch.randn(*s, generator=g).to(torch.bfloat16).to(dev) for s in ((T, d), (E, d)))
+    router = B.make_router(W, None, None)
+    ctx = B.Context(T, d, E, k, R, kw["gate"], kw["n_group"], kw["topk_group"], 1, 1.0)
+    ctx.fb_set_split(0)
+    pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+    results = []
+    for offset in (0, 1, 2, 3):
+        i32 = lambda n: torch.full((n,), -7, dtype=torch.int32, device=dev)
+        counts, early, ids, perm, inv, so, ro, rl = i32(E), i32(T * k), i32(T * k), i32(T * k), i32(T * k), i32(E + 1), i32(R + 1), i32(R)
+        w, z, z_early = (torch.full((n + 8,), -7.0, device=dev) for n in (T * k, T * E, T * E))
+        ctx.fb_predict_load(router, x, T, counts, early, z_early[offset:])
+        ctx.fb_route_dispatch(router, x, T, pi, ids, w, so, ro, perm, inv, rl, z[offset:])
+        assert ctx.fb_device_status() == 0
+        for dump in (z, z_early):
+            assert bool((dump[:offset] == -7).all()) and bool((dump[offset + T * E:] == -7).all())
+        results.append((counts, early, ids, perm, inv, z[offset:offset + T * E], z_early[offset:offset + T * E]))
+    for other in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(results[0], other))
+    ctx.close()
+
+
 @pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
 def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
     # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles

@@ -331,10 +331,12 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   // several pairs and all other gates take the row-per-warp selection (figures: fb_router_rows.cuh).
   // Logit dumps: a block of the ranking kernel writes its rows from registers, 16 bytes a store (row-per-warp selection for
   // dumps instead: serving step with 8192 tokens, 128 experts 75.4 us against 71.6), one tile per pair.  A dump that does
-  // not start on 16 bytes goes to the row-per-warp selection, which stores single words.
+  // not start on 16 bytes goes to the row-per-warp selection, which stores single words, and so does one whose caller
+  // limits the pairs: that kernel writes logits while it walks several tiles.
   const bool dump = logits != nullptr || early_logits != nullptr;
+  const bool over_limit = pairs_avail < ctx->max_clusters[1] && tile_pairs > pairs_avail;
   const bool whole_vectors = (reinterpret_cast<uintptr_t>(logits) | reinterpret_cast<uintptr_t>(early_logits)) % 16 == 0;
-  const bool ranking = J == 1 && ctx->ranking[topk_w != nullptr ? 1 : 0] && whole_vectors;
+  const bool ranking = J == 1 && ctx->ranking[topk_w != nullptr ? 1 : 0] && whole_vectors && !(dump && over_limit);
   const bool several = J == 1 && probe == 0 && tile_pairs > pairs_avail && !(ranking && dump);
   // Both passes of the layer at the same time: nothing could hide the planner behind the second pass, so
   // the dispatch-index kernel counts and plans (see fb_dispatch_kernel).  With several tiles per pair the

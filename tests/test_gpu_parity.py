@@ -931,6 +931,40 @@ def test_logit_dumps_at_any_word(kw):
     ctx.close()
 
 
+@pytest.mark.parametrize("kw", [dict(E=128, gate=0, n_group=1, topk_group=1), dict(E=256, gate=1, n_group=8, topk_group=4)])
+def test_pair_limit_holds_for_logit_dumps(kw):
+    # a dump under a limit walks several tiles on the pairs it is given, as a call without one does; the results are those
+    # of the unlimited call (small integers: exact sums), weights to a few ulp (their sum is formed in another order)
+    dev = torch.device("cuda")
+    T, d, k, R, E = 1300, 448, 6, 4, kw["E"]
+    g = torch.Generator().manual_seed(E)
+    x, W = (torch.randint(-2, 3, s, generator=g).to(torch.bfloat16).to(dev) for s in ((T, d), (E, d)))
+    router = B.make_router(W, None, None)
+    ctx = B.Context(T, d, E, k, R, kw["gate"], kw["n_group"], kw["topk_group"], 1, 1.0)
+    pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+    budget = B.make_budget(max_swaps=4, gamma_num=1, gamma_den=64, alpha_ns=(1, 1), fs_per_byte=(1, 1), expert_bytes=16)
+    results = []
+    for limit in (0, 1, 2, 5):
+        ctx.fb_set_pair_limit(limit)
+        i32 = lambda n: torch.full((n,), -7, dtype=torch.int32, device=dev)
+        counts, early, ids, perm, inv, so, ro, rl = i32(E), i32(T * k), i32(T * k), i32(T * k), i32(T * k), i32(E + 1), i32(R + 1), i32(R)
+        l_counts, pi_out, swaps, n, lb, la = i32(E), i32(E), torch.zeros(16, dtype=torch.int32, device=dev), i32(1), i32(R), i32(R)
+        w, z, z_early, zl, zl_early = (torch.full((m,), -7.0, device=dev) for m in (T * k, T * E, T * E, T * E, T * E))
+        before = ctx.fb_persistent_launch_count()
+        ctx.fb_predict_load(router, x, T, counts, early, z_early)
+        ctx.fb_route_dispatch(router, x, T, pi, ids, w, so, ro, perm, inv, rl, z)
+        first = (counts, early, ids.clone(), perm.clone(), inv.clone(), z, z_early)
+        ctx.fb_layer_step_observed(router, x, x.flip(0).contiguous(), T, pi, budget, 0, l_counts, pi_out, swaps, n, lb, la, ids, w,
+                                   so, ro, perm, inv, rl, early, zl_early, zl)
+        assert ctx.fb_device_status() == 0
+        assert ctx.fb_persistent_launch_count() - before == (3 if limit else 0)
+        results.append((*first, l_counts, pi_out, swaps, n, lb, la, ids, so, ro, perm, inv, rl, early, zl_early, zl, w))
+    for other in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(results[0][:-1], other[:-1]))
+        assert torch.allclose(results[0][-1], other[-1], rtol=0, atol=1e-6)
+    ctx.close()
+
+
 @pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
 def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
     # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles

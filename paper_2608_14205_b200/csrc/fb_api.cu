@@ -1040,16 +1040,19 @@ fb_status fb_row_cosine_mean(const void* a, const void* b, int64_t rows, int32_t
   if (rows > 0 && (!a || !b || !row_scratch)) return FB_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   cudaError_t err = cudaSuccess;
-  if (rows > 0) {
-    const int blocks = static_cast<int>((rows + fb::kCosineWarpsPerBlock - 1) / fb::kCosineWarpsPerBlock);
+  // One launch in all practice: a grid holds 2^31 - 1 blocks, more rows than a part's go in several.
+  constexpr int64_t kPart = int64_t{1} << 31;
+  for (int64_t r0 = 0; r0 < rows && err == cudaSuccess; r0 += kPart) {
+    const int64_t part = rows - r0 < kPart ? rows - r0 : kPart;
+    const int blocks = static_cast<int>((part + fb::kCosineWarpsPerBlock - 1) / fb::kCosineWarpsPerBlock);
     if (dtype == FB_DTYPE_BF16)
       err = launch_dependent(fb::fb_row_cosine_kernel<__nv_bfloat16>, blocks, 32 * fb::kCosineWarpsPerBlock, stream,
-                             static_cast<const __nv_bfloat16*>(a), static_cast<const __nv_bfloat16*>(b),
-                             static_cast<long long>(rows), n, row_scratch);
+                             static_cast<const __nv_bfloat16*>(a) + r0 * n, static_cast<const __nv_bfloat16*>(b) + r0 * n,
+                             static_cast<long long>(part), n, row_scratch + r0);
     else
       err = launch_dependent(fb::fb_row_cosine_kernel<float>, blocks, 32 * fb::kCosineWarpsPerBlock, stream,
-                             static_cast<const float*>(a), static_cast<const float*>(b), static_cast<long long>(rows), n,
-                             row_scratch);
+                             static_cast<const float*>(a) + r0 * n, static_cast<const float*>(b) + r0 * n,
+                             static_cast<long long>(part), n, row_scratch + r0);
   }
   if (err == cudaSuccess)
     err = launch_dependent(fb::fb_mean_kernel, 1, fb::kMeanThreads, stream, row_scratch, static_cast<long long>(rows), mean_out);
@@ -1082,7 +1085,7 @@ fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* 
   qp.out = metrics_out;
   cudaError_t err = cudaSuccess;
   if (T > 0)
-    err = launch_dependent(fb::fb_quality_rows_kernel, (T + fb::kCosineWarpsPerBlock - 1) / fb::kCosineWarpsPerBlock,
+    err = launch_dependent(fb::fb_quality_rows_kernel, (T - 1) / fb::kCosineWarpsPerBlock + 1,
                            32 * fb::kCosineWarpsPerBlock, stream, qp);
   if (err == cudaSuccess) err = launch_dependent(fb::fb_quality_sums_kernel, fb::kQualityBlocks, fb::kMeanThreads, stream, qp);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;

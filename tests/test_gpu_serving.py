@@ -107,6 +107,24 @@ def test_bf16_row_cosines_at_the_edges_of_steps_and_of_the_value_range(n):
     assert torch.allclose(rows.cpu(), want, rtol=0.0, atol=4 * n * 2.0 ** -53, equal_nan=True)
 
 
+def test_row_cosines_of_more_rows_than_one_grid_holds():
+    # 2^32 + 6 rows of one element: 8.6 GB of them and 34 GB of row results
+    rows_n = 2 ** 32 + 6
+    if torch.cuda.mem_get_info()[0] < 60 * 2 ** 30:
+        pytest.skip("needs 60 GB of device memory")
+    dev = torch.device("cuda")
+    a = torch.ones(rows_n, 1, dtype=torch.bfloat16, device=dev)
+    b = torch.ones(rows_n, 1, dtype=torch.bfloat16, device=dev)
+    edges = [0, 2 ** 31 - 1, 2 ** 31, 2 ** 32 - 1, 2 ** 32, 2 ** 32 + 5]
+    for i in edges:
+        b[i] = -2.0
+    rows, mean = torch.zeros(rows_n, dtype=torch.float64, device=dev), torch.zeros(1, dtype=torch.float64, device=dev)
+    B.fb_row_cosine_mean(a, b, rows, mean)
+    assert [rows[i].item() for i in edges] == [-1.0] * len(edges)
+    assert [rows[i + 1].item() for i in edges[1:-2]] == [-1.0 if i + 1 in edges else 1.0 for i in edges[1:-2]]
+    assert mean.item() == (rows_n - 2 * len(edges)) / rows_n      # whole numbers below 2^53: exact sums
+
+
 @pytest.mark.parametrize("T,d,E,k", [(1, 8, 5, 1), (37, 72, 100, 8), (1000, 20, 33, 3), (8200, 64, 8, 2)])
 def test_combined_metrics_match_the_separate_calls(T, d, E, k):
     # row sums are formed alike; the means add them in another order: 1e-12 is far above 2^-53 sqrt(T)

@@ -92,6 +92,12 @@ fb_status fb_set_stamp_buffer(fb_ctx* ctx, uint64_t* stamps);
  * for a NULL context or a limit outside the range. */
 fb_status fb_selftest_wait_timeout(fb_ctx* ctx, uint64_t limit_ns, uint64_t* waited_ns, fb_stream stream);
 
+/* The same for a wait that outlasts its limit because the work it waits for goes on (the end of
+ * a prediction pass in the persistent router kernel): another warp of the block reports `steps`
+ * steps (1 .. 100) of limit_ns / 2 each (limit_ns 1 .. 10 000 000) and then arrives at the
+ * barrier.  Every step restarts the limit, so the wait ends without a status.  Errors as above. */
+fb_status fb_selftest_wait_progress(fb_ctx* ctx, uint64_t limit_ns, int32_t steps, uint64_t* waited_ns, fb_stream stream);
+
 #ifdef __cplusplus
 }
 #endif

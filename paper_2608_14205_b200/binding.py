@@ -60,7 +60,8 @@ EXPORTS = ["fb_create", "fb_destroy", "fb_budget_ns", "fb_swap_cost_ns", "fb_pre
            "fb_set_stamp_buffer", "fb_clock_probe", "fb_attention_begin", "fb_attention_end", "fb_layer_budget_ns",
            "fb_attention_set_time_ns", "fb_attention_reset", "fb_dispatch_slot_counts", "fb_dispatch_globalize",
            "fb_standin_attention", "fb_set_split", "fb_prediction_quality",
-           "fb_layer_step_observed", "fb_staged_row_layout"]
+           "fb_layer_step_observed", "fb_staged_row_layout",
+           "fb_selftest_wait_progress"]
 
 _lib = None
 
@@ -137,6 +138,8 @@ def lib() -> ctypes.CDLL:
     L.fb_set_stamp_buffer.restype = ctypes.c_int
     L.fb_selftest_wait_timeout.argtypes = [vp, u64, vp, vp]
     L.fb_selftest_wait_timeout.restype = ctypes.c_int
+    L.fb_selftest_wait_progress.argtypes = [vp, u64, i32, vp, vp]
+    L.fb_selftest_wait_progress.restype = ctypes.c_int
     L.fb_row_cosine_mean.argtypes = [vp, vp, ctypes.c_int64, i32, i32, vp, vp, vp]
     L.fb_row_cosine_mean.restype = ctypes.c_int
     L.fb_prediction_quality.argtypes = [vp] * 6 + [i32] * 4 + [vp] * 3
@@ -425,6 +428,10 @@ class Context:
     def fb_selftest_wait_timeout(self, limit_ns: int, waited_ns=None, stream=None) -> None:
         _check(lib().fb_selftest_wait_timeout(self._h, limit_ns, _ptr(waited_ns), _stream(stream)),
                "fb_selftest_wait_timeout")
+
+    def fb_selftest_wait_progress(self, limit_ns: int, steps: int, waited_ns=None, stream=None) -> None:
+        _check(lib().fb_selftest_wait_progress(self._h, limit_ns, steps, _ptr(waited_ns), _stream(stream)),
+               "fb_selftest_wait_progress")
 
     def fb_router_floor(self, router, x, T: int, what: int, stream=None) -> None:
         _check(lib().fb_router_floor(self._h, ctypes.byref(router), _ptr(x), T, what, _stream(stream)),

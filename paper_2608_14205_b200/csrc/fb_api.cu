@@ -1299,13 +1299,23 @@ fb_status fb_set_stamp_buffer(fb_ctx* ctx, uint64_t* stamps) {
 #endif
 }
 
-fb_status fb_selftest_wait_timeout(fb_ctx* ctx, uint64_t limit_ns, uint64_t* waited_ns, fb_stream stream_) {
-  if (!ctx || limit_ns == 0 || limit_ns > 100ull * 1000 * 1000) return FB_ERR_INVALID_ARG;
+static fb_status wait_selftest(fb_ctx* ctx, uint64_t limit_ns, int32_t steps, uint64_t* waited_ns, fb_stream stream_) {
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
-  fb::fb_wait_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream_)>>>(limit_ns, ctx->status, waited_ns);
+  fb::fb_wait_selftest_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream_)>>>(limit_ns, steps, ctx->status, waited_ns);
   ++ctx->launches;
   return cudaGetLastError() == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+}
+
+fb_status fb_selftest_wait_timeout(fb_ctx* ctx, uint64_t limit_ns, uint64_t* waited_ns, fb_stream stream) {
+  if (!ctx || limit_ns == 0 || limit_ns > 100ull * 1000 * 1000) return FB_ERR_INVALID_ARG;
+  return wait_selftest(ctx, limit_ns, 0, waited_ns, stream);
+}
+
+fb_status fb_selftest_wait_progress(fb_ctx* ctx, uint64_t limit_ns, int32_t steps, uint64_t* waited_ns, fb_stream stream) {
+  // half a second at most
+  if (!ctx || limit_ns == 0 || limit_ns > 10ull * 1000 * 1000 || steps < 1 || steps > 100) return FB_ERR_INVALID_ARG;
+  return wait_selftest(ctx, limit_ns, steps, waited_ns, stream);
 }
 
 uint64_t fb_persistent_launch_count(const fb_ctx* ctx) { return ctx ? ctx->persistent_launches : 0; }

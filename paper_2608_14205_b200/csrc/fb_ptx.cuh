@@ -28,6 +28,9 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 // Arrive on the barrier at the same shared-memory offset in another CTA of the cluster.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t cta_rank) {
   asm volatile(
@@ -72,18 +75,21 @@ __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_re
 
 // Wait for the phase with the given parity.  Gives up after limit_ns, or as soon
 // as another thread of the block has given up (abort flag in shared memory), and
-// returns false; the caller then skips to its clean-up.
+// returns false; the caller then skips to its clean-up.  progress: the wait is for the end of work that the block
+// reports in steps there; the limit then holds for each step, not for all of them.
 template <bool kCluster = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          uint64_t limit_ns = kWaitLimitNs) {
+                                          uint64_t limit_ns = kWaitLimitNs, const volatile int32_t* progress = nullptr) {
   uint32_t polls = 0;
   uint64_t t0 = 0;
+  int32_t seen = progress != nullptr ? *progress : 0;
   for (;;) {
     const bool ok = kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity);
     if (ok) return true;
     if ((++polls & 0xFFu) == 0) {
       if (*abort_flag) return false;
       const uint64_t now = global_timer_ns();
+      if (progress != nullptr && *progress != seen) { seen = *progress; t0 = now; }
       if (t0 == 0) t0 = now;
       else if (now - t0 > limit_ns) { *abort_flag = 1; return false; }
     }

@@ -1016,18 +1016,32 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 // at most limit_ns, on a barrier that nobody ever arrives at.  The wait gives up, the kernel
 // records FB_ERR_TIMEOUT in the status word and returns normally - the same path a router
 // kernel takes when a copy or an MMA it waits for never completes.
-__global__ void __launch_bounds__(32, 1)
-fb_wait_selftest_kernel(uint64_t limit_ns, int32_t* status, uint64_t* waited_ns) {
+// steps > 0: another warp reports that many steps of half the limit each and then arrives, so the wait lasts longer
+// than the limit and ends well.
+__global__ void __launch_bounds__(64, 1)
+fb_wait_selftest_kernel(uint64_t limit_ns, int32_t steps, int32_t* status, uint64_t* waited_ns) {
   __shared__ uint64_t bar;
   __shared__ int32_t abort_flag;
+  __shared__ int32_t progress;
   if (threadIdx.x == 0) {
     abort_flag = 0;
+    progress = 0;
     mbar_init(smem_u32(&bar), 1);
     fence_mbar_init();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
     const uint64_t t0 = global_timer_ns();
-    const bool ok = mbar_wait<false>(smem_u32(&bar), 0u, &abort_flag, limit_ns);
+    const bool ok = mbar_wait<false>(smem_u32(&bar), 0u, &abort_flag, limit_ns, &progress);
     if (waited_ns != nullptr) *waited_ns = global_timer_ns() - t0;
     if (!ok) atomicCAS(status, 0, FB_ERR_TIMEOUT);
+  } else if (threadIdx.x == 32 && steps > 0) {
+    for (int i = 1; i <= steps; ++i) {
+      const uint64_t t0 = global_timer_ns();
+      while (global_timer_ns() - t0 < limit_ns / 2) { }
+      *static_cast<volatile int32_t*>(&progress) = i;
+    }
+    mbar_arrive(smem_u32(&bar));
   }
 }
 

@@ -39,6 +39,7 @@ struct PersistShared {
   uint32_t tmem_base;
   int32_t abort_flag;
   int32_t accum_ok;
+  int32_t tiles_done;                        // by this block, so far: restarts the limit of the wait on counts_bar
   int32_t any_unranked[4];                   // per row quarter: some row has too many or too few candidates
   int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS];
@@ -63,7 +64,8 @@ __device__ __forceinline__ void finish_early_pass(PersistShared& sh, const Route
     plan_load_placement(p.plan, sh.plan, lane, 32);
     __syncwarp();
   }
-  if (!__all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&sh.counts_bar), 0u, abort_flag))) return;
+  // (the end of a whole pass: under a pair limit a few pairs may walk millions of rows, so the limit is one tile's)
+  if (!__all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&sh.counts_bar), 0u, abort_flag, kWaitLimitNs, &sh.tiles_done))) return;
   int last = 0;
   if (lane == 0) {
     fence_acq_rel_gpu();                                            // what the two blocks added, before the ticket
@@ -110,6 +112,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
 
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
+    sh.tiles_done = 0;
     for (int q = 0; q < 4; ++q) sh.any_unranked[q] = 0;
     sh.issuer_progress[0] = -1;
     sh.issuer_progress[1] = -1;
@@ -221,6 +224,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       named_bar_sync(kAccumBarrierId, kEpilogueThreads);
       if (sh.accum_ok == 0) break;
       ++tiles_done;
+      if (et == 0) *static_cast<volatile int32_t*>(&sh.tiles_done) = static_cast<int32_t>(tiles_done);
       tcgen05_fence_after();
       uint32_t* const hist = mode == kModeDispatch ? sh.tile_hist[tiles_done & 1u] : sh.hist;
 

@@ -50,3 +50,20 @@ def test_selftest_rejects_unbounded_limits():
             ctx.fb_selftest_wait_timeout(bad)
         assert e.value.status == B.FB_ERR_INVALID_ARG
     ctx.close()
+
+
+def test_a_wait_outlasts_its_limit_while_the_work_goes_on():
+    # the persistent router kernel waits for the end of a whole prediction pass, which under a pair limit may take longer
+    # than the limit of one wait: every finished tile restarts it
+    ctx = P.make_context(I.WORKLOADS["tiny"], 128)
+    waited = torch.zeros(1, dtype=torch.int64, device="cuda")
+    limit_ns = 2_000_000
+    ctx.fb_selftest_wait_progress(limit_ns, 8, waited)     # eight steps of half the limit
+    assert ctx.fb_device_status() == 0
+    assert 4 * limit_ns <= int(waited.item()) < 50 * limit_ns
+    ctx.fb_selftest_wait_timeout(limit_ns, waited)         # no step: the limit holds
+    assert ctx.fb_device_status() == B.FB_ERR_TIMEOUT
+    for limit, steps in ((0, 1), (10**8, 1), (1000, 0), (1000, 101)):
+        with pytest.raises(B.FbError):
+            ctx.fb_selftest_wait_progress(limit, steps)
+    ctx.close()

@@ -6,6 +6,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 
 #include "../../include/freebalance.h"
@@ -530,56 +531,62 @@ static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
   return FB_OK;
 }
 
-// The ceiling on a kernel's dynamic shared memory belongs to the function on a device, not
-// to a context: contexts of different shapes share the kernel instances.  It is therefore
-// raised once per device, for every router kernel instance, to the most the device allows
-// beside the kernel's static shared memory, and never lowered again.
-static fb_status ensure_kernel_attributes(int device, const cudaDeviceProp& prop) {
-  static bool done[64] = {};
-  if (device >= 0 && device < 64 && done[device]) return FB_OK;
+// What is set or asked once per device, for all contexts:
+//   * The ceiling on a kernel's dynamic shared memory belongs to the function on a device, not to a context: contexts of
+//     different shapes share the kernel instances.  It is raised for every router kernel instance to the most the
+//     device allows beside the kernel's static shared memory, and never lowered again.
+//   * How many clusters of 2, 4, .. 16 blocks the GPU holds at once.  Every router launch takes more than half of an
+//     SM's shared memory (the operand ring alone is over 136 KB at any width), so one block fits an SM and the answer
+//     is the same for all instances and shapes.
+static fb_status set_up_device(fb_ctx* ctx, int device, const cudaDeviceProp& prop) {
+  static std::mutex mutex;
+  static struct { bool ready; int max_clusters[fb::kMaxPieces + 1]; } known[64] = {};
+  std::lock_guard<std::mutex> lock(mutex);
+  if (device >= 0 && device < 64 && known[device].ready) {
+    memcpy(ctx->max_clusters, known[device].max_clusters, sizeof(ctx->max_clusters));
+    return FB_OK;
+  }
   bool ok = true;
-  auto raise = [&](RouterKernelFn fn) {
+  auto raise = [&](RouterKernelFn fn) -> int {
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(fn)) != cudaSuccess) { ok = false; return; }
+    if (cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(fn)) != cudaSuccess) { ok = false; return 0; }
     const int most = static_cast<int>(prop.sharedMemPerBlockOptin) - static_cast<int>(fa.sharedSizeBytes);
     ok = ok && most > 0 &&
          cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
              cudaSuccess &&
          cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
              cudaSuccess;                                // clusters of 16
+    return most;
   };
   for (int i = 0; i < 4; ++i) {
     raise(ranking_kernel_fn(i / 2 != 0, i % 2 != 0));
     raise(persistent_kernel_fn(i / 2 != 0, i % 2 != 0));
   }
-  for (int i = 0; i < 2 * kRowsKernels; ++i) raise(rows_kernel_fn(i / 2, i % 2 != 0));
+  int smem = 0;
+  for (int i = 0; i < 2 * kRowsKernels; ++i) smem = raise(rows_kernel_fn(i / 2, i % 2 != 0));
   if (!ok) { cudaGetLastError(); return FB_ERR_CUDA; }
-  if (device >= 0 && device < 64) done[device] = true;
-  return FB_OK;
-}
-
-// How many clusters of 2, 4, .. 16 blocks the GPU holds at once.  Counted for the row-per-warp kernel
-// at the largest shared memory of this shape's launches (one block per SM either way).
-static fb_status count_clusters(fb_ctx* ctx) {
   cudaLaunchConfig_t occ;
   memset(&occ, 0, sizeof(occ));
   occ.blockDim = dim3(fb::kRouterThreads, 1, 1);
-  occ.dynamicSmemBytes = ctx->rows_smem[0] > ctx->rows_smem[1] ? ctx->rows_smem[0] : ctx->rows_smem[1];
+  occ.dynamicSmemBytes = static_cast<size_t>(smem);
   cudaLaunchAttribute cl[1];
   cl[0].id = cudaLaunchAttributeClusterDimension;
   occ.attrs = cl;
   occ.numAttrs = 1;
   for (int j = 1; j <= fb::kMaxPieces; ++j) {
     cl[0].val.clusterDim.x = 2u * j; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
-    occ.gridDim = dim3(2u * j * static_cast<unsigned>(ctx->n_sm), 1, 1);
+    occ.gridDim = dim3(2u * j * static_cast<unsigned>(prop.multiProcessorCount), 1, 1);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, rows_kernel_fn(ctx->rows_kernel, ctx->cfg.gate == FB_GATE_SIGMOID_GROUP_TOPK),
-                                       &occ) != cudaSuccess)
-      n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, rows_kernel_fn(kRowsKernels - 1, true), &occ) != cudaSuccess) n = 0;
     ctx->max_clusters[j] = n;
   }
   cudaGetLastError();
-  return ctx->max_clusters[1] >= 1 ? FB_OK : FB_ERR_CUDA;
+  if (ctx->max_clusters[1] < 1) return FB_ERR_CUDA;
+  if (device >= 0 && device < 64) {
+    memcpy(known[device].max_clusters, ctx->max_clusters, sizeof(ctx->max_clusters));
+    known[device].ready = true;
+  }
+  return FB_OK;
 }
 
 // Rows of the histogram table: a launch that cuts its tiles into slices has at most one slice per SM
@@ -634,7 +641,7 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
   ctx->device = device;
   {
     fb_status ss = setup_router_shape(ctx, prop);
-    if (ss == FB_OK) ss = ensure_kernel_attributes(device, prop);
+    if (ss == FB_OK) ss = set_up_device(ctx, device, prop);
     if (ss != FB_OK) { delete ctx; return ss; }
   }
   void* fn = nullptr;
@@ -645,8 +652,7 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
     return FB_ERR_CUDA;
   }
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
-  bool ok = count_clusters(ctx) == FB_OK;
-  ok = ok && dev_alloc(&ctx->counts_scratch, FB_MAX_EXPERTS) && dev_alloc(&ctx->ticket, 1) &&
+  bool ok = dev_alloc(&ctx->counts_scratch, FB_MAX_EXPERTS) && dev_alloc(&ctx->ticket, 1) &&
        dev_alloc(&ctx->status, 1) &&
        dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E)) &&
        dev_alloc(&ctx->early_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E));
@@ -1384,8 +1390,7 @@ extern "C" fb_status fb_predict_load_static(const fb_config* cfg, int device, co
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return FB_ERR_CUDA;
     ctx.cfg = *cfg;
     fb_status ss = setup_router_shape(&ctx, prop);
-    if (ss == FB_OK) ss = ensure_kernel_attributes(device, prop);
-    if (ss == FB_OK) ss = count_clusters(&ctx);
+    if (ss == FB_OK) ss = set_up_device(&ctx, device, prop);
     if (ss != FB_OK) { ctx.cfg.E = -1; return ss; }
     ctx.split_mode = 0;                                  // the sums of an unsplit call, whatever the shape
     for (int i = 0; i < kMapCache; ++i) { ctx.x_maps[i] = MapEntry(); ctx.w_maps[i] = MapEntry(); }

@@ -399,7 +399,9 @@ fb_status fb_apply_swaps_staged(fb_ctx* ctx, void* slot_weights, uint64_t expert
                                 const fb_swap* swaps, const int32_t* n_swaps, int32_t max_swaps,
                                 uint64_t staging_bytes, fb_stream plan_stream, fb_stream copy_stream);
 
-/* ---- prediction-quality metrics (Evaluation, "Metrics"); not part of the per-layer hot path ---- */
+/* ---- prediction-quality metrics (Evaluation, "Metrics"); not part of the per-layer hot path ----
+ * These three take no context and launch on the CURRENT device, which must be the one `stream` and the buffers
+ * belong to. */
 #define FB_DTYPE_BF16 0
 #define FB_DTYPE_F32 1
 /* Mean over the rows (tokens) of the cosine similarity between row i of a and row i of b:

@@ -15,6 +15,7 @@ prints one JSON report per run (synthetic changing-task steps, see inputs.make_s
 from __future__ import annotations
 
 import argparse
+import functools
 import json
 from typing import Dict, Optional
 
@@ -32,6 +33,18 @@ def make_budget_for(wl: I.Workload, T: int, **override) -> B.FbBudget:
               ranks_per_node=wl.ranks_per_node, expert_bytes=wl.expert_bytes)
     kw.update(override)
     return B.make_budget(**kw)
+
+
+def _on_its_device(method):
+    """Run a method of the loop with the loop's device current: the metric calls launch on the current device, and the
+    binding's default stream is the current device's."""
+    @functools.wraps(method)
+    def run(self, *args, **kwargs):
+        if torch._C._cuda_getDevice() == self.dev.index:
+            return method(self, *args, **kwargs)
+        with torch.cuda.device(self.dev):
+            return method(self, *args, **kwargs)
+    return run
 
 
 class ServingLoop:
@@ -72,6 +85,7 @@ class ServingLoop:
                            metrics=torch.zeros(3, dtype=torch.float64).pin_memory())     # the kernel writes to the host
         return self._q
 
+    @_on_its_device
     def layer_step(self, layer: int, router: B.FbRouter, h_prev: torch.Tensor, H: torch.Tensor,
                    budget: B.FbBudget, quality: bool = False) -> dict:
         """Run one layer of one prefill step; commits the new placement for ``layer``.
@@ -103,6 +117,7 @@ class ServingLoop:
         self.placement[layer], self._spare = pi_new, pi
         return dict(out=o, pi_old=pi, pi_new=pi_new, **report)
 
+    @_on_its_device
     def realised_loads(self, r: dict, budget: B.FbBudget):
         """Realised per-expert counts of the last layer step and the rank loads they give under the
         old, the new and the identity placement - all from the library: per-slot counts of the

@@ -264,12 +264,14 @@ fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int
                                 uint32_t* slot_offsets, uint32_t* rank_offsets, uint32_t* rank_load,
                                 fb_stream stream);
 
-/* One whole layer with device buffers: stages 1, 2 and 4 in one call.  Same results, bit for
- * bit, as fb_predict_and_plan followed by fb_route_dispatch under the new placement, but
- * both router passes (the early one on h_prev, the normal one on H) run in ONE kernel
- * launch: the tiles of the normal pass follow those of the early pass on the same blocks
- * (or in the same grid), so the selection and planning tail of the early pass is hidden
- * behind the normal pass.  The dispatch index follows in a second launch.  Arguments as in
+/* One whole layer with device buffers: stages 1, 2 and 4 in one call.  Same results as
+ * fb_predict_and_plan followed by fb_route_dispatch under the new placement - bit for bit
+ * with the k-range split off (fb_set_split), otherwise up to the order of the router GEMM's
+ * additions: how many SM pairs share a tile depends on the tiles of the launch, and this one
+ * has those of both passes.  Both router passes (the early one on h_prev, the normal one on
+ * H) run in ONE kernel launch: the tiles of the normal pass follow those of the early pass on
+ * the same blocks (or in the same grid).  The dispatch index follows in a second launch, which
+ * also counts and plans where both passes run at the same time.  Arguments as in
  * the two calls it replaces; h_prev and H must be different buffers of [T][d] bf16 each,
  * and expert_to_slot_out must not alias expert_to_slot.  Errors as in those calls. */
 fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
@@ -283,8 +285,8 @@ fb_status fb_layer_step(fb_ctx* ctx, const fb_router* router, const void* h_prev
  *   ids_early    dev i32 [T][k]   the early pass's top-k ids (as fb_predict_load's topk_ids)
  *   logits_early dev f32 [T][E]   the early pass's logits
  *   logits       dev f32 [T][E]   the normal pass's logits
- * The other results are those of fb_layer_step; a logit dump may choose another summation order of the
- * router GEMM (see fb_set_split), so logits can differ from the separate calls' in the last bits. */
+ * The other results are those of fb_layer_step (routing weights to a few ulp: a dump may take a kernel that adds
+ * a token's weights in another order). */
 fb_status fb_layer_step_observed(fb_ctx* ctx, const fb_router* router, const void* h_prev, const void* H, int32_t T,
                                  const int32_t* expert_to_slot, const fb_budget* budget, int32_t layer_id,
                                  uint32_t* counts, int32_t* expert_to_slot_out, fb_swap* swaps, int32_t* n_swaps,
@@ -434,8 +436,10 @@ fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* 
  * 256-row tile pairs than the limit (or than fit on the GPU at once, fb_max_pairs) runs
  * the persistent kernel, where each block pair walks several tiles (on as few block pairs as
  * the resulting number of rounds needs: 128 tile pairs run on 64 block pairs, not on all 74);
- * results do not depend on the limit, except that it may switch the k-range split off (see
- * fb_set_split).  Returns FB_ERR_INVALID_ARG for a negative limit. */
+ * results do not depend on the limit beyond rounding: it may change how many pairs share a tile
+ * (see fb_set_split), and a call that dumps logits may take another kernel under a limit, which
+ * adds a token's routing weights in another order.  Returns FB_ERR_INVALID_ARG for a negative
+ * limit. */
 fb_status fb_set_pair_limit(fb_ctx* ctx, int32_t pairs);
 /* k-range split of the router kernel (on by default).  When a call has so few 256-row tile pairs that
  * 2 to 8 block pairs per tile pair fit on the GPU at once, that many pairs share a tile: each sums a
@@ -444,7 +448,10 @@ fb_status fb_set_pair_limit(fb_ctx* ctx, int32_t pairs);
  * function of the shape and of the number of pairs only: a call is reproducible, but its logits
  * differ from an unsplit call's in the order of the fp32 additions (both stay within the
  * library's tolerance of the fp64 product), so a token whose k-th and (k+1)-th keys are closer
- * than that rounding may be routed differently by the two.  mode 0 switches the split off, 1 on.
+ * than that rounding may be routed differently by the two.  Where three pairs or more share a
+ * tile, each block adds the partial sums beginning with its own, so the order also depends on
+ * the row's place in its tile: equal tokens of one batch agree to that rounding only.
+ * mode 0 switches the split off, 1 on.
  * owner_bias_kblocks (-1 .. 1024) is accepted and has no effect: the pieces are equal.
  * FB_ERR_INVALID_ARG for other values. */
 fb_status fb_set_split(fb_ctx* ctx, int32_t mode, int32_t owner_bias_kblocks);

@@ -965,6 +965,57 @@ def test_pair_limit_holds_for_logit_dumps(kw):
     ctx.close()
 
 
+@pytest.mark.parametrize("T,d,kw", [
+    (1000, 2048, dict(E=128, gate=0, n_group=1, topk_group=1)),        # 4 pairs per tile in the layer call, 8 in the separate ones
+    (1000, 2048, dict(E=256, gate=1, n_group=8, topk_group=4)), (4500, 1024, dict(E=60, gate=1, n_group=4, topk_group=2)),
+])
+def test_layer_call_and_separate_calls_on_ordinary_data(T, d, kw):
+    # the split off: the same bits.  On: the order of the additions may differ, so logits agree to rounding and a token is
+    # routed differently only where its k-th and (k+1)-th keys are closer than twice the difference seen (of the keys: a
+    # sigmoid's slope is at most a quarter, its two approximations add 1e-6)
+    dev = torch.device("cuda")
+    E, k, R = kw["E"], 6, 4
+    g = torch.Generator().manual_seed(T + E)
+    x, H, W = (torch.randn(*s, generator=g).to(torch.bfloat16) for s in ((T, d), (T, d), (E, d)))
+    W = (W.float() / d ** 0.5).to(torch.bfloat16)
+    H[1::2] = H[0]                                                       # one token at every place of a tile
+    xd, Hd, Wd = x.to(dev), H.to(dev), W.to(dev)
+    router = B.make_router(Wd, None, None)
+    budget = B.make_budget(max_swaps=4, gamma_num=1, gamma_den=64, alpha_ns=(1, 1), fs_per_byte=(1, 1), expert_bytes=16)
+    pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+    exact = H.double() @ W.double().T
+    ctx = B.Context(T, d, E, k, R, kw["gate"], kw["n_group"], kw["topk_group"], 1, 1.0)
+    i32 = lambda n: torch.zeros(n, dtype=torch.int32, device=dev)
+    for split in (0, 1):
+        ctx.fb_set_split(split)
+        a, b = ([i32(E), i32(E), i32(16), i32(1), i32(R), i32(R), i32(T * k), torch.zeros(T * k, device=dev), i32(E + 1), i32(R + 1),
+                 i32(T * k), i32(T * k), i32(R)] for _ in range(2))
+        z, zl = (torch.zeros(T * E, device=dev) for _ in range(2))
+        ctx.fb_predict_and_plan(router, xd, T, pi, budget, 0, *a[:6])
+        ctx.fb_route_dispatch(router, Hd, T, a[1], *a[6:])
+        ctx.fb_layer_step(router, xd, Hd, T, pi, budget, 0, *b)
+        ids, ids_l = a[6].cpu().numpy().reshape(T, k), b[6].cpu().numpy().reshape(T, k)
+        c = [v.clone() for v in b]
+        ctx.fb_route_dispatch(router, Hd, T, a[1], *c[6:], z)
+        ctx.fb_layer_step_observed(router, xd, Hd, T, pi, budget, 0, *c, None, None, zl)
+        assert ctx.fb_device_status() == 0
+        z, zl = z.cpu().double().view(T, E), zl.cpu().double().view(T, E)
+        # n additions of fp32 products that are exact: n 2^-23 of the sum of their sizes, whatever the order
+        bound = d * 2.0 ** -23 * (H.double().abs() @ W.double().abs().T)
+        assert bool(((z - exact).abs() <= bound).all()) and bool(((zl - exact).abs() <= bound).all())
+        if split == 0:
+            assert all(torch.equal(u, v) for u, v in zip(a, b))
+            assert torch.equal(z, zl) and bool((z[1::2] == z[1]).all())
+            continue
+        diff = max(float((z - zl).abs().max()), float((z[1::2] - z[1]).abs().max()), float((zl[1::2] - z[1]).abs().max()))
+        key_diff = diff if kw["gate"] == 0 else diff / 4 + 1e-6
+        gate = O.Gate(E=E, k=k, gate=kw["gate"], n_group=kw["n_group"], topk_group=kw["topk_group"], renorm=1, route_scale=1.0)
+        key_gap, group_gap = O.near_tie_margins(z.numpy(), gate, None)
+        moved = (np.sort(ids, axis=1) != np.sort(ids_l, axis=1)).any(axis=1)
+        assert not (moved & (key_gap > 2 * key_diff) & (group_gap > 4 * key_diff)).any()
+    ctx.close()
+
+
 @pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
 def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
     # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles

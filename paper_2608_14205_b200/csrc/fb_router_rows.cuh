@@ -487,11 +487,16 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
   // out and lower the sum of 2^rank, at the end of the list they raise the number found - two sums of 2^k - 1 and
   // 2 k in all mean no ties (a test for missing ranks alone would leave it to the order of conflicting stores which
   // of two equal keys at the last rank wins).
-  found = __reduce_add_sync(full, found);
+  const uint32_t total = __reduce_add_sync(full, found);
   const uint32_t want = (1u << p.k) - 1u;
-  if (found != (want | want << 13) + 2u * static_cast<uint32_t>(p.k) * count_one || n[0] > kCandCap || n[1] > kCandCap) {
+  if (total != (want | want << 13) + 2u * static_cast<uint32_t>(p.k) * count_one || n[0] > kCandCap || n[1] > kCandCap) {
+    // which of the two: gates with few kept keys per lane overflow the list often
+    const uint32_t counts = __reduce_add_sync(full, found / count_one << (16 * h));
 #pragma unroll 1
     for (int u = 0; u < 2; ++u) {
+      if ((total >> (13 * u) & 0x1fffu) == want && (counts >> (16 * u) & 0xffffu) == static_cast<uint32_t>(p.k) &&
+          (u == 0 ? n[0] : n[1]) <= kCandCap)
+        continue;
       // scratch: the row's staged words in this block, which nobody else reads (of a shared tile, a block
       // reads the other blocks' copies of its own slice only)
       float* keys = reinterpret_cast<float*>(__cvta_shared_to_generic(row_addr + u * stride));

@@ -115,20 +115,6 @@ struct RowsShared {
 };
 
 // ---------------------------------------------------------------- selection, one warp per token row
-// The ranks that no key took (key still -inf: a row with fewer than k keys above -inf, the others being -inf or no
-// numbers) get the lowest expert ids the row has not named yet, so that a row never names an expert twice.  By one
-// lane; at most 8 ids are taken, so the lowest free one is below 8 and below E.
-__device__ __noinline__ void fill_missing_ranks(const float* win_key, int32_t* win_id, int k) {
-  uint32_t taken = 0;
-  for (int r = 0; r < k; ++r)
-    if (win_key[r] > -INFINITY && win_id[r] < FB_MAX_TOPK) taken |= 1u << win_id[r];
-  for (int r = 0; r < k; ++r)
-    if (!(win_key[r] > -INFINITY)) {
-      win_id[r] = __ffs(~taken) - 1;
-      taken |= 1u << win_id[r];
-    }
-}
-
 // Plain selection of one row by repeated maximum over keys in shared memory (dropped columns hold
 // -inf): the path of rows with more candidates than the list holds, and of rows with equal keys among
 // the candidates (the lower expert id wins).  Rare; kept out of line.
@@ -144,7 +130,21 @@ __device__ __noinline__ void select_slow(float* keys, int E, int k, float* win_k
       const int oa = __shfl_xor_sync(0xffffffffu, at, off);
       if (ob > best || (ob == best && oa < at)) { best = ob; at = oa; }
     }
-    if (at >= E) break;                                     // nothing left (see fill_missing_ranks)
+    if (at >= E) {
+      // Nothing above -inf is left (masked experts, keys that are no numbers): the other ranks get the lowest ids the
+      // row has not named, so that it never names an expert twice.  Fewer than 8 are named: these lie below k <= E.
+      if (lane == 0) {
+        uint32_t named = 0;
+        for (int h = 0; h < r; ++h)
+          if (win_id[h] < FB_MAX_TOPK) named |= 1u << win_id[h];
+        for (int h = r; h < k; ++h) {
+          win_key[h] = -INFINITY;
+          win_id[h] = __ffs(~named) - 1;
+          named |= 1u << win_id[h];
+        }
+      }
+      break;
+    }
     if (lane == 0) { win_key[r] = best; win_id[r] = at; keys[at] = -INFINITY; }
     __syncwarp();
   }
@@ -261,11 +261,23 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
 #pragma unroll
       for (int j = 0; j < kCpl; ++j) key[u][j] = fb_sigmoid(key[u][j]) + sb[j];
   }
-  if (p.ragged) {
+  // Few keys per lane (see below): keys that are no numbers count as -inf, and no number stands for a key that was taken
+  // or a column that does not exist - for the latter once group scores and the softmax denominator are formed.
+  constexpr bool kFewKeys = kCpl <= 4;
+  const float taken = __int_as_float(0x7fffffff);
+  const bool mask_later = p.groups > 1 || want_sum;
+  if (kFewKeys) {
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int j = 0; j < kCpl; ++j) key[u][j] = j < lc.n ? key[u][j] : -INFINITY;
+      for (int j = 0; j < kCpl; ++j) key[u][j] = fmaxf(key[u][j], -INFINITY);
+  }
+  if (p.ragged) {
+    const float missing = kFewKeys && !mask_later ? taken : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j) key[u][j] = j < lc.n ? key[u][j] : missing;
   }
   // ---- groups: score = sum of the two largest keys (the only key of a one-expert group); the best
   // keep_groups are kept, a lower-numbered group wins ties
@@ -341,9 +353,11 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
       for (int u = 0; u < 2; ++u) bound[u] = redux_min_f32(kept[u] ? m2[u] : INFINITY);
     }
   }
-  if (kCpl <= 4) {
+  if (kFewKeys) {
     // Few keys per lane: k rounds of "largest remaining key"; the lowest lane, and in it the lowest column,
-    // has the lowest id on ties.  (Compacting the keys above a bound and ranking them, as below, takes
+    // has the lowest id on ties.  Keys taken, and columns that do not exist, are no numbers, which no maximum takes up:
+    // what is left to take are numbers, -inf for experts that are masked out or in dropped groups, and every row has
+    // E >= k of them.  (Compacting the keys above a bound and ranking them, as below, takes
     // k reductions for the bound alone: layer step 40 tokens x 128 experts 18.5 us that way and 17.3 this way,
     // 5003 x 64 25.4 and 24.6, prediction and plan 2729 x 60 16.0 and 14.3.)
     float lane_max[2];
@@ -360,6 +374,11 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
         const float s = row_exp_sum<kCpl>(key[u], lane_max[u]);
         if (lane == 0) rs.row_sum[2 * pair + u] = s;
       }
+      if (p.ragged && mask_later) {
+#pragma unroll
+        for (int j = 0; j < kCpl; ++j) key[u][j] = j < lc.n ? key[u][j] : taken;
+        lane_max[u] = lc.n > 0 ? lane_max[u] : taken;
+      }
     }
 #pragma unroll 1
     for (int r = 0; r < p.k; ++r) {
@@ -368,7 +387,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
 #pragma unroll
       for (int u = 0; u < 2; ++u) top[u] = redux_max_f32(lane_max[u]);
 #pragma unroll
-      for (int u = 0; u < 2; ++u) holders[u] = __ballot_sync(full, lane_max[u] == top[u] && top[u] > -INFINITY);
+      for (int u = 0; u < 2; ++u) holders[u] = __ballot_sync(full, lane_max[u] == top[u]);
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         if (lane == __ffs(holders[u]) - 1) {
@@ -378,7 +397,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
           rs.win_key[2 * pair + u][r] = top[u];
           rs.win_id[2 * pair + u][r] = lc.c0 + at;
 #pragma unroll
-          for (int j = 0; j < kCpl; ++j) key[u][j] = j == at ? -INFINITY : key[u][j];
+          for (int j = 0; j < kCpl; ++j) key[u][j] = j == at ? taken : key[u][j];
           lane_max[u] = key[u][0];
 #pragma unroll
           for (int j = 1; j < kCpl; ++j) lane_max[u] = fmaxf(lane_max[u], key[u][j]);
@@ -450,10 +469,8 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
   const int h = lane >> 4, c = lane & 15;
   const int most = min(max(n[0], n[1]), kCandCap);
   const float* list = rs.cand_key[h];
-  // Ranks below k that were found: the sum of 2^rank per row in 13 bits each (at most 32 of at most 2^7), and how
-  // many of both rows together above them.
+  // Ranks below k that were found, 16 bits per row: their sum (at most 32 of at most 7) and how many above it.
   uint32_t found = 0;
-  const uint32_t one = 1u << (13 * h), count_one = 1u << 26;
   const float my0 = list[c];
   int r0 = 0;
   if (most <= 16) {
@@ -474,29 +491,24 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
     if (my1 > -INFINITY && r1 < p.k) {
       rs.win_key[2 * pair + h][r1] = my1;
       rs.win_id[2 * pair + h][r1] = rs.cand_id[h][c + 16];
-      found += (one << r1) + count_one;
+      found += 0x100u + r1;
     }
   }
   if (my0 > -INFINITY && r0 < p.k) {
     rs.win_key[2 * pair + h][r0] = my0;
     rs.win_id[2 * pair + h][r0] = rs.cand_id[h][c];
-    found += (one << r0) + count_one;
+    found += 0x100u + r0;
   }
   // Anything but every rank found once means equal keys among the best (or too few candidates): such rows, and rows
-  // whose list overflowed, take the plain path.  Equal keys share a rank: within the best k they leave a later one
-  // out and lower the sum of 2^rank, at the end of the list they raise the number found - two sums of 2^k - 1 and
-  // 2 k in all mean no ties (a test for missing ranks alone would leave it to the order of conflicting stores which
-  // of two equal keys at the last rank wins).
-  const uint32_t total = __reduce_add_sync(full, found);
-  const uint32_t want = (1u << p.k) - 1u;
-  if (total != (want | want << 13) + 2u * static_cast<uint32_t>(p.k) * count_one || n[0] > kCandCap || n[1] > kCandCap) {
-    // which of the two: gates with few kept keys per lane overflow the list often
-    const uint32_t counts = __reduce_add_sync(full, found / count_one << (16 * h));
+  // whose list overflowed, take the plain path.  Equal keys share the first of their ranks: with k ranks found they
+  // lower the sum, at the end of the list they raise the number found.  (A test for missing ranks alone would leave it
+  // to the order of conflicting stores which of two equal keys at the last rank wins.)
+  found = __reduce_add_sync(full, found << (16 * h));
+  const uint32_t want = static_cast<uint32_t>(p.k) << 8 | static_cast<uint32_t>(p.k * (p.k - 1) / 2);
+  if (found != (want | want << 16) || n[0] > kCandCap || n[1] > kCandCap) {
 #pragma unroll 1
     for (int u = 0; u < 2; ++u) {
-      if ((total >> (13 * u) & 0x1fffu) == want && (counts >> (16 * u) & 0xffffu) == static_cast<uint32_t>(p.k) &&
-          (u == 0 ? n[0] : n[1]) <= kCandCap)
-        continue;
+      if ((found >> (16 * u) & 0xffffu) == want && (u == 0 ? n[0] : n[1]) <= kCandCap) continue;
       // scratch: the row's staged words in this block, which nobody else reads (of a shared tile, a block
       // reads the other blocks' copies of its own slice only)
       float* keys = reinterpret_cast<float*>(__cvta_shared_to_generic(row_addr + u * stride));
@@ -515,7 +527,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
 // Expert ids, routing weights (Eq. 3's top-k with the model's weight rule) and histogram of up to 8 rows,
 // four at a time: lane = (row, rank).
 template <bool kSigmoid>
-__device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& sh, RowScratch& rs, int n_rows,
+__device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& sh, const RowScratch& rs, int n_rows,
                                             long long row0, int32_t* out_ids, float* out_w, int lane) {
   const uint32_t full = 0xffffffffu;
   const int rk = lane & 7;
@@ -524,10 +536,6 @@ __device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& s
     const long long row = row0 + i;
     const bool valid = i < n_rows && row < p.T && rk < p.k;
     const float key = rs.win_key[i & 7][rk];
-    if (__any_sync(full, valid && !(key > -INFINITY))) {                    // a row ran out of keys
-      if (valid && rk == 0) fill_missing_ranks(rs.win_key[i & 7], rs.win_id[i & 7], p.k);
-      __syncwarp();
-    }
     const int id = valid ? rs.win_id[i & 7][rk] : 0;
 #ifdef FB_DEBUG
     // what the sanitizer would catch: a chosen expert outside [0, E), a repeated expert
@@ -759,8 +767,6 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
         FB_STAMP(4, 64);
         const long long row0 = static_cast<long long>(tile) * kTileM + first;
         if (got && count > 0 && row0 < p.T) {
-          for (int i = lane; i < 8 * FB_MAX_TOPK; i += 32) rs.win_key[i >> 3][i & 7] = -INFINITY;   // no rank is taken yet
-          __syncwarp();
 #pragma unroll 1
           for (int i = 0; i < count; i += 2)
             if (row0 + i < p.T)

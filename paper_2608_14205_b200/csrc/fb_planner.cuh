@@ -1,7 +1,8 @@
-// Budgeted greedy expert-swap planner (Algorithm 1 lines 2-8, Eqs. 6-9), run by one
-// warp: either a stand-alone one-warp kernel or the tail of the router kernel, in the
-// block that finished last.  Integer arithmetic only, so every rank that replays it on
-// the same count vector gets the same plan.
+// Budgeted greedy expert-swap planner (Algorithm 1 lines 2-8, Eqs. 6-9), decided by one
+// warp: of the stand-alone planner kernel, of the router block that finished last, of the
+// persistent router kernel's last pair (a warp that is idle there), or of every block of the
+// dispatch-index kernel (layer calls with one tile per SM).  Integer arithmetic only, so
+// every block and every rank that replays it on the same count vector gets the same plan.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -107,7 +107,7 @@ __device__ __forceinline__ double row_cosine(CosineSums s) {
   return cosine_of(s.dot, s.na, s.nb);
 }
 // Two rows' cosines at once, with the same additions: where a butterfly step would form a value twice, half of the
-// lanes go on with another sum instead (8 exchanges instead of 30, one square root and division sequence instead
+// lanes go on with another sum instead (10 exchanges instead of 30, one square root and division sequence instead
 // of two).  Lane 0 returns the first row's, lane 16 the second's.
 __device__ __forceinline__ double exchange_add(double keep_low, double keep_high, int lane, int off) {
   const bool high = (lane & off) != 0;

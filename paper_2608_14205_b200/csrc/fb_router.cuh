@@ -80,11 +80,12 @@ constexpr uint32_t kRowBarrierBase = 3;      // named barriers 3..6: the kEpiSub
 
 enum RouterMode : int {
   kModePredict = 0,        // histogram -> counts
-  kModePredictPlan = 1,    // histogram -> counts -> planner in the last block
+  kModePredictPlan = 1,    // histogram -> counts -> planner in the block (or pair) that finishes last
   kModeDispatch = 2,       // ids, weights, per-tile histogram for the dispatch index
-  kModeLayer = 3           // one launch for a whole layer: blocks [0, tiles_first) run the early pass
-                           // (mode 1) on the first input, the others the normal pass (mode 2) on
-                           // the second; the second wave of blocks fills the SMs the first frees
+  kModeLayer = 3           // one launch for a whole layer: the first tiles_first tiles are the early pass
+                           // (mode 1) on the first input, the others the normal pass (mode 2) on the
+                           // second - all at the same time where every block has one tile, otherwise a
+                           // block's tiles of the early pass come first
 };
 
 struct RouterParams {

@@ -3,10 +3,11 @@
 Builds the library once more with -DFB_TIMING (libfreebalance_timing.so, beside the normal
 one), in which one thread per role of every block of the one-tile router kernel writes the
 global nanosecond timer and the SM cycle counter at its phase boundaries, runs the call on the
-seeded inputs of a workload and prints, in microseconds since the first block's start:
-the mean and the latest block per phase boundary, the span of the kernel (first start to last
-exit), how far apart the blocks start and finish, the gap to the next launch, and the SM clock
-each phase ran at (cycles per nanosecond).  The stamps cost a few stores per block.
+seeded inputs of a workload and prints, in microseconds since the launch's turn began (its first
+block's start, or the previous launch's last exit where that is later: blocks start early, on SMs
+that are free, and wait there): the mean and the latest block per phase boundary, the time from one
+launch's last exit to the next one's, how far apart the blocks finish, and the SM clock each phase
+ran at (cycles per nanosecond).  The stamps cost a few stores per block.
 
     python -m paper_2608_14205_b200.phase_timing [--workload dsv3] [--tokens T] [--launches 12]
         [--call predict_and_plan|predict_load] [--json out.json]
@@ -81,7 +82,7 @@ def main(argv=None):
     e1.record()
     torch.cuda.synchronize()
     ctx.fb_set_stamp_buffer(None)
-    per_launch_us = e0.elapsed_time(e1) * 1e3 / n
+    burst_us = e0.elapsed_time(e1) * 1e3
     st = stamps.cpu().numpy()
     used = st[:, :, 0] != 0                                  # blocks that ran
     nblk = int(used[0].sum())
@@ -90,12 +91,14 @@ def main(argv=None):
     cyc = st[:, :, 32:].astype(np.float64)
     rows = []
     out = {"workload": wl.name, "T": T, "call": args.call, "launches": n, "blocks": nblk,
-           "per_launch_us_events": per_launch_us, "phases": {}}
+           "burst_us_events": burst_us, "phases": {}}
+    end = ns_t[:, :, 13].max(axis=1)
     start = ns_t[:, :, 0].min(axis=1, keepdims=True)         # first block start of each launch
-    print(f"{args.call} on {wl.name} T={T}: {nblk} blocks, {per_launch_us:.1f} us per launch "
-          f"(two events around {n} back-to-back launches)")
-    print(f"{'phase boundary':32s} {'mean':>8s} {'latest':>8s}   (us since the launch's first block start; "
-          f"launches 2..{n})")
+    start[1:, 0] = np.maximum(start[1:, 0], end[:-1])        # ... or its turn
+    turn = np.diff(end) / 1e3
+    print(f"{args.call} on {wl.name} T={T}: {nblk} blocks, {turn.mean():.1f} us from exit to exit (launches 2..{n} of a burst; "
+          f"{turn.min():.1f} .. {turn.max():.1f})")
+    print(f"{'phase boundary':32s} {'mean':>8s} {'latest':>8s}   (us since the launch's turn began)")
     sel = slice(1, None)
     for slot in ORDER:
         t = ns_t[sel, :, slot]
@@ -106,23 +109,17 @@ def main(argv=None):
         mean, latest = float(np.nanmean(rel)), float(np.nanmean(np.nanmax(rel, axis=1)))
         out["phases"][SLOTS[slot]] = {"mean_us": mean, "latest_us": latest, "blocks": int(ok[0].sum())}
         print(f"{SLOTS[slot]:32s} {mean:8.2f} {latest:8.2f}   [{int(ok[0].sum())} blocks]")
-    end = ns_t[:, :, 13].max(axis=1)
-    span = (end - start[:, 0]) / 1e3
-    gap = (start[1:, 0] - end[:-1]) / 1e3
-    skew_start = (ns_t[:, :, 0].max(axis=1) - start[:, 0]) / 1e3
     ends = ns_t[:, :, 13]
     skew_end = (end - np.where(ends > 0, ends, np.inf).min(axis=1)) / 1e3
-    own = (ns_t[sel, :, 2] > 0) & (ns_t[sel, :, 11] > 0)          # blocks that own a tile (helper pairs have no epilogue)
+    own = (ns_t[sel, :, 2] > 0) & (ns_t[sel, :, 11] > 0)          # blocks with an epilogue
     main_cyc = (cyc[sel, :, 2] - cyc[sel, :, 1])[own]
     main_ns = (ns_t[sel, :, 2] - ns_t[sel, :, 1])[own]
     epi_cyc = (cyc[sel, :, 11] - cyc[sel, :, 2])[own]
     epi_ns = (ns_t[sel, :, 11] - ns_t[sel, :, 2])[own]
-    out.update(span_us=float(span[sel].mean()), gap_us=float(gap.mean()), start_skew_us=float(skew_start[sel].mean()),
-               end_skew_us=float(skew_end[sel].mean()), main_loop_ghz=float(main_cyc.mean() / main_ns.mean()),
+    out.update(turn_us=float(turn.mean()), end_skew_us=float(skew_end[sel].mean()), main_loop_ghz=float(main_cyc.mean() / main_ns.mean()),
                epilogue_ghz=float(epi_cyc.mean() / epi_ns.mean()), main_loop_cycles=float(main_cyc.mean()))
-    print(f"kernel span (first start .. last exit) {out['span_us']:.2f} us; gap to the next launch's first block "
-          f"{out['gap_us']:.2f} us; blocks start within {out['start_skew_us']:.2f} us and exit within "
-          f"{out['end_skew_us']:.2f} us")
+    print(f"blocks exit within {out['end_skew_us']:.2f} us; the whole burst of {n} launches, the host's first call included: "
+          f"{burst_us:.0f} us between two events")
     print(f"SM clock: main loop {out['main_loop_ghz']:.3f} GHz ({out['main_loop_cycles']:.0f} cycles), "
           f"epilogue {out['epilogue_ghz']:.3f} GHz")
     if args.json:

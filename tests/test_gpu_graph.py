@@ -1,7 +1,7 @@
 """The library's calls inside a CUDA graph: captured once, replayed on new inputs.
 
 The calls allocate nothing, never synchronise and keep no per-launch state on the host that a kernel
-depends on (the k-range split's partial-tile flags are put back by the kernel that consumed them), so a
+depends on (counters and tickets are put back to zero by the kernel that read them), so a
 captured sequence can be replayed; every replay must give the bits the same calls give when made directly.
 """
 import numpy as np
@@ -32,7 +32,7 @@ def _calls(ctx, router, x, H, T, pi, budget, o):
 @pytest.mark.parametrize("name,T,pair_limit", [("qwen3", 2000, 0), ("mixtral", 1000, 0), ("dsv3", 1500, 0),
                                                 ("dsv3", 1500, 2)])
 def test_captured_calls_replay_bit_for_bit(name, T, pair_limit):
-    # qwen3 / mixtral at these sizes run with the k-range split (helper pairs and their flags),
+    # at these sizes several SM pairs share a tile,
     # dsv3 with a pair limit runs the persistent kernel; every form must survive a replay.
     wl = I.WORKLOADS[name]
     layers = [I.make_layer(wl, l, 0, T=T) for l in range(3)]

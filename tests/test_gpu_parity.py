@@ -79,14 +79,15 @@ def test_edge_shapes(kw):
 
 
 @pytest.mark.parametrize("kw,T", [
-    (dict(E=192, k=6, R=8, d=1600), 700),                                    # pairs: 7 stages
-    (dict(E=192, k=6, R=8, d=1600), 100),                                    # one block: 5 stages
-    (dict(E=224, k=8, R=7, d=1096), 450),                                    # pairs: 7 stages
+    (dict(E=192, k=6, R=8, d=1600), 700),                                    # 7 stages
+    (dict(E=192, k=6, R=8, d=1600), 100),
+    (dict(E=224, k=8, R=7, d=1096), 450),                                    # 7 stages
     (dict(gate=1, n_group=6, topk_group=3, k=6, E=192, R=6, d=1600), 700),   # ranking selection, 7 stages
 ])
 def test_widths_whose_operand_ring_has_an_odd_number_of_stages(kw, T):
-    # At these widths as many stages as fit is an odd number, so a stage alternates between the two
-    # MMA issuers without any diagnostic limit being set.
+    # At these widths as many stages as fit is an odd number.  (One MMA issuer there; odd rings that two
+    # issuers share: test_pipeline_depth_does_not_change_results, and gates of 113 to 128 experts with
+    # several tiles per pair, five stages, in test_row_selection_of_restricted_gates_at_every_lane_layout.)
     _run(_wl(**kw), T, with_logit_bias=True)
     _run(_wl(**kw), T, layer=1)
 
@@ -172,8 +173,8 @@ def test_plan_swaps_alone_on_random_counts(seed):
 
 @pytest.mark.parametrize("seed", range(24))
 def test_planner_variants_random_plans_exact(seed):
-    """The one-pass sweep, the widened frontier, per-expert sizes and ranks of more than 16
-    experts all run the general planner loop: exact agreement with the oracle's variant."""
+    """The one-pass sweep, the widened frontier and per-expert sizes run the general planner loop:
+    exact agreement with the oracle's variant."""
     rng = np.random.default_rng(500 + seed)
     R = int(rng.choice([2, 3, 4, 8, 16, 64]))
     m = int(rng.choice([1, 2, 4, 8, 32]))
@@ -536,11 +537,12 @@ def test_pair_limit_does_not_change_results():
 
 
 @pytest.mark.parametrize("name,T,split,d", [("dsv3", 3000, 0, None), ("qwen3", 2500, 0, None), ("dsv3", 1100, 1, None),
-                                             ("dsv3", 1300, 0, 2112)])
+                                             ("dsv3", 1300, 0, 2112), ("qwen3", 1300, 0, 2112)])
 def test_pipeline_depth_does_not_change_results(name, T, split, d):
-    # Short operand rings, and rings with an odd number of stages (a stage then alternates between
-    # the two MMA issuers, which keep each other informed of their progress): same bits as the full
-    # depth, through the one-tile kernel, its k-range split and the persistent kernel.  With three
+    # Short operand rings, and rings with an odd number of stages (where two MMA issuers work, at up to
+    # 128 columns, a stage then alternates between them and they keep each other informed of their
+    # progress): same bits as the full depth, through the one-tile kernel, tiles shared by several pairs
+    # and the persistent kernel.  With three
     # stages an issuer that took a stale phase of a "full" barrier for its own would read operands
     # that have not arrived.  d = 2112 gives an odd number of k-blocks: in the persistent kernel the
     # issuer that owns a ring position then changes from tile to tile.
@@ -571,9 +573,9 @@ def test_pipeline_depth_does_not_change_results(name, T, split, d):
 @pytest.mark.parametrize("name,T,d", [("qwen3", 8192, None), ("mixtral", 4096, None), ("dsv3", 4096, None),
                                        ("qwen3", 1000, None), ("dsv3", 2049, 2112), ("mixtral", 300, 2048)])
 def test_k_range_split_on_and_off_agree_with_the_oracle(name, T, d):
-    # Shapes that leave at least half of the SM pairs without a tile run with helper pairs that
-    # sum the tail of every tile's k-range; both settings must satisfy the oracle, and the counts
-    # may differ between them only in near-tie tokens.
+    # Where two to eight times as many SM pairs as tile pairs fit, that many share a tile's k-range;
+    # both settings must satisfy the oracle, and the counts may differ between them only in
+    # near-tie tokens.
     wl = I.WORKLOADS[name]
     if d is not None:
         wl = dataclasses.replace(wl, d=d)
@@ -589,7 +591,7 @@ def test_k_range_split_on_and_off_agree_with_the_oracle(name, T, d):
         counts[mode] = gpu["counts"]
         ctx.close()
     assert int(np.abs(counts[0] - counts[1]).sum()) <= 2 * wl.k * max(1, T // 200)
-    for bias in (0, 5):                                   # other owner shares: still the oracle's results
+    for bias in (0, 5):                                   # accepted, without effect: still the oracle's results
         ctx = P.make_context(wl, T)
         ctx.fb_set_split(1, bias)
         gpu = P.run_gpu_layer(ctx, wl, li, bkw, want_logits=False)
@@ -707,8 +709,8 @@ def test_persistent_kernel_narrow_and_wide_gates(kw, T, limit):
 
 
 def test_dispatch_index_with_several_tiles_per_block():
-    # more tiles than resident blocks of the dispatch-index kernel: every block walks a run of
-    # three tiles (the rotation of its mask buffers and the carried counts are exercised)
+    # more tiles than SMs: every block of the dispatch-index kernel walks a run of six tiles, a batch
+    # of four and one of two (the carried counts are exercised)
     wl = _wl(E=64, k=4, R=8, gate=0, d=64, max_swaps=6)
     T = 100_000
     rng = np.random.default_rng(0)
@@ -737,7 +739,7 @@ def test_dispatch_index_over_table_widths_and_runs_of_tiles(E, k, R, T):
     dict(E=100, k=6, R=4),                                            # four
     dict(E=200, k=8, R=8, renorm=0), dict(E=250, k=8, R=5),           # eight; the last lane's second vector is padding
     dict(gate=1, n_group=5, topk_group=2, k=7, E=250, R=5),           # sixteen; bound from the lanes, idle lanes
-    dict(gate=1, n_group=8, topk_group=3, k=6, E=160, R=8),           # groups of 20: five per lane, single loads
+    dict(gate=1, n_group=8, topk_group=3, k=6, E=160, R=8),           # groups of 20 over four lanes: two vectors per lane
     dict(gate=1, n_group=32, topk_group=4, k=8, E=64, R=8),           # groups of two
     dict(gate=1, n_group=3, topk_group=3, k=5, E=96, R=6, route_scale=2.5),   # every group kept
     dict(E=128, k=8, R=8), dict(gate=1, n_group=8, topk_group=4, k=8, E=256, R=32),   # ranking gates, tiles shared by pairs

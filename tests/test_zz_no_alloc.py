@@ -50,8 +50,8 @@ def test_static_entry_matches_context_entry_twice(name, T):
     B.fb_predict_load_static(cfg, 0, router, x, T, got_counts, got_ids, status)
     torch.cuda.synchronize(dev)
     assert torch.cuda.mem_get_info(dev)[0] >= free_before
-    # the reference results, through a context running the same kernel (the static entry has no
-    # room for the partial tiles of the k-range split, so the context switches its split off)
+    # the reference results, through a context running the same kernel (the static entry never
+    # shares a tile between SM pairs, so the context switches its split off)
     ctx = P.make_context(wl, T)
     ctx.fb_set_split(0)
     for router, x, want_counts, want_ids, _, _, _ in prepared:

@@ -465,9 +465,24 @@ bool dev_alloc(Tp** p, size_t count) {
 
 }  // namespace
 
+// What the host side needs to know of a device.  Three attributes: the whole property record takes the driver 2.5 ms
+// and, with other processes on the machine, now and then a hundred (2.7 -> 0.2 ms per context).
+struct DeviceLimits {
+  int n_sm = 0, smem_optin = 0;
+  bool usable = false;                                 // built for sm_100a only; no fallback
+};
+static DeviceLimits device_limits(int device) {
+  DeviceLimits d;
+  int major = 0;
+  d.usable = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) == cudaSuccess && major == 10 &&
+             cudaDeviceGetAttribute(&d.n_sm, cudaDevAttrMultiProcessorCount, device) == cudaSuccess &&
+             cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) == cudaSuccess;
+  return d;
+}
+
 // Shape-dependent launch parameters of the router kernels (host arithmetic only): padded width, TMEM
 // columns, gate layout, pipeline depths and dynamic shared memory.
-static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
+static fb_status setup_router_shape(fb_ctx* ctx, const DeviceLimits& dev) {
   const fb_config& c = ctx->cfg;
   ctx->N = (c.E + 15) / 16 * 16;
   fb::RouterParams& g = ctx->gate;
@@ -485,7 +500,7 @@ static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
   ctx->rows_kernel = 0;
   while ((1 << ctx->rows_kernel) < cpl) ++ctx->rows_kernel;
   if (ctx->rows_kernel >= kRowsKernels) return FB_ERR_UNSUPPORTED_SHAPE;   // (no gate within the limits has more columns per lane)
-  const size_t optin = static_cast<size_t>(prop.sharedMemPerBlockOptin) - 2048 - 1024;
+  const size_t optin = static_cast<size_t>(dev.smem_optin) - 2048 - 1024;
   const size_t stage_bytes = fb::kATileBytes + static_cast<size_t>(ctx->N / 2) * fb::kBlockK * 2;
   auto depth = [&](size_t bytes) {
     const int n = static_cast<int>(bytes / stage_bytes);
@@ -527,7 +542,7 @@ static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
   }
   if (ctx->rows_stages[1] < 2) return FB_ERR_UNSUPPORTED_SHAPE;
   ctx->max_tiles = (c.T_max + fb::kTileM - 1) / fb::kTileM;
-  ctx->n_sm = prop.multiProcessorCount;
+  ctx->n_sm = dev.n_sm;
   return FB_OK;
 }
 
@@ -538,7 +553,7 @@ static fb_status setup_router_shape(fb_ctx* ctx, const cudaDeviceProp& prop) {
 //   * How many clusters of 2, 4, .. 16 blocks the GPU holds at once.  Every router launch takes more than half of an
 //     SM's shared memory (the operand ring alone is over 136 KB at any width), so one block fits an SM and the answer
 //     is the same for all instances and shapes.
-static fb_status set_up_device(fb_ctx* ctx, int device, const cudaDeviceProp& prop) {
+static fb_status set_up_device(fb_ctx* ctx, int device, const DeviceLimits& dev) {
   static std::mutex mutex;
   static struct { bool ready; int max_clusters[fb::kMaxPieces + 1]; } known[64] = {};
   std::lock_guard<std::mutex> lock(mutex);
@@ -550,7 +565,7 @@ static fb_status set_up_device(fb_ctx* ctx, int device, const cudaDeviceProp& pr
   auto raise = [&](RouterKernelFn fn) -> int {
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(fn)) != cudaSuccess) { ok = false; return 0; }
-    const int most = static_cast<int>(prop.sharedMemPerBlockOptin) - static_cast<int>(fa.sharedSizeBytes);
+    const int most = dev.smem_optin - static_cast<int>(fa.sharedSizeBytes);
     ok = ok && most > 0 &&
          cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
              cudaSuccess &&
@@ -575,7 +590,7 @@ static fb_status set_up_device(fb_ctx* ctx, int device, const cudaDeviceProp& pr
   occ.numAttrs = 1;
   for (int j = 1; j <= fb::kMaxPieces; ++j) {
     cl[0].val.clusterDim.x = 2u * j; cl[0].val.clusterDim.y = 1; cl[0].val.clusterDim.z = 1;
-    occ.gridDim = dim3(2u * j * static_cast<unsigned>(prop.multiProcessorCount), 1, 1);
+    occ.gridDim = dim3(2u * j * static_cast<unsigned>(dev.n_sm), 1, 1);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, rows_kernel_fn(kRowsKernels - 1, true), &occ) != cudaSuccess) n = 0;
     ctx->max_clusters[j] = n;
@@ -632,16 +647,15 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) return FB_ERR_CUDA;
   DeviceGuard guard(device);
   if (!guard.ok) return FB_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return FB_ERR_CUDA;
-  if (prop.major != 10) return FB_ERR_CUDA;            // built for sm_100a only; no fallback
+  const DeviceLimits limits = device_limits(device);
+  if (!limits.usable) return FB_ERR_CUDA;
   fb_ctx* ctx = new (std::nothrow) fb_ctx();
   if (!ctx) return FB_ERR_CUDA;
   ctx->cfg = *cfg;
   ctx->device = device;
   {
-    fb_status ss = setup_router_shape(ctx, prop);
-    if (ss == FB_OK) ss = set_up_device(ctx, device, prop);
+    fb_status ss = setup_router_shape(ctx, limits);
+    if (ss == FB_OK) ss = set_up_device(ctx, device, limits);
     if (ss != FB_OK) { delete ctx; return ss; }
   }
   void* fn = nullptr;
@@ -1368,8 +1382,7 @@ extern "C" fb_status fb_predict_load_static(const fb_config* cfg, int device, co
     // One-time set-up for this device, with the device current.  In host code the name
     // of a __device__ array is only a handle: the address a kernel can use has to be
     // asked for.
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess || prop.major != 10) return FB_ERR_CUDA;
+    if (!device_limits(device).usable) return FB_ERR_CUDA;
     void* addr = nullptr;
     if (cudaGetSymbolAddress(&addr, g_static_scratch) != cudaSuccess || addr == nullptr) return FB_ERR_CUDA;
     void* fn = nullptr;
@@ -1386,11 +1399,11 @@ extern "C" fb_status fb_predict_load_static(const fb_config* cfg, int device, co
   fb_ctx& ctx = st.ctx;
   if (memcmp(&ctx.cfg, cfg, sizeof(fb_config)) != 0) {
     // shape-dependent launch parameters (host arithmetic and function attributes only)
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return FB_ERR_CUDA;
+    const DeviceLimits limits = device_limits(device);
+    if (!limits.usable) return FB_ERR_CUDA;
     ctx.cfg = *cfg;
-    fb_status ss = setup_router_shape(&ctx, prop);
-    if (ss == FB_OK) ss = set_up_device(&ctx, device, prop);
+    fb_status ss = setup_router_shape(&ctx, limits);
+    if (ss == FB_OK) ss = set_up_device(&ctx, device, limits);
     if (ss != FB_OK) { ctx.cfg.E = -1; return ss; }
     ctx.split_mode = 0;                                  // the sums of an unsplit call, whatever the shape
     for (int i = 0; i < kMapCache; ++i) { ctx.x_maps[i] = MapEntry(); ctx.w_maps[i] = MapEntry(); }

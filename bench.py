@@ -731,7 +731,7 @@ def main():
         persistent = persistent_launches > 0
         roof = None
         if router_ms:
-            kname = ("fb_router_persistent_kernel" if persistent else "fb_router_kernel") + \
+            kname = ("fb_router_persistent_kernel" if persistent else "fb_router_kernel / fb_router_rows_kernel") + \
                     (" (fb_layer_step: both router passes in one launch)" if layer_api else " (fb_predict_and_plan)")
             k1_ms = statistics.median(router_ms)
             roof = roofline(k1_ms, alg_bytes, alg_flops, kname)
@@ -744,7 +744,7 @@ def main():
         if pp_b2b:
             pp_bytes, pp_flops = 2 * T * d + 2 * d * E + 4 * E, 2 * T * d * E
             roof_pp = roofline(statistics.median(pp_b2b), pp_bytes, pp_flops,
-                               "fb_router_kernel + planner tail (fb_predict_and_plan)")
+                               "router kernel + planner tail (fb_predict_and_plan)")
             roof_pp["timing"] = f"{pp_n} launches back to back between two events, median of {len(pp_b2b)} repeats"
             roof_pp["spread"] = spread(pp_b2b)
             roof_pp["tokens_per_s"] = T / (statistics.median(pp_b2b) * 1e-3)

@@ -190,6 +190,8 @@ uint64_t fb_swap_cost_ns(const fb_budget* budget, int32_t rank_a, int32_t rank_b
  *   counts      dev u32 [E]      out: n_e = number of tokens whose top-k contains e
  *   topk_ids    dev i32 [T][k]   out, optional (NULL to skip): chosen experts per token,
  *                                descending selection key, equal keys -> lower id first
+ *                                (a token whose keys are no numbers: k distinct experts,
+ *                                unspecified which; other tokens are not affected)
  *   logits      dev f32 [T][E]   out, optional debug dump of g(x) (NULL to skip)
  * T == 0 writes zero counts. */
 fb_status fb_predict_load(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T,

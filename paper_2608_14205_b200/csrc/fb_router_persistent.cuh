@@ -41,7 +41,7 @@ struct PersistShared {
   int32_t accum_ok;
   int32_t tiles_done;                        // by this block, so far: restarts the limit of the wait on counts_bar
   int32_t any_unranked[4];                   // per row quarter: some row has too many or too few candidates
-  int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
+  int32_t issuer_progress[2];                // where both issuers use a stage: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];
   alignas(16) uint32_t hist[FB_MAX_EXPERTS];          // early pass: over all of the block's tiles
@@ -369,15 +369,13 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
 
       // ---------------- rank the candidates (many equal keys can overflow the list: handled below)
       const uint32_t n_cand = sh.cand_count[row_in_tile];
+      if (n_cand < static_cast<uint32_t>(k)) sh.any_unranked[quarter] = 1;
       const bool overflow = rank_candidates(cand, n_cand, sub, row_in_tile, out_hi, out_lo);
-      if (overflow || n_cand < static_cast<uint32_t>(k)) sh.any_unranked[quarter] = 1;
+      if (overflow) sh.any_unranked[quarter] = 1;
       row_sync();
       TopK top;
       top.init();
-      if (sub == 0) {
-        sh.cand_count[row_in_tile] = 0;                      // ready for the next tile
-        if (!overflow) read_ranked(top, k, out_hi, out_lo, row_in_tile);
-      }
+      if (sub == 0 && !overflow) read_ranked(top, k, out_hi, out_lo, row_in_tile);
       if (sh.any_unranked[quarter] != 0) {
         // Some of these rows had more than kCandCap keys at or above its floor (many equal
         // keys).  Such rows are selected by plain insertion: every thread scans its own kept
@@ -408,8 +406,10 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
             if (x > -INFINITY) top.insert_any_order(x, static_cast<int32_t>(static_cast<uint32_t>(w)));
           }
         }
-        if (sub == 0) fill_missing_ranks(top, overflow ? ranks_taken(top) : n_cand, k);   // fewer than k: no numbers
+        if (sub == 0) fill_missing_ranks(top, overflow ? ranks_taken(top) : sh.cand_count[row_in_tile], k);   // no numbers
       }
+
+      if (sub == 0) sh.cand_count[row_in_tile] = 0;          // ready for the next tile
 
       // ---------------- outputs per row
       const bool writer = valid && sub == 0;

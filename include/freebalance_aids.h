@@ -30,9 +30,9 @@ fb_status fb_time_next_router_launch(fb_ctx* ctx, void* event_before, void* even
 /* Diagnostic: later router launches of this context use at most `stages` stages of the
  * operand pipeline (0 lifts the limit; 1 is not a pipeline: FB_ERR_INVALID_ARG).  Results do
  * not depend on the depth, only the speed does.  Exists so that tests can run short rings and
- * rings with an odd number of stages, in which a stage alternates between the two MMA issuers
- * (they then keep each other informed of their progress; with an even number a stage always
- * serves the same issuer). */
+ * rings in which a stage alternates between the two MMA issuers (an odd number of stages, or an
+ * odd number of k-blocks and several tiles per pair: they then keep each other informed of
+ * their progress). */
 fb_status fb_set_stage_limit(fb_ctx* ctx, int32_t stages);
 
 /* Where a row's logits lie in shared memory between the router GEMM and the row-per-warp

@@ -208,7 +208,7 @@ struct RouterShared {
   int32_t abort_flag;
   int32_t is_last;
   int32_t accum_ok;
-  int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
+  int32_t issuer_progress[2];                // where both issuers use a stage: see issuer_turn_wait
   float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];
   alignas(16) uint32_t hist[FB_MAX_EXPERTS];
@@ -495,13 +495,13 @@ __device__ __forceinline__ void write_slice_counts(uint8_t* table, int slice, in
   }
 }
 
-// Two MMA issuers share one ring of stages.  With an even number of stages a stage always serves
-// the same issuer, which therefore sees every phase of the stage's "full" barrier.  With an odd
-// number a stage alternates between them, and a parity wait alone cannot tell "the other issuer's
-// use of this stage is still being filled" (a wait for my parity passes on the phase before it)
-// from "my use is complete".  So each issuer publishes the ring position of the last k-block whose
-// operands it has seen arrive, and before it waits for position g on a stage whose previous use
-// (position g - stages) was the other issuer's, it waits until the other one has got that far.
+// Two MMA issuers share one ring of stages.  Where a stage always serves the same issuer - an even number of stages, and
+// one tile per pair or an even number of k-blocks per tile - that issuer sees every phase of the stage's "full" barrier.
+// With an odd number of stages a stage alternates between them, and with an odd number of k-blocks the issuers' ring
+// positions trade places from tile to tile; a parity wait alone cannot tell "the other issuer's use of this stage is
+// still being filled" (a wait for my parity passes on the phase before it) from "my use is complete".  So each issuer
+// publishes the ring position of the last k-block whose operands it has seen arrive, and before it waits for position g on
+// a stage whose previous use (position g - stages) was the other issuer's, it waits until the other one has got that far.
 __device__ __forceinline__ bool issuer_turn_wait(const volatile int32_t* other_progress, int32_t need,
                                                  volatile int* abort_flag) {
   uint32_t polls = 0;
@@ -575,7 +575,8 @@ __device__ __forceinline__ void issue_mmas(const RouterParams& p, const TileWalk
   const bool leader = elect_one();
   const int stages = p.stages, step = p.issuers;
   const uint32_t idesc = umma_idesc_bf16_f32(kTileM * 2, static_cast<uint32_t>(p.N));
-  const bool odd_ring = step == 2 && (stages & 1) != 0;
+  const bool several = w.pair_first + w.pair_stride < w.total_pairs;
+  const bool shared_stages = step == 2 && ((stages & 1) != 0 || (several && (w.n_kb & 1) != 0));   // see issuer_turn_wait
   volatile int32_t* my_progress = progress + issuer;
   const volatile int32_t* other_progress = progress + (issuer ^ 1);
   int s0 = 0;                                  // stage and phase of the tile's first k-block
@@ -595,7 +596,7 @@ __device__ __forceinline__ void issue_mmas(const RouterParams& p, const TileWalk
     uint32_t phase = phase0;
     if (s >= stages) { s -= stages; phase ^= 1u; }
     for (int kb = issuer; kb < w.n_kb; kb += step) {
-      if (odd_ring && g0 + kb >= stages) {
+      if (shared_stages && g0 + kb >= stages) {
         // whose was the stage's previous use (ring position g0 + kb - stages)?  Its k-block index
         // inside its own tile decides, as for every k-block.
         int kbp = kb - stages;
@@ -605,7 +606,7 @@ __device__ __forceinline__ void issue_mmas(const RouterParams& p, const TileWalk
       }
       ok = ok && __all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&full_bar[s]), phase, abort_flag));
       if (!ok) break;
-      if (odd_ring && leader) *my_progress = g0 + kb;
+      if (shared_stages && leader) *my_progress = g0 + kb;
       tcgen05_fence_after();
       if (kb == 0) FB_STAMP(16, 32);
       const uint32_t a_addr = smem_base + static_cast<uint32_t>(s) * stage_bytes;

@@ -106,7 +106,7 @@ struct RowsShared {
   int32_t abort_flag;
   int32_t is_last;
   int32_t accum_ok;
-  int32_t issuer_progress[2];                // rings with an odd number of stages: see issuer_turn_wait
+  int32_t issuer_progress[2];                // where both issuers use a stage: see issuer_turn_wait
   uint16_t quad_word[FB_MAX_EXPERTS / 4];    // where columns 4 q .. 4 q + 3 lie in a staged row
   alignas(16) float logit_bias[FB_MAX_EXPERTS];
   alignas(16) float select_bias[FB_MAX_EXPERTS];

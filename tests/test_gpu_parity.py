@@ -1018,6 +1018,38 @@ def test_layer_call_and_separate_calls_on_ordinary_data(T, d, kw):
     ctx.close()
 
 
+@pytest.mark.parametrize("kw", [
+    dict(E=96, k=5, R=6), dict(E=128, k=6, R=8, gate=1, n_group=4, topk_group=3),        # persistent kernel
+    dict(E=60, k=4, R=5), dict(E=120, k=6, R=8, gate=1, n_group=6, topk_group=3),        # row-per-warp kernel
+])
+@pytest.mark.parametrize("d", [192, 448, 1088])          # 3, 7 and 17 k-blocks
+def test_odd_numbers_of_k_blocks_with_several_tiles_per_pair(kw, d):
+    # two MMA issuers, several tiles per pair: with an odd number of k-blocks their ring positions trade places from tile
+    # to tile, whatever the number of stages; small integers, so every result is exact
+    dev = torch.device("cuda")
+    kw = dict(dict(gate=0, n_group=1, topk_group=1), **kw)
+    T, E, k, R = 2700, kw["E"], kw["k"], kw["R"]
+    g = torch.Generator().manual_seed(E + d)
+    x, W = (torch.randint(-3, 4, s, generator=g).to(torch.bfloat16).to(dev) for s in ((T, d), (E, d)))
+    router = B.make_router(W, None, None)
+    ctx = B.Context(T, d, E, k, R, kw["gate"], kw["n_group"], kw["topk_group"], 1, 1.0)
+    pi = torch.randperm(E, generator=g).to(torch.int32).to(dev)
+    i32 = lambda n: torch.full((n,), -7, dtype=torch.int32, device=dev)
+    results = []
+    for limit, stages in ((0, 0), (1, 0), (3, 0), (1, 2), (2, 2), (1, 3), (2, 4)):
+        ctx.fb_set_pair_limit(limit)
+        ctx.fb_set_stage_limit(stages)
+        for _ in range(3 if limit else 1):
+            counts, early, ids, perm, inv, so, ro, rl = i32(E), i32(T * k), i32(T * k), i32(T * k), i32(T * k), i32(E + 1), i32(R + 1), i32(R)
+            ctx.fb_predict_load(router, x, T, counts, early)
+            ctx.fb_route_dispatch(router, x, T, pi, ids, torch.zeros(T * k, device=dev), so, ro, perm, inv, rl)
+            assert ctx.fb_device_status() == 0, (limit, stages)
+            results.append((counts, early, ids, perm, inv, so, ro, rl))
+    for other in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(results[0], other))
+    ctx.close()
+
+
 @pytest.mark.parametrize("pieces", [2, 3, 4, 5, 6, 7, 8])
 def test_any_number_of_pairs_per_tile_gives_the_unshared_results(pieces):
     # small integers: every order of the sums is exact.  Token counts around the edges of row slices and tiles

@@ -15,7 +15,6 @@ prints one JSON report per run (synthetic changing-task steps, see inputs.make_s
 from __future__ import annotations
 
 import argparse
-import functools
 import json
 from typing import Dict, Optional
 
@@ -35,23 +34,12 @@ def make_budget_for(wl: I.Workload, T: int, **override) -> B.FbBudget:
     return B.make_budget(**kw)
 
 
-def _on_its_device(method):
-    """Run a method of the loop with the loop's device current: the metric calls launch on the current device, and the
-    binding's default stream is the current device's."""
-    @functools.wraps(method)
-    def run(self, *args, **kwargs):
-        if torch._C._cuda_getDevice() == self.dev.index:
-            return method(self, *args, **kwargs)
-        with torch.cuda.device(self.dev):
-            return method(self, *args, **kwargs)
-    return run
-
-
 class ServingLoop:
     """Per-layer placement state plus the output buffers of one layer step."""
 
     def __init__(self, wl: I.Workload, T_max: int, device: int = 0):
         self.wl, self.T_max = wl, T_max
+        self.device = device
         self.dev = torch.device("cuda", device)
         self.ctx = B.Context(T_max, wl.d, wl.E, wl.k, wl.R, wl.gate, wl.n_group, wl.topk_group, wl.renorm,
                              wl.route_scale, device=device)
@@ -85,13 +73,16 @@ class ServingLoop:
                            metrics=torch.zeros(3, dtype=torch.float64).pin_memory())     # the kernel writes to the host
         return self._q
 
-    @_on_its_device
     def layer_step(self, layer: int, router: B.FbRouter, h_prev: torch.Tensor, H: torch.Tensor,
                    budget: B.FbBudget, quality: bool = False) -> dict:
         """Run one layer of one prefill step; commits the new placement for ``layer``.
 
         Returns the output buffers (device tensors, overwritten by the next call) and, with
         ``quality=True``, the metrics as Python floats."""
+        # The metric calls launch on the current device, and the binding's default stream is the current device's.
+        if torch._C._cuda_getDevice() != self.device:
+            with torch.cuda.device(self.device):
+                return self.layer_step(layer, router, h_prev, H, budget, quality)
         T, o, ctx = h_prev.shape[0], self.out, self.ctx
         pi, pi_new = self.placement_of(layer), self._spare
         report = {}
@@ -117,12 +108,14 @@ class ServingLoop:
         self.placement[layer], self._spare = pi_new, pi
         return dict(out=o, pi_old=pi, pi_new=pi_new, **report)
 
-    @_on_its_device
     def realised_loads(self, r: dict, budget: B.FbBudget):
         """Realised per-expert counts of the last layer step and the rank loads they give under the
         old, the new and the identity placement - all from the library: per-slot counts of the
         dispatch index, `rank_load` of the step, and the planner's own rank-load aggregation
         (fb_plan_swaps with no swap allowed) for the other two placements."""
+        if torch._C._cuda_getDevice() != self.device:
+            with torch.cuda.device(self.device):
+                return self.realised_loads(r, budget)
         ctx, o, E, R = self.ctx, self.out, self.wl.E, self.wl.R
         i32 = lambda n: torch.zeros(max(1, n), dtype=torch.int32, device=self.dev)
         slot_counts, before, vanilla, scratch = i32(E), i32(R), i32(R), i32(R)

@@ -466,7 +466,7 @@ bool dev_alloc(Tp** p, size_t count) {
 }  // namespace
 
 // What the host side needs to know of a device.  Three attributes: the whole property record takes the driver 2.5 ms
-// and, with other processes on the machine, now and then a hundred (2.7 -> 0.2 ms per context).
+// and, with other processes on the machine, now and then a hundred (2.9 -> 0.4 ms per context).
 struct DeviceLimits {
   int n_sm = 0, smem_optin = 0;
   bool usable = false;                                 // built for sm_100a only; no fallback
@@ -551,7 +551,7 @@ static fb_status setup_router_shape(fb_ctx* ctx, const DeviceLimits& dev) {
 //     different shapes share the kernel instances.  It is raised for every router kernel instance to the most the
 //     device allows beside the kernel's static shared memory, and never lowered again.
 //   * How many clusters of 2, 4, .. 16 blocks the GPU holds at once.  Every router launch takes more than half of an
-//     SM's shared memory (the operand ring alone is over 136 KB at any width), so one block fits an SM and the answer
+//     SM's shared memory (the operand ring alone is 136 KB or more at any width), so one block fits an SM and the answer
 //     is the same for all instances and shapes.
 static fb_status set_up_device(fb_ctx* ctx, int device, const DeviceLimits& dev) {
   static std::mutex mutex;

@@ -360,6 +360,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
     p.tmem_cols = next_pow2_at_least_32(2 * p.issuers * ctx->N);
   }
   const int blocks = 2 * J * clusters;
+  p.prefetch_kb = probe == 0 ? fb::kPrefetchBytes / fb::kATileBytes / blocks : 0;
   // every block publishes its counts once: as many tickets as blocks that own a tile of the counted pass
   p.ticket_target = blocks < p.tiles_first * J ? blocks : p.tiles_first * J;
   RouterKernelFn fn;
@@ -436,6 +437,7 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   dp.inv_perm = inv_perm;
   dp.rank_load = rank_load;
   dp.status = ctx->status;
+  dp.stamps = ctx->stamps;
   // one block per SM at most: more tiles than that are walked in runs (every block reads the whole
   // histogram table once, so more blocks would only read it more often)
   const int blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;

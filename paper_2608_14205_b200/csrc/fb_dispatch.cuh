@@ -12,6 +12,11 @@
 // everything a block needs from global memory is requested at once, before anything depends on it
 // (placement, first tile's ids, the whole histogram table 16 experts per load), and the launch may
 // overlap the end of the router kernel (programmatic dependent launch).
+// The next kernel of the stream may set itself up, and a router kernel bring rows into L2 (prefetch_operands), while a
+// kernel of this file or the planner kernel runs - but not before its wait is over: allowed earlier, a whole chain of small kernels
+// starts during the main loop of the router kernel before them, and the next router kernel takes SMs and bandwidth
+// from it (layer calls back to back, allowed before and after the wait: 1733 tokens, 256 experts 31.6 and 30.7 us, 1000 x 128
+// 19.8 and 18.9; a shard's six launches 58.0 and 56.6).
 // Measured on whole layer steps back to back (B200), against 32-bit tables read column by column
 // behind a serialised launch: 1733 tokens, 256 experts 48.5 -> 44.4 us; 8192 tokens, 128 experts
 // 37.9 -> 36.2 us; 131072 tokens, 128 experts 256.5 -> 252.4 us.  Without the dependent launch the
@@ -23,6 +28,30 @@
 #include "../../include/freebalance.h"
 #include "fb_planner.cuh"
 #include "fb_ptx.cuh"
+
+// Phase time stamps (builds with -DFB_TIMING only; see fb_set_stamp_buffer): one designated
+// thread per role writes %globaltimer (slot i) and clock64 (slot 32 + i) of its block at the
+// phase boundaries below.  Without the flag the macro is empty and the kernels carry none of it.
+//   0 block start          1 set-up done            2 accumulators complete  3 keys computed
+//   4 barrier              5 groups chosen          7 candidates collected   8 candidates ranked
+//   9 top-k read back     10 outputs written       11 counts published      12 planner done
+//  13 block exit          14 first load issued     15 last load issued      16 first operands landed
+//  17 last MMA issued     18 planner entered       19 rank loads formed    20 greedy loop left
+// and in the dispatch-index kernel
+//  21 block start         22 wait over             23 tables read           24 barrier
+//  25 totals formed       26 planner done          27 offsets formed        28 block exit
+#ifdef FB_TIMING
+#define FB_STAMP(i, who)                                                                    \
+  do {                                                                                      \
+    if (p.stamps != nullptr && threadIdx.x == (who)) {                                      \
+      unsigned long long* st_ = p.stamps + static_cast<size_t>(blockIdx.x) * 64;           \
+      st_[i] = global_timer_ns();                                                           \
+      st_[32 + (i)] = static_cast<unsigned long long>(clock64());                           \
+    }                                                                                       \
+  } while (0)
+#else
+#define FB_STAMP(i, who) do { } while (0)
+#endif
 
 namespace fb {
 
@@ -54,6 +83,7 @@ struct DispatchParams {
   const uint8_t* early_counts;     // [num_slices][slice_row_bytes(E)]
   uint32_t* counts_out;            // [E]
   PlanParams plan;
+  unsigned long long* stamps;      // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
 };
 
 // Four bytes as two pairs of 16-bit counters.
@@ -176,9 +206,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int E = p.E, k = p.k;
   const int tile = static_cast<int>(blockIdx.x);
-  // The next router kernel of the stream may set itself up while this grid runs (it waits for
-  // this grid's completion before it reads anything).
-  pdl_launch_dependents();
+  FB_STAMP(21, 0);
   if (t == 0) bad = 0;
   if (t < FB_MAX_EXPERTS) { expert_at[t] = -1; mask[t] = make_uint4(0, 0, 0, 0); }
   if constexpr (kPlan) plan_clear(plan, t, kDispatchThreads);
@@ -193,6 +221,8 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   const int first_slice = tile * p.slices_per_tile;
   __syncthreads();
   pdl_wait();                                    // from here on: what the router kernel wrote
+  pdl_launch_dependents();
+  FB_STAMP(22, 0);
   // ---- everything the block needs from global memory, before anything depends on it
   const int my_slot = t < E ? p.expert_to_slot[t] : 0;
   int e = (t < kDispatchTile * k && flat < n_assign) ? p.topk_ids[flat] : -1;
@@ -220,7 +250,9 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     }
   }
   if constexpr (kPlan) plan_place_ranks(p.plan, plan, t, kDispatchThreads);
+  FB_STAMP(23, 0);
   __syncthreads();
+  FB_STAMP(24, 0);
   if (st < 8 * U) {
     uint32_t all0 = 0, all1 = 0, bef0 = 0, bef1 = 0;
     const int w0 = warp - warp % kSumWarps;
@@ -240,10 +272,12 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     }
   }
   __syncthreads();
+  FB_STAMP(25, 0);
   if constexpr (kPlan)
     if (warp == 0) plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
   const uint32_t ahead = e >= 0 ? rows_before(mask[e], row) : 0u;
   if constexpr (kPlan) __syncthreads();
+  FB_STAMP(26, 0);
   bool usable = bad == 0;
   if constexpr (kPlan) usable = plan.bad == 0;
   uint32_t count = 0, all = 0;
@@ -266,6 +300,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     if (!kPlan && t == 0 && tile == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
     return;
   }
+  FB_STAMP(27, 0);
   if (tile == 0) write_offsets(p, offs, t);
   if (e >= 0) {
     const long long pos = static_cast<long long>(base[e]) + ahead;
@@ -277,6 +312,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
       p.inv_perm[flat] = static_cast<int32_t>(pos);
     }
   }
+  FB_STAMP(28, 0);
 }
 
 // A run of consecutive tiles per block (more tiles than SMs).
@@ -308,9 +344,6 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
   const int per_block = (p.num_tiles + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
   const int tile_begin = static_cast<int>(blockIdx.x) * per_block;
   const int tile_end = min(p.num_tiles, tile_begin + per_block);
-  // The next router kernel of the stream may set itself up while this grid runs (it waits for
-  // this grid's completion before it reads anything).
-  pdl_launch_dependents();
   if (t == 0) bad = 0;
   if (t < FB_MAX_EXPERTS) owner[t] = -1;
   // Thread t owns assignment t of the tile: row t / k, choice t % k (exact for t < 8192, k <= 8).
@@ -326,6 +359,7 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
     return (e < 0 || e >= E) ? 0 : e;
   };
   pdl_wait();                                    // from here on: what the router kernel wrote
+  pdl_launch_dependents();
   const int my_slot_in = t < E ? p.expert_to_slot[t] : 0;
   int ids[kBatch];
 #pragma unroll
@@ -484,8 +518,8 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
 // counts[p] = number of local assignments in slot p
 __global__ void fb_slot_counts_kernel(const uint32_t* __restrict__ slot_offsets, int E, uint32_t* __restrict__ counts) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();
   if (p < E) counts[p] = __ldcg(slot_offsets + p + 1) - __ldcg(slot_offsets + p);
 }
 
@@ -513,8 +547,8 @@ fb_dispatch_globalize_kernel(const __grid_constant__ GlobalizeParams p) {
   __shared__ int32_t slot_of[FB_MAX_EXPERTS];
   static_assert(kGlobalizeThreads == FB_MAX_EXPERTS, "one thread per slot");
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();
   const long long n = static_cast<long long>(p.T) * p.k;
   long long q = static_cast<long long>(blockIdx.x) * kGlobalizeThreads + t;
   int e = q < n ? p.topk_ids[q] : -1;

@@ -39,6 +39,7 @@ struct PersistShared {
   uint32_t tmem_base;
   int32_t abort_flag;
   int32_t accum_ok;
+  int32_t started;                           // the wait for the kernels before this one is over (prefetch_operands)
   int32_t tiles_done;                        // by this block, so far: restarts the limit of the wait on counts_bar
   int32_t any_unranked[4];                   // per row quarter: some row has too many or too few candidates
   int32_t issuer_progress[2];                // where both issuers use a stage: see issuer_turn_wait
@@ -112,6 +113,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
 
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
+    sh.started = 0;
     sh.tiles_done = 0;
     for (int q = 0; q < 4; ++q) sh.any_unranked[q] = 0;
     sh.issuer_progress[0] = -1;
@@ -146,9 +148,19 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   __syncthreads();
   cluster_arrive_relaxed(); cluster_wait();  // the partner's barriers and tensor memory are ready too
   tcgen05_fence_after();
+  TileWalk walk;
+  walk.pair_first = pair_first;
+  walk.pair_stride = pair_stride;
+  walk.total_pairs = total_pairs;
+  walk.pairs_per_pass = pairs_per_pass;
+  walk.kb0 = 0;
+  walk.n_kb = p.num_kb;
+  walk.cluster_rank = cta_rank;
+  if (warp == kSecondIssuerWarp) prefetch_operands(p, &tmap_x, &tmap_x2, walk, &sh.started);
   // Everything above touched only this block's own state and the call's parameters; from here on
   // the kernel reads memory that earlier work of the stream may have written.
   pdl_wait();
+  if (threadIdx.x == 0) *static_cast<volatile int32_t*>(&sh.started) = 1;
   // From here on the next kernel of the stream may be scheduled (if it was launched with
   // programmatic stream serialization - the library's own router launches are): its blocks
   // take the SMs as this grid's blocks leave them and do their set-up while the last blocks
@@ -161,14 +173,6 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   if (warp == kSecondIssuerWarp && cta_rank == 1) {
     if (p.mode != kModeDispatch && pair_first < pairs_per_pass) finish_early_pass(sh, p, lane, abort_flag);
   } else if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
-    TileWalk walk;
-    walk.pair_first = pair_first;
-    walk.pair_stride = pair_stride;
-    walk.total_pairs = total_pairs;
-    walk.pairs_per_pass = pairs_per_pass;
-    walk.kb0 = 0;
-    walk.n_kb = p.num_kb;
-    walk.cluster_rank = cta_rank;
     if (warp == 0)
       produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
     else if (cta_rank == 0 && (warp == 1 || p.issuers == 2))

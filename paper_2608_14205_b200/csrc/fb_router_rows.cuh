@@ -106,6 +106,7 @@ struct RowsShared {
   int32_t abort_flag;
   int32_t is_last;
   int32_t accum_ok;
+  int32_t started;                           // the wait for the kernels before this one is over (prefetch_operands)
   int32_t issuer_progress[2];                // where both issuers use a stage: see issuer_turn_wait
   uint16_t quad_word[FB_MAX_EXPERTS / 4];    // where columns 4 q .. 4 q + 3 lie in a staged row
   alignas(16) float logit_bias[FB_MAX_EXPERTS];
@@ -603,6 +604,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   if (threadIdx.x == 0) {
     sh.abort_flag = 0;
     sh.is_last = 0;
+    sh.started = 0;
     sh.issuer_progress[0] = -1;
     sh.issuer_progress[1] = -1;
     for (int s = 0; s < p.stages; ++s) {
@@ -632,22 +634,24 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   __syncthreads();
   cluster_arrive_relaxed(); cluster_wait();  // the other blocks' barriers and tensor memory are ready too
   tcgen05_fence_after();
+  TileWalk walk;
+  walk.pair_first = pair_first;
+  walk.pair_stride = pair_stride;
+  walk.total_pairs = total_pairs;
+  walk.pairs_per_pass = pairs_per_pass;
+  walk.kb0 = kb0;
+  walk.n_kb = n_kb;
+  walk.cluster_rank = cluster_rank;
+  if (warp == kSecondIssuerWarp) prefetch_operands(p, &tmap_x, &tmap_x2, walk, &sh.started);
   // (see fb_router_kernel for these two)
   pdl_wait();
+  if (threadIdx.x == 0) *static_cast<volatile int32_t*>(&sh.started) = 1;
   pdl_launch_dependents();
   const uint32_t tmem_base = sh.tmem_base;
   FB_STAMP(1, 64);
   bool closing_arrived = false;              // this warp has delivered its arrival for the closing cluster barrier
 
   if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
-    TileWalk walk;
-    walk.pair_first = pair_first;
-    walk.pair_stride = pair_stride;
-    walk.total_pairs = total_pairs;
-    walk.pairs_per_pass = pairs_per_pass;
-    walk.kb0 = kb0;
-    walk.n_kb = n_kb;
-    walk.cluster_rank = cluster_rank;
     if (warp == 0)
       produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
     else if (cta_rank == 0 && (warp == 1 || p.issuers == 2))

@@ -80,3 +80,38 @@ def test_captured_calls_replay_bit_for_bit(name, T, pair_limit):
     assert ctx.fb_device_status() == 0
     ctx.fb_set_pair_limit(0)
     ctx.close()
+
+
+@pytest.mark.parametrize("name,T,pair_limit", [("tiny", 300, 0), ("qwen3", 8192, 0), ("dsv3", 1500, 0), ("dsv3", 1500, 2)])
+def test_inputs_written_right_before_a_call_are_the_ones_it_uses(name, T, pair_limit):
+    # A router kernel brings rows of its input into L2 while earlier kernels of the stream still run: calls queued back to
+    # back, with the hidden states written in between, must see what was written last.
+    wl = I.WORKLOADS[name]
+    layers = [I.make_layer(wl, l, 0, T=T) for l in range(2)]
+    ctx = P.make_context(wl, T)
+    ctx.fb_set_pair_limit(pair_limit)
+    dev = torch.device("cuda", ctx.device)
+    sb = layers[0].select_bias.to(dev) if layers[0].select_bias is not None else None
+    router = B.make_router(layers[0].W.to(dev), None, sb)
+    pi = layers[0].expert_to_slot.to(dev)
+    budget = B.make_budget(**P.budget_kwargs(wl, T))
+    src = [(li.h_prev.to(dev), li.H.to(dev)) for li in layers]
+    x, H = src[0][0].clone(), src[0][1].clone()
+    want = []
+    for a, b in src:
+        o = _buffers(wl, T, dev)
+        _calls(ctx, router, a, b, T, pi, budget, o)
+        torch.cuda.synchronize(dev)
+        want.append(o)
+    got = [_buffers(wl, T, dev) for _ in range(6)]
+    torch.cuda.synchronize(dev)
+    for i, o in enumerate(got):
+        a, b = src[i % 2]
+        _calls(ctx, router, a, b, T, pi, budget, _buffers(wl, T, dev))     # something to run ahead of
+        x.copy_(a); H.copy_(b)
+        _calls(ctx, router, x, H, T, pi, budget, o)
+    torch.cuda.synchronize(dev)
+    for i, o in enumerate(got):
+        for key in ("counts", "pi_out", "l_counts", "l_pi_out", "ids", "w", "so", "ro", "perm", "inv", "rl"):
+            assert torch.equal(o[key], want[i % 2][key]), (i, key)
+    assert ctx.fb_device_status() == 0

@@ -174,6 +174,8 @@ fb_status fill_plan(const fb_ctx* ctx, const fb_budget* b, const int32_t* pi, in
   if (b->gamma_num > FB_MAX_GAMMA_NUM) return FB_ERR_INVALID_ARG;
   pp->E = ctx->cfg.E;
   pp->R = ctx->cfg.R;
+  pp->per_rank = pp->E / pp->R;
+  pp->per_rank_inv = fb::per_rank_inverse(pp->per_rank);
   pp->max_swaps = b->max_swaps;
   pp->global_ns = b->global_ns;
   pp->rank_ns = b->rank_ns;
@@ -257,7 +259,8 @@ cudaError_t launch_dependent(void (*kernel)(Params...), int blocks, int threads,
 }
 
 fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* counts, cudaStream_t stream) {
-  const cudaError_t err = launch_dependent(fb::fb_plan_kernel, 1, fb::kPlanThreads, stream, pp, counts, ctx->status);
+  const cudaError_t err = launch_dependent(fb::plan_needs_general_loop(pp) ? fb::fb_plan_kernel<true> : fb::fb_plan_kernel<false>, 1,
+                                           fb::kPlanThreads, stream, pp, counts, ctx->status);
   ++ctx->launches;
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }

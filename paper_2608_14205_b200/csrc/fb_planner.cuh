@@ -17,6 +17,8 @@ constexpr uint32_t kPlanBarrierId = 1;    // named barrier of the router kernel'
 
 struct PlanParams {
   int32_t E, R;
+  int32_t per_rank;                     // E / R, and what replaces the division by it (rank_of_slot); host
+  uint32_t per_rank_inv;
   uint32_t max_swaps;
   uint64_t global_ns, rank_ns, link_ns;
   uint32_t tau_tokens;
@@ -38,19 +40,25 @@ struct PlanParams {
   int32_t* n_swaps;                     // device [1]
   uint32_t* load_before;                // device [R]
   uint32_t* load_after;                 // device [R]
-  unsigned long long* stamps;           // this block's 64 phase-stamp words (FB_TIMING builds) or nullptr
 };
+
+// s / per_rank for a slot s < 256: with inv = ceil(65536 / m) the quotient is at most s / 65536 < 1 / 256 too large, and
+// the fraction of s / m is at most 1 - 1 / m.
+__host__ __device__ constexpr uint32_t per_rank_inverse(int m) { return (65536u + static_cast<uint32_t>(m) - 1u) / static_cast<uint32_t>(m); }
+__device__ __forceinline__ int rank_of_slot(const PlanParams& p, int s) {
+  return static_cast<int>(static_cast<uint32_t>(s) * p.per_rank_inv >> 16);
+}
 
 // Phase stamps of the planner (FB_TIMING builds only): 18 planner entered, 19 rank loads formed,
 // 20 greedy loop left.
 #ifdef FB_TIMING
 #define FB_PLAN_STAMP(i)                                                                    \
   do {                                                                                      \
-    if (p.stamps != nullptr && lane == 0) {                                                 \
+    if (stamps != nullptr && lane == 0) {                                                   \
       unsigned long long t_;                                                                \
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_));                                \
-      p.stamps[i] = t_;                                                                     \
-      p.stamps[32 + (i)] = static_cast<unsigned long long>(clock64());                      \
+      stamps[i] = t_;                                                                       \
+      stamps[32 + (i)] = static_cast<unsigned long long>(clock64());                        \
     }                                                                                       \
   } while (0)
 #else
@@ -71,8 +79,8 @@ struct PlanShared {
   int32_t slot_of[FB_MAX_EXPERTS];       // expert -> slot (current placement)
   int32_t expert_at[FB_MAX_EXPERTS];     // slot -> expert
   uint8_t moved[FB_MAX_EXPERTS];
-  // fast loop: one word per slot - the expert placed there in bits 0..7, its count above (kSlotMoved once
-  // the expert has moved)
+  // fast loop: one word per slot - the expert placed there in bits 0..7, twice its count above (kSlotMoved in the
+  // place of a count once the expert has moved)
   alignas(16) uint32_t slot_cnt[FB_MAX_EXPERTS];
   uint8_t rank_of[FB_MAX_EXPERTS];       // expert -> rank under the placement as given
   uint8_t node_of[FB_MAX_RANKS];         // rank -> node (all 0 when every rank is in one node)
@@ -85,9 +93,9 @@ struct PlanShared {
   int32_t fast;                          // the fast loop ran: the placement is in slot_cnt, not in expert_at
 };
 
-constexpr uint32_t kSlotMoved = 1u << 23;       // as a count
-static_assert(FB_MAX_COUNT_SUM <= kSlotMoved / 4 && FB_MAX_EXPERTS <= 256, "slot word layout");
-__device__ __forceinline__ uint32_t slot_word(uint32_t count, int expert) { return count << 8 | static_cast<uint32_t>(expert); }
+constexpr uint32_t kSlotMoved = 1u << 22;       // as a count
+static_assert(2 * FB_MAX_COUNT_SUM <= kSlotMoved && FB_MAX_EXPERTS <= 256, "slot word layout");
+__device__ __forceinline__ uint32_t slot_word(uint32_t count, int expert) { return count << 9 | static_cast<uint32_t>(expert); }
 
 // true if x is a better choice than y: larger benefit / cost, compared exactly as
 // cross products in 128 bits; equal ratios -> smaller (a, b, ea, eb).
@@ -119,7 +127,7 @@ __device__ __forceinline__ void plan_place(const PlanParams& p, PlanShared& sh, 
   const bool inside = s >= 0 && s < p.E;
   sh.slot_of[e] = s;
   sh.moved[e] = 0;
-  sh.rank_of[e] = static_cast<uint8_t>(inside ? s / (p.E / p.R) : 0);
+  sh.rank_of[e] = static_cast<uint8_t>(inside ? rank_of_slot(p, s) : 0);
   if (!inside || atomicExch(&sh.expert_at[s], e) != -1) sh.bad = 1;
 }
 __device__ __forceinline__ void plan_place_ranks(const PlanParams& p, PlanShared& sh, int t, int nthreads) {
@@ -173,28 +181,36 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 // constant up to v = 2 M2 - La - Lb.  A pair is useful exactly if v < D (0 < d < D), and with
 // gamma_num = 0 also M2 < La, which the same comparison tests.  The best pair is therefore the one
 // with the smallest v (clamped from below when gamma_num = 0), ties to the smallest pair.
-// A moved expert counts as 2^23 tokens: paired with an unmoved one v is beyond any D, with a moved one it is
-// D, so no candidate has to be tested - only the smallest v is, against D.
+// A moved expert counts as 2^22 tokens (kSlotMoved): paired with an unmoved one v is 2^21 or more, beyond any D that it
+// could be less than, with a moved one it is D, so no candidate has to be tested - only the smallest v is, against D.
 //
 // Lane l tries expert slot l / g of the heavy rank with kPerLane slots of the light one, g lanes per
-// heavy slot; slots beyond m repeat the last one (the same pair twice changes nothing).  kPerLane == 0: more
+// heavy slot; slots beyond m repeat the last one (the same pair twice in a lane changes nothing; lanes with nothing
+// but repeats stand aside).  kPerLane == 0: more
 // than 16 experts per rank, lane l takes the heavy slots l, l + 32, ... with every light one (20 experts per
 // rank, 4 tokens: layer step 63 us with the general loop below, 22 with this one).  A lane keeps the
-// packed (load, rank) keys of its two ranks, so an iteration is: two warp reductions for the frontier, the
-// slot words, the smallest v of the lane, one reduction for v, one for the pair (the lane rides along), one
-// shuffle for the moved tokens.
+// packed (load, rank) keys of its two ranks.
+//
+// What an iteration waits for: the slot words, a few operations, and ONE warp reduction, over v, the sign of 2 d - D and
+// the lane - d follows from v and the sign in every lane.  The frontier of the next iteration is the larger
+// (smaller) of the two new loads and of the other ranks' largest (smallest), which is reduced meanwhile.  Only where
+// two lanes hold the smallest v a second reduction finds the smaller pair.  (Integer operations issue every other cycle
+// from a single warp: 600 cycles per iteration with 16 experts per rank, 385 with 8.)  In line in its kernels, with the
+// parameters out of constant memory, everything around the loop takes 630 cycles; as a function with a pointer to them it
+// took 1400: layer calls of 8192 tokens, 128 experts 25.9 -> 24.3 us, 40 x 128 16.7 -> 15.3, 1733 x 256 30.7 -> 29.6.
 // kBooks: two cost classes, or per-rank or per-link budgets that can bind.  Otherwise the budgets allow
 // a fixed number of swaps (swap_cap) and the loop keeps no books at all.
 template <int kPerLane, bool kBooks>
 __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanShared& sh, int lane,
                                                       int& L0, int& L1, bool write) {
-  const int R = p.R, m = p.E / R;
+  const int m = p.per_rank;
   const uint32_t full = 0xffffffffu;
-  constexpr uint32_t kNone = 0xffffffffu;
+  constexpr uint32_t kNone = 0xffffffffu, kNoPair = (1u << 24) - 1;
   constexpr int kNarrow = kPerLane == 0 ? 1 : kPerLane;
   constexpr int g = kPerLane == 8 ? 2 : (kPerLane == 2 ? 4 : 8);     // m <= 16, <= 8, <= 4
   const int ia = min(lane / g, m - 1), j0 = (lane % g) * kNarrow;
   const bool whole = m == g * kNarrow;                            // the lane's light slots are contiguous and exist
+  const bool aside = kPerLane != 0 && (lane / g >= m || j0 >= m);
   const bool flat = p.gamma_den == 0 || p.gamma_num == 0;
   const uint32_t tau = p.tau_tokens, max_swaps = kBooks ? p.max_swaps : p.swap_cap;
   // frontier keys (lowest index on ties): max of load << 6 | (63 - rank), min of load << 6 | rank
@@ -206,15 +222,14 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
   uint32_t my_links[4] = {kNone, kNone, kNone, kNone};            // lane i keeps the links of swaps i, i+32, ...
   unsigned long long global_spent = 0;
   uint32_t n = 0;
-  __syncwarp();
+  uint32_t hi_key = __reduce_max_sync(full, max(h0, h1));
+  uint32_t lo_key = __reduce_min_sync(full, min(l0, l1));
   while (n < max_swaps) {
-    const uint32_t hi_key = __reduce_max_sync(full, max(h0, h1));
-    const uint32_t lo_key = __reduce_min_sync(full, min(l0, l1));
     const int a = 63 - static_cast<int>(hi_key & 63u), b = static_cast<int>(lo_key & 63u);
     const int La = static_cast<int>(hi_key >> 6), Lb = static_cast<int>(lo_key >> 6);
     const int D = La - Lb;
     const int base_a = a * m, base_b = b * m;
-    uint32_t wa = 0, wb[kNarrow];                                 // slot words: count, expert
+    uint32_t wa = 0, wb[kNarrow];                                 // slot words: twice the count, expert
     if constexpr (kPerLane != 0) {
       wa = sh.slot_cnt[base_a + ia];
       if (kPerLane == 8 && whole) {
@@ -254,56 +269,64 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
       }
       if (stop) break;
     }
-    int v_floor = 0;
-    if (flat) {
-      const uint32_t m2 = max(lane != a && lane != b ? h0 >> 6 : 0u, lane + 32 != a && lane + 32 != b ? h1 >> 6 : 0u);
-      v_floor = 2 * static_cast<int>(__reduce_max_sync(full, m2)) - La - Lb;
-    }
-    // ---- smallest v of this lane, ties -> smallest pair; where its experts are, and the tokens moved a -> b
-    uint32_t mine = (1u << 24) - 1, pair = 0;
-    int sa = 0, sb = 0, delta = 0;
+    // the other ranks' largest and smallest load
+    const bool in0 = lane == a || lane == b, in1 = lane + 32 == a || lane + 32 == b;
+    const uint32_t hi_rest = __reduce_max_sync(full, max(in0 ? 0u : h0, in1 ? 0u : h1));
+    const uint32_t lo_rest = __reduce_min_sync(full, min(in0 ? kNone : l0, in1 ? kNone : l1));
+    const int v_floor = flat ? 2 * static_cast<int>(hi_rest >> 6) - La - Lb : 0;
+    // ---- smallest v of this lane, ties -> smallest pair; where its experts are, and 2 d - D
+    uint32_t mine = kNoPair, pair = 0;
+    int sa = 0, sb = 0, off = 0;
     if constexpr (kPerLane != 0) {
-      const int x = 2 * static_cast<int>(wa >> 8) - D;
+      const int y = static_cast<int>(wa >> 8) - D;
       uint32_t key[kNarrow];
 #pragma unroll
-      for (int t = 0; t < kNarrow; ++t) {
-        const int v = max(abs(x - 2 * static_cast<int>(wb[t] >> 8)), v_floor);
-        key[t] = static_cast<uint32_t>(min(v, (1 << 24) - 1)) << 8 | (wb[t] & 0xffu);
-      }
+      for (int t = 0; t < kNarrow; ++t)                           // v << 8 | expert of the light rank
+        key[t] = __byte_perm(static_cast<uint32_t>(max(abs(y - static_cast<int>(wb[t] >> 8)), v_floor)), wb[t], 0x2104);
       uint32_t best = key[0];
 #pragma unroll
       for (int t = 1; t < kNarrow; ++t) best = min(best, key[t]);
-      mine = best >> 8;
+      mine = aside ? kNoPair : best >> 8;
       pair = (wa & 0xffu) << 8 | (best & 0xffu);
       sa = base_a + ia;
+      uint32_t w_best = wb[0];
+      sb = base_b + min(j0, m - 1);
 #pragma unroll
-      for (int t = kNarrow - 1; t >= 0; --t)
-        if (key[t] == best) { sb = base_b + min(j0 + t, m - 1); delta = static_cast<int>(wa >> 8) - static_cast<int>(wb[t] >> 8); }
+      for (int t = kNarrow - 1; t > 0; --t)
+        if (key[t] == best) { sb = base_b + min(j0 + t, m - 1); w_best = wb[t]; }
+      off = y - static_cast<int>(w_best >> 8);
     } else {
       for (int i = lane; i < m; i += 32) {
         const uint32_t wi = sh.slot_cnt[base_a + i];
-        const int x = 2 * static_cast<int>(wi >> 8) - D;
+        const int y = static_cast<int>(wi >> 8) - D;
         for (int jj = 0; jj < m; jj += 8) {
           uint32_t wj[8];
 #pragma unroll
           for (int t = 0; t < 8; ++t) wj[t] = sh.slot_cnt[base_b + min(jj + t, m - 1)];
 #pragma unroll
           for (int t = 0; t < 8; ++t) {
-            const uint32_t v = static_cast<uint32_t>(min(max(abs(x - 2 * static_cast<int>(wj[t] >> 8)), v_floor), (1 << 24) - 1));
+            const int o = y - static_cast<int>(wj[t] >> 8);
+            const uint32_t v = static_cast<uint32_t>(max(abs(o), v_floor));
             const uint32_t pr = (wi & 0xffu) << 8 | (wj[t] & 0xffu);
             if (v < mine || (v == mine && pr < pair)) {
               mine = v; pair = pr; sa = base_a + i; sb = base_b + min(jj + t, m - 1);
-              delta = static_cast<int>(wi >> 8) - static_cast<int>(wj[t] >> 8);
+              off = o;
             }
           }
         }
       }
     }
-    const uint32_t top = __reduce_min_sync(full, mine);
+    const uint32_t sign_lane = (off < 0 ? 32u : 0u) | static_cast<uint32_t>(lane);
+    uint32_t win = __reduce_min_sync(full, mine << 6 | sign_lane);
+    const uint32_t top = win >> 6;
     if (top >= static_cast<uint32_t>(D)) break;                   // Algorithm 1 lines 6-7
-    const uint32_t win = __reduce_min_sync(full, mine == top ? pair << 5 | static_cast<uint32_t>(lane) : kNone);
+    const uint32_t holders = __ballot_sync(full, mine == top);
+    if ((holders & (holders - 1)) != 0)                           // (the same in all lanes)
+      win = __reduce_min_sync(full, mine == top ? pair << 6 | sign_lane : kNone);
     const int src = static_cast<int>(win & 31u);
-    const int dlt = __shfl_sync(full, delta, src);
+    // tokens moved a -> b: (D + off) / 2 of the chosen lane
+    const int dlt = flat ? __shfl_sync(full, (D + off) >> 1, src)
+                         : (D + ((win & 32u) != 0 ? -static_cast<int>(top) : static_cast<int>(top))) >> 1;
     if (lane == src) {
       // the two experts trade slots
       sh.slot_cnt[sa] = slot_word(kSlotMoved, static_cast<int>(pair & 0xffu));
@@ -312,13 +335,16 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
       // The accepted swap stays in shared memory until the loop is over (ranks and expert ids
       // are below 256: one word; link_key is otherwise unused on this path): a global store
       // here would be waited for at the warp barrier below, once per iteration.
-      sh.link_key[n] = static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 | (win >> 5);
+      sh.link_key[n] = static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 | pair;
     }
     const uint32_t moved = static_cast<uint32_t>(dlt) << 6;
     if (lane == a) { h0 -= moved; l0 -= moved; }
     if (lane + 32 == a) { h1 -= moved; l1 -= moved; }
     if (lane == b) { h0 += moved; l0 += moved; }
     if (lane + 32 == b) { h1 += moved; l1 += moved; }
+    const uint32_t new_a = static_cast<uint32_t>(La - dlt) << 6, new_b = static_cast<uint32_t>(Lb + dlt) << 6;
+    hi_key = max(hi_rest, max(new_a | static_cast<uint32_t>(63 - a), new_b | static_cast<uint32_t>(63 - b)));
+    lo_key = min(lo_rest, min(new_a | static_cast<uint32_t>(a), new_b | static_cast<uint32_t>(b)));
     if (kBooks) {
       if (static_cast<int>(n & 31u) == lane) {
 #pragma unroll
@@ -505,10 +531,11 @@ __device__ __noinline__ void plan_loop_general(const PlanParams& p, PlanShared& 
 // registers and code would otherwise weigh on every router kernel.
 // write: whether this warp's results go to global memory (several blocks may replay a plan, see the
 // dispatch index); only for instances without the general loop.
+// In line: its parameters come out of constant memory that way (see plan_loop_uniform).
 template <bool kGeneral>
-__device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh, int lane, int* status,
-                                             bool write = true) {
-  const int E = p.E, R = p.R, m = E / R;
+__device__ __forceinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh, int lane, int* status,
+                                                bool write = true, unsigned long long* stamps = nullptr) {
+  const int R = p.R, m = p.per_rank;
   const uint32_t full = 0xffffffffu;
   __syncwarp();
   FB_PLAN_STAMP(18);
@@ -571,5 +598,12 @@ __device__ __noinline__ void plan_swaps_warp(const PlanParams& p, PlanShared& sh
   }
 }
 
+// The same as a function of its own, for the router kernels, where most calls do not reach it: with the planner's code in the
+// kernel a layer call of 8192 tokens took 23.0 us and takes 22.8 without, of 131072 tokens 219 and 217; prediction and
+// plan of 300 tokens, which reaches it, 13.8 and 13.9.
+__device__ __noinline__ void plan_swaps_apart(const PlanParams& p, PlanShared& sh, int lane, int* status,
+                                              unsigned long long* stamps) {
+  plan_swaps_warp<false>(p, sh, lane, status, true, stamps);
+}
 
 }  // namespace fb

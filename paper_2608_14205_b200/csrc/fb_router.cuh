@@ -450,15 +450,9 @@ __device__ __forceinline__ void publish_counts(Shared& sh, const RouterParams& p
     if (sh.abort_flag) { if (et == 0) atomicCAS(p.status, 0, FB_ERR_TIMEOUT); }
     if (run_planner) {
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
-      if (warp == 2) {
-#ifdef FB_TIMING
-        PlanParams pt = p.plan;
-        pt.stamps = p.stamps != nullptr ? p.stamps + static_cast<size_t>(blockIdx.x) * 64 : nullptr;
-        plan_swaps_warp<false>(pt, sh.plan, lane, p.status);
-#else
-        plan_swaps_warp<false>(p.plan, sh.plan, lane, p.status);
-#endif
-      }
+      if (warp == 2)
+        plan_swaps_apart(p.plan, sh.plan, lane, p.status,
+                         p.stamps != nullptr ? p.stamps + static_cast<size_t>(blockIdx.x) * 64 : nullptr);
       named_bar_sync(kPlanBarrierId, kEpilogueThreads);
       plan_write_placement(p.plan, sh.plan, et, kEpilogueThreads);
     }
@@ -1061,6 +1055,8 @@ fb_wait_selftest_kernel(uint64_t limit_ns, int32_t steps, int32_t* status, uint6
 
 // Stand-alone planner: placement and counts by one thread per expert (both loads in flight at once;
 // a single warp walking them took 11 of the kernel's 13 us), the decision by one warp.
+// kGeneral: for plans that need the general loop (plan_needs_general_loop).
+template <bool kGeneral>
 __global__ void __launch_bounds__(kPlanThreads, 1)
 fb_plan_kernel(const __grid_constant__ PlanParams p, const uint32_t* __restrict__ counts, int32_t* status) {
   __shared__ PlanShared sh;
@@ -1075,7 +1071,7 @@ fb_plan_kernel(const __grid_constant__ PlanParams p, const uint32_t* __restrict_
   __syncthreads();
   if (t < p.E) plan_put_count(sh, t, count);
   __syncthreads();
-  if (t < 32) plan_swaps_warp<true>(p, sh, t, status);
+  if (t < 32) plan_swaps_warp<kGeneral>(p, sh, t, status);
   __syncthreads();
   plan_write_placement(p, sh, t, kPlanThreads);
 }

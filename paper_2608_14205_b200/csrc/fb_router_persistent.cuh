@@ -82,7 +82,7 @@ __device__ __forceinline__ void finish_early_pass(PersistShared& sh, const Route
   }
   if (lane == 0) *p.ticket = 0;
   if (!planner) return;
-  plan_swaps_warp<false>(p.plan, sh.plan, lane, p.status);
+  plan_swaps_apart(p.plan, sh.plan, lane, p.status, nullptr);
   __syncwarp();
   plan_write_placement(p.plan, sh.plan, lane, 32);
 }

@@ -65,7 +65,8 @@ struct fb_ctx {
   uint32_t* counts_scratch = nullptr;   // [256], zero between calls
   uint32_t* ticket = nullptr;           // [1],   zero between calls
   int32_t* status = nullptr;            // [1]
-  uint8_t* early_counts = nullptr;      // the same for the early pass of a layer call whose plan is made with the index
+  uint32_t* totals = nullptr;           // [2][256], zero between calls: its sums, and the early pass's where the plan is made with the index
+  uint32_t* index_ticket = nullptr;     // [1],   zero between calls
   uint8_t* slice_counts = nullptr;      // [max_slices][slice_row_bytes(E)]: per-slice histograms for the dispatch index
   // descriptor cache
   MapEntry x_maps[kMapCache];
@@ -302,6 +303,8 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.early_ids = early_ids;
   p.early_logits = early_logits;
   p.slice_counts = ctx->slice_counts;
+  p.totals = ctx->totals;
+  p.early_totals = ctx->totals != nullptr ? ctx->totals + FB_MAX_EXPERTS : nullptr;
   p.stamps = ctx->stamps;
   p.probe = probe;
   if (plan) p.plan = *plan;
@@ -349,7 +352,6 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.defer_counts = (mode == fb::kModeLayer && !several && tile_per_block && p.fuse_planner && deferred_out != nullptr) ? 1 : 0;
   if (p.defer_counts) {
     p.fuse_planner = 0;
-    p.early_counts = ctx->early_counts;
     *deferred_out = true;
   }
   int clusters = tile_pairs;
@@ -430,7 +432,8 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   const int rows = fb::slice_rows(slices_per_tile);
   dp.num_slices = T / fb::kDispatchTile * slices_per_tile + (T % fb::kDispatchTile + rows - 1) / rows;
   dp.slice_counts = ctx->slice_counts;
-  dp.early_counts = ctx->early_counts;
+  dp.totals = ctx->totals;
+  dp.ticket = ctx->index_ticket;
   dp.counts_out = counts_out;
   if (plan) dp.plan = *plan;
   dp.expert_to_slot = expert_to_slot;
@@ -449,7 +452,9 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
                                                                  : fb::fb_dispatch_kernel<false>,
                                            blocks, fb::kDispatchThreads, stream, dp);
   ++ctx->launches;
-  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+  if (err == cudaSuccess) return FB_OK;
+  cudaMemsetAsync(ctx->totals, 0, 2 * FB_MAX_EXPERTS * sizeof(uint32_t), stream);   // what the router kernel has added
+  return FB_ERR_CUDA;
 }
 
 // The device that owns a device pointer (-1 if it is not device memory).
@@ -674,8 +679,10 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
   bool ok = dev_alloc(&ctx->counts_scratch, FB_MAX_EXPERTS) && dev_alloc(&ctx->ticket, 1) &&
        dev_alloc(&ctx->status, 1) &&
        dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E)) &&
-       dev_alloc(&ctx->early_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E));
+       dev_alloc(&ctx->totals, 2 * FB_MAX_EXPERTS) && dev_alloc(&ctx->index_ticket, 1);
   ok = ok && cudaMemset(ctx->counts_scratch, 0, FB_MAX_EXPERTS * sizeof(uint32_t)) == cudaSuccess &&
+       cudaMemset(ctx->totals, 0, 2 * FB_MAX_EXPERTS * sizeof(uint32_t)) == cudaSuccess &&
+       cudaMemset(ctx->index_ticket, 0, sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->ticket, 0, sizeof(uint32_t)) == cudaSuccess &&
        cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess;
   if (!ok) { fb_destroy(ctx); return FB_ERR_CUDA; }
@@ -687,7 +694,7 @@ fb_status fb_destroy(fb_ctx* ctx) {
   if (!ctx) return FB_OK;
   DeviceGuard guard(ctx->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->early_counts, ctx->st_hprev, ctx->st_H,
+  void* ptrs[] = {ctx->counts_scratch, ctx->ticket, ctx->status, ctx->slice_counts, ctx->totals, ctx->index_ticket, ctx->st_hprev, ctx->st_H,
                   ctx->st_pi, ctx->st_pi_out, ctx->st_counts, ctx->st_swaps, ctx->st_nswaps, ctx->st_load_before,
                   ctx->st_load_after, ctx->st_ids, ctx->st_w, ctx->st_slot_offsets, ctx->st_rank_offsets,
                   ctx->st_perm, ctx->st_inv_perm, ctx->st_rank_load};

@@ -3,10 +3,12 @@
 // come from prefix sums and population counts only - no atomic decides an output
 // position - so the result is unique and reproducible.
 //
-// Input: the router kernel's top-k ids and its per-slice expert histogram
+// Input: the router kernel's top-k ids, its per-slice expert histogram
 // slice_counts[slice][e] (slices_per_tile slices of slice_rows tokens per tile, one byte per expert: a
-// token names an expert at most once, so a count is at most 128).  One block per 128-token tile,
-// or per run of consecutive tiles when there are more tiles than blocks.
+// token names an expert at most once, so a count is at most 128) and its totals per expert, which the router blocks add up in
+// global memory.  One block per 128-token tile, or per run of consecutive tiles when there are more tiles than blocks.
+// A block needs, besides the totals, the counts of the tiles before its own: it adds up the rows of the table before it or
+// those from its first on, whichever are fewer.
 //
 // What bounds it: latency, not bandwidth (16 T k bytes of output are 2 MB at 16k tokens).  So
 // everything a block needs from global memory is requested at once, before anything depends on it
@@ -71,6 +73,8 @@ struct DispatchParams {
   int32_t num_slices, slices_per_tile;
   const int32_t* topk_ids;         // [T][k]
   const uint8_t* slice_counts;     // [num_slices][slice_row_bytes(E)]
+  uint32_t* totals;                // [2][FB_MAX_EXPERTS]: normal, early pass; this grid's last block puts them back to zero
+  uint32_t* ticket;                // zero on entry, zero again on exit
   const int32_t* expert_to_slot;   // [E]
   uint32_t* slot_offsets;          // [E+1]
   uint32_t* rank_offsets;          // [R+1]
@@ -78,9 +82,8 @@ struct DispatchParams {
   int32_t* inv_perm;               // [T*k]
   uint32_t* rank_load;             // [R]
   int32_t* status;
-  // fb_dispatch_kernel<true>: the histogram table of the early pass, the count vector and the plan that
-  // are formed from it, and whose output placement the index is made under
-  const uint8_t* early_counts;     // [num_slices][slice_row_bytes(E)]
+  // fb_dispatch_kernel<true>: the count vector and the plan that are formed from the early pass's totals, and whose
+  // output placement the index is made under
   uint32_t* counts_out;            // [E]
   PlanParams plan;
   unsigned long long* stamps;      // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
@@ -92,50 +95,43 @@ __device__ __forceinline__ void add_bytes(uint32_t& even, uint32_t& odd, uint32_
   odd += (w >> 8) & 0x00ff00ffu;
 }
 
-// What a thread holds of one 16-byte unit's column sums, and the sums over a warp: word i of a unit holds
-// bytes (4 (i / 2) + (i & 1)) and that + 2 as 16-bit counters.
-struct UnitSums {
-  uint32_t all[8], earlier[8];
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) all[i] = earlier[i] = 0;
+// Column sums over rows [first, last) of the histogram table.  A row is W = row_bytes / 4 words of four experts; a
+// warp reads 32 / W rows at a time (one where W > 16), lane l word l % W - and word l + 32 where W > 32 - and the warps take
+// turns, so that a lane adds one or two words per step and no sums have to be exchanged but those of the rows of one
+// step.  (With 16 bytes per lane, eight rows per warp and step, the sums went through 32 shuffles per warp.)
+struct RowSums {
+  uint32_t even[2], odd[2];          // two 16-bit counters each: bytes 0 and 2, bytes 1 and 3 of the lane's words
+};
+__device__ __forceinline__ RowSums add_rows(const uint8_t* table, int row_bytes, int first, int last, int warp, int warps,
+                                            int lane) {
+  RowSums s = {{0, 0}, {0, 0}};
+  const int W = row_bytes >> 2, at_once = W <= 16 ? 32 / W : 1;
+  const int sub = W <= 16 ? lane / W : 0, word = W <= 16 ? lane % W : lane;
+  const bool one = sub < at_once && word < W, two = lane + 32 < W;
+  const uint8_t* at = table + static_cast<size_t>(word) * 4;
+#pragma unroll 4
+  for (int r = first + warp * at_once + sub; r < last; r += warps * at_once) {
+    const uint8_t* row = at + static_cast<size_t>(r) * row_bytes;
+    const uint32_t v = one ? __ldcg(reinterpret_cast<const uint32_t*>(row)) : 0u;
+    const uint32_t w = two ? __ldcg(reinterpret_cast<const uint32_t*>(row + 128)) : 0u;
+    add_bytes(s.even[0], s.odd[0], v);
+    add_bytes(s.even[1], s.odd[1], w);
   }
-  __device__ __forceinline__ void add(const uint4& v, bool is_earlier) {
-    const uint32_t keep = is_earlier ? 0xffffffffu : 0u;
-    add_bytes(all[0], all[1], v.x); add_bytes(all[2], all[3], v.y);
-    add_bytes(all[4], all[5], v.z); add_bytes(all[6], all[7], v.w);
-    add_bytes(earlier[0], earlier[1], v.x & keep); add_bytes(earlier[2], earlier[3], v.y & keep);
-    add_bytes(earlier[4], earlier[5], v.z & keep); add_bytes(earlier[6], earlier[7], v.w & keep);
-  }
-  // Adds up the warp's threads and leaves the result in part[0 = all, 1 = earlier][i * U + unit]; U units
-  // per row, lane l of the warp holds unit (l + first) % U (nothing if !holds).  The whole warp calls it.
-  __device__ __forceinline__ void to_warp(uint32_t (*part)[FB_MAX_EXPERTS / 2], int U, int unit, int lane, bool holds) {
-    if ((U & (U - 1)) == 0) {                      // units of a warp repeat every U lanes
-      for (int off = U; off < 32; off <<= 1) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          all[i] += __shfl_xor_sync(0xffffffffu, all[i], off);
-          earlier[i] += __shfl_xor_sync(0xffffffffu, earlier[i], off);
-        }
-      }
-      if (lane < U) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { part[0][i * U + lane] = all[i]; part[1][i * U + lane] = earlier[i]; }
-      }
-    } else {
-      // a unit count that does not divide a warp (E = 160, say): shared-memory adds
-      for (int i = lane; i < 8 * U; i += 32) { part[0][i] = 0; part[1][i] = 0; }
-      __syncwarp();
-      if (holds) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (all[i]) atomicAdd(&part[0][i * U + unit], all[i]);
-          if (earlier[i]) atomicAdd(&part[1][i * U + unit], earlier[i]);
-        }
-      }
+  __syncwarp();
+  if (W <= 16) {                     // the rows of one step: lanes W apart
+    for (int off = at_once / 2 * W; off >= W; off = off / W / 2 * W) {
+      s.even[0] += __shfl_down_sync(0xffffffffu, s.even[0], off);
+      s.odd[0] += __shfl_down_sync(0xffffffffu, s.odd[0], off);
     }
   }
-};
+  return s;
+}
+// ... to part[word] = experts 4 w, 4 w + 2 in word 2 w and the two others in word 2 w + 1.
+__device__ __forceinline__ void store_row_sums(const RowSums& s, uint32_t* part, int row_bytes, int lane) {
+  const int W = row_bytes >> 2;
+  if (lane < W) *reinterpret_cast<uint2*>(part + 2 * lane) = make_uint2(s.even[0], s.odd[0]);
+  if (lane + 32 < W) *reinterpret_cast<uint2*>(part + 2 * lane + 64) = make_uint2(s.even[1], s.odd[1]);
+}
 
 template <bool kFirst, class A, class B> struct Choose { using type = A; };
 template <class A, class B> struct Choose<false, A, B> { using type = B; };
@@ -178,20 +174,31 @@ __device__ __forceinline__ void write_offsets(const DispatchParams& p, const uin
   for (int r = t; r < p.R; r += kDispatchThreads) p.rank_load[r] = offs[(r + 1) * m] - offs[r * m];
 }
 
+// The totals have been read by all blocks: the last one puts them back to zero for the next call.  By one warp, after a
+// barrier behind the block's reads (their values have arrived: nothing of this grid is still to be read).
+__device__ __forceinline__ uint32_t take_index_ticket(const DispatchParams& p, int lane) {
+  return lane == 0 ? atomicAdd(p.ticket, 1u) : 0u;
+}
+__device__ __forceinline__ void clear_totals(const DispatchParams& p, uint32_t ticket, int lane) {
+  if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
+  for (int i = lane; i < 2 * FB_MAX_EXPERTS; i += 32) p.totals[i] = 0;
+  if (lane == 0) *p.ticket = 0;
+}
+
 // One tile per block (at most as many tiles as SMs).  The work per expert does not depend on the
 // placement; the slots come in with one scan at the end.
 // kPlan: the swap planner runs in here as well, in every block (its decisions are integer and reproducible,
 // so no block waits for another; block 0 writes the outputs).  Used where a layer launch runs both passes at
-// the same time: counting through global memory, electing the last block of the early pass and planning in
-// it were 3 to 5 us at the end of the router kernel with every other SM idle; here the planner works beside
-// the loads of the index.  Layer steps: 512 tokens x 8 experts 15.3 -> 13.6 us, 40 x 128 20.1 -> 19.3,
-// 1733 x 256 36.0 -> 35.2, 8192 x 128 32.0 -> 31.5.
+// the same time: electing the last block of the early pass and planning in
+// it were 3 to 5 us at the end of the router kernel with every other SM idle.  Layer steps: 512 tokens x 8 experts 15.3 ->
+// 13.6 us, 40 x 128 20.1 -> 19.3, 1733 x 256 36.0 -> 35.2, 8192 x 128 32.0 -> 31.5.
+// The first warp plans as soon as totals and placement have arrived; the others add up the table and find every
+// assignment's place among its tile's meanwhile.  Against totals out of the tables of both passes, with the planner behind
+// them: 8192 x 128 24.2 -> 23.0 us, 1733 x 256 29.1 -> 28.1, 1000 x 128 17.6 -> 16.7, 40 x 128 15.1 -> 14.7.
+constexpr uint32_t kIndexPlanBarrier = 1, kIndexTableBarrier = 2;     // named barriers
 template <bool kPlan>
 __global__ void __launch_bounds__(kDispatchThreads, 1)
 fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
-  // threads [0, 512) add up the table of the normal pass, [512, 1024) that of the early pass (kPlan)
-  constexpr int kSumThreads = kPlan ? kDispatchThreads / 2 : kDispatchThreads;
-  constexpr int kSumWarps = kSumThreads / 32;
   struct Empty {};
   __shared__ int32_t expert_at[FB_MAX_EXPERTS];    // slot -> expert
   __shared__ uint32_t base[FB_MAX_EXPERTS];        // expert: assignments in earlier tiles; then the tile's first position
@@ -199,7 +206,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   __shared__ uint32_t offs[FB_MAX_EXPERTS + 1];    // exclusive prefix of total over slots
   __shared__ uint4 mask[FB_MAX_EXPERTS];           // rows of the tile that chose the expert
   __shared__ uint32_t warp_sum[FB_MAX_EXPERTS / 32];
-  __shared__ uint32_t part[kDispatchWarps][2][FB_MAX_EXPERTS / 2];
+  __shared__ alignas(8) uint32_t part[kDispatchWarps][FB_MAX_EXPERTS / 2];    // see store_row_sums
   __shared__ typename Choose<kPlan, PlanShared, Empty>::type plan;
   __shared__ int32_t bad;
 
@@ -209,75 +216,77 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   FB_STAMP(21, 0);
   if (t == 0) bad = 0;
   if (t < FB_MAX_EXPERTS) { expert_at[t] = -1; mask[t] = make_uint4(0, 0, 0, 0); }
-  if constexpr (kPlan) plan_clear(plan, t, kDispatchThreads);
+  if constexpr (kPlan) {
+    plan_clear(plan, t, kDispatchThreads);
+    plan_place_ranks(p.plan, plan, t, kDispatchThreads);
+  }
   // Thread t owns assignment t of the tile: row t / k, choice t % k (exact for t < 8192, k <= 8).
   const int row = (t * ((65536 + k - 1) / k)) >> 16;
   const long long flat = static_cast<long long>(tile) * kDispatchTile * k + t;
   const long long n_assign = static_cast<long long>(p.T) * k;
-  const int row_bytes = slice_row_bytes(E), U = row_bytes >> 4;
-  const int P = kSumThreads / U, st = t % kSumThreads;
-  const int unit = st % U, slice0 = st / U;
-  const uint8_t* table = t < kSumThreads ? p.slice_counts : p.early_counts;
+  const bool owns = t < kDispatchTile * k && flat < n_assign;
+  const int row_bytes = slice_row_bytes(E), W = row_bytes >> 2;
   const int first_slice = tile * p.slices_per_tile;
+  const bool later = 2 * first_slice > p.num_slices;               // fewer rows from this tile's first on than before it
+  const int row_first = later ? first_slice : 0, row_last = later ? p.num_slices : first_slice;
   __syncthreads();
   pdl_wait();                                    // from here on: what the router kernel wrote
   pdl_launch_dependents();
   FB_STAMP(22, 0);
   // ---- everything the block needs from global memory, before anything depends on it
   const int my_slot = t < E ? p.expert_to_slot[t] : 0;
-  int e = (t < kDispatchTile * k && flat < n_assign) ? p.topk_ids[flat] : -1;
-  UnitSums sums;
-  sums.clear();
-  if (slice0 < P) {
-#pragma unroll 4
-    for (int s = slice0; s < p.num_slices; s += P)
-      sums.add(__ldg(reinterpret_cast<const uint4*>(table + static_cast<size_t>(s) * row_bytes) + unit), s < first_slice);
-  }
-  if (t < kDispatchTile * k && flat < n_assign) {
+  const uint32_t my_total = t < E ? __ldcg(p.totals + t) : 0u;
+  const uint32_t my_early = kPlan && t < E ? __ldcg(p.totals + FB_MAX_EXPERTS + t) : 0u;
+  int e = owns ? p.topk_ids[flat] : 0;
 #ifdef FB_DEBUG
-    if (e < 0 || e >= E) atomicCAS(p.status, 0, FB_ERR_INTERNAL);       // an expert id outside [0, E)
+  if (e < 0 || e >= E) atomicCAS(p.status, 0, FB_ERR_INTERNAL);         // an expert id outside [0, E)
 #endif
-    if (e < 0 || e >= E) e = 0;
-    atomicOr(reinterpret_cast<uint32_t*>(&mask[e]) + (row >> 5), 1u << (row & 31));
-  }
-  const int warps = min(kSumWarps, (min(P, p.num_slices) * U + 31) >> 5);
-  if (warp % kSumWarps < warps) sums.to_warp(part[warp], U, unit, lane, slice0 < P);
+  if (e < 0 || e >= E) e = 0;
   if (t < E) {
+    total[t] = my_total;
     if constexpr (kPlan) {
       plan_place(p.plan, plan, t, my_slot);
+      plan_put_count_at(plan, t, my_slot, my_early, E);
+      if (tile == 0) p.counts_out[t] = my_early;
     } else {
       if (my_slot < 0 || my_slot >= E || atomicExch(&expert_at[my_slot], t) != -1) bad = 1;
     }
   }
-  if constexpr (kPlan) plan_place_ranks(p.plan, plan, t, kDispatchThreads);
-  FB_STAMP(23, 0);
-  __syncthreads();
-  FB_STAMP(24, 0);
-  if (st < 8 * U) {
-    uint32_t all0 = 0, all1 = 0, bef0 = 0, bef1 = 0;
-    const int w0 = warp - warp % kSumWarps;
-    for (int w = w0; w < w0 + warps; ++w) {
-      const uint32_t a = part[w][0][st], b = part[w][1][st];
-      all0 += a & 0xffffu; all1 += a >> 16;
-      bef0 += b & 0xffffu; bef1 += b >> 16;
-    }
-    const int un = st % U, i = st / U;
-    const int e0 = 16 * un + 4 * (i >> 1) + (i & 1), e1 = e0 + 2;
-    if (t < kSumThreads) {
-      if (e0 < E) { total[e0] = all0; base[e0] = bef0; }
-      if (e1 < E) { total[e1] = all1; base[e1] = bef1; }
-    } else if constexpr (kPlan) {
-      if (e0 < E) { plan_put_count(plan, e0, all0); if (tile == 0) p.counts_out[e0] = all0; }
-      if (e1 < E) { plan_put_count(plan, e1, all1); if (tile == 0) p.counts_out[e1] = all1; }
+  if (owns) atomicOr(reinterpret_cast<uint32_t*>(&mask[e]) + (row >> 5), 1u << (row & 31));
+  if constexpr (kPlan) {
+    if (warp < FB_MAX_EXPERTS / 32) named_bar_sync(kIndexPlanBarrier, FB_MAX_EXPERTS);
+    FB_STAMP(25, 0);
+    if (warp == 0) {
+      named_bar_arrive(kIndexTableBarrier, kDispatchThreads);
+      plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
     }
   }
+  uint32_t ticket = 0, ahead = 0;
+  if (!kPlan || warp != 0) {
+    constexpr int kFirst = kPlan ? 1 : 0;          // the first warp that adds rows
+    store_row_sums(add_rows(p.slice_counts, row_bytes, row_first, row_last, warp - kFirst, kDispatchWarps - kFirst, lane),
+                   part[warp], row_bytes, lane);
+    FB_STAMP(23, 32);
+    named_bar_sync(kIndexTableBarrier, kDispatchThreads);
+    FB_STAMP(24, 32);
+    if (warp == kDispatchWarps - 1) ticket = take_index_ticket(p, lane);
+    const int j = t - 32 * kFirst;
+    if (j < 2 * W) {
+      uint32_t s0 = 0, s1 = 0;
+#pragma unroll 8
+      for (int w = kFirst; w < kDispatchWarps; ++w) {
+        const uint32_t v = part[w][j];
+        s0 += v & 0xffffu; s1 += v >> 16;
+      }
+      const int e0 = 4 * (j >> 1) + (j & 1), e1 = e0 + 2;
+      if (e0 < E) base[e0] = later ? total[e0] - s0 : s0;
+      if (e1 < E) base[e1] = later ? total[e1] - s1 : s1;
+    }
+    ahead = rows_before(mask[e], row);
+  }
   __syncthreads();
-  FB_STAMP(25, 0);
-  if constexpr (kPlan)
-    if (warp == 0) plan_swaps_warp<false>(p.plan, plan, lane, p.status, tile == 0);
-  const uint32_t ahead = e >= 0 ? rows_before(mask[e], row) : 0u;
-  if constexpr (kPlan) __syncthreads();
   FB_STAMP(26, 0);
+  if (kPlan && warp == 0) ahead = rows_before(mask[e], row);
   bool usable = bad == 0;
   if constexpr (kPlan) usable = plan.bad == 0;
   uint32_t count = 0, all = 0;
@@ -294,24 +303,25 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
     if (t == E - 1) offs[E] = all;
   }
   __syncthreads();
+  FB_STAMP(27, 0);
   if constexpr (kPlan)
     if (tile == 0) plan_write_placement(p.plan, plan, t, kDispatchThreads);
-  if (!usable) {                                // not a bijection: report (the planner has), write no index
-    if (!kPlan && t == 0 && tile == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
-    return;
-  }
-  FB_STAMP(27, 0);
-  if (tile == 0) write_offsets(p, offs, t);
-  if (e >= 0) {
-    const long long pos = static_cast<long long>(base[e]) + ahead;
+  if (usable) {
+    if (tile == 0) write_offsets(p, offs, t);
+    if (owns) {
+      const long long pos = static_cast<long long>(base[e]) + ahead;
 #ifdef FB_DEBUG
-    if (pos < 0 || pos >= n_assign) atomicCAS(p.status, 0, FB_ERR_INTERNAL);   // a position outside [0, T k)
+      if (pos < 0 || pos >= n_assign) atomicCAS(p.status, 0, FB_ERR_INTERNAL);   // a position outside [0, T k)
 #endif
-    if (pos < n_assign) {
-      p.perm[pos] = static_cast<int32_t>(flat);
-      p.inv_perm[flat] = static_cast<int32_t>(pos);
+      if (pos < n_assign) {
+        p.perm[pos] = static_cast<int32_t>(flat);
+        p.inv_perm[flat] = static_cast<int32_t>(pos);
+      }
     }
+  } else if (!kPlan && t == 0 && tile == 0) {      // not a bijection: report (the planner has), write no index
+    atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
   }
+  if (warp == kDispatchWarps - 1) clear_totals(p, ticket, lane);
   FB_STAMP(28, 0);
 }
 
@@ -328,8 +338,8 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
   __shared__ uint16_t ahead_of[kBatch][FB_MAX_EXPERTS];   // the batch's assignments to this slot in earlier tiles
   // The per-warp sums of the histogram table are read before the tile loop starts and share their
   // memory with what the loop works on.
-  __shared__ union {
-    uint32_t part[kDispatchWarps][2][FB_MAX_EXPERTS / 2];   // [all / earlier slices][two 16-bit counters per word]
+  __shared__ alignas(16) union {
+    uint32_t part[kDispatchWarps][FB_MAX_EXPERTS / 2];      // see store_row_sums
     struct {
       uint4 mask[kBatch][FB_MAX_EXPERTS];                   // rows of the tile that go to the slot
       uint32_t sorted[kBatch * kDispatchThreads];   // the batch's assignments in slot order: slot << 16 | tile, thread
@@ -364,35 +374,25 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
   int ids[kBatch];
 #pragma unroll
   for (int i = 0; i < kBatch; ++i) ids[i] = load_id(tile_begin + i);
-  // ---- column sums of the histogram table, split at this block's first slice.  Thread (part, unit)
-  // adds 16 experts of every P-th slice; a warp's threads of the same unit are then combined by
-  // shuffles.  16-bit counters: a thread adds at most 2^16 / 2^7 / (32 / U) slices between two flushes.
-  const int row_bytes = slice_row_bytes(E), U = row_bytes >> 4;
-  const int P = kDispatchThreads / U;
-  const int unit = t % U, slice0 = t / U;
-  const int first_slice = tile_begin * p.slices_per_tile;
-  const int chunk = 15 * (U < 16 ? 1 : 16);      // slices per thread and flush: 15 * 128 * 32 < 2^16, 240 * 128 * 2 < 2^16
-  const bool active_part = slice0 < P;
-  uint32_t sum_all0 = 0, sum_all1 = 0, sum_bef0 = 0, sum_bef1 = 0;      // thread w < row_bytes / 2: experts 2 w, 2 w + 1
-  for (int s_base = 0; s_base < p.num_slices; s_base += chunk * P) {
-    UnitSums sums;
-    sums.clear();
-    const int s_end = min(p.num_slices, s_base + chunk * P);
-    if (active_part) {
-#pragma unroll 4
-      for (int s = s_base + slice0; s < s_end; s += P)
-        sums.add(__ldg(reinterpret_cast<const uint4*>(p.slice_counts + static_cast<size_t>(s) * row_bytes) + unit), s < first_slice);
-    }
-    const int span = min(P, s_end - s_base);     // threads of slices beyond it hold nothing
-    const int warps = min(kDispatchWarps, (span * U + 31) >> 5);
-    if (s_base > 0) __syncthreads();             // the previous flush has been read
-    if (warp < warps) sums.to_warp(u.part[warp], U, unit, lane, active_part);
+  const uint32_t my_total = t < E ? __ldcg(p.totals + t) : 0u;
+  // ---- column sums of the histogram table before this block's first slice, or from it on.  16-bit counters: a lane
+  // adds 500 slices of at most 128 at most between two flushes.
+  const int row_bytes = slice_row_bytes(E), W = row_bytes >> 2;
+  const int first_slice = min(tile_begin * p.slices_per_tile, p.num_slices);
+  const bool later = 2 * first_slice > p.num_slices;
+  const int row_first = later ? first_slice : 0, row_last = later ? p.num_slices : first_slice;
+  constexpr int kFlush = 500 * kDispatchWarps;
+  uint32_t sum0 = 0, sum1 = 0;                   // thread j < 2 W: experts 4 (j / 2) + j % 2 and that + 2
+  for (int s_base = row_first; s_base < row_last; s_base += kFlush) {
+    const RowSums sums = add_rows(p.slice_counts, row_bytes, s_base, min(row_last, s_base + kFlush), warp, kDispatchWarps, lane);
+    if (s_base > row_first) __syncthreads();     // the previous flush has been read
+    store_row_sums(sums, u.part[warp], row_bytes, lane);
     __syncthreads();
-    if (t < 8 * U) {
-      for (int w = 0; w < warps; ++w) {
-        const uint32_t a = u.part[w][0][t], b = u.part[w][1][t];
-        sum_all0 += a & 0xffffu; sum_all1 += a >> 16;
-        sum_bef0 += b & 0xffffu; sum_bef1 += b >> 16;
+    if (t < 2 * W) {
+#pragma unroll 8
+      for (int w = 0; w < kDispatchWarps; ++w) {
+        const uint32_t v = u.part[w][t];
+        sum0 += v & 0xffffu; sum1 += v >> 16;
       }
     }
   }
@@ -400,18 +400,19 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
     if (my_slot_in < 0 || my_slot_in >= E) bad = 1;
     else if (atomicExch(&owner[my_slot_in], t) != -1) bad = 1;
     slot_of[t] = (my_slot_in < 0 || my_slot_in >= E) ? 0 : my_slot_in;
+    total[slot_of[t]] = my_total;
   }
   __syncthreads();
-  if (bad) {                                    // not a bijection: report, write nothing
-    if (t == 0 && blockIdx.x == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
+  const uint32_t ticket = warp == kDispatchWarps - 1 ? take_index_ticket(p, lane) : 0u;
+  if (bad || tile_begin >= tile_end) {
+    if (warp == kDispatchWarps - 1) clear_totals(p, ticket, lane);
+    if (bad && t == 0 && blockIdx.x == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);   // not a bijection: report, write nothing
     return;
   }
-  if (tile_begin >= tile_end) return;
-  if (t < 8 * U) {
-    const int un = t % U, i = t / U;
-    const int e0 = 16 * un + 4 * (i >> 1) + (i & 1), e1 = e0 + 2;
-    if (e0 < E) { total[slot_of[e0]] = sum_all0; gbase[slot_of[e0]] = sum_bef0; }
-    if (e1 < E) { total[slot_of[e1]] = sum_all1; gbase[slot_of[e1]] = sum_bef1; }
+  if (t < 2 * W) {
+    const int e0 = 4 * (t >> 1) + (t & 1), e1 = e0 + 2;
+    if (e0 < E) { const int sl = slot_of[e0]; gbase[sl] = later ? total[sl] - sum0 : sum0; }
+    if (e1 < E) { const int sl = slot_of[e1]; gbase[sl] = later ? total[sl] - sum1 : sum1; }
   }
   static_assert(kDispatchThreads == kDispatchBatch * FB_MAX_EXPERTS, "one mask per thread");
   u.b.mask[t / FB_MAX_EXPERTS][t % FB_MAX_EXPERTS] = make_uint4(0, 0, 0, 0);
@@ -503,6 +504,7 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
     mark_rows();
     __syncthreads();
   }
+  if (warp == kDispatchWarps - 1) clear_totals(p, ticket, lane);
 }
 
 // ---- token-sharded dispatch (several GPUs, each with a contiguous token range in rank order)

@@ -156,6 +156,15 @@ __device__ __forceinline__ void plan_put_count(PlanShared& sh, int e, uint32_t c
   atomicAdd(&sh.load[sh.rank_of[e]], c);
 }
 
+// The same by the thread that has placed the expert (slot: its slot as given), with no barrier in between.
+__device__ __forceinline__ void plan_put_count_at(PlanShared& sh, int e, int slot, uint32_t c, int E) {
+  sh.cnt[e] = c;
+  if (c > FB_MAX_COUNT_SUM) { sh.bad_range = 1; return; }
+  if (slot < 0 || slot >= E) return;
+  sh.slot_cnt[slot] = slot_word(c, e);
+  atomicAdd(&sh.load[sh.rank_of[e]], c);
+}
+
 // The new placement (called by all those threads after the planner warp is done and a
 // barrier): slot s holds the expert its slot word names (fast loop) or expert_at[s].  An
 // unusable input keeps the placement as given.

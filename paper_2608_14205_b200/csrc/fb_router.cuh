@@ -81,8 +81,8 @@ struct RouterParams {
   int32_t tiles_first;               // kModeLayer: blocks below this index (even) belong to the early pass
   int32_t ticket_target;             // number of tickets taken: one per block that publishes counts (persistent kernel: per pair)
   int32_t fuse_planner;              // prediction modes: the block that finishes last runs the planner
-  int32_t defer_counts;              // kModeLayer: the early pass leaves its histograms in early_counts and the
-                                     // dispatch-index kernel counts and plans (fb_dispatch_kernel<true>)
+  int32_t defer_counts;              // kModeLayer: the early pass adds its counts to early_totals and leaves the count
+                                     // vector and the plan to the dispatch-index kernel (fb_dispatch_kernel<true>)
   // fb_router_rows_kernel only: J block pairs per tile pair (cluster size / 2), the rows staged at a time
   // while the operand ring is busy with the next tile, and the column layout of a row over the lanes of a
   // warp: lane l holds columns g group_size + (l % lanes_per_group) cols_per_lane + j of group
@@ -104,7 +104,8 @@ struct RouterParams {
   int32_t* early_ids;                // kModeLayer: the early pass's ids and logits, or nullptr
   float* early_logits;
   uint8_t* slice_counts;             // [tiles * pieces][slice_row_bytes(E)] (dispatch mode)
-  uint8_t* early_counts;             // the same table for the early pass (defer_counts)
+  uint32_t* totals;                  // [E] sums of that table over all slices, zero on entry (dispatch mode)
+  uint32_t* early_totals;            // [E] the early pass's, zero on entry (defer_counts)
   unsigned long long* stamps;        // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
   int32_t probe;                     // measurement aid: 1 = operands are loaded but no MMA is issued and nothing
                                      // follows the main loop; 2 = with the MMAs, still nothing after them
@@ -468,6 +469,13 @@ __device__ __forceinline__ void write_slice_counts(uint8_t* table, int slice, in
     reinterpret_cast<uint32_t*>(table + static_cast<size_t>(slice) * row_bytes)[w] =
         h.x | h.y << 8 | h.z << 16 | h.w << 24;
   }
+}
+
+// A block's counts into the sums over all blocks that the dispatch-index kernel reads: thread et adds expert et's.
+// Nothing here waits for the additions, the end of the grid does.
+__device__ __forceinline__ void add_to_totals(uint32_t* totals, int E, uint32_t count, int et) {
+  static_assert(kEpilogueThreads >= FB_MAX_EXPERTS, "one thread per expert");
+  if (et < E && count != 0) atomicAdd(totals + et, count);
 }
 
 // Two MMA issuers share one ring of stages.  Where a stage always serves the same issuer - an even number of stages, and
@@ -996,8 +1004,10 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     }
     named_bar_sync(kPlanBarrierId, kEpilogueThreads);
     if (mode == kModeDispatch || p.defer_counts) {
-      if (static_cast<long long>(tile) * kTileM < p.T)       // the padding block of an odd pair owns no tile
-        write_slice_counts(mode == kModeDispatch ? p.slice_counts : p.early_counts, tile, E, sh.hist, et);
+      if (static_cast<long long>(tile) * kTileM < p.T) {     // the padding block of an odd pair owns no tile
+        add_to_totals(mode == kModeDispatch ? p.totals : p.early_totals, E, et < FB_MAX_EXPERTS ? sh.hist[et] : 0u, et);
+        if (mode == kModeDispatch) write_slice_counts(p.slice_counts, tile, E, sh.hist, et);
+      }
     } else if (p.probe == 0) {
       publish_counts(sh, p, et, warp, lane, mode == kModePredictPlan && p.fuse_planner != 0);
     }

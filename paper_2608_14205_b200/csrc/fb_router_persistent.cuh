@@ -212,6 +212,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     // for the layer call; no difference at 16384 tokens, 256 experts.
     auto row_sync = [&]() { named_bar_sync(kRowBarrierBase + static_cast<uint32_t>(quarter), kEpiSubs * 32); };
     uint32_t tiles_done = 0;
+    uint32_t my_total = 0;                                 // expert et's assignments in this block's tiles of the normal pass
     for (int pt = pair_first; pt < total_pairs; pt += pair_stride) {
       const bool second_pass = pt >= pairs_per_pass;
       const int mode = p.mode == kModeLayer ? (second_pass ? kModeDispatch : kModePredictPlan) : p.mode;
@@ -429,7 +430,11 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
       if (et < 4) sh.any_unranked[et] = 0;                    // everyone has read it
       if (mode == kModeDispatch) {
         const bool owns = static_cast<long long>(tile) * kTileM < p.T;   // the padding block of an odd pair owns no tile
-        if (owns) write_slice_counts(p.slice_counts, tile, E, hist, et);
+        if (owns) {
+          if (et < FB_MAX_EXPERTS) my_total += hist[et];
+          write_slice_counts(p.slice_counts, tile, E, hist, et);
+        }
+        if (pt + pair_stride >= total_pairs) add_to_totals(p.totals, E, my_total, et);
         // the other one was written out before the last barrier; the next tile counts into it
         for (int e = et; e < E; e += kEpilogueThreads) sh.tile_hist[(tiles_done & 1u) ^ 1u][e] = 0;
       } else if (pt + pair_stride >= pairs_per_pass) {

@@ -685,6 +685,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
     if ((p.mode == kModePredictPlan || p.mode == kModeLayer) && !p.defer_counts) plan_load_placement(p.plan, sh.plan, et, kEpilogueThreads);
 
     uint32_t tiles_done = 0;
+    uint32_t my_total = 0;                                   // expert et's assignments in this block's tiles for the index
     for (int pt = pair_first; pt < total_pairs; pt += pair_stride) {
       const bool second_pass = pt >= pairs_per_pass;
       const int mode = p.mode == kModeLayer ? (second_pass ? kModeDispatch : kModePredictPlan) : p.mode;
@@ -788,8 +789,11 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
         // measurement launch: nothing is published
       } else if (mode == kModeDispatch || p.defer_counts) {
         const int slice = tile * J + piece;
-        if (static_cast<long long>(tile) * kTileM + piece * slice_rows(J) < p.T)  // (one beyond the last token owns no row)
-          write_slice_counts(mode == kModeDispatch ? p.slice_counts : p.early_counts, slice, E, sh.hist, et);
+        if (static_cast<long long>(tile) * kTileM + piece * slice_rows(J) < p.T) {  // (one beyond the last token owns no row)
+          if (et < FB_MAX_EXPERTS) my_total += sh.hist[et];
+          if (mode == kModeDispatch) write_slice_counts(p.slice_counts, slice, E, sh.hist, et);
+        }
+        if (last_tile) add_to_totals(mode == kModeDispatch ? p.totals : p.early_totals, E, my_total, et);
         if (several_tiles) {
           named_bar_sync(kPlanBarrierId, kEpilogueThreads);
           for (int e = et; e < E; e += kEpilogueThreads) sh.hist[e] = 0;

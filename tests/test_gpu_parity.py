@@ -463,6 +463,40 @@ def test_planner_with_many_experts_per_rank(E, R, bud):
     _run(_wl(E=E, k=4, R=R, d=64, max_swaps=12), 700, placement=I.random_placement(E, seed=R), **bud)
 
 
+@pytest.mark.parametrize("m", [1, 2, 3, 4, 5, 7, 8, 9, 15, 16, 17])
+@pytest.mark.parametrize("gamma_num,most", [(1, 4), (0, 4), (1, 2**21)])
+def test_planner_at_the_edges_of_its_lane_layouts(m, gamma_num, most):
+    # whole numbers: exact.  Counts below 4 make nearly every choice a tie; the largest add up to the planner's range.
+    R, rng = 8, np.random.default_rng(m)
+    E, ms = R * m, max(1, min(R * m // 2, 20))
+    counts = rng.integers(0, max(4, most // E), E)
+    if most > 4:
+        counts[rng.integers(0, E)] += most - int(counts.sum())
+    pi = I.random_placement(E, m)
+    bkw = dict(max_swaps=ms, gamma_num=gamma_num, gamma_den=7)
+    ctx = B.Context(128, 64, E, 1, R)
+    dev = torch.device("cuda")
+    z = lambda n: torch.zeros(n, dtype=torch.int32, device=dev)
+    out_pi, swaps, n, lb, la = z(E), z(4 * ms), z(1), z(R), z(R)
+    ctx.fb_plan_swaps(torch.tensor(counts, dtype=torch.int32, device=dev), pi.to(dev), B.make_budget(**bkw), 0, out_pi, swaps,
+                      n, lb, la)
+    assert ctx.fb_device_status() == 0
+    want = O.plan_swaps(counts.tolist(), pi.tolist(), R, O.Budget(**bkw), layer_id=0)
+    got = [tuple(r) for r in swaps.cpu().numpy().reshape(-1, 4)[:int(n.item())].tolist()]
+    assert (got, out_pi.cpu().tolist(), lb.cpu().tolist(), la.cpu().tolist()) == want
+
+
+@pytest.mark.parametrize("name,T", [("qwen3", 700), ("dsv3", 1500), ("qwen3", 19000)])
+def test_a_refused_placement_leaves_nothing_behind_for_the_next_call(name, T):
+    # the sums that the router kernel hands to the dispatch index are put back to zero whatever comes of the index
+    wl = I.WORKLOADS[name]
+    li = I.make_layer(wl, 0, 0, T=T)
+    ctx, bkw = P.make_context(wl, T), P.budget_kwargs(wl, T)
+    assert P.run_gpu_layer(ctx, wl, li, bkw, placement=torch.zeros(wl.E, dtype=torch.int32))["status"] == B.FB_ERR_BAD_PLACEMENT
+    gpu = P.run_gpu_layer(ctx, wl, li, bkw)
+    P.compare_layer(wl, li, bkw, gpu, sample_rows=np.arange(0, T, 37))
+
+
 # ------------------------------------------------------------------ persistent router kernel (several tiles per block pair)
 @pytest.mark.parametrize("name,T,limit,d,lb", [
     ("dsv3", 777, 1, None, False), ("dsv3", 1500, 2, None, False), ("dsv3", 2049, 3, None, True),

@@ -200,13 +200,16 @@ __device__ __forceinline__ void plan_write_placement(const PlanParams& p, PlanSh
 // rank, 4 tokens: layer step 63 us with the general loop below, 22 with this one).  A lane keeps the
 // packed (load, rank) keys of its two ranks.
 //
-// What an iteration waits for: the slot words, a few operations, and ONE warp reduction, over v, the sign of 2 d - D and
-// the lane - d follows from v and the sign in every lane.  The frontier of the next iteration is the larger
-// (smaller) of the two new loads and of the other ranks' largest (smallest), which is reduced meanwhile.  Only where
-// two lanes hold the smallest v a second reduction finds the smaller pair.  (Integer operations issue every other cycle
-// from a single warp: 600 cycles per iteration with 16 experts per rank, 385 with 8.)  In line in its kernels, with the
-// parameters out of constant memory, everything around the loop takes 630 cycles; as a function with a pointer to them it
-// took 1400: layer calls of 8192 tokens, 128 experts 25.9 -> 24.3 us, 40 x 128 16.7 -> 15.3, 1733 x 256 30.7 -> 29.6.
+// What an iteration waits for: the slot words, a few operations, and two warp reductions, one over v and one over the
+// pair, the sign of 2 d - D and the lane - d follows from v and the sign in every lane.  The frontier of the next iteration is
+// the larger (smaller) of the two new loads and of the other ranks' largest (smallest), which is reduced meanwhile.
+// One branch per iteration: each costs as much as a reduction (22 cycles) or more, and integer operations
+// issue every other cycle from a single warp.  With 16 experts per rank 360 cycles per iteration, with 8 240; with
+// branches for "balanced", "no pair", ties and the chosen lane 520 and 355, before that (reductions for the frontier as
+// well, a shuffle for d, more operations per slot word) 610 and 390.
+// In line in its kernels, with the parameters out of constant memory, everything around the loop takes 600 cycles; as a
+// function with a pointer to them it took 1400: layer calls of 8192 tokens, 128 experts 25.9 -> 24.3 us, 40 x 128 16.7 ->
+// 15.3, 1733 x 256 30.7 -> 29.6.
 // kBooks: two cost classes, or per-rank or per-link budgets that can bind.  Otherwise the budgets allow
 // a fixed number of swaps (swap_cap) and the loop keeps no books at all.
 template <int kPerLane, bool kBooks>
@@ -222,17 +225,17 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
   const bool aside = kPerLane != 0 && (lane / g >= m || j0 >= m);
   const bool flat = p.gamma_den == 0 || p.gamma_num == 0;
   const uint32_t tau = p.tau_tokens, max_swaps = kBooks ? p.max_swaps : p.swap_cap;
-  // frontier keys (lowest index on ties): max of load << 6 | (63 - rank), min of load << 6 | rank
+  // frontier keys (lowest index on ties): max of load << 6 | (63 - rank), min of load << 6 | rank - the same but for
+  // the six bits of the rank, which are the other's complement
+  const uint32_t none0 = L0 >= 0 ? 0u : kNone, none1 = L1 >= 0 ? 0u : kNone;      // no such rank
   uint32_t h0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(63 - lane)) : 0u;
   uint32_t h1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(31 - lane)) : 0u;
-  uint32_t l0 = L0 >= 0 ? (static_cast<uint32_t>(L0) << 6 | static_cast<uint32_t>(lane)) : kNone;
-  uint32_t l1 = L1 >= 0 ? (static_cast<uint32_t>(L1) << 6 | static_cast<uint32_t>(lane + 32)) : kNone;
   // books
   uint32_t my_links[4] = {kNone, kNone, kNone, kNone};            // lane i keeps the links of swaps i, i+32, ...
   unsigned long long global_spent = 0;
   uint32_t n = 0;
   uint32_t hi_key = __reduce_max_sync(full, max(h0, h1));
-  uint32_t lo_key = __reduce_min_sync(full, min(l0, l1));
+  uint32_t lo_key = __reduce_min_sync(full, min(h0 ^ 63u | none0, h1 ^ 63u | none1));
   while (n < max_swaps) {
     const int a = 63 - static_cast<int>(hi_key & 63u), b = static_cast<int>(lo_key & 63u);
     const int La = static_cast<int>(hi_key >> 6), Lb = static_cast<int>(lo_key >> 6);
@@ -252,7 +255,7 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
         for (int t = 0; t < kNarrow; ++t) wb[t] = sh.slot_cnt[base_b + min(j0 + t, m - 1)];
       }
     }
-    if (static_cast<uint32_t>(D) <= tau) break;                   // (the same in all lanes)
+    bool stop = static_cast<uint32_t>(D) <= tau;                  // (the same in all lanes, as everything that ends the loop)
     unsigned long long c_ns = 0, rs_a = 0, rs_b = 0;
     uint32_t lkey = 0;
     if (kBooks) {
@@ -265,7 +268,7 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
       const int ka = cls ? node_a : a, kb = cls ? node_b : b;
       lkey = static_cast<uint32_t>(cls) << 16 | static_cast<uint32_t>(ka < kb ? ka : kb) << 8 |
              static_cast<uint32_t>(ka < kb ? kb : ka);
-      bool stop = p.global_ns != FB_BUDGET_OFF && (c_ns > p.global_ns || global_spent > p.global_ns - c_ns);
+      stop = stop || (p.global_ns != FB_BUDGET_OFF && (c_ns > p.global_ns || global_spent > p.global_ns - c_ns));
       const unsigned long long rs = rs_a > rs_b ? rs_a : rs_b;
       stop = stop || (p.rank_ns != FB_BUDGET_OFF && (c_ns > p.rank_ns || rs > p.rank_ns - c_ns));
       if (p.link_ns != FB_BUDGET_OFF) {
@@ -276,12 +279,11 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
           if (n > 32u * q) used += __popc(__ballot_sync(full, my_links[q] == lkey));    // n is the same in all lanes
         stop = stop || used >= p.uniform_link_cap[cls];
       }
-      if (stop) break;
     }
     // the other ranks' largest and smallest load
     const bool in0 = lane == a || lane == b, in1 = lane + 32 == a || lane + 32 == b;
     const uint32_t hi_rest = __reduce_max_sync(full, max(in0 ? 0u : h0, in1 ? 0u : h1));
-    const uint32_t lo_rest = __reduce_min_sync(full, min(in0 ? kNone : l0, in1 ? kNone : l1));
+    const uint32_t lo_rest = __reduce_min_sync(full, min(in0 ? kNone : h0 ^ 63u | none0, in1 ? kNone : h1 ^ 63u | none1));
     const int v_floor = flat ? 2 * static_cast<int>(hi_rest >> 6) - La - Lb : 0;
     // ---- smallest v of this lane, ties -> smallest pair; where its experts are, and 2 d - D
     uint32_t mine = kNoPair, pair = 0;
@@ -291,10 +293,16 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
       uint32_t key[kNarrow];
 #pragma unroll
       for (int t = 0; t < kNarrow; ++t)                           // v << 8 | expert of the light rank
-        key[t] = __byte_perm(static_cast<uint32_t>(max(abs(y - static_cast<int>(wb[t] >> 8)), v_floor)), wb[t], 0x2104);
-      uint32_t best = key[0];
+        key[t] = __byte_perm(static_cast<uint32_t>(abs(y - static_cast<int>(wb[t] >> 8))), wb[t], 0x2104);
+      if (flat) {
 #pragma unroll
-      for (int t = 1; t < kNarrow; ++t) best = min(best, key[t]);
+        for (int t = 0; t < kNarrow; ++t)
+          key[t] = __byte_perm(static_cast<uint32_t>(max(static_cast<int>(key[t] >> 8), v_floor)), wb[t], 0x2104);
+      }
+      uint32_t best = key[0];
+      if constexpr (kNarrow == 8) best = __vimin3_u32(__vimin3_u32(key[0], key[1], key[2]), __vimin3_u32(key[3], key[4], key[5]),
+                                                      min(key[6], key[7]));
+      else if constexpr (kNarrow == 2) best = min(key[0], key[1]);
       mine = aside ? kNoPair : best >> 8;
       pair = (wa & 0xffu) << 8 | (best & 0xffu);
       sa = base_a + ia;
@@ -326,34 +334,26 @@ __device__ __forceinline__ uint32_t plan_loop_uniform(const PlanParams& p, PlanS
       }
     }
     const uint32_t sign_lane = (off < 0 ? 32u : 0u) | static_cast<uint32_t>(lane);
-    uint32_t win = __reduce_min_sync(full, mine << 6 | sign_lane);
-    const uint32_t top = win >> 6;
-    if (top >= static_cast<uint32_t>(D)) break;                   // Algorithm 1 lines 6-7
-    const uint32_t holders = __ballot_sync(full, mine == top);
-    if ((holders & (holders - 1)) != 0)                           // (the same in all lanes)
-      win = __reduce_min_sync(full, mine == top ? pair << 6 | sign_lane : kNone);
+    const uint32_t top = __reduce_min_sync(full, mine);
+    const uint32_t win = __reduce_min_sync(full, mine == top ? pair << 6 | sign_lane : kNone);
+    if (stop || top >= static_cast<uint32_t>(D)) break;           // Algorithm 1 lines 6-7
     const int src = static_cast<int>(win & 31u);
-    // tokens moved a -> b: (D + off) / 2 of the chosen lane
-    const int dlt = flat ? __shfl_sync(full, (D + off) >> 1, src)
-                         : (D + ((win & 32u) != 0 ? -static_cast<int>(top) : static_cast<int>(top))) >> 1;
-    if (lane == src) {
-      // the two experts trade slots
-      sh.slot_cnt[sa] = slot_word(kSlotMoved, static_cast<int>(pair & 0xffu));
-      sh.slot_cnt[sb] = slot_word(kSlotMoved, static_cast<int>(pair >> 8));
-      if (kBooks) { sh.rank_spent[a] = rs_a + c_ns; sh.rank_spent[b] = rs_b + c_ns; }
-      // The accepted swap stays in shared memory until the loop is over (ranks and expert ids
-      // are below 256: one word; link_key is otherwise unused on this path): a global store
-      // here would be waited for at the warp barrier below, once per iteration.
-      sh.link_key[n] = static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 | pair;
-    }
-    const uint32_t moved = static_cast<uint32_t>(dlt) << 6;
-    if (lane == a) { h0 -= moved; l0 -= moved; }
-    if (lane + 32 == a) { h1 -= moved; l1 -= moved; }
-    if (lane == b) { h0 += moved; l0 += moved; }
-    if (lane + 32 == b) { h1 += moved; l1 += moved; }
-    const uint32_t new_a = static_cast<uint32_t>(La - dlt) << 6, new_b = static_cast<uint32_t>(Lb + dlt) << 6;
-    hi_key = max(hi_rest, max(new_a | static_cast<uint32_t>(63 - a), new_b | static_cast<uint32_t>(63 - b)));
-    lo_key = min(lo_rest, min(new_a | static_cast<uint32_t>(a), new_b | static_cast<uint32_t>(b)));
+    // tokens moved a -> b, in the place of a load: (D + off) / 2 of the chosen lane
+    const uint32_t moved = static_cast<uint32_t>(flat ? __shfl_sync(full, D + off, src)
+                                                 : D + ((win & 32u) != 0 ? -static_cast<int>(top) : static_cast<int>(top))) << 5;
+    // The two experts trade slots.  The accepted swap stays in shared memory until the loop is over (ranks and expert ids
+    // are below 256: one word; link_key is otherwise unused on this path): a global store here would be waited for at the
+    // warp barrier below, once per iteration.
+    const uint32_t chosen = lane == src ? 1u : 0u;
+    st_shared_if(chosen, smem_u32(&sh.slot_cnt[sa]), slot_word(kSlotMoved, static_cast<int>(pair & 0xffu)));
+    st_shared_if(chosen, smem_u32(&sh.slot_cnt[sb]), slot_word(kSlotMoved, static_cast<int>(pair >> 8)));
+    st_shared_if(chosen, smem_u32(&sh.link_key[n]), static_cast<uint32_t>(a) << 24 | static_cast<uint32_t>(b) << 16 | pair);
+    if (kBooks && chosen != 0) { sh.rank_spent[a] = rs_a + c_ns; sh.rank_spent[b] = rs_b + c_ns; }
+    if (in0) h0 += lane == a ? 0u - moved : moved;
+    if (in1) h1 += lane + 32 == a ? 0u - moved : moved;
+    const uint32_t new_a = hi_key - moved, new_b = lo_key + moved;
+    hi_key = __vimax3_u32(hi_rest, new_a, new_b ^ 63u);
+    lo_key = __vimin3_u32(lo_rest, new_a ^ 63u, new_b);
     if (kBooks) {
       if (static_cast<int>(n & 31u) == lane) {
 #pragma unroll

@@ -328,6 +328,10 @@ __device__ __forceinline__ float redux_min_f32(float x) {
   asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
   return r;
 }
+// A word to shared memory when pred != 0; a predicated store, not a branch.
+__device__ __forceinline__ void st_shared_if(uint32_t pred, uint32_t addr, uint32_t v) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %0, 0;\n@p st.shared.u32 [%1], %2;\n}\n" ::"r"(pred), "r"(addr), "r"(v) : "memory");
+}
 // Both 32-bit words to shared memory when pred != 0; a predicated store, not a branch.
 __device__ __forceinline__ void st_shared_v2_if(uint32_t pred, uint32_t addr, uint32_t lo, uint32_t hi) {
   asm volatile(

@@ -297,36 +297,51 @@ __device__ __forceinline__ float kth_largest_known(const float* tab, int n_chunk
 // share the candidates (candidate c belongs to thread c % kEpiSubs); a candidate with fewer
 // than FB_MAX_TOPK larger ones is written to out_hi/out_lo[rank][row].  Returns true when
 // the row had more candidates than the list holds (nothing is written for it then).
+// A thread ranks kMine candidates at a time, from c0 on.  (Always four: a warp whose longest list has a
+// candidate or two more than 16 went through twice the comparisons.)
+template <int kMine>
+__device__ __forceinline__ void rank_some(const unsigned long long* cand, uint32_t n, uint32_t n_most, uint32_t c0, int sub,
+                                          int row_in_tile, uint32_t* out_hi, uint32_t* out_lo) {
+  unsigned long long mykey[kMine];
+  uint32_t rank[kMine];
+#pragma unroll
+  for (int t = 0; t < kMine; ++t) {
+    const uint32_t c = c0 + t * kEpiSubs + sub;
+    mykey[t] = cand[(c < n ? c : 0) * kTileM + row_in_tile];
+    rank[t] = 0;
+  }
+#pragma unroll 2
+  for (uint32_t d = 0; d < n_most; ++d) {
+    const unsigned long long other = d < n ? cand[d * kTileM + row_in_tile] : 0ull;
+#pragma unroll
+    for (int t = 0; t < kMine; ++t) rank[t] += other > mykey[t] ? 1u : 0u;
+  }
+#pragma unroll
+  for (int t = 0; t < kMine; ++t) {
+    const uint32_t c = c0 + t * kEpiSubs + sub;
+    if (c < n && rank[t] < static_cast<uint32_t>(FB_MAX_TOPK)) {
+      out_hi[rank[t] * kTileM + row_in_tile] = static_cast<uint32_t>(mykey[t] >> 32);
+      out_lo[rank[t] * kTileM + row_in_tile] = static_cast<uint32_t>(mykey[t]);
+    }
+  }
+}
 __device__ __forceinline__ bool rank_candidates(const unsigned long long* cand, uint32_t n_all, int sub,
                                                 int row_in_tile, uint32_t* out_hi, uint32_t* out_lo) {
   const bool overflow = n_all > kCandCap;
   const uint32_t n = overflow ? 0u : n_all;
   const uint32_t n_most = __reduce_max_sync(0xffffffffu, n);
-#pragma unroll 1
-  for (uint32_t tier = 0; tier * 4 * kEpiSubs < n_most; ++tier) {
-    unsigned long long mykey[4];
-    uint32_t rank[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const uint32_t c = (tier * 4 + t) * kEpiSubs + sub;
-      mykey[t] = cand[(c < n ? c : 0) * kTileM + row_in_tile];
-      rank[t] = 0;
-    }
-#pragma unroll 2
-    for (uint32_t d = 0; d < n_most; ++d) {
-      const unsigned long long other = d < n ? cand[d * kTileM + row_in_tile] : 0ull;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) rank[t] += other > mykey[t] ? 1u : 0u;
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const uint32_t c = (tier * 4 + t) * kEpiSubs + sub;
-      if (c < n && rank[t] < static_cast<uint32_t>(FB_MAX_TOPK)) {
-        out_hi[rank[t] * kTileM + row_in_tile] = static_cast<uint32_t>(mykey[t] >> 32);
-        out_lo[rank[t] * kTileM + row_in_tile] = static_cast<uint32_t>(mykey[t]);
-      }
+  uint32_t c0 = 0;
+  if (n_most > 2 * kEpiSubs) {
+    if (n_most <= 3 * kEpiSubs) {
+      rank_some<3>(cand, n, n_most, 0, sub, row_in_tile, out_hi, out_lo);
+      c0 = 3 * kEpiSubs;
+    } else {
+      rank_some<4>(cand, n, n_most, 0, sub, row_in_tile, out_hi, out_lo);
+      c0 = 4 * kEpiSubs;
     }
   }
+#pragma unroll 1
+  for (; c0 < n_most; c0 += 2 * kEpiSubs) rank_some<2>(cand, n, n_most, c0, sub, row_in_tile, out_hi, out_lo);
   return overflow;
 }
 
@@ -389,10 +404,18 @@ __device__ __forceinline__ void write_row_outputs(const TopK& top, const RouterP
     if (bad) atomicCAS(p.status, 0, FB_ERR_INTERNAL);
   }
 #endif
+  // 16 bytes a store where every row starts on 16 bytes (a warp's rows lie k words apart)
+  const bool whole = k % 4 == 0;
   if (out_ids != nullptr) {
+    if (whole && reinterpret_cast<uintptr_t>(out_ids) % 16 == 0) {
 #pragma unroll
-    for (int j = 0; j < FB_MAX_TOPK; ++j)
-      if (j < k) out_ids[row * k + j] = top.i[j];
+      for (int j = 0; j < FB_MAX_TOPK; j += 4)
+        if (j < k) *reinterpret_cast<int4*>(out_ids + row * k + j) = make_int4(top.i[j], top.i[j + 1], top.i[j + 2], top.i[j + 3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < FB_MAX_TOPK; ++j)
+        if (j < k) out_ids[row * k + j] = top.i[j];
+    }
   }
   if (out_w != nullptr) {
     float w[FB_MAX_TOPK];
@@ -407,9 +430,16 @@ __device__ __forceinline__ void write_row_outputs(const TopK& top, const RouterP
     float scale;
     if (!sigmoid_gate) scale = 1.0f / wsum;
     else scale = p.renorm ? p.route_scale / wsum : p.route_scale;
+    if (whole && reinterpret_cast<uintptr_t>(out_w) % 16 == 0) {
 #pragma unroll
-    for (int j = 0; j < FB_MAX_TOPK; ++j)
-      if (j < k) out_w[row * k + j] = w[j] * scale;
+      for (int j = 0; j < FB_MAX_TOPK; j += 4)
+        if (j < k)
+          *reinterpret_cast<float4*>(out_w + row * k + j) = make_float4(w[j] * scale, w[j + 1] * scale, w[j + 2] * scale, w[j + 3] * scale);
+    } else {
+#pragma unroll
+      for (int j = 0; j < FB_MAX_TOPK; ++j)
+        if (j < k) out_w[row * k + j] = w[j] * scale;
+    }
   }
 }
 

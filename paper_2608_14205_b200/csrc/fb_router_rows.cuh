@@ -63,8 +63,7 @@ constexpr int kListStride = kCandCap + 12;     // + the last lane's columns, rou
 struct RowScratch {                    // one per epilogue warp
   alignas(16) float cand_key[2][kListStride];  // keys of two rows' candidates in ascending id order; -inf behind the last one
   alignas(16) int32_t cand_id[2][kListStride];
-  alignas(16) float win_key[8][FB_MAX_TOPK];   // the rows' top-k in order of rank
-  alignas(16) int32_t win_id[8][FB_MAX_TOPK];
+  alignas(16) int2 win[8][FB_MAX_TOPK];        // the rows' top-k in order of rank: key (its bits), expert id
   float row_sum[8];                            // softmax denominators relative to the row's largest key
 };
 __host__ __device__ constexpr size_t staging_bytes(int rows, int N) {
@@ -119,7 +118,7 @@ struct RowsShared {
 // Plain selection of one row by repeated maximum over keys in shared memory (dropped columns hold
 // -inf): the path of rows with more candidates than the list holds, and of rows with equal keys among
 // the candidates (the lower expert id wins).  Rare; kept out of line.
-__device__ __noinline__ void select_slow(float* keys, int E, int k, float* win_key, int32_t* win_id, int lane) {
+__device__ __noinline__ void select_slow(float* keys, int E, int k, int2* win, int lane) {
   for (int r = 0; r < k; ++r) {
     float best = -INFINITY;
     int at = E;
@@ -137,16 +136,15 @@ __device__ __noinline__ void select_slow(float* keys, int E, int k, float* win_k
       if (lane == 0) {
         uint32_t named = 0;
         for (int h = 0; h < r; ++h)
-          if (win_id[h] < FB_MAX_TOPK) named |= 1u << win_id[h];
+          if (win[h].y < FB_MAX_TOPK) named |= 1u << win[h].y;
         for (int h = r; h < k; ++h) {
-          win_key[h] = -INFINITY;
-          win_id[h] = __ffs(~named) - 1;
-          named |= 1u << win_id[h];
+          win[h] = make_int2(__float_as_int(-INFINITY), __ffs(~named) - 1);
+          named |= 1u << win[h].y;
         }
       }
       break;
     }
-    if (lane == 0) { win_key[r] = best; win_id[r] = at; keys[at] = -INFINITY; }
+    if (lane == 0) { win[r] = make_int2(__float_as_int(best), at); keys[at] = -INFINITY; }
     __syncwarp();
   }
 }
@@ -355,31 +353,73 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
     }
   }
   if (kFewKeys) {
-    // Few keys per lane: k rounds of "largest remaining key"; the lowest lane, and in it the lowest column,
-    // has the lowest id on ties.  Keys taken, and columns that do not exist, are no numbers, which no maximum takes up:
-    // what is left to take are numbers, -inf for experts that are masked out or in dropped groups, and every row has
-    // E >= k of them.  (Compacting the keys above a bound and ranking them, as below, takes
-    // k reductions for the bound alone: layer step 40 tokens x 128 experts 18.5 us that way and 17.3 this way,
+    // Few keys per lane: k rounds of "largest remaining key".  (Compacting the keys above a bound and ranking them, as
+    // below, takes k reductions for the bound alone: layer step 40 tokens x 128 experts 18.5 us that way and 17.3 this way,
     // 5003 x 64 25.4 and 24.6, prediction and plan 2729 x 60 16.0 and 14.3.)
+    // A lane first puts its keys into descending order, so that a round is one reduction over the lanes' first keys: the lane that
+    // holds the largest stores it and moves up, without a branch.  Equal keys in one lane keep their order; if two lanes ever
+    // hold the largest, or it is -inf (masked experts, dropped groups, keys that are no numbers, columns that do not exist),
+    // the rows are selected once more below, where the lower id is looked for.  Against that form for all rows: layer call
+    // 5003 x 64 20.5 -> 18.9 us, 40 x 128 14.5 -> 14.0, 2000 x 60 15.6 -> 15.0, prediction and plan 8192 x 128 19.7 -> 18.3.
+    float first[2][kCpl];
+    int id[2][kCpl];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+#pragma unroll
+      for (int j = 0; j < kCpl; ++j) {
+        if (p.groups > 1) key[u][j] = kept[u] ? key[u][j] : -INFINITY;
+        first[u][j] = j < lc.n ? key[u][j] : -INFINITY;
+        id[u][j] = lc.c0 + j;
+      }
+#pragma unroll
+      for (int pass = 0; pass < kCpl; ++pass)
+#pragma unroll
+        for (int j = pass & 1; j + 1 < kCpl; j += 2) {
+          const bool swap = first[u][j + 1] > first[u][j];
+          const float hi = fmaxf(first[u][j], first[u][j + 1]), lo = fminf(first[u][j], first[u][j + 1]);
+          const int ih = swap ? id[u][j + 1] : id[u][j], il = swap ? id[u][j] : id[u][j + 1];
+          first[u][j] = hi; first[u][j + 1] = lo;
+          id[u][j] = ih; id[u][j + 1] = il;
+        }
+      if (want_sum) {
+        const float s = row_exp_sum<kCpl>(key[u], first[u][0]);
+        if (lane == 0) rs.row_sum[2 * pair + u] = s;
+      }
+    }
+    uint32_t several = 0;
+    float last[2] = {0.0f, 0.0f};
+#pragma unroll 1
+    for (int r = 0; r < p.k; ++r) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) last[u] = redux_max_f32(first[u][0]);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const bool mine = first[u][0] == last[u];
+        const uint32_t holders = __ballot_sync(full, mine);
+        several |= holders & (holders - 1);
+        if (mine) rs.win[2 * pair + u][r] = make_int2(__float_as_int(first[u][0]), id[u][0]);
+#pragma unroll
+        for (int j = 0; j < kCpl; ++j) {
+          first[u][j] = mine ? (j + 1 < kCpl ? first[u][j + 1] : -INFINITY) : first[u][j];
+          if (j + 1 < kCpl) id[u][j] = mine ? id[u][j + 1] : id[u][j];
+        }
+      }
+    }
+    if (several == 0 && fminf(last[0], last[1]) > -INFINITY) return;
+    // Once more: the lowest lane, and in it the lowest column, has the lowest id on ties.  Keys taken, and columns that do
+    // not exist, are no numbers, which no maximum takes up: what is left to take are numbers, -inf for experts that are masked
+    // out or in dropped groups, and every row has E >= k of them.
+    __syncwarp();
     float lane_max[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      if (p.groups > 1) {
+      if (p.ragged && mask_later) {
 #pragma unroll
-        for (int j = 0; j < kCpl; ++j) key[u][j] = kept[u] ? key[u][j] : -INFINITY;
+        for (int j = 0; j < kCpl; ++j) key[u][j] = j < lc.n ? key[u][j] : taken;
       }
       lane_max[u] = key[u][0];
 #pragma unroll
       for (int j = 1; j < kCpl; ++j) lane_max[u] = fmaxf(lane_max[u], key[u][j]);
-      if (want_sum) {
-        const float s = row_exp_sum<kCpl>(key[u], lane_max[u]);
-        if (lane == 0) rs.row_sum[2 * pair + u] = s;
-      }
-      if (p.ragged && mask_later) {
-#pragma unroll
-        for (int j = 0; j < kCpl; ++j) key[u][j] = j < lc.n ? key[u][j] : taken;
-        lane_max[u] = lc.n > 0 ? lane_max[u] : taken;
-      }
     }
 #pragma unroll 1
     for (int r = 0; r < p.k; ++r) {
@@ -395,8 +435,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
           int at = 0;
 #pragma unroll
           for (int j = kCpl - 1; j >= 0; --j) at = key[u][j] == top[u] ? j : at;
-          rs.win_key[2 * pair + u][r] = top[u];
-          rs.win_id[2 * pair + u][r] = lc.c0 + at;
+          rs.win[2 * pair + u][r] = make_int2(__float_as_int(top[u]), lc.c0 + at);
 #pragma unroll
           for (int j = 0; j < kCpl; ++j) key[u][j] = j == at ? taken : key[u][j];
           lane_max[u] = key[u][0];
@@ -490,14 +529,12 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
       count_greater(r1, o.x, my1); count_greater(r1, o.y, my1); count_greater(r1, o.z, my1); count_greater(r1, o.w, my1);
     }
     if (my1 > -INFINITY && r1 < p.k) {
-      rs.win_key[2 * pair + h][r1] = my1;
-      rs.win_id[2 * pair + h][r1] = rs.cand_id[h][c + 16];
+      rs.win[2 * pair + h][r1] = make_int2(__float_as_int(my1), rs.cand_id[h][c + 16]);
       found += 0x100u + r1;
     }
   }
   if (my0 > -INFINITY && r0 < p.k) {
-    rs.win_key[2 * pair + h][r0] = my0;
-    rs.win_id[2 * pair + h][r0] = rs.cand_id[h][c];
+    rs.win[2 * pair + h][r0] = make_int2(__float_as_int(my0), rs.cand_id[h][c]);
     found += 0x100u + r0;
   }
   // Anything but every rank found once means equal keys among the best (or too few candidates): such rows, and rows
@@ -520,7 +557,7 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
       for (int j = 0; j < kCpl; ++j)
         if (j < lc.n && (u == 0 ? kept[0] : kept[1])) keys[lc.c0 + j] = u == 0 ? key[0][j] : key[1][j];
       __syncwarp();
-      select_slow(keys, p.E, p.k, rs.win_key[2 * pair + u], rs.win_id[2 * pair + u], lane);
+      select_slow(keys, p.E, p.k, rs.win[2 * pair + u], lane);
     }
   }
 }
@@ -536,8 +573,9 @@ __device__ __forceinline__ void finish_rows(const RouterParams& p, RowsShared& s
     const int i = base + (lane >> 3);
     const long long row = row0 + i;
     const bool valid = i < n_rows && row < p.T && rk < p.k;
-    const float key = rs.win_key[i & 7][rk];
-    const int id = valid ? rs.win_id[i & 7][rk] : 0;
+    const int2 found = rs.win[i & 7][rk];
+    const float key = __int_as_float(found.x);
+    const int id = valid ? found.y : 0;
 #ifdef FB_DEBUG
     // what the sanitizer would catch: a chosen expert outside [0, E), a repeated expert
     {

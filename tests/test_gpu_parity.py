@@ -825,6 +825,29 @@ def test_row_selection_breaks_ties_and_survives_overfull_lists(T):
         ctx.close()
 
 
+@pytest.mark.parametrize("kw", [dict(E=8, k=2, R=4), dict(E=64, k=6, R=8, gate=1), dict(E=64, k=8, R=8), dict(E=128, k=7, R=8),
+                                dict(E=60, k=4, R=4, renorm=0)])
+def test_few_keys_per_lane_break_ties_between_lanes(kw):
+    # one, two and four columns per lane; experts e and e + E / 2 have equal weights and lie in different lanes, which the
+    # branch-free rounds leave to the exact ones - in every third row only, the others have no ties
+    T, wl = 190, _wl(d=256, **kw)
+    li = I.make_layer(wl, 1, 0, T=T)
+    half = wl.E // 2
+    li.W[half:, :128] = li.W[:half, :128]
+    li.h_prev[::3, 128:] = 0
+    li.H[::3, 128:] = 0
+    if li.select_bias is not None:
+        li.select_bias = torch.zeros(wl.E)
+    ctx = P.make_context(wl, T)
+    bkw = P.budget_kwargs(wl, T)
+    gpu = P.run_gpu_layer(ctx, wl, li, bkw, want_logits=False)
+    P.compare_layer(wl, li, bkw, gpu)
+    ids = gpu["ids"][::3]
+    assert (ids[:, 0] < half).all()
+    assert ((ids[:, 1:] < half) | (ids[:, 1:] == ids[:, :-1] + half)).all()
+    ctx.close()
+
+
 @pytest.mark.parametrize("E,kw", [
     (256, dict(gate=0, n_group=1, topk_group=1)), (200, dict(gate=0, n_group=1, topk_group=1)),      # eight columns per lane
     (256, dict(gate=1, n_group=8, topk_group=4)), (250, dict(gate=1, n_group=5, topk_group=2)),      # bound from the groups; sixteen

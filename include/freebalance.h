@@ -216,7 +216,8 @@ fb_status fb_plan_swaps(fb_ctx* ctx, const uint32_t* counts, const int32_t* expe
                         int32_t* expert_to_slot_out, fb_swap* swaps, int32_t* n_swaps,
                         uint32_t* load_before, uint32_t* load_after, fb_stream stream);
 
-/* Stages 1 + 2 in one launch: the thread block that finishes last runs the planner. */
+/* Stages 1 + 2 in one call: the planner's kernel starts under the end of the prediction pass (calls with more tiles than
+ * the GPU holds at once plan beside their last tiles instead, in one launch). */
 fb_status fb_predict_and_plan(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T,
                               const int32_t* expert_to_slot, const fb_budget* budget,
                               int32_t layer_id, uint32_t* counts, int32_t* expert_to_slot_out,

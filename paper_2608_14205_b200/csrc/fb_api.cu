@@ -259,11 +259,14 @@ cudaError_t launch_dependent(void (*kernel)(Params...), int blocks, int threads,
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, const uint32_t* counts, cudaStream_t stream) {
+// counts_out: counts are the totals of a prediction pass (see fb_plan_kernel).
+fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, uint32_t* counts, uint32_t* counts_out, cudaStream_t stream) {
   const cudaError_t err = launch_dependent(fb::plan_needs_general_loop(pp) ? fb::fb_plan_kernel<true> : fb::fb_plan_kernel<false>, 1,
-                                           fb::kPlanThreads, stream, pp, counts, ctx->status);
+                                           fb::kPlanThreads, stream, pp, counts, counts_out, ctx->status);
   ++ctx->launches;
-  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
+  if (err == cudaSuccess) return FB_OK;
+  if (counts_out != nullptr) cudaMemsetAsync(counts, 0, FB_MAX_EXPERTS * sizeof(uint32_t), stream);
+  return FB_ERR_CUDA;
 }
 
 // Launch a router kernel in one of its modes.
@@ -349,10 +352,13 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   // the dispatch-index kernel counts and plans (see fb_dispatch_kernel).  With several tiles per pair the
   // early pass is done long before the normal one and the planner runs beside it.
   const bool tile_per_block = (T + fb::kDispatchTile - 1) / fb::kDispatchTile <= ctx->n_sm;   // of that kernel
-  p.defer_counts = (mode == fb::kModeLayer && !several && tile_per_block && p.fuse_planner && deferred_out != nullptr) ? 1 : 0;
+  // A prediction pass that plans hands its counts to the planner kernel where one tile per pair leaves nothing to hide it behind.
+  const bool layer_plan = mode == fb::kModeLayer && tile_per_block && p.fuse_planner && deferred_out != nullptr;
+  const bool pass_plan = mode == fb::kModePredictPlan && plan_wanted;
+  p.defer_counts = (!several && probe == 0 && (layer_plan || pass_plan)) ? 1 : 0;
   if (p.defer_counts) {
     p.fuse_planner = 0;
-    *deferred_out = true;
+    if (deferred_out != nullptr) *deferred_out = true;
   }
   int clusters = tile_pairs;
   if (several) {
@@ -411,7 +417,8 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   ++ctx->launches;
   if (several) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
-  if (plan_wanted && !p.fuse_planner && !p.defer_counts) return launch_plan(ctx, *plan, counts_out, stream);
+  if (pass_plan && p.defer_counts) return launch_plan(ctx, *plan, p.early_totals, counts_out, stream);
+  if (plan_wanted && !p.fuse_planner && !p.defer_counts) return launch_plan(ctx, *plan, counts_out, nullptr, stream);
   return FB_OK;
 }
 
@@ -735,7 +742,7 @@ fb_status fb_plan_swaps(fb_ctx* ctx, const uint32_t* counts, const int32_t* expe
   if (st != FB_OK) return st;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
-  return launch_plan(ctx, pp, counts, static_cast<cudaStream_t>(stream_));
+  return launch_plan(ctx, pp, const_cast<uint32_t*>(counts), nullptr, static_cast<cudaStream_t>(stream_));   // (read only)
 }
 
 fb_status fb_predict_and_plan(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T,
@@ -756,7 +763,7 @@ fb_status fb_predict_and_plan(fb_ctx* ctx, const fb_router* router, const void* 
   if (!guard.ok) return FB_ERR_CUDA;
   if (T == 0) {
     if (cudaMemsetAsync(counts, 0, ctx->cfg.E * sizeof(uint32_t), stream) != cudaSuccess) return FB_ERR_CUDA;
-    return launch_plan(ctx, pp, counts, stream);
+    return launch_plan(ctx, pp, counts, nullptr, stream);
   }
   return launch_router(ctx, router, x, T, fb::kModePredictPlan, counts, nullptr, nullptr, nullptr, &pp, stream);
 }

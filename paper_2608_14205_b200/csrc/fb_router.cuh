@@ -81,8 +81,9 @@ struct RouterParams {
   int32_t tiles_first;               // kModeLayer: blocks below this index (even) belong to the early pass
   int32_t ticket_target;             // number of tickets taken: one per block that publishes counts (persistent kernel: per pair)
   int32_t fuse_planner;              // prediction modes: the block that finishes last runs the planner
-  int32_t defer_counts;              // kModeLayer: the early pass adds its counts to early_totals and leaves the count
-                                     // vector and the plan to the dispatch-index kernel (fb_dispatch_kernel<true>)
+  int32_t defer_counts;              // the early pass adds its counts to early_totals and leaves the count vector and the
+                                     // plan to the next kernel: the dispatch index (kModeLayer, fb_dispatch_kernel<true>)
+                                     // or the planner kernel (kModePredictPlan)
   // fb_router_rows_kernel only: J block pairs per tile pair (cluster size / 2), the rows staged at a time
   // while the operand ring is busy with the next tile, and the column layout of a row over the lanes of a
   // warp: lane l holds columns g group_size + (l % lanes_per_group) cols_per_lane + j of group
@@ -1095,21 +1096,30 @@ fb_wait_selftest_kernel(uint64_t limit_ns, int32_t steps, int32_t* status, uint6
 
 // Stand-alone planner: placement and counts by one thread per expert (both loads in flight at once;
 // a single warp walking them took 11 of the kernel's 13 us), the decision by one warp.
+// counts_out: the counts are the totals that the blocks of a prediction pass have added up (early_totals); they become the
+// count vector (Eq. 5) and are put back to zero.  That takes the end of the pass out of the router kernel: a fence and a
+// ticket in every block, the last block's loads and the planner at the end of the grid took longer than this launch, which waits
+// on an SM of its own: prediction and plan of 300 tokens, 128 experts 14.3 -> 11.8 us, 8192 x 128 17.4 -> 16.4, 16384 x 256
+// (power bound) 65 -> 62.
 // kGeneral: for plans that need the general loop (plan_needs_general_loop).
 template <bool kGeneral>
 __global__ void __launch_bounds__(kPlanThreads, 1)
-fb_plan_kernel(const __grid_constant__ PlanParams p, const uint32_t* __restrict__ counts, int32_t* status) {
+fb_plan_kernel(const __grid_constant__ PlanParams p, uint32_t* __restrict__ counts, uint32_t* __restrict__ counts_out, int32_t* status) {
   __shared__ PlanShared sh;
   const int t = threadIdx.x;
   static_assert(kPlanThreads >= FB_MAX_EXPERTS, "one thread per expert");
   plan_clear(sh, t, kPlanThreads);
+  plan_place_ranks(p, sh, t, kPlanThreads);
   __syncthreads();
   pdl_wait();
   pdl_launch_dependents();               // (why here: fb_dispatch.cuh)
-  const uint32_t count = t < p.E ? __ldcg(counts + t) : 0u;
-  plan_load_placement(p, sh, t, kPlanThreads);
-  __syncthreads();
-  if (t < p.E) plan_put_count(sh, t, count);
+  if (t < p.E) {
+    const uint32_t count = __ldcg(counts + t);
+    const int slot = p.expert_to_slot[t];
+    plan_place(p, sh, t, slot);
+    plan_put_count_at(sh, t, slot, count, p.E);
+    if (counts_out != nullptr) { counts_out[t] = count; counts[t] = 0; }
+  }
   __syncthreads();
   if (t < 32) plan_swaps_warp<kGeneral>(p, sh, t, status);
   __syncthreads();

@@ -577,7 +577,9 @@ __device__ __forceinline__ void produce_operands(const RouterParams& p, const CU
                                                  const CUtensorMap* map_w, const TileWalk& w, uint32_t smem_base,
                                                  uint32_t stage_bytes, uint64_t* full_bar, uint64_t* empty_bar,
                                                  volatile int* abort_flag) {
-  const uint64_t pol_x = l2_policy_evict_first();            // x is streamed once
+  // x is streamed once - unless the logits are written as well: who asks for them compares the two passes and reads the
+  // hidden states again (call and quality figures, 8192 x 2048, 128 experts: 49.7 -> 47.7 us)
+  const uint64_t pol_x = p.logits != nullptr ? l2_policy_evict_normal() : l2_policy_evict_first();
   const uint64_t pol_w = l2_policy_evict_last();             // W is re-read by every pair
   const bool leader = elect_one();
   const uint32_t cta_rank = w.cluster_rank & 1u;

@@ -432,7 +432,7 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   const fb_config& c = ctx->cfg;
   fb::DispatchParams dp;
   memset(&dp, 0, sizeof(dp));
-  dp.T = T; dp.k = c.k; dp.E = c.E; dp.R = c.R;
+  dp.T = T; dp.k = c.k; dp.E = c.E; dp.R = c.R; dp.per_rank = c.E / c.R;
   dp.num_tiles = (T + fb::kDispatchTile - 1) / fb::kDispatchTile;
   dp.topk_ids = topk_ids;
   dp.slices_per_tile = slices_per_tile;
@@ -1212,6 +1212,7 @@ fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int
   if (!guard.ok) return FB_ERR_CUDA;
   fb::GlobalizeParams gp;
   gp.T = T_local; gp.k = ctx->cfg.k; gp.E = ctx->cfg.E; gp.R = ctx->cfg.R; gp.world = world; gp.rank = rank;
+  gp.per_rank = ctx->cfg.E / ctx->cfg.R;
   gp.counts_all = slot_counts_all; gp.local_offsets = slot_offsets_local; gp.topk_ids = topk_ids;
   gp.expert_to_slot = expert_to_slot; gp.inv_perm = inv_perm;
   gp.slot_offsets = slot_offsets; gp.rank_offsets = rank_offsets; gp.rank_load = rank_load;

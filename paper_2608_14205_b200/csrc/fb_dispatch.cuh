@@ -71,6 +71,7 @@ __host__ __device__ constexpr int slice_row_bytes(int E) { return (E + 15) & ~15
 struct DispatchParams {
   int32_t T, k, E, R, num_tiles;
   int32_t num_slices, slices_per_tile;
+  int32_t per_rank;                // E / R
   const int32_t* topk_ids;         // [T][k]
   const uint8_t* slice_counts;     // [num_slices][slice_row_bytes(E)]
   uint32_t* totals;                // [2][FB_MAX_EXPERTS]: normal, early pass; this grid's last block puts them back to zero
@@ -168,10 +169,15 @@ __device__ __forceinline__ uint32_t block_prefix(uint32_t count, uint32_t* warp_
 }
 
 __device__ __forceinline__ void write_offsets(const DispatchParams& p, const uint32_t* offs, int t) {
-  const int m = p.E / p.R;
-  for (int s = t; s <= p.E; s += kDispatchThreads) p.slot_offsets[s] = offs[s];
-  for (int r = t; r <= p.R; r += kDispatchThreads) p.rank_offsets[r] = offs[r * m];
-  for (int r = t; r < p.R; r += kDispatchThreads) p.rank_load[r] = offs[(r + 1) * m] - offs[r * m];
+  // (with loops over E and R and a division by R in block 0: layer call 1733 x 256 27.8 -> 27.1 us, 1000 x 128 14.9 -> 14.5,
+  // 40 x 128 13.4 -> 12.9)
+  static_assert(kDispatchThreads > FB_MAX_EXPERTS + FB_MAX_RANKS + 1, "one element per thread");
+  const int m = p.per_rank, r = t - (kDispatchThreads - FB_MAX_RANKS - 1);      // ranks: the last threads
+  if (t <= p.E) p.slot_offsets[t] = offs[t];
+  if (r >= 0 && r <= p.R) {
+    p.rank_offsets[r] = offs[r * m];
+    if (r < p.R) p.rank_load[r] = offs[(r + 1) * m] - offs[r * m];
+  }
 }
 
 // The totals have been read by all blocks: the last one puts them back to zero for the next call.  By one warp, after a
@@ -304,8 +310,8 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   }
   __syncthreads();
   FB_STAMP(27, 0);
-  if constexpr (kPlan)
-    if (tile == 0) plan_write_placement(p.plan, plan, t, kDispatchThreads);
+  if constexpr (kPlan)                             // (not by the block that writes the offsets, where there is another)
+    if (tile == (gridDim.x > 1 ? 1 : 0)) plan_write_placement(p.plan, plan, t, kDispatchThreads);
   if (usable) {
     if (tile == 0) write_offsets(p, offs, t);
     if (owns) {
@@ -529,6 +535,7 @@ constexpr int kGlobalizeThreads = 256;   // >= FB_MAX_EXPERTS: one thread per sl
 
 struct GlobalizeParams {
   int32_t T, k, E, R, world, rank;
+  int32_t per_rank;                  // E / R
   const uint32_t* counts_all;        // [world][E]
   const uint32_t* local_offsets;     // [E+1]
   const int32_t* topk_ids;           // [T][k] (local)
@@ -584,7 +591,7 @@ fb_dispatch_globalize_kernel(const __grid_constant__ GlobalizeParams p) {
   }
   __syncthreads();
   if (blockIdx.x == 0) {
-    const int m = p.E / p.R;
+    const int m = p.per_rank;
     for (int s = t; s <= p.E; s += kGlobalizeThreads) p.slot_offsets[s] = G[s];
     for (int r = t; r <= p.R; r += kGlobalizeThreads) p.rank_offsets[r] = G[r * m];
     for (int r = t; r < p.R; r += kGlobalizeThreads) p.rank_load[r] = G[(r + 1) * m] - G[r * m];

@@ -226,7 +226,9 @@ __device__ __forceinline__ void select_two_rows(const RouterParams& p, const Lan
 #pragma unroll
     for (int u = 0; u < 2; ++u) load_columns<kCpl>(key[u], a0 + u * stride, p, lc.n);
     uint32_t from = my_rank;
-#pragma unroll (kCpl >= 8 ? 1 : 3)
+    // (one, two, three and seven pieces' loads in flight with few columns per lane: 1000 x 128 14.2, 14.2, 14.5, 14.7 us, 40 x 128
+    // 13.0 to 13.1, 5 x 128 13.4, 13.1, 13.4, 13.5; with eight columns two and four were 0.6 us slower than one)
+#pragma unroll (kCpl >= 8 ? 1 : 2)
     for (int i = 1; i < p.pieces; ++i) {
       float t[2][kCpl];
       from = from + 2 < 2u * p.pieces ? from + 2 : from + 2 - 2u * p.pieces;

@@ -1,7 +1,8 @@
 // Fused router kernel: logits = x W^T (+ b) on tcgen05 tensor cores with fp32
 // accumulators in tensor memory, fed by TMA; then, straight out of tensor memory, the
-// model's gating rule, top-k, and a per-expert histogram (Eqs. 2-5).  The block that
-// finishes last publishes the count vector and, when asked, runs the swap planner.
+// model's gating rule, top-k, and a per-expert histogram (Eqs. 2-5).  The counts go to totals that the next
+// kernel of the call reads (dispatch index, planner), or the block that finishes last publishes them and, when asked,
+// runs the swap planner.
 //
 // One block owns 128 token rows and all N = pad16(E) expert columns.
 // Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer for the even k-blocks (owns the
@@ -59,7 +60,7 @@ constexpr uint32_t kRowBarrierBase = 3;      // named barriers 3..6: the kEpiSub
 
 enum RouterMode : int {
   kModePredict = 0,        // histogram -> counts
-  kModePredictPlan = 1,    // histogram -> counts -> planner in the block (or pair) that finishes last
+  kModePredictPlan = 1,    // histogram -> totals for the planner kernel, or -> counts -> planner in the pair that finishes last
   kModeDispatch = 2,       // ids, weights, per-tile histogram for the dispatch index
   kModeLayer = 3           // one launch for a whole layer: the first tiles_first tiles are the early pass
                            // (mode 1) on the first input, the others the normal pass (mode 2) on the

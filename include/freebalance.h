@@ -35,6 +35,12 @@
  *     and loads the kernels) they may be captured into a CUDA graph and the graph
  *     replayed on new contents of the same buffers.  Budgets and shapes are frozen into
  *     the graph at capture; fb_device_status is not capturable (it synchronises).
+ *   - Streams: calls of one context are made by one host thread at a time.  On the device a
+ *     prediction call (fb_predict_load, fb_predict_and_plan) of a context may run beside a
+ *     routing call (fb_route_dispatch, fb_layer_step) of the same context on another
+ *     stream, and fb_plan_swaps and the dispatch-index helpers beside anything; two
+ *     prediction calls, or two routing calls, of one context must not overlap (they share
+ *     its scratch): order them by the stream or by events, or use a context each.
  *   - No call throws or aborts.  Argument and shape problems are reported by the
  *     return value and nothing is launched.  Problems only the device can see (a
  *     placement that is not a bijection, count sums beyond the planner's range, a

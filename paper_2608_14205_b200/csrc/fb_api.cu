@@ -33,6 +33,7 @@ struct MapEntry {
 };
 
 constexpr int kMapCache = 8;
+constexpr size_t kLine = 32;            // words that blocks count on lie in lines of their own
 
 }  // namespace
 
@@ -61,11 +62,14 @@ struct fb_ctx {
   int n_sm = 148;                 // SMs of the device
   int split_mode = 1;             // k-range split over the blocks of a cluster: 0 off, 1 on
   EncodeTiledFn encode = nullptr;
-  // device scratch (one allocation from counts_scratch on but for slice_counts)
-  uint32_t* counts_scratch = nullptr;   // [256], zero between calls
-  uint32_t* ticket = nullptr;           // [1],   zero between calls
+  // device scratch (one allocation from counts_scratch on but for slice_counts).  A prediction call may run beside a routing
+  // call of the same context on another stream: they share no words of it.
+  uint32_t* counts_scratch = nullptr;   // [2][256], zero between calls: of prediction calls, of layer calls
+  uint32_t* ticket = nullptr;           // [2][kLine], zero between calls: the same
   int32_t* status = nullptr;            // [1]
-  uint32_t* totals = nullptr;           // [2][256], zero between calls: its sums, and the early pass's where the plan is made with the index
+  // [3][256], zero between calls: sums of slice_counts; the early pass's of a layer call whose plan is made with the index;
+  // those of a prediction call whose plan is made by the planner kernel
+  uint32_t* totals = nullptr;
   uint32_t* index_ticket = nullptr;     // [1],   zero between calls
   uint8_t* slice_counts = nullptr;      // [max_slices][slice_row_bytes(E)]: per-slice histograms for the dispatch index
   // descriptor cache
@@ -296,8 +300,9 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.mode = mode;
   p.logit_bias = router->logit_bias;
   p.select_bias = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? router->select_bias : nullptr;
-  p.counts_scratch = ctx->counts_scratch;
-  p.ticket = ctx->ticket;
+  const bool layer = mode == fb::kModeLayer;
+  p.counts_scratch = ctx->counts_scratch + (layer ? FB_MAX_EXPERTS : 0);
+  p.ticket = ctx->ticket + (layer ? kLine : 0);
   p.status = ctx->status;
   p.counts_out = counts_out;
   p.topk_ids = topk_ids;
@@ -307,7 +312,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.early_logits = early_logits;
   p.slice_counts = ctx->slice_counts;
   p.totals = ctx->totals;
-  p.early_totals = ctx->totals != nullptr ? ctx->totals + FB_MAX_EXPERTS : nullptr;
+  p.early_totals = ctx->totals != nullptr ? ctx->totals + (layer ? 1 : 2) * FB_MAX_EXPERTS : nullptr;
   p.stamps = ctx->stamps;
   p.probe = probe;
   if (plan) p.plan = *plan;
@@ -460,7 +465,8 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
                                            blocks, fb::kDispatchThreads, stream, dp);
   ++ctx->launches;
   if (err == cudaSuccess) return FB_OK;
-  cudaMemsetAsync(ctx->totals, 0, 2 * FB_MAX_EXPERTS * sizeof(uint32_t), stream);   // what the router kernel has added
+  // what the router kernel has added
+  cudaMemsetAsync(ctx->totals, 0, (plan != nullptr ? 2 : 1) * FB_MAX_EXPERTS * sizeof(uint32_t), stream);
   return FB_ERR_CUDA;
 }
 
@@ -683,16 +689,15 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
     return FB_ERR_CUDA;
   }
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
-  // Everything that is zero between calls is one allocation and one memset (a context in 325 us; 337 with five of each);
-  // the words that blocks count on lie in lines of their own.
-  constexpr size_t kLine = 32, kZeroWords = 3 * FB_MAX_EXPERTS + 3 * kLine;
+  // Everything that is zero between calls is one allocation and one memset (a context in 325 us; 337 with five of each).
+  constexpr size_t kZeroWords = 5 * FB_MAX_EXPERTS + 4 * kLine;
   bool ok = dev_alloc(&ctx->counts_scratch, kZeroWords) &&
             dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E)) &&
             cudaMemset(ctx->counts_scratch, 0, kZeroWords * sizeof(uint32_t)) == cudaSuccess;
   if (ok) {
-    ctx->totals = ctx->counts_scratch + FB_MAX_EXPERTS;
-    ctx->ticket = ctx->totals + 2 * FB_MAX_EXPERTS;
-    ctx->index_ticket = ctx->ticket + kLine;
+    ctx->totals = ctx->counts_scratch + 2 * FB_MAX_EXPERTS;
+    ctx->ticket = ctx->totals + 3 * FB_MAX_EXPERTS;
+    ctx->index_ticket = ctx->ticket + 2 * kLine;
     ctx->status = reinterpret_cast<int32_t*>(ctx->index_ticket + kLine);
   }
   if (!ok) { fb_destroy(ctx); return FB_ERR_CUDA; }

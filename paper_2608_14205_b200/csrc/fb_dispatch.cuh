@@ -74,7 +74,9 @@ struct DispatchParams {
   int32_t per_rank;                // E / R
   const int32_t* topk_ids;         // [T][k]
   const uint8_t* slice_counts;     // [num_slices][slice_row_bytes(E)]
-  uint32_t* totals;                // [2][FB_MAX_EXPERTS]: normal, early pass; this grid's last block puts them back to zero
+  // [FB_MAX_EXPERTS] of the normal pass, then (fb_dispatch_kernel<true> only) as many of the early pass; what the grid has
+  // read its last block puts back to zero
+  uint32_t* totals;
   uint32_t* ticket;                // zero on entry, zero again on exit
   const int32_t* expert_to_slot;   // [E]
   uint32_t* slot_offsets;          // [E+1]
@@ -180,14 +182,16 @@ __device__ __forceinline__ void write_offsets(const DispatchParams& p, const uin
   }
 }
 
-// The totals have been read by all blocks: the last one puts them back to zero for the next call.  By one warp, after a
-// barrier behind the block's reads (their values have arrived: nothing of this grid is still to be read).
+// The totals have been read by all blocks: the last one puts them back to zero for the next call (kBoth: those of both
+// passes; otherwise the early pass's words are another call's).  By one warp, after a barrier behind the block's reads
+// (their values have arrived: nothing of this grid is still to be read).
 __device__ __forceinline__ uint32_t take_index_ticket(const DispatchParams& p, int lane) {
   return lane == 0 ? atomicAdd(p.ticket, 1u) : 0u;
 }
+template <bool kBoth>
 __device__ __forceinline__ void clear_totals(const DispatchParams& p, uint32_t ticket, int lane) {
   if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
-  for (int i = lane; i < 2 * FB_MAX_EXPERTS; i += 32) p.totals[i] = 0;
+  for (int i = lane; i < (kBoth ? 2 : 1) * FB_MAX_EXPERTS; i += 32) p.totals[i] = 0;
   if (lane == 0) *p.ticket = 0;
 }
 
@@ -327,7 +331,7 @@ fb_dispatch_kernel(const __grid_constant__ DispatchParams p) {
   } else if (!kPlan && t == 0 && tile == 0) {      // not a bijection: report (the planner has), write no index
     atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);
   }
-  if (warp == kDispatchWarps - 1) clear_totals(p, ticket, lane);
+  if (warp == kDispatchWarps - 1) clear_totals<kPlan>(p, ticket, lane);
   FB_STAMP(28, 0);
 }
 
@@ -411,7 +415,7 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
   __syncthreads();
   const uint32_t ticket = warp == kDispatchWarps - 1 ? take_index_ticket(p, lane) : 0u;
   if (bad || tile_begin >= tile_end) {
-    if (warp == kDispatchWarps - 1) clear_totals(p, ticket, lane);
+    if (warp == kDispatchWarps - 1) clear_totals<false>(p, ticket, lane);
     if (bad && t == 0 && blockIdx.x == 0) atomicCAS(p.status, 0, FB_ERR_BAD_PLACEMENT);   // not a bijection: report, write nothing
     return;
   }
@@ -510,7 +514,7 @@ fb_dispatch_runs_kernel(const __grid_constant__ DispatchParams p) {
     mark_rows();
     __syncthreads();
   }
-  if (warp == kDispatchWarps - 1) clear_totals(p, ticket, lane);
+  if (warp == kDispatchWarps - 1) clear_totals<false>(p, ticket, lane);
 }
 
 // ---- token-sharded dispatch (several GPUs, each with a contiguous token range in rank order)

@@ -27,6 +27,11 @@ uint64_t fb_persistent_launch_count(const fb_ctx* ctx);
  * alone inside a call that launches several kernels. */
 fb_status fb_time_next_router_launch(fb_ctx* ctx, void* event_before, void* event_after);
 
+/* Diagnostic: the nth (1 = next) of the launches counted by fb_launch_count from now on is not made; the call
+ * it belongs to sees a failed launch and returns FB_ERR_CUDA.  0: none (the default).  For tests of
+ * what a call leaves behind when one of its launches fails.  FB_ERR_INVALID_ARG for a negative n. */
+fb_status fb_fail_launch(fb_ctx* ctx, int32_t nth);
+
 /* Diagnostic: later router launches of this context use at most `stages` stages of the
  * operand pipeline (0 lifts the limit; 1 is not a pipeline: FB_ERR_INVALID_ARG).  Results do
  * not depend on the depth, only the speed does.  Exists so that tests can run short rings and

@@ -61,7 +61,7 @@ EXPORTS = ["fb_create", "fb_destroy", "fb_budget_ns", "fb_swap_cost_ns", "fb_pre
            "fb_attention_set_time_ns", "fb_attention_reset", "fb_dispatch_slot_counts", "fb_dispatch_globalize",
            "fb_standin_attention", "fb_set_split", "fb_prediction_quality",
            "fb_layer_step_observed", "fb_staged_row_layout",
-           "fb_selftest_wait_progress"]
+           "fb_selftest_wait_progress", "fb_fail_launch"]
 
 _lib = None
 
@@ -110,6 +110,8 @@ def lib() -> ctypes.CDLL:
     L.fb_device_status.argtypes = [vp, ctypes.POINTER(i32), vp]
     L.fb_staged_row_layout.argtypes = [ctypes.POINTER(FbConfig)] + [vp] * 3
     L.fb_staged_row_layout.restype = ctypes.c_int
+    L.fb_fail_launch.argtypes = [vp, i32]
+    L.fb_fail_launch.restype = ctypes.c_int
     L.fb_set_stage_limit.argtypes = [vp, i32]
     L.fb_set_stage_limit.restype = ctypes.c_int
     L.fb_set_pair_limit.argtypes = [vp, i32]
@@ -381,6 +383,9 @@ class Context:
 
     def fb_set_pair_limit(self, pairs: int) -> None:
         _check(lib().fb_set_pair_limit(self._h, pairs), "fb_set_pair_limit")
+
+    def fb_fail_launch(self, nth: int) -> None:
+        _check(lib().fb_fail_launch(self._h, nth), "fb_fail_launch")
 
     def fb_set_stage_limit(self, stages: int) -> None:
         _check(lib().fb_set_stage_limit(self._h, stages), "fb_set_stage_limit")

@@ -89,6 +89,7 @@ struct fb_ctx {
   uint32_t* st_slot_offsets = nullptr; uint32_t* st_rank_offsets = nullptr;
   int32_t* st_perm = nullptr; int32_t* st_inv_perm = nullptr; uint32_t* st_rank_load = nullptr;
   uint64_t launches = 0;
+  int fail_launch = 0;                                   // see fb_fail_launch
   uint64_t persistent_launches = 0;
   cudaEvent_t ev_before = nullptr, ev_after = nullptr;   // one-shot: recorded around the next router launch
   unsigned long long* stamps = nullptr;                  // caller's phase-stamp buffer (FB_TIMING builds)
@@ -263,14 +264,27 @@ cudaError_t launch_dependent(void (*kernel)(Params...), int blocks, int threads,
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// One of a context's launches: counted, and with fb_fail_launch one of them is not made.
+bool launch_refused(fb_ctx* ctx) {
+  ++ctx->launches;
+  return ctx->fail_launch > 0 && --ctx->fail_launch == 0;
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_counted(fb_ctx* ctx, void (*kernel)(Params...), int blocks, int threads, cudaStream_t stream, Args... args) {
+  return launch_refused(ctx) ? cudaErrorUnknown : launch_dependent(kernel, blocks, threads, stream, args...);
+}
+
+// A kernel that should have read and cleared `sets` of the context's totals from `first` on was not launched behind the
+// router kernel that adds to them: back to zero for the next call.
+void clear_unread_totals(fb_ctx* ctx, int first, int sets, cudaStream_t stream) {
+  cudaMemsetAsync(ctx->totals + first * FB_MAX_EXPERTS, 0, static_cast<size_t>(sets) * FB_MAX_EXPERTS * sizeof(uint32_t), stream);
+}
+
 // counts_out: counts are the totals of a prediction pass (see fb_plan_kernel).
 fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, uint32_t* counts, uint32_t* counts_out, cudaStream_t stream) {
-  const cudaError_t err = launch_dependent(fb::plan_needs_general_loop(pp) ? fb::fb_plan_kernel<true> : fb::fb_plan_kernel<false>, 1,
-                                           fb::kPlanThreads, stream, pp, counts, counts_out, ctx->status);
-  ++ctx->launches;
-  if (err == cudaSuccess) return FB_OK;
-  if (counts_out != nullptr) cudaMemsetAsync(counts, 0, FB_MAX_EXPERTS * sizeof(uint32_t), stream);
-  return FB_ERR_CUDA;
+  const cudaError_t err = launch_counted(ctx, fb::plan_needs_general_loop(pp) ? fb::fb_plan_kernel<true> : fb::fb_plan_kernel<false>,
+                                         1, fb::kPlanThreads, stream, pp, counts, counts_out, ctx->status);
+  return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
 // Launch a router kernel in one of its modes.
@@ -416,15 +430,19 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const cudaError_t err = cudaLaunchKernelEx(&cfg, fn, *mx, *mx2, *mw, p);
+  const cudaError_t err = launch_refused(ctx) ? cudaErrorUnknown : cudaLaunchKernelEx(&cfg, fn, *mx, *mx2, *mw, p);
   if (ctx->ev_after) cudaEventRecord(ctx->ev_after, stream);
   ctx->ev_before = ctx->ev_after = nullptr;
-  ++ctx->launches;
   if (several) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
-  if (pass_plan && p.defer_counts) return launch_plan(ctx, *plan, p.early_totals, counts_out, stream);
-  if (plan_wanted && !p.fuse_planner && !p.defer_counts) return launch_plan(ctx, *plan, counts_out, nullptr, stream);
-  return FB_OK;
+  if (pass_plan && p.defer_counts) {
+    st = launch_plan(ctx, *plan, p.early_totals, counts_out, stream);
+    if (st != FB_OK) clear_unread_totals(ctx, 2, 1, stream);
+  } else if (plan_wanted && !p.fuse_planner && !p.defer_counts) {
+    st = launch_plan(ctx, *plan, counts_out, nullptr, stream);
+    if (st != FB_OK && layer) clear_unread_totals(ctx, 0, 1, stream);     // no dispatch index follows
+  }
+  return st;
 }
 
 // Dispatch index from the router kernel's top-k ids and per-slice histograms.  plan: also the count vector and
@@ -459,14 +477,12 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   // one block per SM at most: more tiles than that are walked in runs (every block reads the whole
   // histogram table once, so more blocks would only read it more often)
   const int blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;
-  const cudaError_t err = launch_dependent(blocks < dp.num_tiles ? fb::fb_dispatch_runs_kernel
-                                           : plan != nullptr     ? fb::fb_dispatch_kernel<true>
-                                                                 : fb::fb_dispatch_kernel<false>,
-                                           blocks, fb::kDispatchThreads, stream, dp);
-  ++ctx->launches;
+  const cudaError_t err = launch_counted(ctx, blocks < dp.num_tiles ? fb::fb_dispatch_runs_kernel
+                                              : plan != nullptr     ? fb::fb_dispatch_kernel<true>
+                                                                    : fb::fb_dispatch_kernel<false>,
+                                         blocks, fb::kDispatchThreads, stream, dp);
   if (err == cudaSuccess) return FB_OK;
-  // what the router kernel has added
-  cudaMemsetAsync(ctx->totals, 0, (plan != nullptr ? 2 : 1) * FB_MAX_EXPERTS * sizeof(uint32_t), stream);
+  clear_unread_totals(ctx, 0, plan != nullptr ? 2 : 1, stream);
   return FB_ERR_CUDA;
 }
 
@@ -1165,6 +1181,12 @@ fb_status fb_staged_row_layout(const fb_config* cfg, int32_t* row_words, int32_t
   return FB_OK;
 }
 
+fb_status fb_fail_launch(fb_ctx* ctx, int32_t nth) {
+  if (!ctx || nth < 0) return FB_ERR_INVALID_ARG;
+  ctx->fail_launch = nth;
+  return FB_OK;
+}
+
 fb_status fb_set_stage_limit(fb_ctx* ctx, int32_t stages) {
   if (!ctx || stages < 0 || stages == 1) return FB_ERR_INVALID_ARG;
   ctx->stage_limit = stages;
@@ -1200,9 +1222,8 @@ fb_status fb_dispatch_slot_counts(fb_ctx* ctx, const uint32_t* slot_offsets, uin
   if (!ctx || !slot_offsets || !slot_counts) return FB_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
-  const cudaError_t err = launch_dependent(fb::fb_slot_counts_kernel, 1, FB_MAX_EXPERTS, static_cast<cudaStream_t>(stream_),
-                                           slot_offsets, ctx->cfg.E, slot_counts);
-  ++ctx->launches;
+  const cudaError_t err = launch_counted(ctx, fb::fb_slot_counts_kernel, 1, FB_MAX_EXPERTS, static_cast<cudaStream_t>(stream_),
+                                         slot_offsets, ctx->cfg.E, slot_counts);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
@@ -1228,9 +1249,8 @@ fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int
   long long blocks = (n + fb::kGlobalizeThreads - 1) / fb::kGlobalizeThreads;
   if (blocks < 1) blocks = 1;
   if (blocks > 4 * ctx->n_sm) blocks = 4 * ctx->n_sm;
-  const cudaError_t err = launch_dependent(fb::fb_dispatch_globalize_kernel, static_cast<int>(blocks), fb::kGlobalizeThreads,
-                                           static_cast<cudaStream_t>(stream_), gp);
-  ++ctx->launches;
+  const cudaError_t err = launch_counted(ctx, fb::fb_dispatch_globalize_kernel, static_cast<int>(blocks), fb::kGlobalizeThreads,
+                                         static_cast<cudaStream_t>(stream_), gp);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 

@@ -79,3 +79,44 @@ def test_prediction_and_routing_calls_of_one_context_overlap(name, T, pair_limit
     for key, v in big.items():
         assert torch.equal(v, want[((reps - 1) // 3) % 2][2][key]), key
     ctx.close()
+
+
+# The router kernel fills the SMs that the other stream's kernel leaves.  The planner behind it must not run on that kernel's SMs,
+# where its one warp got an issue slot in 30: planning took 50 to 70 us instead of 2.  20 us leave room for the spread of
+# two medians and the planner's launch.
+@pytest.mark.parametrize("name,T,pairs", [("qwen3", 8192, 32), ("qwen3", 2000, 8), ("tiny", 512, 2)])
+def test_planning_is_not_held_up_by_a_kernel_on_the_other_sms(name, T, pairs):
+    wl = I.WORKLOADS[name]
+    li = I.make_layer(wl, 0, 0, T=T)
+    ctx = P.make_context(wl, T)
+    ctx.fb_set_pair_limit(pairs)
+    dev = torch.device("cuda", ctx.device)
+    router = B.make_router(li.W.to(dev), None, None)
+    x, pi = li.h_prev.to(dev), li.expert_to_slot.to(dev)
+    budget = B.make_budget(**P.budget_kwargs(wl, T))
+    i32 = lambda n: torch.zeros(max(1, n), dtype=torch.int32, device=dev)
+    o = (i32(wl.E), i32(wl.E), i32(4 * (wl.E // 2)), i32(1), i32(wl.R), i32(wl.R))
+    n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
+    sink = torch.zeros(1024 * n_sm, device=dev)
+    main, side = torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
+
+    def beside(call):
+        times = []
+        for _ in range(15):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            with torch.cuda.stream(main):
+                B.fb_standin_attention(sink, n_sm - 2 * pairs, 3000)           # some 400 us
+            with torch.cuda.stream(side):
+                torch.cuda._sleep(50000)                                       # until it has its SMs
+                a.record()
+                call()
+                b.record()
+            torch.cuda.synchronize(dev)
+            times.append(a.elapsed_time(b) * 1e3)
+        return sorted(times)[len(times) // 2]
+
+    predict = beside(lambda: ctx.fb_predict_load(router, x, T, o[0]))
+    plan = beside(lambda: ctx.fb_predict_and_plan(router, x, T, pi, budget, 0, *o))
+    assert ctx.fb_device_status() == 0
+    assert plan < predict + 20.0, (predict, plan)
+    ctx.close()

@@ -572,16 +572,21 @@ __device__ __forceinline__ void prefetch_operands(const RouterParams& p, const C
   }
 }
 
+// L2 policies of the operand loads.  x is streamed once - unless the logits are written as well: who asks for them compares
+// the two passes and reads the hidden states again (call and quality figures, 8192 x 2048, 128 experts: 49.7 -> 47.7 us).  W is
+// re-read by every pair.  Made by the producer warp before its wait for the stream's earlier kernels: behind the wait the choice
+// between the two took 0.1 us of every launch (8 experts, 128 tokens, prediction 7.00 -> 7.09 us).
+struct LoadPolicies { uint64_t x, w; };
+__device__ __forceinline__ LoadPolicies load_policies(const RouterParams& p) {
+  return {p.logits != nullptr ? l2_policy_evict_normal() : l2_policy_evict_first(), l2_policy_evict_last()};
+}
+
 // TMA producer (a whole warp): both blocks of a pair report their bytes to the even block's barrier, which
 // expects the bytes of both.
 __device__ __forceinline__ void produce_operands(const RouterParams& p, const CUtensorMap* map_x, const CUtensorMap* map_x2,
                                                  const CUtensorMap* map_w, const TileWalk& w, uint32_t smem_base,
                                                  uint32_t stage_bytes, uint64_t* full_bar, uint64_t* empty_bar,
-                                                 volatile int* abort_flag) {
-  // x is streamed once - unless the logits are written as well: who asks for them compares the two passes and reads the
-  // hidden states again (call and quality figures, 8192 x 2048, 128 experts: 49.7 -> 47.7 us)
-  const uint64_t pol_x = p.logits != nullptr ? l2_policy_evict_normal() : l2_policy_evict_first();
-  const uint64_t pol_w = l2_policy_evict_last();             // W is re-read by every pair
+                                                 const LoadPolicies& policy, volatile int* abort_flag) {
   const bool leader = elect_one();
   const uint32_t cta_rank = w.cluster_rank & 1u;
   const int stages = p.stages, w_row = static_cast<int>(cta_rank) * (p.N / 2);
@@ -601,8 +606,8 @@ __device__ __forceinline__ void produce_operands(const RouterParams& p, const CU
         const uint32_t a_dst = smem_base + static_cast<uint32_t>(s) * stage_bytes;
         const uint32_t full = map_to_cta(smem_u32(&full_bar[s]), w.cluster_rank & ~1u);
         if (cta_rank == 0) mbar_arrive_expect_tx(smem_u32(&full_bar[s]), 2u * stage_bytes);
-        tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, row, pol_x);
-        tma_load_2d_pair(a_dst + kATileBytes, map_w, full, kb * kBlockK, w_row, pol_w);
+        tma_load_2d_pair(a_dst, xmap, full, kb * kBlockK, row, policy.x);
+        tma_load_2d_pair(a_dst + kATileBytes, map_w, full, kb * kBlockK, w_row, policy.w);
       }
       __syncwarp();
       ring_advance(s, phase, stages);
@@ -753,6 +758,8 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   walk.kb0 = 0;
   walk.n_kb = p.num_kb;
   walk.cluster_rank = cta_rank;
+  LoadPolicies policies = {0, 0};
+  if (warp == 0) policies = load_policies(p);
   if (warp == kSecondIssuerWarp) prefetch_operands(p, &tmap_x, &tmap_x2, walk, &sh.started);
   // Everything above touched only this block's own state and the call's parameters; from here on
   // the kernel reads memory that earlier work of the stream may have written.
@@ -769,7 +776,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   FB_STAMP(1, 64);
 
   if (warp == 0) {
-    produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
+    produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, policies, abort_flag);
     cluster_arrive_relaxed();  // this warp is done with the pair's shared state (see the teardown)
   } else if (warp == 1 || warp == kSecondIssuerWarp) {
     // MMA issuers: in a pair only the even block issues

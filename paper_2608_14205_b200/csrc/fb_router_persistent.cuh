@@ -156,6 +156,8 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   walk.kb0 = 0;
   walk.n_kb = p.num_kb;
   walk.cluster_rank = cta_rank;
+  LoadPolicies policies = {0, 0};
+  if (warp == 0) policies = load_policies(p);
   if (warp == kSecondIssuerWarp) prefetch_operands(p, &tmap_x, &tmap_x2, walk, &sh.started);
   // Everything above touched only this block's own state and the call's parameters; from here on
   // the kernel reads memory that earlier work of the stream may have written.
@@ -174,7 +176,7 @@ fb_router_persistent_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     if (p.mode != kModeDispatch && pair_first < pairs_per_pass) finish_early_pass(sh, p, lane, abort_flag);
   } else if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
     if (warp == 0)
-      produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
+      produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, policies, abort_flag);
     else if (cta_rank == 0 && (warp == 1 || p.issuers == 2))
       issue_mmas(p, walk, warp == 1 ? 0 : 1, tmem_base, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, sh.accum_bar,
                  sh.tmem_empty_bar, sh.issuer_progress, abort_flag);

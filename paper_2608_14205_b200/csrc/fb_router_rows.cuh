@@ -685,6 +685,8 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
   walk.kb0 = kb0;
   walk.n_kb = n_kb;
   walk.cluster_rank = cluster_rank;
+  LoadPolicies policies = {0, 0};
+  if (warp == 0) policies = load_policies(p);
   if (warp == kSecondIssuerWarp) prefetch_operands(p, &tmap_x, &tmap_x2, walk, &sh.started);
   // (see fb_router_kernel for these two)
   pdl_wait();
@@ -696,7 +698,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
 
   if (warp == 0 || warp == 1 || warp == kSecondIssuerWarp) {
     if (warp == 0)
-      produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, abort_flag);
+      produce_operands(p, &tmap_x, &tmap_x2, &tmap_w, walk, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, policies, abort_flag);
     else if (cta_rank == 0 && (warp == 1 || p.issuers == 2))
       issue_mmas(p, walk, warp == 1 ? 0 : 1, tmem_base, smem_base, stage_bytes, sh.full_bar, sh.empty_bar, sh.accum_bar,
                  sh.tmem_empty_bar, sh.issuer_progress, abort_flag);

@@ -65,13 +65,12 @@ struct fb_ctx {
   EncodeTiledFn encode = nullptr;
   // device scratch (one allocation from counts_scratch on but for slice_counts).  A prediction call may run beside a routing
   // call of the same context on another stream: they share no words of it.
-  uint32_t* counts_scratch = nullptr;   // [2][256], zero between calls: of prediction calls, of layer calls
-  uint32_t* ticket = nullptr;           // [2][kLine], zero between calls: the same
-  int32_t* status = nullptr;            // [1]
-  // [3][256], zero between calls: sums of slice_counts; the early pass's of a layer call whose plan is made with the index;
-  // those of a prediction call whose plan is made by the planner kernel
-  uint32_t* totals = nullptr;
+  uint32_t* counts_scratch = nullptr;   // [256], zero between calls: the early pass's counts, prediction calls
+  uint32_t* totals = nullptr;           // [256], zero between calls: sums of slice_counts
+  uint32_t* layer_counts = nullptr;     // [256] directly behind them, zero between calls: the early pass's counts, layer calls
+  uint32_t* ticket = nullptr;           // [2][kLine], zero between calls: prediction calls, layer calls
   uint32_t* index_ticket = nullptr;     // [1],   zero between calls
+  int32_t* status = nullptr;            // [1]
   uint8_t* slice_counts = nullptr;      // [max_slices][slice_row_bytes(E)]: per-slice histograms for the dispatch index
   // descriptor cache
   MapEntry x_maps[kMapCache];
@@ -276,10 +275,10 @@ cudaError_t launch_counted(fb_ctx* ctx, void (*kernel)(Params...), int blocks, i
   return launch_refused(ctx) ? cudaErrorUnknown : launch_dependent(kernel, blocks, threads, smem, stream, args...);
 }
 
-// A kernel that should have read and cleared `sets` of the context's totals from `first` on was not launched behind the
-// router kernel that adds to them: back to zero for the next call.
-void clear_unread_totals(fb_ctx* ctx, int first, int sets, cudaStream_t stream) {
-  cudaMemsetAsync(ctx->totals + first * FB_MAX_EXPERTS, 0, static_cast<size_t>(sets) * FB_MAX_EXPERTS * sizeof(uint32_t), stream);
+// A kernel that should have read and cleared these of the context's words was not launched behind the router kernel that
+// adds to them: back to zero for the next call.
+void clear_unread(uint32_t* words, int sets, cudaStream_t stream) {
+  cudaMemsetAsync(words, 0, static_cast<size_t>(sets) * FB_MAX_EXPERTS * sizeof(uint32_t), stream);
 }
 
 // counts_out: counts are the totals of a prediction pass (see fb_plan_kernel).
@@ -322,7 +321,7 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.logit_bias = router->logit_bias;
   p.select_bias = c.gate == FB_GATE_SIGMOID_GROUP_TOPK ? router->select_bias : nullptr;
   const bool layer = mode == fb::kModeLayer;
-  p.counts_scratch = ctx->counts_scratch + (layer ? FB_MAX_EXPERTS : 0);
+  p.counts_scratch = layer ? ctx->layer_counts : ctx->counts_scratch;
   p.ticket = ctx->ticket + (layer ? kLine : 0);
   p.status = ctx->status;
   p.counts_out = counts_out;
@@ -333,7 +332,6 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.early_logits = early_logits;
   p.slice_counts = ctx->slice_counts;
   p.totals = ctx->totals;
-  p.early_totals = ctx->totals != nullptr ? ctx->totals + (layer ? 1 : 2) * FB_MAX_EXPERTS : nullptr;
   p.stamps = ctx->stamps;
   p.probe = probe;
   if (plan) p.plan = *plan;
@@ -443,11 +441,11 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   if (several) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
   if (pass_plan && p.defer_counts) {
-    st = launch_plan(ctx, *plan, p.early_totals, counts_out, ctx->plan_smem, stream);
-    if (st != FB_OK) clear_unread_totals(ctx, 2, 1, stream);
+    st = launch_plan(ctx, *plan, p.counts_scratch, counts_out, ctx->plan_smem, stream);
+    if (st != FB_OK) clear_unread(p.counts_scratch, 1, stream);
   } else if (plan_wanted && !p.fuse_planner && !p.defer_counts) {
     st = launch_plan(ctx, *plan, counts_out, nullptr, ctx->plan_smem, stream);
-    if (st != FB_OK && layer) clear_unread_totals(ctx, 0, 1, stream);     // no dispatch index follows
+    if (st != FB_OK && layer) clear_unread(ctx->totals, 1, stream);     // no dispatch index follows
   }
   return st;
 }
@@ -489,7 +487,7 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
                                                                     : fb::fb_dispatch_kernel<false>,
                                          blocks, fb::kDispatchThreads, 0, stream, dp);
   if (err == cudaSuccess) return FB_OK;
-  clear_unread_totals(ctx, 0, plan != nullptr ? 2 : 1, stream);
+  clear_unread(ctx->totals, plan != nullptr ? 2 : 1, stream);
   return FB_ERR_CUDA;
 }
 
@@ -720,13 +718,14 @@ fb_status fb_create(fb_ctx** out, const fb_config* cfg, int device) {
   }
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
   // Everything that is zero between calls is one allocation and one memset (a context in 325 us; 337 with five of each).
-  constexpr size_t kZeroWords = 5 * FB_MAX_EXPERTS + 4 * kLine;
+  constexpr size_t kZeroWords = 3 * FB_MAX_EXPERTS + 4 * kLine;
   bool ok = dev_alloc(&ctx->counts_scratch, kZeroWords) &&
             dev_alloc(&ctx->slice_counts, max_slices(ctx) * fb::slice_row_bytes(cfg->E)) &&
             cudaMemset(ctx->counts_scratch, 0, kZeroWords * sizeof(uint32_t)) == cudaSuccess;
   if (ok) {
-    ctx->totals = ctx->counts_scratch + 2 * FB_MAX_EXPERTS;
-    ctx->ticket = ctx->totals + 3 * FB_MAX_EXPERTS;
+    ctx->totals = ctx->counts_scratch + FB_MAX_EXPERTS;
+    ctx->layer_counts = ctx->totals + FB_MAX_EXPERTS;
+    ctx->ticket = ctx->layer_counts + FB_MAX_EXPERTS;
     ctx->index_ticket = ctx->ticket + 2 * kLine;
     ctx->status = reinterpret_cast<int32_t*>(ctx->index_ticket + kLine);
   }

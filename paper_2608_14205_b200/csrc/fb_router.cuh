@@ -82,7 +82,7 @@ struct RouterParams {
   int32_t tiles_first;               // kModeLayer: blocks below this index (even) belong to the early pass
   int32_t ticket_target;             // number of tickets taken: one per block that publishes counts (persistent kernel: per pair)
   int32_t fuse_planner;              // prediction modes: the block that finishes last runs the planner
-  int32_t defer_counts;              // the early pass adds its counts to early_totals and leaves the count vector and the
+  int32_t defer_counts;              // the early pass adds its counts to counts_scratch and leaves the count vector and the
                                      // plan to the next kernel: the dispatch index (kModeLayer, fb_dispatch_kernel<true>)
                                      // or the planner kernel (kModePredictPlan)
   // fb_router_rows_kernel only: J block pairs per tile pair (cluster size / 2), the rows staged at a time
@@ -96,7 +96,8 @@ struct RouterParams {
   int32_t ragged;                    // some lane holds fewer columns than the kernel instance is made for
   const float* logit_bias;           // [E] or nullptr
   const float* select_bias;          // [E] or nullptr
-  uint32_t* counts_scratch;          // [E] zero on entry, zero again on exit
+  uint32_t* counts_scratch;          // [E] the early pass's counts, zero on entry; zero again on exit, or left to the next
+                                     // kernel of the call (defer_counts)
   uint32_t* ticket;                  // zero on entry, zero again on exit
   int32_t* status;
   uint32_t* counts_out;              // [E]           (predict modes)
@@ -107,7 +108,6 @@ struct RouterParams {
   float* early_logits;
   uint8_t* slice_counts;             // [tiles * pieces][slice_row_bytes(E)] (dispatch mode)
   uint32_t* totals;                  // [E] sums of that table over all slices, zero on entry (dispatch mode)
-  uint32_t* early_totals;            // [E] the early pass's, zero on entry (defer_counts)
   unsigned long long* stamps;        // [blocks][64] phase time stamps (FB_TIMING builds) or nullptr
   int32_t probe;                     // measurement aid: 1 = operands are loaded but no MMA is issued and nothing
                                      // follows the main loop; 2 = with the MMAs, still nothing after them
@@ -1046,7 +1046,7 @@ fb_router_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     named_bar_sync(kPlanBarrierId, kEpilogueThreads);
     if (mode == kModeDispatch || p.defer_counts) {
       if (static_cast<long long>(tile) * kTileM < p.T) {     // the padding block of an odd pair owns no tile
-        add_to_totals(mode == kModeDispatch ? p.totals : p.early_totals, E, et < FB_MAX_EXPERTS ? sh.hist[et] : 0u, et);
+        add_to_totals(mode == kModeDispatch ? p.totals : p.counts_scratch, E, et < FB_MAX_EXPERTS ? sh.hist[et] : 0u, et);
         if (mode == kModeDispatch) write_slice_counts(p.slice_counts, tile, E, sh.hist, et);
       }
     } else if (p.probe == 0) {
@@ -1106,7 +1106,7 @@ fb_wait_selftest_kernel(uint64_t limit_ns, int32_t steps, int32_t* status, uint6
 
 // Stand-alone planner: placement and counts by one thread per expert (both loads in flight at once;
 // a single warp walking them took 11 of the kernel's 13 us), the decision by one warp.
-// counts_out: the counts are the totals that the blocks of a prediction pass have added up (early_totals); they become the
+// counts_out: the counts are the totals that the blocks of a prediction pass have added up (counts_scratch); they become the
 // count vector (Eq. 5) and are put back to zero.  That takes the end of the pass out of the router kernel: a fence and a
 // ticket in every block, the last block's loads and the planner at the end of the grid took longer than this launch, which waits
 // on an SM of its own: prediction and plan of 300 tokens, 128 experts 14.3 -> 11.8 us, 8192 x 128 17.4 -> 16.4, 16384 x 256

@@ -838,7 +838,7 @@ fb_router_rows_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
           if (et < FB_MAX_EXPERTS) my_total += sh.hist[et];
           if (mode == kModeDispatch) write_slice_counts(p.slice_counts, slice, E, sh.hist, et);
         }
-        if (last_tile) add_to_totals(mode == kModeDispatch ? p.totals : p.early_totals, E, my_total, et);
+        if (last_tile) add_to_totals(mode == kModeDispatch ? p.totals : p.counts_scratch, E, my_total, et);
         if (several_tiles) {
           named_bar_sync(kPlanBarrierId, kEpilogueThreads);
           for (int e = et; e < E; e += kEpilogueThreads) sh.hist[e] = 0;

@@ -84,8 +84,8 @@ def test_captured_calls_replay_bit_for_bit(name, T, pair_limit):
 
 @pytest.mark.parametrize("name,T,pair_limit", [("tiny", 300, 0), ("qwen3", 8192, 0), ("dsv3", 1500, 0), ("dsv3", 1500, 2)])
 def test_inputs_written_right_before_a_call_are_the_ones_it_uses(name, T, pair_limit):
-    # A router kernel brings rows of its input into L2 while earlier kernels of the stream still run: calls queued back to
-    # back, with the hidden states written in between, must see what was written last.
+    # Calls queued back to back, with the hidden states written in between, must see what was written last.  (These copies do
+    # not let the call behind them start early; test_gpu_early_start.py has a writer that does.)
     wl = I.WORKLOADS[name]
     layers = [I.make_layer(wl, l, 0, T=T) for l in range(2)]
     ctx = P.make_context(wl, T)

@@ -35,6 +35,13 @@ struct MapEntry {
 constexpr int kMapCache = 8;
 constexpr size_t kLine = 32;            // words that blocks count on lie in lines of their own
 
+// What a small kernel's launch asks of the SMs that its blocks go to: so much dynamic shared memory, and, where that is
+// not zero, an execution priority.
+struct SmShare {
+  int smem = 0, priority = 0;
+};
+constexpr SmShare kAnyShare;
+
 }  // namespace
 
 struct fb_ctx {
@@ -60,7 +67,7 @@ struct fb_ctx {
   int pair_limit = 0;             // the caller's limit on the block pairs to use (0 = none)
   int stage_limit = 0;            // diagnostic: pipeline stages at most (0 = as many as fit)
   int n_sm = 148;                 // SMs of the device
-  int plan_smem = 0;              // dynamic shared memory of the planner kernel behind a router kernel (see launch_plan)
+  SmShare own_sm;                 // for the planner kernel behind a router kernel (see launch_plan)
   int split_mode = 1;             // k-range split over the blocks of a cluster: 0 off, 1 on
   EncodeTiledFn encode = nullptr;
   // device scratch (one allocation from counts_scratch on but for slice_counts).  A prediction call may run beside a routing
@@ -250,18 +257,20 @@ static RouterKernelFn rows_kernel_fn(int log_cpl, bool sigmoid) {
 // Launch of a small kernel that may start under the end of the stream's previous kernel (it waits for
 // that kernel's completion - griddepcontrol.wait - before it touches global memory).
 template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(Params...), int blocks, int threads, int smem, cudaStream_t stream, Args... args) {
+cudaError_t launch_dependent(void (*kernel)(Params...), int blocks, int threads, const SmShare& share, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
   cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
-  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg.dynamicSmemBytes = static_cast<size_t>(share.smem);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePriority;
+  attr[1].val.priority = share.priority;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = share.smem > 0 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -271,8 +280,8 @@ bool launch_refused(fb_ctx* ctx) {
   return ctx->fail_launch > 0 && --ctx->fail_launch == 0;
 }
 template <typename... Params, typename... Args>
-cudaError_t launch_counted(fb_ctx* ctx, void (*kernel)(Params...), int blocks, int threads, int smem, cudaStream_t stream, Args... args) {
-  return launch_refused(ctx) ? cudaErrorUnknown : launch_dependent(kernel, blocks, threads, smem, stream, args...);
+cudaError_t launch_counted(fb_ctx* ctx, void (*kernel)(Params...), int blocks, int threads, const SmShare& share, cudaStream_t stream, Args... args) {
+  return launch_refused(ctx) ? cudaErrorUnknown : launch_dependent(kernel, blocks, threads, share, stream, args...);
 }
 
 // A kernel that should have read and cleared these of the context's words was not launched behind the router kernel that
@@ -282,14 +291,16 @@ void clear_unread(uint32_t* words, int sets, cudaStream_t stream) {
 }
 
 // counts_out: counts are the totals of a prediction pass (see fb_plan_kernel).
-// smem: behind a router kernel the block asks for all of an SM's shared memory.  It is launched while the router blocks run,
-// and the only SMs with room for it would be those that another stream's kernel (the attention the prediction runs beside)
-// keeps busy: its one deciding warp starved there.  This way it waits for the first SM that the router kernel leaves.
-// Prediction and plan beside a kernel that fills the other SMs with multiply-adds, with and without: 8192 x 128 on 32 pairs
-// 23.6 and 99 us, 2000 x 128 on 8 pairs 25.6 and 97, 2048 x 256 on 8 pairs 52 and 109.
-fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, uint32_t* counts, uint32_t* counts_out, int smem, cudaStream_t stream) {
+// share: behind a router kernel the block asks for an SM of its own (all of the shared memory), ahead of other kernels' blocks
+// (the highest priority).  It is launched while the router blocks run, and beside another stream's kernel - the attention that
+// the prediction is meant to run beside - the only SMs with room for it would be the busy ones of that kernel, where its one
+// deciding warp starved; without the priority the SM that the first router block leaves went to that kernel's waiting blocks.
+// Prediction and plan of 8192 x 128 beside a kernel of multiply-adds: on 32 pairs, the other SMs taken, 99 us without either
+// and 24 with; on all SMs, with the other kernel launched 2 us later, 109 without either, 611 with the SM alone, 23 with both.
+fb_status launch_plan(fb_ctx* ctx, const fb::PlanParams& pp, uint32_t* counts, uint32_t* counts_out, const SmShare& share,
+                      cudaStream_t stream) {
   const cudaError_t err = launch_counted(ctx, fb::plan_needs_general_loop(pp) ? fb::fb_plan_kernel<true> : fb::fb_plan_kernel<false>,
-                                         1, fb::kPlanThreads, smem, stream, pp, counts, counts_out, ctx->status);
+                                         1, fb::kPlanThreads, share, stream, pp, counts, counts_out, ctx->status);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
@@ -441,10 +452,10 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   if (several) ++ctx->persistent_launches;
   if (err != cudaSuccess) return FB_ERR_CUDA;
   if (pass_plan && p.defer_counts) {
-    st = launch_plan(ctx, *plan, p.counts_scratch, counts_out, ctx->plan_smem, stream);
+    st = launch_plan(ctx, *plan, p.counts_scratch, counts_out, ctx->own_sm, stream);
     if (st != FB_OK) clear_unread(p.counts_scratch, 1, stream);
   } else if (plan_wanted && !p.fuse_planner && !p.defer_counts) {
-    st = launch_plan(ctx, *plan, counts_out, nullptr, ctx->plan_smem, stream);
+    st = launch_plan(ctx, *plan, counts_out, nullptr, ctx->own_sm, stream);
     if (st != FB_OK && layer) clear_unread(ctx->totals, 1, stream);     // no dispatch index follows
   }
   return st;
@@ -485,7 +496,7 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   const cudaError_t err = launch_counted(ctx, blocks < dp.num_tiles ? fb::fb_dispatch_runs_kernel
                                               : plan != nullptr     ? fb::fb_dispatch_kernel<true>
                                                                     : fb::fb_dispatch_kernel<false>,
-                                         blocks, fb::kDispatchThreads, 0, stream, dp);
+                                         blocks, fb::kDispatchThreads, kAnyShare, stream, dp);
   if (err == cudaSuccess) return FB_OK;
   clear_unread(ctx->totals, plan != nullptr ? 2 : 1, stream);
   return FB_ERR_CUDA;
@@ -599,11 +610,11 @@ static fb_status setup_router_shape(fb_ctx* ctx, const DeviceLimits& dev) {
 //     is the same for all instances and shapes.
 static fb_status set_up_device(fb_ctx* ctx, int device, const DeviceLimits& dev) {
   static std::mutex mutex;
-  static struct { bool ready; int max_clusters[fb::kMaxPieces + 1]; int plan_smem; } known[64] = {};
+  static struct { bool ready; int max_clusters[fb::kMaxPieces + 1]; SmShare own_sm; } known[64] = {};
   std::lock_guard<std::mutex> lock(mutex);
   if (device >= 0 && device < 64 && known[device].ready) {
     memcpy(ctx->max_clusters, known[device].max_clusters, sizeof(ctx->max_clusters));
-    ctx->plan_smem = known[device].plan_smem;
+    ctx->own_sm = known[device].own_sm;
     return FB_OK;
   }
   bool ok = true;
@@ -628,7 +639,9 @@ static fb_status set_up_device(fb_ctx* ctx, int device, const DeviceLimits& dev)
   for (int i = 0; i < 2 * kRowsKernels; ++i) smem = raise_router(rows_kernel_fn(i / 2, i % 2 != 0));
   const int plan_general = raise(reinterpret_cast<const void*>(fb::fb_plan_kernel<true>));
   const int plan_uniform = raise(reinterpret_cast<const void*>(fb::fb_plan_kernel<false>));
-  ctx->plan_smem = plan_general < plan_uniform ? plan_general : plan_uniform;
+  ctx->own_sm.smem = plan_general < plan_uniform ? plan_general : plan_uniform;
+  int least = 0;
+  ok = ok && cudaDeviceGetStreamPriorityRange(&least, &ctx->own_sm.priority) == cudaSuccess;
   if (!ok) { cudaGetLastError(); return FB_ERR_CUDA; }
   cudaLaunchConfig_t occ;
   memset(&occ, 0, sizeof(occ));
@@ -649,7 +662,7 @@ static fb_status set_up_device(fb_ctx* ctx, int device, const DeviceLimits& dev)
   if (ctx->max_clusters[1] < 1) return FB_ERR_CUDA;
   if (device >= 0 && device < 64) {
     memcpy(known[device].max_clusters, ctx->max_clusters, sizeof(ctx->max_clusters));
-    known[device].plan_smem = ctx->plan_smem;
+    known[device].own_sm = ctx->own_sm;
     known[device].ready = true;
   }
   return FB_OK;
@@ -779,7 +792,7 @@ fb_status fb_plan_swaps(fb_ctx* ctx, const uint32_t* counts, const int32_t* expe
   if (st != FB_OK) return st;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
-  return launch_plan(ctx, pp, const_cast<uint32_t*>(counts), nullptr, 0, static_cast<cudaStream_t>(stream_));   // (read only)
+  return launch_plan(ctx, pp, const_cast<uint32_t*>(counts), nullptr, kAnyShare, static_cast<cudaStream_t>(stream_));   // (read only)
 }
 
 fb_status fb_predict_and_plan(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T,
@@ -800,7 +813,7 @@ fb_status fb_predict_and_plan(fb_ctx* ctx, const fb_router* router, const void* 
   if (!guard.ok) return FB_ERR_CUDA;
   if (T == 0) {
     if (cudaMemsetAsync(counts, 0, ctx->cfg.E * sizeof(uint32_t), stream) != cudaSuccess) return FB_ERR_CUDA;
-    return launch_plan(ctx, pp, counts, nullptr, 0, stream);
+    return launch_plan(ctx, pp, counts, nullptr, kAnyShare, stream);
   }
   return launch_router(ctx, router, x, T, fb::kModePredictPlan, counts, nullptr, nullptr, nullptr, &pp, stream);
 }
@@ -1122,16 +1135,16 @@ fb_status fb_row_cosine_mean(const void* a, const void* b, int64_t rows, int32_t
     const int64_t part = rows - r0 < kPart ? rows - r0 : kPart;
     const int blocks = static_cast<int>((part + fb::kCosineWarpsPerBlock - 1) / fb::kCosineWarpsPerBlock);
     if (dtype == FB_DTYPE_BF16)
-      err = launch_dependent(fb::fb_row_cosine_kernel<__nv_bfloat16>, blocks, 32 * fb::kCosineWarpsPerBlock, 0, stream,
+      err = launch_dependent(fb::fb_row_cosine_kernel<__nv_bfloat16>, blocks, 32 * fb::kCosineWarpsPerBlock, kAnyShare, stream,
                              static_cast<const __nv_bfloat16*>(a) + r0 * n, static_cast<const __nv_bfloat16*>(b) + r0 * n,
                              static_cast<long long>(part), n, row_scratch + r0);
     else
-      err = launch_dependent(fb::fb_row_cosine_kernel<float>, blocks, 32 * fb::kCosineWarpsPerBlock, 0, stream,
+      err = launch_dependent(fb::fb_row_cosine_kernel<float>, blocks, 32 * fb::kCosineWarpsPerBlock, kAnyShare, stream,
                              static_cast<const float*>(a) + r0 * n, static_cast<const float*>(b) + r0 * n,
                              static_cast<long long>(part), n, row_scratch + r0);
   }
   if (err == cudaSuccess)
-    err = launch_dependent(fb::fb_mean_kernel, 1, fb::kMeanThreads, 0, stream, row_scratch, static_cast<long long>(rows), mean_out);
+    err = launch_dependent(fb::fb_mean_kernel, 1, fb::kMeanThreads, kAnyShare, stream, row_scratch, static_cast<long long>(rows), mean_out);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
@@ -1139,7 +1152,7 @@ fb_status fb_topk_hits(const int32_t* ids_a, const int32_t* ids_b, int32_t T, in
                        fb_stream stream_) {
   if (T < 0 || k < 1 || k > FB_MAX_TOPK || !hits_out || (T > 0 && (!ids_a || !ids_b))) return FB_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-  return launch_dependent(fb::fb_topk_hits_kernel, fb::kHitsBlocks, fb::kHitsThreads, 0, stream, ids_a, ids_b, T, k, hits_out) ==
+  return launch_dependent(fb::fb_topk_hits_kernel, fb::kHitsBlocks, fb::kHitsThreads, kAnyShare, stream, ids_a, ids_b, T, k, hits_out) ==
                  cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
@@ -1162,8 +1175,8 @@ fb_status fb_prediction_quality(const void* h_prev, const void* H, const float* 
   cudaError_t err = cudaSuccess;
   if (T > 0)
     err = launch_dependent(fb::fb_quality_rows_kernel, (T - 1) / fb::kCosineWarpsPerBlock + 1,
-                           32 * fb::kCosineWarpsPerBlock, 0, stream, qp);
-  if (err == cudaSuccess) err = launch_dependent(fb::fb_quality_sums_kernel, fb::kQualityBlocks, fb::kMeanThreads, 0, stream, qp);
+                           32 * fb::kCosineWarpsPerBlock, kAnyShare, stream, qp);
+  if (err == cudaSuccess) err = launch_dependent(fb::fb_quality_sums_kernel, fb::kQualityBlocks, fb::kMeanThreads, kAnyShare, stream, qp);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
 
@@ -1235,7 +1248,7 @@ fb_status fb_dispatch_slot_counts(fb_ctx* ctx, const uint32_t* slot_offsets, uin
   if (!ctx || !slot_offsets || !slot_counts) return FB_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
   if (!guard.ok) return FB_ERR_CUDA;
-  const cudaError_t err = launch_counted(ctx, fb::fb_slot_counts_kernel, 1, FB_MAX_EXPERTS, 0, static_cast<cudaStream_t>(stream_),
+  const cudaError_t err = launch_counted(ctx, fb::fb_slot_counts_kernel, 1, FB_MAX_EXPERTS, kAnyShare, static_cast<cudaStream_t>(stream_),
                                          slot_offsets, ctx->cfg.E, slot_counts);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }
@@ -1262,7 +1275,7 @@ fb_status fb_dispatch_globalize(fb_ctx* ctx, int32_t T_local, int32_t world, int
   long long blocks = (n + fb::kGlobalizeThreads - 1) / fb::kGlobalizeThreads;
   if (blocks < 1) blocks = 1;
   if (blocks > 4 * ctx->n_sm) blocks = 4 * ctx->n_sm;
-  const cudaError_t err = launch_counted(ctx, fb::fb_dispatch_globalize_kernel, static_cast<int>(blocks), fb::kGlobalizeThreads, 0,
+  const cudaError_t err = launch_counted(ctx, fb::fb_dispatch_globalize_kernel, static_cast<int>(blocks), fb::kGlobalizeThreads, kAnyShare,
                                          static_cast<cudaStream_t>(stream_), gp);
   return err == cudaSuccess ? FB_OK : FB_ERR_CUDA;
 }

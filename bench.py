@@ -744,7 +744,7 @@ def main():
         if pp_b2b:
             pp_bytes, pp_flops = 2 * T * d + 2 * d * E + 4 * E, 2 * T * d * E
             roof_pp = roofline(statistics.median(pp_b2b), pp_bytes, pp_flops,
-                               "router kernel + planner tail (fb_predict_and_plan)")
+                               "router kernel, then the planner's (fb_predict_and_plan)")
             roof_pp["timing"] = f"{pp_n} launches back to back between two events, median of {len(pp_b2b)} repeats"
             roof_pp["spread"] = spread(pp_b2b)
             roof_pp["tokens_per_s"] = T / (statistics.median(pp_b2b) * 1e-3)

@@ -9,7 +9,7 @@
  *   2. fb_plan_swaps        rank loads under the placement pi (Alg. 1 line 2), cost
  *                           model (Eq. 9), budgets (Eq. 10), deterministic greedy
  *                           pairwise swaps under the load objective (Eqs. 6-8)
- *      fb_predict_and_plan  1 + 2 in a single kernel launch
+ *      fb_predict_and_plan  1 + 2 in one call
  *      fb_layer_step        1 + 2 + 4 for one layer: both router passes in one launch
  *   3. fb_apply_swaps       the accepted swaps applied to the expert weights (logical ranks
  *                           on one GPU: an exchange of slot images inside one buffer)
@@ -222,8 +222,9 @@ fb_status fb_plan_swaps(fb_ctx* ctx, const uint32_t* counts, const int32_t* expe
                         int32_t* expert_to_slot_out, fb_swap* swaps, int32_t* n_swaps,
                         uint32_t* load_before, uint32_t* load_after, fb_stream stream);
 
-/* Stages 1 + 2 in one call: the planner's kernel starts under the end of the prediction pass (calls with more tiles than
- * the GPU holds at once plan beside their last tiles instead, in one launch). */
+/* Stages 1 + 2 in one call of two launches: the planner's kernel takes the first SM that the prediction pass leaves.  Calls
+ * with more tiles than the GPU holds at once, or than fb_set_pair_limit allows, plan beside their last tiles instead, in one
+ * launch - unless the plan needs the general loop (expert_bytes_table, or a mode other than FB_PLAN_LOOP). */
 fb_status fb_predict_and_plan(fb_ctx* ctx, const fb_router* router, const void* x, int32_t T,
                               const int32_t* expert_to_slot, const fb_budget* budget,
                               int32_t layer_id, uint32_t* counts, int32_t* expert_to_slot_out,

@@ -78,14 +78,15 @@ fb_status fb_standin_attention(float* out, int32_t blocks, int32_t iters, fb_str
  * Errors: FB_ERR_INVALID_ARG for a NULL or non-device buffer or a size out of range. */
 fb_status fb_clock_probe(uint64_t* samples, int32_t n, uint32_t period_ns, fb_stream stream);
 
-/* Phase time stamps of the one-tile router kernel.  Only a library built with -DFB_TIMING
+/* Phase time stamps of the one-tile router kernels and of the dispatch index behind them.  Only a library built with -DFB_TIMING
  * carries the stamp code (paper_2608_14205_b200/phase_timing.py builds one beside the normal
  * library and prints the table); the normal build returns FB_ERR_UNSUPPORTED_SHAPE here and
  * its kernels contain none of it.  stamps: dev u64 [blocks][64], or NULL to stop stamping:
- * every block of every following router launch through ctx writes the global nanosecond
- * timer in slots 0..31 and the SM cycle counter in slots 32..63 at its phase boundaries
- * (the slot list is at the top of csrc/fb_router.cuh).  The buffer must hold 64 words per
- * block of the largest launch. */
+ * every block of every following launch of these kernels through ctx writes the global
+ * nanosecond timer in slots 0..31 and the SM cycle counter in slots 32..63 at its phase
+ * boundaries (the slot list is at the top of csrc/fb_dispatch.cuh).  The buffer must hold 64
+ * words per block of the largest launch, the dispatch index's among them (a block per 128
+ * tokens, as many as the GPU has SMs at most). */
 fb_status fb_set_stamp_buffer(fb_ctx* ctx, uint64_t* stamps);
 
 /* Self-test of the bounded wait that every kernel of the library uses for its barriers: a

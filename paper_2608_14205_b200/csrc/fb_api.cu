@@ -346,9 +346,8 @@ fb_status launch_router(fb_ctx* ctx, const fb_router* router, const void* x, int
   p.stamps = ctx->stamps;
   p.probe = probe;
   if (plan) p.plan = *plan;
-  // The fused tail serves the common plans; a plan that needs the general loop (per-expert sizes,
-  // a planner variant) gets the stand-alone planner kernel behind
-  // the router kernel instead.
+  // A launch of more tiles than the GPU holds at once plans itself (fuse_planner); a plan that needs the general loop (per-expert sizes, a
+  // planner variant) gets the planner kernel behind the router kernel instead.
   const bool plan_wanted = plan != nullptr && (mode == fb::kModePredictPlan || mode == fb::kModeLayer);
   p.fuse_planner = (plan_wanted && !fb::plan_needs_general_loop(*plan)) ? 1 : 0;
   const int tiles = (T + fb::kTileM - 1) / fb::kTileM;
@@ -490,8 +489,8 @@ fb_status launch_dispatch_index(fb_ctx* ctx, int32_t T, int slices_per_tile, con
   dp.rank_load = rank_load;
   dp.status = ctx->status;
   dp.stamps = ctx->stamps;
-  // one block per SM at most: more tiles than that are walked in runs (every block reads the whole
-  // histogram table once, so more blocks would only read it more often)
+  // one block per SM at most: more tiles than that are walked in runs (every block reads up to half of the
+  // histogram table, so more blocks would only read it more often)
   const int blocks = dp.num_tiles < ctx->n_sm ? dp.num_tiles : ctx->n_sm;
   const cudaError_t err = launch_counted(ctx, blocks < dp.num_tiles ? fb::fb_dispatch_runs_kernel
                                               : plan != nullptr     ? fb::fb_dispatch_kernel<true>

@@ -12,17 +12,14 @@
 //
 // What bounds it: latency, not bandwidth (16 T k bytes of output are 2 MB at 16k tokens).  So
 // everything a block needs from global memory is requested at once, before anything depends on it
-// (placement, first tile's ids, the whole histogram table 16 experts per load), and the launch may
-// overlap the end of the router kernel (programmatic dependent launch).
+// (placement, totals, first tile's ids, its part of the histogram table four experts per load), and the launch may
+// overlap the end of the router kernel (programmatic dependent launch; layer calls back to back without and with it: 512
+// tokens, 8 experts 12.4 and 9.7 us, 1000 x 128 16.5 and 14.1, 8192 x 128 22.7 and 20.3, 131072 x 128 no difference).
 // The next kernel of the stream may set itself up, and a router kernel bring rows into L2 (prefetch_operands), while a
 // kernel of this file or the planner kernel runs - but not before its wait is over: allowed earlier, a whole chain of small kernels
 // starts during the main loop of the router kernel before them, and the next router kernel takes SMs and bandwidth
 // from it (layer calls back to back, allowed before and after the wait: 1733 tokens, 256 experts 31.6 and 30.7 us, 1000 x 128
 // 19.8 and 18.9; a shard's six launches 58.0 and 56.6).
-// Measured on whole layer steps back to back (B200), against 32-bit tables read column by column
-// behind a serialised launch: 1733 tokens, 256 experts 48.5 -> 44.4 us; 8192 tokens, 128 experts
-// 37.9 -> 36.2 us; 131072 tokens, 128 experts 256.5 -> 252.4 us.  Without the dependent launch the
-// first two are 1.6 us slower; two blocks per SM of half the length are 5 us slower (each reads the table).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -65,7 +62,7 @@ constexpr int kDispatchWarps = kDispatchThreads / 32;
 __host__ __device__ constexpr int slice_rows(int pieces) { return (kDispatchTile + 2 * pieces - 1) / (2 * pieces) * 2; }
 constexpr int kDispatchBatch = 4;        // tiles a block works on at a time
 static_assert(kDispatchTile * FB_MAX_TOPK == kDispatchThreads, "one thread per assignment of a tile");
-// Bytes of one row of the histogram table: 16-byte units, so that a thread reads 16 experts at once.
+// Bytes of one row of the histogram table: 16-byte units (a lane reads four experts at once, see add_rows).
 __host__ __device__ constexpr int slice_row_bytes(int E) { return (E + 15) & ~15; }
 
 struct DispatchParams {
@@ -198,10 +195,9 @@ __device__ __forceinline__ void clear_totals(const DispatchParams& p, uint32_t t
 // One tile per block (at most as many tiles as SMs).  The work per expert does not depend on the
 // placement; the slots come in with one scan at the end.
 // kPlan: the swap planner runs in here as well, in every block (its decisions are integer and reproducible,
-// so no block waits for another; block 0 writes the outputs).  Used where a layer launch runs both passes at
-// the same time: electing the last block of the early pass and planning in
-// it were 3 to 5 us at the end of the router kernel with every other SM idle.  Layer steps: 512 tokens x 8 experts 15.3 ->
-// 13.6 us, 40 x 128 20.1 -> 19.3, 1733 x 256 36.0 -> 35.2, 8192 x 128 32.0 -> 31.5.
+// so no block waits for another; block 0 writes counts and plan, block 1 - or block 0 alone - the placement).  Used where a
+// layer launch runs both passes at the same time: electing the last block of the early pass and planning in
+// it were 3 to 5 us at the end of the router kernel with every other SM idle.
 // The first warp plans as soon as totals and placement have arrived; the others add up the table and find every
 // assignment's place among its tile's meanwhile.  Against totals out of the tables of both passes, with the planner behind
 // them: 8192 x 128 24.2 -> 23.0 us, 1733 x 256 29.1 -> 28.1, 1000 x 128 17.6 -> 16.7, 40 x 128 15.1 -> 14.7.

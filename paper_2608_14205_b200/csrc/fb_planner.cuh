@@ -1,7 +1,7 @@
 // Budgeted greedy expert-swap planner (Algorithm 1 lines 2-8, Eqs. 6-9), decided by one
-// warp: of the stand-alone planner kernel, of the router block that finished last, of the
-// persistent router kernel's last pair (a warp that is idle there), or of every block of the
-// dispatch-index kernel (layer calls with one tile per SM).  Integer arithmetic only, so
+// warp: of the planner kernel (alone or behind a prediction pass), of every block of the dispatch-index kernel
+// (layer calls with one tile per SM), or, with more tiles than the GPU holds at once, of the persistent router kernel's last
+// pair (a warp that is idle there) or of the other router kernels' last block.  Integer arithmetic only, so
 // every block and every rank that replays it on the same count vector gets the same plan.
 #pragma once
 #include <cuda_runtime.h>
@@ -534,10 +534,9 @@ __device__ __noinline__ void plan_loop_general(const PlanParams& p, PlanShared& 
 // placement arrays and plan_put_count has turned the count vector into counts per slot.  A single
 // warp keeps the rank loads in registers (lane r holds ranks r and r + 32) and needs no block barrier.  Writes the swaps, their number and the rank loads
 // before and after; the new placement is written afterwards by plan_write_placement.
-// kGeneral: the instance carries the general loop as well.  The router kernels' fused tail uses
-// the instance without it (the host launches the stand-alone planner kernel behind the router
-// kernel when a plan needs the general loop - see plan_needs_general_loop): the general loop's
-// registers and code would otherwise weigh on every router kernel.
+// kGeneral: the instance carries the general loop as well.  Only a planner kernel's does (the host launches it behind
+// the router kernel when a plan needs the general loop - see plan_needs_general_loop): the general loop's registers
+// and code would otherwise weigh on every other kernel that plans.
 // write: whether this warp's results go to global memory (several blocks may replay a plan, see the
 // dispatch index); only for instances without the general loop.
 // In line: its parameters come out of constant memory that way (see plan_loop_uniform).
@@ -607,9 +606,10 @@ __device__ __forceinline__ void plan_swaps_warp(const PlanParams& p, PlanShared&
   }
 }
 
-// The same as a function of its own, for the router kernels, where most calls do not reach it: with the planner's code in the
-// kernel a layer call of 8192 tokens took 23.0 us and takes 22.8 without, of 131072 tokens 219 and 217; prediction and
-// plan of 300 tokens, which reaches it, 13.8 and 13.9.
+// The same as a function of its own, for the router kernels: only launches of more tiles than the GPU holds at once plan there.
+// In line and apart, calls that do not reach it: layer 40 tokens, 128 experts 13.1 and 12.9 us, 512 x 8 9.9 and 9.7, 8192 x 128
+// 20.2 and 20.3; that do: layer 131072 x 128 182.0 and 180.9 (spread 1.5), prediction and plan 24000 x 256 93.6 and 94.1
+// (spread 1), 20000 x 128 33.5 and 34.7.
 __device__ __noinline__ void plan_swaps_apart(const PlanParams& p, PlanShared& sh, int lane, int* status,
                                               unsigned long long* stamps) {
   plan_swaps_warp<false>(p, sh, lane, status, true, stamps);

@@ -547,8 +547,9 @@ struct TileWalk {
 // While a block waits for the stream's earlier kernels (blocks start as soon as SMs are free) its second issuer warp brings
 // the first of its rows of x into L2.  Nothing is read early: L2 is where this GPU's writes meet its reads, so a line
 // that an earlier kernel still writes is written there and read after the wait.  Memory is idle meanwhile where the kernel
-// before is a dispatch index or a planner: layer calls back to back, 8192 tokens x 2048, 128 experts 28.4 -> 26.5 us,
-// 4096 x 4096, 8 experts 22.3 -> 20.0, prediction and plan of 8192 x 2048 21.2 -> 19.7.
+// before is a dispatch index or a planner: layer calls back to back without and with it, 8192 tokens x 2048, 128 experts 23.8
+// and 22.4 us, 4096 x 4096, 8 experts 20.1 and 18.7, prediction and plan of 8192 x 2048 17.1 and 16.2.  Behind a kernel that
+// does not let this one start early there is nothing to gain: 24.0 and 24.7, 21.2 and 21.2, 17.3 and 17.3.
 // After as many k-blocks as the ring holds, one every kPrefetchCycles - an SM's share of the memory bandwidth - so that the
 // loads that follow the wait never queue behind many of these; the limit on all blocks' together (prefetch_kb) keeps
 // what is brought in well inside the 126 MB of L2.

@@ -16,14 +16,14 @@ def _us_per_call(call, n=60, reps=9):
     times = []
     for _ in range(reps):
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        torch.cuda._sleep(400000)                       # the launches are queued before the first one starts
+        torch.cuda._sleep(1000000)                      # the launches are queued before the first one starts
         a.record()
         for _ in range(n):
             call()
         b.record()
         torch.cuda.synchronize()
         times.append(a.elapsed_time(b) / n * 1e3)
-    return sorted(times)[reps // 2]
+    return min(times)                                   # (a busy host only ever adds to it)
 
 
 # The same context and buffers for both, so that only the number of tokens differs: the second selection took 0.8 and 0.6 us of
